@@ -6,7 +6,6 @@
 #include <new>
 #include <string>
 
-#include "sg_df.cuh"
 #include "sg_internal.h"
 
 namespace {
@@ -22,17 +21,6 @@ sg_status fail(sg_ctx *ctx, sg_status st, const std::string &msg)
 sg_status cuda_fail(sg_ctx *ctx, cudaError_t e, const char *where)
 {
     return fail(ctx, SG_ECUDA, std::string(where) + ": " + cudaGetErrorString(e));
-}
-
-// FP64 values as double-float pairs (hi = fl32(d), lo = fl32(d - hi))
-std::vector<float2> df_pairs(const std::vector<double> &v)
-{
-    std::vector<float2> out(v.size());
-    for (size_t i = 0; i < v.size(); i++) {
-        const sg::df2 d(v[i]);
-        out[i] = make_float2(d.hi, d.lo);
-    }
-    return out;
 }
 
 template <typename T>
@@ -52,57 +40,80 @@ sg_status upload(sg_ctx *ctx, const std::vector<T> &v, const T **dst)
     return SG_OK;
 }
 
+void free_workspace(sg_ctx *ctx)
+{
+    if (ctx->acc) cudaFree(ctx->acc);
+    if (ctx->maxbits) cudaFree(ctx->maxbits);
+    if (ctx->xs) cudaFree(ctx->xs);
+    if (ctx->flags) cudaFree(ctx->flags);
+    ctx->acc = nullptr;
+    ctx->maxbits = nullptr;
+    ctx->xs = nullptr;
+    ctx->flags = nullptr;
+    ctx->acc_nvec = 0;
+}
+
 void free_all(sg_ctx *ctx)
 {
     for (void *p : ctx->allocations) cudaFree(p);
     ctx->allocations.clear();
+    sg::free_rows(ctx);
     if (ctx->stage_x) cudaFree(ctx->stage_x);
     if (ctx->stage_y) cudaFree(ctx->stage_y);
     ctx->stage_x = ctx->stage_y = nullptr;
-    if (ctx->acc) cudaFree(ctx->acc);
-    if (ctx->maxbits) cudaFree(ctx->maxbits);
-    if (ctx->xs) cudaFree(ctx->xs);
-    ctx->acc = nullptr;
-    ctx->maxbits = nullptr;
-    ctx->xs = nullptr;
-    ctx->acc_nvec = 0;
+    free_workspace(ctx);
 }
 
-// Apply workspace for nvec vectors: fixed-point accumulators (zeroed here and
-// left zeroed by every apply), the per-vector max|x| words and, for the fast
-// path, the entry-major input copy.
+// Apply workspace for nvec vectors.  Row form: per-vector flags (zero between
+// applies) and the entry-major input copy.  Term-by-term kernel: fixed-point
+// accumulators (zeroed here and left zeroed by every apply) and the
+// per-vector max|x| words.
 sg_status ensure_workspace(sg_ctx *ctx, int nvec, cudaStream_t s)
 {
     if (nvec <= ctx->acc_nvec) return SG_OK;
     cudaError_t e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "stream synchronize");
-    if (ctx->acc) cudaFree(ctx->acc);
-    if (ctx->maxbits) cudaFree(ctx->maxbits);
-    if (ctx->xs) cudaFree(ctx->xs);
-    ctx->acc = nullptr;
-    ctx->maxbits = nullptr;
-    ctx->xs = nullptr;
-    ctx->kp.xs = nullptr;
-    ctx->kp.xs_nvec = 0;
-    ctx->acc_nvec = 0;
-    const size_t words = (size_t)ctx->host.n_cs * nvec * sg::acc_words(ctx->fp32);
-    if ((e = cudaMalloc(&ctx->acc, words * sizeof(unsigned long long))) != cudaSuccess ||
-        (e = cudaMalloc(&ctx->maxbits, sizeof(long long) * nvec)) != cudaSuccess)
-        return fail(ctx, SG_ENOMEM, std::string("workspace cudaMalloc: ") + cudaGetErrorString(e));
-#if SG_STAGE_X
-    if (ctx->kp.fast.enabled) {
-        const size_t xs_bytes = (size_t)ctx->host.n_cs * sg::xs_stride(nvec) * (ctx->fp32 ? 4 : 8);
-        if ((e = cudaMalloc(&ctx->xs, xs_bytes)) != cudaSuccess)
+    free_workspace(ctx);
+    if (ctx->host.rows) {
+        const size_t xs_bytes = (size_t)ctx->host.n_cs * sg::xs_stride(nvec) * sg::row_value_bytes(ctx->prob.prec);
+        if ((e = cudaMalloc(&ctx->flags, sizeof(unsigned) * nvec)) != cudaSuccess ||
+            (e = cudaMalloc(&ctx->xs, xs_bytes)) != cudaSuccess)
             return fail(ctx, SG_ENOMEM, std::string("workspace cudaMalloc: ") + cudaGetErrorString(e));
-        ctx->kp.xs = ctx->xs;
-        ctx->kp.xs_nvec = nvec;
+        if ((e = cudaMemsetAsync(ctx->flags, 0, sizeof(unsigned) * nvec, s)) != cudaSuccess)
+            return cuda_fail(ctx, e, "workspace memset");
+    } else {
+        const size_t words = (size_t)ctx->host.n_cs * nvec * sg::acc_words(ctx->fp32);
+        if ((e = cudaMalloc(&ctx->acc, words * sizeof(unsigned long long))) != cudaSuccess ||
+            (e = cudaMalloc(&ctx->maxbits, sizeof(long long) * nvec)) != cudaSuccess)
+            return fail(ctx, SG_ENOMEM, std::string("workspace cudaMalloc: ") + cudaGetErrorString(e));
+        if ((e = cudaMemsetAsync(ctx->acc, 0, words * sizeof(unsigned long long), s)) != cudaSuccess)
+            return cuda_fail(ctx, e, "workspace memset");
+        ctx->kp.acc = ctx->acc;
     }
-#endif
-    if ((e = cudaMemsetAsync(ctx->acc, 0, words * sizeof(unsigned long long), s)) != cudaSuccess)
-        return cuda_fail(ctx, e, "workspace memset");
     ctx->acc_nvec = nvec;
-    ctx->kp.acc = ctx->acc;
     return SG_OK;
+}
+
+sg::RowIO row_io(const sg_ctx *ctx, const double *x, double *y, int nvec)
+{
+    sg::RowIO io{};
+    io.x = x;
+    io.xs = ctx->xs;
+    io.y = y;
+    io.flags = ctx->flags;
+    io.nvec = nvec;
+    io.stride = sg::xs_stride(nvec);
+    io.words = sg::acc_words(ctx->fp32);
+    io.part = 0;
+    io.nparts = 1;
+    return io;
+}
+
+// The launches of one apply (workspace ready).
+cudaError_t enqueue_apply(sg_ctx *ctx, const double *x, double *y, int nvec, cudaStream_t s)
+{
+    if (!ctx->host.rows) return sg::launch_apply(ctx->kp, ctx->fp32, x, y, nvec, ctx->maxbits, s);
+    return sg::apply_rows(ctx, row_io(ctx, x, y, nvec), s);
 }
 
 // Device shared-memory opt-in limit of sm_100-class GPUs, used to size plans
@@ -180,6 +191,114 @@ sg_status plan(int D, int L, const sg_basis *basis, const sg_grid *grids,
 
 namespace sg {
 
+// Input copies small enough to stay in the caches are not made: the row
+// kernel then gathers from x itself.
+constexpr int64_t kDirectElems = 65536;
+
+cudaError_t apply_rows(sg_ctx *ctx, RowIO io, cudaStream_t s)
+{
+    const sg_precision prec = ctx->prob.prec;
+    cudaError_t e = cudaSuccess;
+    if (prec == SG_FP64 && io.nvec == 1) io.xs = io.x;  // x is its own entry-major copy
+    else if (!io.xs || ctx->host.n_cs * (int64_t)io.nvec <= kDirectElems) io.xs = nullptr;
+    else e = launch_row_stage(ctx->rop, io, prec, s);
+    if (e == cudaSuccess) e = launch_rows(ctx->rop, io, prec, row_vt(ctx->host, prec), s);
+    if (e == cudaSuccess && io.y) e = launch_row_settle(io, ctx->rop.n, s);
+    return e;
+}
+
+void free_rows(sg_ctx *ctx)
+{
+    for (void *p : ctx->row_allocs) cudaFree(p);
+    ctx->row_allocs.clear();
+    ctx->bytes_device -= ctx->row_bytes;
+    ctx->row_bytes = 0;
+    ctx->rop = RowOp{};
+}
+
+namespace {
+
+template <typename T>
+cudaError_t row_upload(std::vector<void *> &own, const T *src, size_t n, T **dst, int64_t *bytes)
+{
+    *dst = nullptr;
+    const size_t b = std::max<size_t>(1, n) * sizeof(T);
+    cudaError_t e = cudaMalloc(reinterpret_cast<void **>(dst), b);
+    if (e != cudaSuccess) return e;
+    own.push_back(*dst);
+    if (bytes) *bytes += (int64_t)b;
+    return src && n ? cudaMemcpy(*dst, src, n * sizeof(T), cudaMemcpyHostToDevice) : cudaSuccess;
+}
+
+}  // namespace
+
+cudaError_t build_rows(sg_ctx *ctx)
+{
+    free_rows(ctx);
+    const HostTables &T = ctx->host;
+    const KParams &kp = ctx->kp;
+    const sg_precision prec = ctx->prob.prec;
+    const size_t n = (size_t)T.n_cs;
+    std::vector<void *> tmp;  // set-up tables, released below
+    RowShifts S{};
+    S.nshift = (int)T.sh_off.size() - 1;
+    int *cnt = nullptr;
+    long long *start = nullptr;
+    cudaError_t e = cudaSuccess;
+    auto ints = [&](const std::vector<int> &v, const int **dst) {
+        int *p = nullptr;
+        if (e == cudaSuccess) e = row_upload(tmp, v.data(), v.size(), &p, nullptr);
+        *dst = p;
+    };
+    ints(T.sh_off, &S.off); ints(T.sh_mode, &S.mode); ints(T.sh_d, &S.d);
+    ints(T.sh_src_off, &S.src_off); ints(T.sh_src, &S.src);
+    ints(T.pr_off, &S.prod_off); ints(T.pr_mode, &S.fmode); ints(T.pr_op, &S.fop);
+    double *coef = nullptr;
+    if (e == cudaSuccess) e = row_upload(tmp, T.pr_coef.data(), T.pr_coef.size(), &coef, nullptr);
+    S.coef = coef;
+    if (e == cudaSuccess) e = row_upload<int>(tmp, nullptr, n, &cnt, nullptr);
+    if (e == cudaSuccess) e = row_upload<long long>(tmp, nullptr, n, &start, nullptr);
+    if (e == cudaSuccess) e = launch_row_count(kp, S, cnt, 0);
+    std::vector<int> hc(n);
+    if (e == cudaSuccess) e = cudaMemcpy(hc.data(), cnt, n * sizeof(int), cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) {
+        const int rb = row_value_bytes(prec);
+        const RowWindows W = cut_rows(hc, row_window_rows((int64_t)n, row_window_units(T)), row_budget(T, prec), rb);
+        RowOp R{};
+        RowWin *wins = nullptr;
+        uint2 *meta = nullptr;
+        int *cols = nullptr;
+        unsigned char *vals = nullptr;
+        int64_t bytes = 0;
+        e = row_upload(ctx->row_allocs, W.wins.data(), W.wins.size(), &wins, &bytes);
+        if (e == cudaSuccess) e = row_upload(ctx->row_allocs, W.meta.data(), W.meta.size(), &meta, &bytes);
+        if (e == cudaSuccess) e = row_upload<int>(ctx->row_allocs, nullptr, (size_t)W.entries, &cols, &bytes);
+        if (e == cudaSuccess)
+            e = row_upload<unsigned char>(ctx->row_allocs, nullptr, (size_t)W.entries * rb, &vals, &bytes);
+        if (e == cudaSuccess) e = cudaMemcpy(start, W.start.data(), n * sizeof(long long), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = launch_row_fill(kp, S, prec, start, cols, vals, 0);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(0);
+        R.cols = cols; R.vals = vals; R.wins = wins; R.meta = meta;
+        R.esplit = kp.esplit;
+        R.err = kp.err;
+        R.nwin = (int)W.wins.size();
+        R.n = (int)n;
+        R.cap = W.cap;
+        R.wrows = W.wrows;
+        ctx->rop = R;
+        ctx->win_entries.resize(W.wins.size());
+        for (size_t w = 0; w < W.wins.size(); w++) ctx->win_entries[w] = W.wins[w].nent;
+        ctx->row_bytes = bytes;
+        ctx->bytes_device += bytes;
+    }
+    for (void *p : tmp) cudaFree(p);
+    if (e != cudaSuccess) {
+        free_rows(ctx);
+        (void)cudaGetLastError();  // reported here; not by a later launch
+    }
+    return e;
+}
+
 int64_t planned_device_bytes(const sg_ctx *ctx)
 {
     const HostTables &T = ctx->host;
@@ -188,12 +307,7 @@ int64_t planned_device_bytes(const sg_ctx *ctx)
     int64_t bytes = b(T.levels) + b(T.coefs) + b(T.order) + b(T.rank_tab) + b(T.lmin_tab) + b(T.lvl) +
                     b(T.tabd) * 3 / 2 + b(p.mcoef) + b(p.mnfac) + b(p.mfoff) + b(p.mfmode) + b(p.mfpow) +
                     b(T.harm_mono) + b(T.esplit);
-    if (T.fast)
-        bytes += b(T.pair_modes) + b(T.h1off) + b(T.goff) + b(T.ioff) + b(T.soff) + b(T.spoff) + b(T.fsc) +
-                 b(T.ftab) * 3 / 2 + b(T.fdesc) + b(T.fdesc_off) + T.franks * (int64_t)sizeof(int) +
-                 b(T.fimg) / (ctx->fp32 ? 2 : 1) + b(T.fimg_off) + b(T.fvt_off) + b(T.frank_start) +
-                 (T.fvt_off.empty() ? 0 : T.fvt_off.back()) * (ctx->fp32 ? 4 : 8);
-    return bytes;
+    return bytes + std::max(term_form(p, T).bytes, row_form_bytes(T, p.prec));
 }
 
 }  // namespace sg
@@ -225,7 +339,6 @@ sg_status sg_create(int D, int L, const sg_basis *basis, const sg_grid *grids,
     HostTables &T = ctx->host;
     KParams &kp = ctx->kp;
     std::vector<float> tabf(T.tabd.begin(), T.tabd.end());
-    std::vector<float> ftabf(T.ftab.begin(), T.ftab.end());
     std::vector<int> zero(1, 0);
     sg_status st = SG_OK;
     const int *errp = nullptr;
@@ -244,25 +357,7 @@ sg_status sg_create(int D, int L, const sg_basis *basis, const sg_grid *grids,
         (st = upload(ctx, p.mfpow, &kp.mfpow)) != SG_OK ||
         (st = upload(ctx, T.harm_mono, &kp.harm_mono)) != SG_OK ||
         (st = upload(ctx, T.esplit, &kp.esplit)) != SG_OK ||
-        (st = upload(ctx, zero, &errp)) != SG_OK ||
-        (T.fast && ((st = upload(ctx, T.pair_modes, &kp.fast.pair_modes)) != SG_OK ||
-                    (st = upload(ctx, T.h1off, &kp.fast.h1off)) != SG_OK ||
-                    (st = upload(ctx, T.goff, &kp.fast.goff)) != SG_OK ||
-                    (st = upload(ctx, T.ioff, &kp.fast.ioff)) != SG_OK ||
-                    (st = upload(ctx, T.soff, &kp.fast.soff)) != SG_OK ||
-                    (st = upload(ctx, T.spoff, &kp.fast.spoff)) != SG_OK ||
-                    (st = upload(ctx, T.fsc, &kp.fast.sc)) != SG_OK ||
-                    (st = upload(ctx, T.ftab, &kp.fast.tabd)) != SG_OK ||
-                    (st = upload(ctx, ftabf, &kp.fast.tabf)) != SG_OK ||
-                    (st = upload(ctx, T.fdesc, &kp.fast.desc)) != SG_OK ||
-                    (st = upload(ctx, T.fdesc_off, &kp.fast.desc_off)) != SG_OK ||
-                    (st = upload(ctx, T.fimg_off, &kp.fast.img_off)) != SG_OK ||
-                    (st = upload(ctx, T.fvt_off, &kp.fast.mt_off)) != SG_OK ||
-                    (st = upload(ctx, T.frank_start, &kp.fast.rank_start)) != SG_OK ||
-                    (ctx->fp32 ? (st = upload(ctx, std::vector<float>(T.fimg.begin(), T.fimg.end()),
-                                              &kp.fast.imgf)) != SG_OK
-                     : p.prec == SG_DF64 ? (st = upload(ctx, df_pairs(T.fimg), &kp.fast.imgx)) != SG_OK
-                                         : (st = upload(ctx, T.fimg, &kp.fast.imgd)) != SG_OK)))) {
+        (st = upload(ctx, zero, &errp)) != SG_OK) {
         g_create_error = ctx->last_error;
         free_all(ctx);
         delete ctx;
@@ -270,69 +365,28 @@ sg_status sg_create(int D, int L, const sg_basis *basis, const sg_grid *grids,
     }
     kp.err = const_cast<int *>(errp);
     ctx->has_device = true;
-    if (p.prec == SG_DF64 && !T.fast) {
+    if (p.prec == SG_DF64 && (!T.rows || !term_form(p, T).fits)) {
         st = fail(nullptr, SG_EUNSUPPORTED,
-                  "SG_DF64 needs the fast path (a potential with one- and two-mode monomials of a chain)");
+                  "SG_DF64 needs the pair form (a potential with one- and two-mode monomials of a chain)");
         free_all(ctx);
         delete ctx;
         return st;
     }
-    if (T.fast) {
-        kp.fast.enabled = 1;
-        kp.fast.df = p.prec == SG_DF64;
-        kp.fast.nb1 = T.nb1;
-        kp.fast.nq1 = T.nq1;
-        kp.fast.npairs = (int)T.pair_modes.size() / 2;
-        kp.fast.c0const = T.c0const;
-        kp.fast.desccap = T.fdesccap;
-        kp.fast.gcap = T.fgcap;
-        kp.fast.nbocap = T.fnbocap;
-        kp.fast.n_big = T.fn_big;
-        kp.fast.work_cta = T.fwork_cta;
-        kp.fast.work_warp = T.fwork_warp;
-        kp.matcap = T.matcap;
-        kp.cap = T.fast_cap;
-        // M^B in the fast kernel's layout order, built on the device
-        void *rp = nullptr;
-        e = cudaMalloc(&rp, std::max<size_t>(1, (size_t)T.franks) * sizeof(int));
-        if (e != cudaSuccess) {
-            st = fail(nullptr, SG_ENOMEM, std::string("cudaMalloc (index maps): ") + cudaGetErrorString(e));
+    if (T.rows) {
+        e = build_rows(ctx);
+        if (e == cudaErrorMemoryAllocation) {
+            st = fail(nullptr, SG_ENOMEM, std::string("cudaMalloc (row operator): ") + cudaGetErrorString(e));
             free_all(ctx);
             delete ctx;
             return st;
         }
-        ctx->allocations.push_back(rp);
-        ctx->bytes_device += (int64_t)T.franks * (int64_t)sizeof(int);
-        kp.fast.ranks = static_cast<const int *>(rp);
-        // the inner-block tables of every term with a grid, in the context's precision
-        void *vp = nullptr;
-        const size_t nvt = std::max<size_t>(1, (size_t)T.fvt_off.back());
-        // 16 bytes of padding: the term kernel prefetches 16-byte rounded ranges
-        e = cudaMalloc(&vp, nvt * (ctx->fp32 ? sizeof(float) : sizeof(double)) + 16);
-        if (e != cudaSuccess) {
-            st = fail(nullptr, SG_ENOMEM, std::string("cudaMalloc (inner-block tables): ") + cudaGetErrorString(e));
-            free_all(ctx);
-            delete ctx;
-            return st;
-        }
-        ctx->allocations.push_back(vp);
-        ctx->bytes_device += (int64_t)nvt * (ctx->fp32 ? 4 : 8);
-        if (ctx->fp32) kp.fast.mtabf = static_cast<const float *>(vp);
-        else if (kp.fast.df) kp.fast.mtabx = static_cast<const float2 *>(vp);
-        else kp.fast.mtabd = static_cast<const double *>(vp);
-        e = launch_build_ranks(kp, static_cast<int *>(rp), 0);
-        if (e == cudaSuccess) e = launch_build_mtab(kp, ctx->fp32, 0);
-        if (e == cudaSuccess) e = cudaDeviceSynchronize();
-        if (e == cudaSuccess) {
-            ctx->smem_bytes = fast_smem_bytes(kp, ctx->fp32);
-            e = configure_fast_kernels(kp, ctx->fp32);
-        }
+        if (e == cudaSuccess) e = configure_rows();
     } else {
         ctx->smem_bytes = apply_smem_bytes(kp, ctx->fp32);
         e = configure_kernels(ctx->smem_bytes, ctx->fp32);
     }
     if (e != cudaSuccess) {
-        st = cuda_fail(nullptr, e, "cudaFuncSetAttribute");
+        st = cuda_fail(nullptr, e, "context set-up");
         free_all(ctx);
         delete ctx;
         return st;
@@ -366,8 +420,7 @@ sg_status sg_apply_H(sg_ctx *ctx, const double *x, double *y, int nvec, void *st
     if ((x < y + n) && (y < x + n)) return fail(ctx, SG_EINVAL, "x and y overlap");
     sg_status st = ensure_workspace(ctx, nvec, (cudaStream_t)stream);
     if (st != SG_OK) return st;
-    cudaError_t e = sg::launch_apply(ctx->kp, ctx->fp32, x, y, nvec, ctx->maxbits, nullptr,
-                                     (cudaStream_t)stream);
+    cudaError_t e = enqueue_apply(ctx, x, y, nvec, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "apply launch");
     return SG_OK;
 }
@@ -380,8 +433,17 @@ sg_status sg_apply_H_part(sg_ctx *ctx, const double *x, int nvec, int part, int 
     if (!x || !acc) return fail(ctx, SG_EINVAL, "x or acc is NULL");
     if (nvec < 1) return fail(ctx, SG_EINVAL, "nvec must be >= 1");
     if (nparts < 1 || part < 0 || part >= nparts) return fail(ctx, SG_EINVAL, "need 0 <= part < nparts");
-    sg_status st = ensure_workspace(ctx, nvec, (cudaStream_t)stream);  // the per-vector exponents
+    sg_status st = ensure_workspace(ctx, nvec, (cudaStream_t)stream);
     if (st != SG_OK) return st;
+    if (ctx->host.rows) {
+        sg::RowIO io = row_io(ctx, x, nullptr, nvec);
+        io.acc = reinterpret_cast<unsigned long long *>(acc);
+        io.part = part;
+        io.nparts = nparts;
+        const cudaError_t er = sg::apply_rows(ctx, io, (cudaStream_t)stream);
+        if (er != cudaSuccess) return cuda_fail(ctx, er, "partial apply launch");
+        return SG_OK;
+    }
     sg::KParams kp = ctx->kp;
     kp.acc = reinterpret_cast<unsigned long long *>(acc);
     kp.part = part;
@@ -403,6 +465,14 @@ sg_status sg_apply_H_finish(sg_ctx *ctx, const double *x, int64_t *acc, double *
     if ((x < y + n) && (y < x + n)) return fail(ctx, SG_EINVAL, "x and y overlap");
     sg_status st = ensure_workspace(ctx, nvec, (cudaStream_t)stream);
     if (st != SG_OK) return st;
+    if (ctx->host.rows) {
+        sg::RowIO io = row_io(ctx, x, y, nvec);
+        io.acc = reinterpret_cast<unsigned long long *>(acc);
+        cudaError_t er = sg::launch_row_finish(ctx->rop, io, (cudaStream_t)stream);
+        if (er == cudaSuccess) er = sg::launch_row_settle(io, ctx->rop.n, (cudaStream_t)stream);
+        if (er != cudaSuccess) return cuda_fail(ctx, er, "finish launch");
+        return SG_OK;
+    }
     sg::KParams kp = ctx->kp;
     kp.acc = reinterpret_cast<unsigned long long *>(acc);
     cudaError_t e = sg::launch_maxabs(kp, x, nvec, ctx->maxbits, (cudaStream_t)stream);
@@ -449,8 +519,7 @@ sg_status sg_apply_H_host(sg_ctx *ctx, const double *x_host, double *y_host, int
         return cuda_fail(ctx, e, "H2D copy");
     sg_status st = ensure_workspace(ctx, nvec, s);
     if (st != SG_OK) return st;
-    if ((e = sg::launch_apply(ctx->kp, ctx->fp32, ctx->stage_x, ctx->stage_y, nvec, ctx->maxbits,
-                              nullptr, s)) != cudaSuccess)
+    if ((e = enqueue_apply(ctx, ctx->stage_x, ctx->stage_y, nvec, s)) != cudaSuccess)
         return cuda_fail(ctx, e, "apply launch");
     if ((e = cudaMemcpyAsync(y_host, ctx->stage_y, n * sizeof(double), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
         return cuda_fail(ctx, e, "D2H copy");

@@ -1,4 +1,6 @@
-// Smolyak operator action on the GPU (sm_103a).
+// Term-by-term Smolyak operator action on the GPU (sm_103a), for the problems
+// whose row form (sg_rows.cu) is not built: levels above kRowMaxL, or more
+// index shifts or entries than it holds.
 //
 // One thread block per Smolyak term (terms ordered most-expensive first).  For
 // term l the block performs Alg. 1 of arXiv 2111.13655:
@@ -398,47 +400,6 @@ __global__ void k_maxabs(const double *__restrict__ x, int n, long long *__restr
     if ((threadIdx.x & 31) == 0 && mb) atomicMax(maxbits + v, mb);
 }
 
-// Entry-major copy of the input vectors in the contraction type (rows of
-// `stride` elements, a multiple of 4): thread r reads x_v[r] for every vector
-// (coalesced across threads per vector) and writes the first xs_stride(nvec)
-// values of its row (zero beyond nvec) as 16-byte stores.
-template <typename T>
-__device__ __forceinline__ void stage_rows(const double *__restrict__ x, long long n, int nvec, int stride,
-                                           T *__restrict__ xs, long long r0, long long rstep)
-{
-    constexpr int U = 16 / (int)sizeof(T);
-    struct alignas(16) Unit { T v[U]; };
-    const int w = xs_stride(nvec);
-    for (long long r = r0; r < n; r += rstep) {
-        T *row = xs + (size_t)r * stride;
-        for (int v0 = 0; v0 < w; v0 += U) {
-            Unit t;
-#pragma unroll
-            for (int e = 0; e < U; e++) t.v[e] = v0 + e < nvec ? (T)x[(size_t)(v0 + e) * n + r] : T(0);
-            *reinterpret_cast<Unit *>(row + v0) = t;
-        }
-    }
-}
-
-template <typename T>
-__global__ void k_stage_x(const double *__restrict__ x, int n, int nvec, int stride, T *__restrict__ xs)
-{
-    stage_rows<T>(x, n, nvec, stride, xs, blockIdx.x * (long long)blockDim.x + threadIdx.x,
-                  (long long)gridDim.x * blockDim.x);
-}
-
-// Many problems (blockIdx.z = problem j, its vectors from nvec * cs_prefix[j],
-// its rows from cs_prefix[j]).
-template <typename T>
-__global__ void k_stage_x_batch(const double *__restrict__ x, const long long *__restrict__ cs_prefix, int nvec,
-                                int stride, T *__restrict__ xs)
-{
-    const int j = blockIdx.z;
-    const long long c0 = cs_prefix[j], n = cs_prefix[j + 1] - c0;
-    stage_rows<T>(x + (size_t)nvec * c0, n, nvec, stride, xs + (size_t)c0 * stride,
-                  blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
-}
-
 // The accumulated integer of one entry times 2^E (E from the vector's max|x|
 // bits; NaN when x held a non-finite value); clears the accumulator words.
 // FP32 contexts: one signed word; FP64: four signed 32-bit digits.
@@ -474,49 +435,6 @@ __global__ void k_finalize(const KParams P, const double *__restrict__ x, double
         const int v = (int)(i / P.n_cs);
         const size_t r = i - (size_t)v * P.n_cs;
         y[i] = finalize_value(P.acc + (r * nvec + v) * acc_words(fp32), maxbits[v], fp32) + P.esplit[r] * x[i];
-    }
-}
-
-// Many problems (vectors problem after problem, problem j from nvec * cs_prefix[j]):
-// per-vector max|x| bits into maxbits[j * nvec + v]; blockIdx.z = problem.
-__global__ void k_maxabs_batch(const double *__restrict__ x, const long long *__restrict__ cs_prefix, int nvec,
-                               long long *__restrict__ maxbits)
-{
-    const int j = blockIdx.z, v = blockIdx.y;
-    const long long c0 = cs_prefix[j];
-    const long long n = cs_prefix[j + 1] - c0;
-    const double *xv = x + (size_t)nvec * c0 + (size_t)v * n;
-    long long mb = 0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const long long b = __double_as_longlong(xv[i]) & 0x7FFFFFFFFFFFFFFFll;
-        mb = b > mb ? b : mb;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        const long long other = __shfl_xor_sync(0xffffffffu, mb, o);
-        mb = other > mb ? other : mb;
-    }
-    if ((threadIdx.x & 31) == 0 && mb) atomicMax(maxbits + (size_t)j * nvec + v, mb);
-}
-
-// Many problems: y = (accumulated integer) * 2^E + esplit_j * x, entry by entry;
-// blockIdx.y = problem (its entries start at nvec * cs_prefix[j]); clears the
-// accumulators.
-__global__ void k_finalize_batch(const KParams *__restrict__ kps, const long long *__restrict__ cs_prefix,
-                                 const double *__restrict__ x, double *__restrict__ y,
-                                 unsigned long long *acc, const long long *__restrict__ maxbits, int nvec,
-                                 int fp32)
-{
-    const int j = blockIdx.y;
-    const size_t base = (size_t)nvec * (size_t)cs_prefix[j];
-    const size_t n = (size_t)(cs_prefix[j + 1] - cs_prefix[j]);
-    const size_t total = (size_t)nvec * n;
-    const double *esplit = kps[j].esplit;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int v = (int)(i / n);
-        const size_t r = i - (size_t)v * n;
-        const size_t a = base + r * nvec + v;  // entry-major in its problem
-        y[base + i] = finalize_value(acc + a * acc_words(fp32), maxbits[(size_t)j * nvec + v], fp32) +
-                      esplit[r] * x[base + i];
     }
 }
 
@@ -578,9 +496,8 @@ cudaError_t configure_kernels(size_t smem, bool fp32)
 }
 
 cudaError_t launch_apply(const KParams &kp, bool fp32, const double *x, double *y, int nvec,
-                         long long *maxbits, int *lsb_exp, cudaStream_t stream)
+                         long long *maxbits, cudaStream_t stream)
 {
-    (void)lsb_exp;
     cudaError_t e = launch_maxabs(kp, x, nvec, maxbits, stream);
     if (e == cudaSuccess) e = launch_apply_terms(kp, fp32, x, maxbits, nvec, stream);
     if (e == cudaSuccess) e = launch_finalize(kp, fp32, x, y, nvec, maxbits, stream);
@@ -592,33 +509,6 @@ cudaError_t launch_maxabs(const KParams &kp, const double *x, int nvec, long lon
     cudaError_t e = cudaMemsetAsync(maxbits, 0, sizeof(long long) * nvec, stream);
     if (e != cudaSuccess) return e;
     k_maxabs<<<dim3(64, nvec), 256, 0, stream>>>(x, kp.n_cs, maxbits);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_stage_x(const KParams &kp, bool fp32, const double *x, int nvec, cudaStream_t stream)
-{
-    if (!kp.xs || nvec > kp.xs_nvec) return cudaErrorInvalidValue;
-    const int stride = xs_stride(kp.xs_nvec);
-    const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((kp.n_cs + 255) / 256, 152 * 16));
-    void *xs = const_cast<void *>(kp.xs);
-    if (fp32) k_stage_x<float><<<blocks, 256, 0, stream>>>(x, kp.n_cs, nvec, stride, static_cast<float *>(xs));
-    else if (kp.fast.df) k_stage_x<df2><<<blocks, 256, 0, stream>>>(x, kp.n_cs, nvec, stride, static_cast<df2 *>(xs));
-    else k_stage_x<double><<<blocks, 256, 0, stream>>>(x, kp.n_cs, nvec, stride, static_cast<double *>(xs));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_stage_x_batch(bool fp32, const double *x, const long long *cs_prefix, int nprob, int64_t max_ncs,
-                                 int nvec, int xs_nvec, void *xs, cudaStream_t stream)
-{
-    if (!xs || nvec > xs_nvec) return cudaErrorInvalidValue;
-    const int stride = xs_stride(xs_nvec);
-    const unsigned bx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(64, (max_ncs + 255) / 256));
-    if (fp32)
-        k_stage_x_batch<float><<<dim3(bx, 1, nprob), 256, 0, stream>>>(x, cs_prefix, nvec, stride,
-                                                                       static_cast<float *>(xs));
-    else
-        k_stage_x_batch<double><<<dim3(bx, 1, nprob), 256, 0, stream>>>(x, cs_prefix, nvec, stride,
-                                                                        static_cast<double *>(xs));
     return cudaGetLastError();
 }
 
@@ -634,15 +524,6 @@ cudaError_t launch_finalize(const KParams &kp, bool fp32, const double *x, doubl
 cudaError_t launch_apply_terms(const KParams &kp, bool fp32, const double *x, const long long *maxbits, int nvec,
                                cudaStream_t stream)
 {
-    if (kp.fast.enabled) {
-        if (kp.xs && nvec <= kp.xs_nvec) {
-            cudaError_t e = launch_stage_x(kp, fp32, x, nvec, stream);
-            return e == cudaSuccess ? launch_apply_fast(kp, fp32, x, nvec, maxbits, stream) : e;
-        }
-        KParams k2 = kp;  // no staged copy of this size: the term kernels read x
-        k2.xs = nullptr;
-        return launch_apply_fast(k2, fp32, x, nvec, maxbits, stream);
-    }
     if (kp.n_terms <= kp.part) return cudaSuccess;
     const size_t smem = apply_smem_bytes(kp, fp32);
     dim3 grid((unsigned)((kp.n_terms - kp.part + kp.nparts - 1) / kp.nparts));
@@ -650,30 +531,6 @@ cudaError_t launch_apply_terms(const KParams &kp, bool fp32, const double *x, co
         k_apply<float><<<grid, kThreads, smem, stream>>>(kp, x, maxbits, nvec);
     else
         k_apply<double><<<grid, kThreads, smem, stream>>>(kp, x, maxbits, nvec);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_maxabs_batch(const double *x, const long long *cs_prefix, int nprob, int64_t max_ncs, int nvec,
-                                long long *maxbits, cudaStream_t stream)
-{
-    cudaError_t e = cudaMemsetAsync(maxbits, 0, sizeof(long long) * (size_t)nprob * nvec, stream);
-    if (e != cudaSuccess) return e;
-    const unsigned bx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(64, (max_ncs + 255) / 256));
-    k_maxabs_batch<<<dim3(bx, nvec, nprob), 256, 0, stream>>>(x, cs_prefix, nvec, maxbits);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_finalize_batch(const KParams *kps, const long long *cs_prefix, int nprob, int64_t max_ncs,
-                                  const double *x, double *y, unsigned long long *acc, const long long *maxbits,
-                                  int nvec, bool fp32, cudaStream_t stream)
-{
-    // blocks per problem: enough for the largest problem, within about 16 blocks per SM in all
-    // (at least 64 per problem)
-    const size_t per = (size_t)nvec * (size_t)max_ncs;
-    const size_t cap = std::max<size_t>(64, (152 * 16 + (size_t)nprob - 1) / (size_t)std::max(1, nprob));
-    const unsigned bx = (unsigned)std::max<size_t>(1, std::min<size_t>((per + 255) / 256, cap));
-    k_finalize_batch<<<dim3(bx, (unsigned)nprob), 256, 0, stream>>>(kps, cs_prefix, x, y, acc, maxbits, nvec,
-                                                                    fp32 ? 1 : 0);
     return cudaGetLastError();
 }
 

@@ -8,12 +8,14 @@
 // GPU up front, so a fresh cudaMalloc would fail or fragment it), and a
 // latency-critical loop that cannot take the implicit device-wide
 // synchronisation a cudaMalloc/cudaFree may cause.  sg_apply_H allocates its
-// fixed-point accumulators on the first call with a larger nvec; this entry
+// workspace on the first call with a larger nvec; this entry
 // point never allocates.
 //
-// The scratch holds, per call, the per-vector scale exponents (kNoAllocMaxVec
-// words) followed by the fixed-point accumulators of the compact vectors
-// (sg::acc_words words per element: four for FP64 contexts, one for mixed).  It is one array shared by every call on a
+// The scratch holds, per call, the per-vector flags and the entry-major input
+// copy of the row kernels, or, for a problem applied term by term, the
+// per-vector scale exponents (kNoAllocMaxVec words) followed by the fixed-point
+// accumulators of the compact vectors (sg::acc_words words per element: four
+// for FP64 contexts, one for mixed).  It is one array shared by every call on a
 // device, and keeps whatever the last call left in it: each call clears the
 // part it uses before its kernels run.  Two calls whose GPU work overlaps
 // (different streams, host threads or contexts on the same device) use the
@@ -34,6 +36,10 @@ constexpr size_t kNoAllocAccWords = kNoAllocWords - kNoAllocMaxVec;
 static_assert(SG_NOALLOC_SCRATCH_BYTES % 256 == 0, "scratch size must keep 256-byte alignment");
 static_assert(kNoAllocAccWords / sg::acc_words(false) == SG_NOALLOC_MAX_ELEMS, "header limit out of date");
 static_assert(kNoAllocAccWords / sg::acc_words(true) == SG_NOALLOC_MAX_ELEMS_MIXED, "header limit out of date");
+// the widest input copy of the row kernels at these limits: rows of xs_stride(nvec) <= 8/5 nvec elements
+static_assert((size_t)SG_NOALLOC_MAX_ELEMS_MIXED * 8 / 5 * 4 <= kNoAllocAccWords * 8 &&
+                  (size_t)SG_NOALLOC_MAX_ELEMS * 8 / 5 * 8 <= kNoAllocAccWords * 8,
+              "scratch too small for the input copy");
 
 static __device__ __align__(256) unsigned long long g_noalloc_scratch[kNoAllocWords];
 
@@ -94,6 +100,23 @@ extern "C" sg_status sg_apply_H_noalloc(sg_ctx *ctx, const double *x, double *y,
     }
 
     cudaStream_t s = (cudaStream_t)stream;
+    if (ctx->host.rows) {
+        // per-vector flags, then the entry-major input copy: rows of at most
+        // 8/5 (nvec = 5) elements per element, within the scratch at the limits above
+        e = cudaMemsetAsync(scratch, 0, kNoAllocMaxVec * sizeof(unsigned long long), s);
+        if (e != cudaSuccess) return noalloc_fail(ctx, SG_ECUDA, std::string("memset: ") + cudaGetErrorString(e));
+        sg::RowIO io{};
+        io.x = x;
+        io.y = y;
+        io.xs = scratch + kNoAllocMaxVec;
+        io.flags = reinterpret_cast<unsigned *>(scratch);
+        io.nvec = nvec;
+        io.stride = sg::xs_stride(nvec);
+        io.nparts = 1;
+        e = sg::apply_rows(ctx, io, s);
+        if (e != cudaSuccess) return noalloc_fail(ctx, SG_ECUDA, std::string("apply launch: ") + cudaGetErrorString(e));
+        return SG_OK;
+    }
     long long *maxbits = reinterpret_cast<long long *>(scratch);
     unsigned long long *acc = scratch + kNoAllocMaxVec;
     // The accumulators are summed into and must start at zero; the exponents
@@ -103,8 +126,7 @@ extern "C" sg_status sg_apply_H_noalloc(sg_ctx *ctx, const double *x, double *y,
 
     sg::KParams kp = ctx->kp;
     kp.acc = acc;
-    kp.xs = nullptr;  // no staged input copy: the term kernels read x
-    e = sg::launch_apply(kp, ctx->fp32, x, y, nvec, maxbits, nullptr, s);
+    e = sg::launch_apply(kp, ctx->fp32, x, y, nvec, maxbits, s);
     if (e != cudaSuccess) return noalloc_fail(ctx, SG_ECUDA, std::string("apply launch: ") + cudaGetErrorString(e));
     return SG_OK;
 }

@@ -1,28 +1,18 @@
-// Many Smolyak problems per apply (declared in include/smolyak.h): the terms
-// of all problems of one kernel variant go to the device in one launch per
-// form (block / warp), ordered by estimated cost over all problems, so a
-// batch of small and large problems keeps every SM busy until the end.
+// Many Smolyak problems per apply (declared in include/smolyak.h): the row
+// windows of all problems go to the device in one launch, so a batch of small
+// and large problems keeps every SM busy until the end.
 #include <algorithm>
-#include <map>
 #include <new>
 #include <string>
-#include <tuple>
 #include <vector>
 
 #include "sg_internal.h"
 
-// Order of the batched work items: 0 = by term cost over all problems,
-// 1 = problem-major (problems by total cost, then their terms by cost).
-#ifndef SG_BATCH_ORDER
-#define SG_BATCH_ORDER 0
-#endif
-// A fast-path problem with at least this many block-form terms fills the GPU
-// for several waves by itself: it runs as its own launches (parameters in the
-// kernel's parameter bank, as in sg_apply_H) inside the batch's sequence, and
-// only the smaller problems share the packed launches.
-#ifndef SG_BATCH_SOLO_TERMS
-#define SG_BATCH_SOLO_TERMS 16384
-#endif
+// A problem with at least this many rows fills the GPU for several waves by
+// itself: it runs as its own launches (parameters in the kernel's parameter
+// bank, windows of its own plan) inside the batch's sequence, and only the
+// smaller problems share the packed launches.
+constexpr int64_t kSoloRows = 131072;
 
 struct sg_batch {
     std::vector<sg_ctx *> ctxs;
@@ -30,21 +20,21 @@ struct sg_batch {
     int device = 0;
     bool fp32 = false;
     std::vector<long long> cs_prefix;  // host copy
-    int64_t n_terms = 0, max_ncs = 0;
+    int64_t n_terms = 0;
     const long long *d_cs_prefix = nullptr;
-    const sg::KParams *d_kps = nullptr;
-    struct Group {
-        sg::KParams kp_any;
-        sg::FastBatchGroup g;
-    };
-    std::vector<Group> groups;
-    std::vector<int> generic;          // problems outside the fast path: one launch each
-    std::vector<int> solo;             // large fast-path problems: their own launches
+    const sg::RowOp *d_ops = nullptr;  // one per problem
+    const int2 *items = nullptr;       // (problem, window) of the packed problems, most entries first
+    const int2 *stage_items = nullptr; // (problem, chunk of 256 rows) of the packed problems
+    int n_items = 0, n_stage = 0, cap = 4, wrows = 16;
+    std::vector<int> packed, solo;     // row-form problems: shared launches, launches of their own
+    std::vector<int> generic;          // problems applied term by term
     std::vector<void *> allocations;
-    std::vector<sg::KParams> h_kps;    // host copy of d_kps (the input-copy pointers change with the workspace)
+    // workspace: input copies and flags of the row-form problems, accumulators
+    // and exponents of the others (all from the start of the problem's vectors)
+    void *xs = nullptr;
+    unsigned *flags = nullptr;
     unsigned long long *acc = nullptr;
     long long *maxbits = nullptr;
-    void *xs = nullptr;                // entry-major input copies of the fast-path problems
     int acc_nvec = 0;
     // the apply's launch sequence captured as a graph, for the last (x, y, nvec, stream)
     cudaGraphExec_t graph = nullptr;
@@ -88,17 +78,25 @@ void drop_graph(sg_batch *b)
     b->gstream = nullptr;
 }
 
+void free_workspace(sg_batch *b)
+{
+    if (b->acc) cudaFree(b->acc);
+    if (b->maxbits) cudaFree(b->maxbits);
+    if (b->xs) cudaFree(b->xs);
+    if (b->flags) cudaFree(b->flags);
+    b->acc = nullptr;
+    b->maxbits = nullptr;
+    b->xs = nullptr;
+    b->flags = nullptr;
+    b->acc_nvec = 0;
+}
+
 void free_all(sg_batch *b)
 {
     drop_graph(b);
     for (void *p : b->allocations) cudaFree(p);
     b->allocations.clear();
-    if (b->acc) cudaFree(b->acc);
-    if (b->maxbits) cudaFree(b->maxbits);
-    if (b->xs) cudaFree(b->xs);
-    b->acc = nullptr;
-    b->maxbits = nullptr;
-    b->xs = nullptr;
+    free_workspace(b);
 }
 
 }  // namespace
@@ -113,7 +111,7 @@ extern "C" sg_status sg_batch_create(sg_ctx *const *ctxs, int n, sg_batch **out)
     for (int j = 0; j < n; j++) {
         sg_ctx *c = ctxs[j];
         if (!c || !c->has_device) { delete b; return SG_EINVAL; }
-        if (c->kp.fast.df) { delete b; return SG_EUNSUPPORTED; }  // double-float contexts are applied one by one
+        if (c->prob.prec == SG_DF64) { delete b; return SG_EUNSUPPORTED; }  // double-float contexts are applied one by one
         if (j > 0 && (c->device != b->device || c->fp32 != b->fp32)) { delete b; return SG_EINVAL; }
         b->device = c->device;
         b->fp32 = c->fp32;
@@ -124,71 +122,35 @@ extern "C" sg_status sg_batch_create(sg_ctx *const *ctxs, int n, sg_batch **out)
     if (cudaGetDevice(&cur) != cudaSuccess || cur != b->device) { delete b; return SG_EINVAL; }
 
     b->cs_prefix.assign(n + 1, 0);
-    std::vector<sg::KParams> kps(n);
+    std::vector<sg::RowOp> ops(n);
+    struct Item { int nent, j, w; };
+    std::vector<Item> it;
+    std::vector<int2> stage;
     for (int j = 0; j < n; j++) {
         const sg_ctx *c = ctxs[j];
         b->cs_prefix[j + 1] = b->cs_prefix[j] + c->host.n_cs;
-        b->max_ncs = std::max<int64_t>(b->max_ncs, c->host.n_cs);
         b->n_terms += c->host.n_terms;
-        kps[j] = c->kp;
-        kps[j].acc = nullptr;  // the batch kernels take the batch's accumulators explicitly
-        kps[j].xs = nullptr;   // set with the workspace (the batch's own input copies)
-        kps[j].xs_nvec = 0;
+        ops[j] = c->rop;
+        if (!c->host.rows) { b->generic.push_back(j); continue; }
+        if (c->host.n_cs >= kSoloRows) { b->solo.push_back(j); continue; }
+        b->packed.push_back(j);
+        b->cap = std::max(b->cap, c->rop.cap);
+        b->wrows = std::max(b->wrows, c->rop.wrows);
+        for (int w = 0; w < c->rop.nwin; w++) it.push_back({c->win_entries[w], j, w});
+        for (int q = 0; q * (int64_t)256 < c->host.n_cs; q++) stage.push_back(make_int2(j, q));
     }
-
-    // every fast-path problem (of the batch's one precision) shares the launches
-    std::map<int, std::vector<int>> by_variant;
-    for (int j = 0; j < n; j++) {
-        const sg::KParams &kp = ctxs[j]->kp;
-        if (!kp.fast.enabled) b->generic.push_back(j);
-        else if (kp.fast.n_big >= SG_BATCH_SOLO_TERMS) b->solo.push_back(j);
-        else by_variant[0].push_back(j);
-    }
+    if (it.size() > (size_t)0x7FFFFFFF) { delete b; return SG_EUNSUPPORTED; }
+    std::stable_sort(it.begin(), it.end(), [](const Item &a, const Item &c) { return a.nent > c.nent; });
+    std::vector<int2> items(it.size());
+    for (size_t q = 0; q < it.size(); q++) items[q] = make_int2(it[q].j, it[q].w);
+    b->n_items = (int)items.size();
+    b->n_stage = (int)stage.size();
     sg_status st;
-    b->h_kps = kps;
-    if ((st = bupload(b, kps, &b->d_kps)) != SG_OK || (st = bupload(b, b->cs_prefix, &b->d_cs_prefix)) != SG_OK) {
+    if ((st = bupload(b, ops, &b->d_ops)) != SG_OK || (st = bupload(b, b->cs_prefix, &b->d_cs_prefix)) != SG_OK ||
+        (st = bupload(b, items, &b->items)) != SG_OK || (st = bupload(b, stage, &b->stage_items)) != SG_OK) {
         free_all(b);
         delete b;
         return st;
-    }
-    for (auto &kv : by_variant) {
-        sg_batch::Group G{};
-        G.kp_any = ctxs[kv.second[0]]->kp;
-        G.kp_any.xs = nullptr;
-        G.g.kps = b->d_kps;
-        for (int f = 0; f < 2; f++) {
-            struct Item { int64_t cost; int j, p; };
-            std::vector<Item> it;
-            size_t part = 0;
-            for (int j : kv.second) {
-                const sg::HostTables &T = ctxs[j]->host;
-                const int nb = ctxs[j]->kp.fast.n_big;
-                const int64_t p0 = f == 0 ? 0 : nb, p1 = f == 0 ? nb : T.n_terms;
-                if (p1 > p0) part = std::max(part, sg::fast_part_bytes(ctxs[j]->kp, b->fp32, f == 1));
-                for (int64_t p = p0; p < p1; p++) it.push_back({T.pcost[p], j, (int)p});
-            }
-            if (SG_BATCH_ORDER == 0) {
-                std::stable_sort(it.begin(), it.end(), [](const Item &a, const Item &c) { return a.cost > c.cost; });
-            } else {
-                // problem-major: problems by decreasing total cost, each problem's
-                // terms by decreasing cost (a few problems in flight at a time)
-                std::map<int, int64_t> tot;
-                for (const Item &t : it) tot[t.j] += t.cost;
-                std::stable_sort(it.begin(), it.end(), [&](const Item &a, const Item &c) {
-                    if (a.j != c.j) return tot[a.j] != tot[c.j] ? tot[a.j] > tot[c.j] : a.j < c.j;
-                    return a.cost > c.cost;
-                });
-            }
-            std::vector<int2> items(it.size());
-            for (size_t q = 0; q < it.size(); q++) items[q] = make_int2(it[q].j, it[q].p);
-            if (it.size() > (size_t)0x7FFFFFFF) { free_all(b); delete b; return SG_EUNSUPPORTED; }
-            G.g.count[f] = (int)it.size();
-            G.g.part[f] = (int)part;
-            if ((st = bupload(b, items, &G.g.items[f])) != SG_OK) { free_all(b); delete b; return st; }
-        }
-        cudaError_t e = sg::configure_fast_batch(G.kp_any, b->fp32, G.g);
-        if (e != cudaSuccess) { free_all(b); delete b; return SG_ECUDA; }
-        b->groups.push_back(G);
     }
     *out = b;
     return SG_OK;
@@ -201,17 +163,8 @@ extern "C" sg_status sg_batch_size(const sg_batch *b, int64_t *n_cs_total, int64
     if (n_cs_total) *n_cs_total = b->cs_prefix.back();
     if (n_terms_total) *n_terms_total = b->n_terms;
     if (launches_per_apply) {
-        // max|x|, finalisation, the input copies
-        int l = 2 + (SG_STAGE_X && (!b->groups.empty() || !b->solo.empty()));
-        for (const auto &G : b->groups) l += (G.g.count[0] > 0) + (G.g.count[1] > 0);
-        for (int j : b->solo) {
-            const sg::KParams &kp = b->ctxs[j]->kp;
-            l += (kp.fast.n_big > 0) + (kp.n_terms > kp.fast.n_big);
-        }
-        for (int j : b->generic) {
-            const sg::KParams &kp = b->ctxs[j]->kp;
-            l += kp.n_terms > 0;
-        }
+        // row form: input copies, rows, settle; term by term: max|x|, terms, finalisation
+        const int l = (b->packed.empty() ? 0 : 3) + 3 * (int)(b->solo.size() + b->generic.size());
         *launches_per_apply = l;
     }
     return SG_OK;
@@ -239,35 +192,23 @@ extern "C" sg_status sg_apply_H_batch(sg_batch *b, const double *x, double *y, i
         drop_graph(b);  // it names the old workspace
         if ((e = cudaStreamSynchronize(s)) != cudaSuccess)
             return bfail(b, SG_ECUDA, std::string("stream synchronize: ") + cudaGetErrorString(e));
-        if (b->acc) cudaFree(b->acc);
-        if (b->maxbits) cudaFree(b->maxbits);
-        if (b->xs) cudaFree(b->xs);
-        b->acc = nullptr;
-        b->maxbits = nullptr;
-        b->xs = nullptr;
-        b->acc_nvec = 0;
-        const size_t words = total * sg::acc_words(b->fp32);
-        if ((e = cudaMalloc(&b->acc, words * sizeof(unsigned long long))) != cudaSuccess ||
-            (e = cudaMalloc(&b->maxbits, sizeof(long long) * (size_t)nprob * nvec)) != cudaSuccess)
-            return bfail(b, SG_ENOMEM, std::string("workspace cudaMalloc: ") + cudaGetErrorString(e));
-#if SG_STAGE_X
-        if (!b->groups.empty() || !b->solo.empty()) {
-            // the fast-path problems gather from entry-major copies, problem j's rows from cs_prefix[j]
-            const size_t rb = b->fp32 ? 4 : 8, stride = (size_t)sg::xs_stride(nvec);
-            if ((e = cudaMalloc(&b->xs, (size_t)b->cs_prefix.back() * stride * rb)) != cudaSuccess)
+        free_workspace(b);
+        if (!b->packed.empty() || !b->solo.empty()) {
+            const size_t rb = b->fp32 ? 4 : 8, nf = (size_t)nprob * nvec * sizeof(unsigned);
+            if ((e = cudaMalloc(&b->xs, (size_t)b->cs_prefix.back() * sg::xs_stride(nvec) * rb)) != cudaSuccess ||
+                (e = cudaMalloc(&b->flags, nf)) != cudaSuccess)
                 return bfail(b, SG_ENOMEM, std::string("workspace cudaMalloc: ") + cudaGetErrorString(e));
-            for (int j = 0; j < nprob; j++) {
-                if (!b->ctxs[j]->kp.fast.enabled) continue;
-                b->h_kps[j].xs = static_cast<unsigned char *>(b->xs) + (size_t)b->cs_prefix[j] * stride * rb;
-                b->h_kps[j].xs_nvec = nvec;
-            }
-            if ((e = cudaMemcpy(const_cast<sg::KParams *>(b->d_kps), b->h_kps.data(),
-                                sizeof(sg::KParams) * b->h_kps.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
-                return bfail(b, SG_ECUDA, std::string("parameter upload: ") + cudaGetErrorString(e));
+            if ((e = cudaMemsetAsync(b->flags, 0, nf, s)) != cudaSuccess)
+                return bfail(b, SG_ECUDA, std::string("workspace memset: ") + cudaGetErrorString(e));
         }
-#endif
-        if ((e = cudaMemsetAsync(b->acc, 0, words * sizeof(unsigned long long), s)) != cudaSuccess)
-            return bfail(b, SG_ECUDA, std::string("workspace memset: ") + cudaGetErrorString(e));
+        if (!b->generic.empty()) {
+            const size_t words = total * sg::acc_words(b->fp32);
+            if ((e = cudaMalloc(&b->acc, words * sizeof(unsigned long long))) != cudaSuccess ||
+                (e = cudaMalloc(&b->maxbits, sizeof(long long) * (size_t)nprob * nvec)) != cudaSuccess)
+                return bfail(b, SG_ENOMEM, std::string("workspace cudaMalloc: ") + cudaGetErrorString(e));
+            if ((e = cudaMemsetAsync(b->acc, 0, words * sizeof(unsigned long long), s)) != cudaSuccess)
+                return bfail(b, SG_ECUDA, std::string("workspace memset: ") + cudaGetErrorString(e));
+        }
         b->acc_nvec = nvec;
     }
     // Replay the captured launch sequence when the same buffers, block size and
@@ -300,40 +241,48 @@ extern "C" sg_status sg_apply_H_batch(sg_batch *b, const double *x, double *y, i
     return enqueue_apply(b, x, y, nvec, s);
 }
 
-// The launch sequence of one batched apply: max|x|, term kernels, finalisation.
+// The launch sequence of one batched apply.
 sg_status enqueue_apply(sg_batch *b, const double *x, double *y, int nvec, cudaStream_t s)
 {
-    const int nprob = (int)b->ctxs.size();
+    const sg_precision prec = b->fp32 ? SG_MIXED : SG_FP64;
+    const size_t rb = b->fp32 ? 4 : 8;
     cudaError_t e;
-    if ((e = sg::launch_maxabs_batch(x, b->d_cs_prefix, nprob, b->max_ncs, nvec, b->maxbits, s)) != cudaSuccess)
-        return bfail(b, SG_ECUDA, std::string("max|x| launch: ") + cudaGetErrorString(e));
-    if (b->xs && (e = sg::launch_stage_x_batch(b->fp32, x, b->d_cs_prefix, nprob, b->max_ncs, nvec, b->acc_nvec,
-                                               b->xs, s)) != cudaSuccess)
-        return bfail(b, SG_ECUDA, std::string("input copy launch: ") + cudaGetErrorString(e));
+    sg::RowIO io{};
+    io.x = x;
+    io.y = y;
+    io.xs = b->xs;
+    io.flags = b->flags;
+    io.nvec = nvec;
+    io.stride = sg::xs_stride(nvec);
+    io.nparts = 1;
     for (int j : b->solo) {
-        sg::KParams kp = b->h_kps[j];  // with the batch's input copy of problem j
-        const size_t off = (size_t)nvec * (size_t)b->cs_prefix[j];
-        kp.acc = b->acc + off * sg::acc_words(b->fp32);
-        if (!kp.xs || nvec > kp.xs_nvec) kp.xs = nullptr;
-        if ((e = sg::launch_apply_fast(kp, b->fp32, x + off, nvec, b->maxbits + (size_t)j * nvec, s)) != cudaSuccess)
-            return bfail(b, SG_ECUDA, std::string("term launch: ") + cudaGetErrorString(e));
+        const size_t c0 = (size_t)b->cs_prefix[j];
+        sg::RowIO o = io;
+        o.x += c0 * nvec;
+        o.y += c0 * nvec;
+        o.xs = static_cast<unsigned char *>(b->xs) + c0 * io.stride * rb;
+        o.flags += (size_t)j * nvec;
+        const sg_ctx *c = b->ctxs[j];
+        if ((e = sg::launch_row_stage(c->rop, o, prec, s)) != cudaSuccess ||
+            (e = sg::launch_rows(c->rop, o, prec, sg::row_vt(c->host, prec), s)) != cudaSuccess ||
+            (e = sg::launch_row_settle(o, c->rop.n, s)) != cudaSuccess)
+            return bfail(b, SG_ECUDA, std::string("row launch: ") + cudaGetErrorString(e));
     }
-    for (const auto &G : b->groups)
-        if ((e = sg::launch_fast_batch(G.kp_any, b->fp32, G.g, x, b->acc, b->maxbits, b->d_cs_prefix, nvec, s)) !=
-            cudaSuccess)
-            return bfail(b, SG_ECUDA, std::string("batched term launch: ") + cudaGetErrorString(e));
+    if (!b->packed.empty()) {
+        const int vt = b->fp32 ? SG_F32_VT : SG_F64_VT;
+        if ((e = sg::launch_row_stage_batch(io, prec, b->d_cs_prefix, b->stage_items, b->n_stage, s)) != cudaSuccess ||
+            (e = sg::launch_rows_batch(b->d_ops, b->items, b->n_items, b->cap, b->wrows, io, prec, vt, b->d_cs_prefix,
+                                       s)) != cudaSuccess ||
+            (e = sg::launch_row_settle_batch(io, b->d_cs_prefix, (int)b->ctxs.size(), s)) != cudaSuccess)
+            return bfail(b, SG_ECUDA, std::string("batched row launch: ") + cudaGetErrorString(e));
+    }
     for (int j : b->generic) {
         sg::KParams kp = b->ctxs[j]->kp;
         const size_t off = (size_t)nvec * (size_t)b->cs_prefix[j];
         kp.acc = b->acc + off * sg::acc_words(b->fp32);
-        kp.xs = nullptr;  // the context's own input copy is not the batch's
-        if ((e = sg::launch_apply_terms(kp, b->fp32, x + off, b->maxbits + (size_t)j * nvec, nvec, s)) !=
-            cudaSuccess)
+        if ((e = sg::launch_apply(kp, b->fp32, x + off, y + off, nvec, b->maxbits + (size_t)j * nvec, s)) != cudaSuccess)
             return bfail(b, SG_ECUDA, std::string("term launch: ") + cudaGetErrorString(e));
     }
-    if ((e = sg::launch_finalize_batch(b->d_kps, b->d_cs_prefix, nprob, b->max_ncs, x, y, b->acc,
-                                       b->maxbits, nvec, b->fp32, s)) != cudaSuccess)
-        return bfail(b, SG_ECUDA, std::string("finalise launch: ") + cudaGetErrorString(e));
     return SG_OK;
 }
 

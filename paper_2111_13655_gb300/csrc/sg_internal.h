@@ -40,157 +40,82 @@ constexpr int kAcc32LsbBelowMax = 40;
 // 64-bit words per accumulated entry of a context's precision
 __host__ __device__ constexpr int acc_words(bool fp32) { return fp32 ? 1 : kAccDigits; }
 
-constexpr int kMaxPairs = 64;  // coupled mode pairs handled by the fast path
+constexpr int kMaxPairs = 64;  // coupled mode pairs of the pair form (below)
 
-// Tuning of the fast kernels (FP32 / FP64): the shared-memory budget per
-// block that the host plans terms with, the resident blocks per SM the kernels
-// are compiled for, and the vectors per chunk below which a term is sliced.
+// ---------------------------------------------------------------------------
+// The row form of H_S (sg_rows.cu, sg_rows_setup.cpp).  With U_i(l) the
+// operator of mode i on level l and Delta_i(l) = U_i(l) - U_i(l-1), Eq. (16)'s
+// sum over the terms l in R(l) with the coefficients D_l of Eq. (8) is
+//     H_S = sum_{|l| <= L} (x)_i Delta_i(l_i)
+// for every product operator (x)_i U_i.  The potential is a sum of monomials,
+// and a mode that a monomial does not touch contributes B^T W B = I on its
+// nb(l) functions (nq >= nb), so Delta_i(l)[k] = 1 exactly for l = lmin_i(k).
+// A monomial over the modes S therefore couples k and k' (equal outside S) by
+//     c sum_{l_S: |l_S| <= T} prod_{i in S} Delta M_i(l_i)[k_i][k'_i],
+//     T = L - sum_{i not in S} lmin_i(k_i),
+// M_i(l) = B^T W diag(Q^p) B the quadrature matrix of the monomial's power on
+// level l (the kinetic part: K).  These elements, quadrature errors included,
+// are those of the term-by-term sum; M_i(l) is a power of the tridiagonal
+// Jacobi matrix of the grid, so a monomial of power p couples k_i to
+// k_i - p .. k_i + p only (every second one when q0 = 0), and few of these
+// shifts stay inside the compact basis: 15 per row at D=12 L=10.  The
+// elements are formed once per context in FP64 and stored row by row.
+
+// Rows of one window (consecutive compact indices) and their entries.
+struct RowWin {
+    long long ent0;  // first entry (a multiple of 4: 16-byte copies)
+    int row0, nrows;
+    int nent, pad;
+};
+// One problem's row operator on the device.
+struct RowOp {
+    const int *cols;        // compact index of each entry's column
+    const void *vals;       // its element (float, double or float2 = (hi, lo))
+    const RowWin *wins;
+    const uint2 *meta;      // per row, rows of a window by decreasing length: {start | local row << 24, length}
+    const double *esplit;   // harmonic diagonal (FP64)
+    int *err;
+    int nwin, n;
+    int cap;                // entries of a window staged at a time (the largest window, or the budget)
+    int wrows;              // rows per window (a power of two)
+};
+// What a row kernel reads and writes.
+struct RowIO {
+    const double *x;        // input vectors, column after column
+    const void *xs;         // entry-major copy in the contraction type (rows of `stride`), or nullptr: gather from x
+    double *y;              // result, or nullptr: the sums go to acc
+    unsigned long long *acc;
+    unsigned *flags;        // per vector: set when x holds a non-finite value
+    int nvec, stride, words;
+    int part, nparts;       // windows w with w % nparts == part
+};
+// Largest level and number of distinct index shifts the row form is built for.
+constexpr int kRowMaxL = 63;
+constexpr int kRowMaxShifts = 65536;
+// Largest row operator (bytes); larger ones use the term-by-term kernel.
+constexpr int64_t kRowMaxBytes = (int64_t)64 << 30;
+
+// Default plan of the row kernels (sg_tune measures the alternatives).
+#ifndef SG_F32_VT
+#define SG_F32_VT 4
+#endif
+#ifndef SG_F64_VT
+#define SG_F64_VT 2
+#endif
+#ifndef SG_ROW_WINDOW
+#define SG_ROW_WINDOW 2  // rows per window, in units of 64
+#endif
 #ifndef SG_F32_SMEM_KB
 #define SG_F32_SMEM_KB 52
-#endif
-#ifndef SG_F32_MINBLOCKS
-#define SG_F32_MINBLOCKS 4
-#endif
-// (defaults: the plan sg_tune picks at D=12 L=10 in both precisions; FP64
-// 165.6 -> 149.2 ms per 8-vector apply against a target of 4 vectors)
-#ifndef SG_F32_SLICE_VT
-#define SG_F32_SLICE_VT 1
-#endif
-#ifndef SG_F64_SLICE_VT
-#define SG_F64_SLICE_VT 1
-#endif
-// Warp form: terms that fit a quarter of the block's shared memory with a
-// chunk of SG_WARP_VT vectors (sliced when SG_WARP_SLICE is 1) run one per warp.
-// Measured at D=12 L=10 (mixed): 1 vector 31.29 ms per 8-vector apply, 4
-// vectors 31.85, 2 vectors 30.9 (sg_tune's pick there); slicing in the warp
-// form 43-60 ms.  1 is kept: the 256-wavepacket batch (nb = nq = l+1) is 12%
-// slower with 2.
-#ifndef SG_WARP_VT
-#define SG_WARP_VT 1
-#endif
-#ifndef SG_WARP_SLICE
-#define SG_WARP_SLICE 0
 #endif
 #ifndef SG_F64_SMEM_KB
 #define SG_F64_SMEM_KB 70
 #endif
-#ifndef SG_F64_MINBLOCKS
-#define SG_F64_MINBLOCKS 3
-#endif
 
-// Inner positions of the fast kernel: up to fast_rmax level-1 modes whose
-// action at each outer grid point is tabulated per term (inner-block table,
-// NBI = nb1^R <= 9 values per inner block).  Level 1 must have the same basis
-// size nb1 in every mode (2 or 3); otherwise no position is inner.
-inline int fast_inner_nb(int nb1) { return nb1 == 2 || nb1 == 3 ? nb1 : 1; }
-inline int fast_rmax(int nb1) { return nb1 == 2 ? 3 : nb1 == 3 ? 2 : 0; }
-
-// Sizes shared by the host planner and the fast kernels.
-// Padding of a buffer of n elements to a multiple of u elements (16 bytes).
-__host__ __device__ inline int64_t pad_elems(int64_t n, int u) { return (n + u - 1) / u * u; }
-#ifndef SG_STAGE_X
-#define SG_STAGE_X 1  // the fast path gathers from an entry-major copy of x
-#endif
 // Row length (elements) of the entry-major input copy for nvec vectors.
-__host__ __device__ inline int xs_stride(int nvec) { return (nvec + 3) & ~3; }
-// Elements (of a type with u per 16 bytes) that hold a term's NB int32
-// compact indices, padded to 16 bytes.
-__host__ __device__ inline int64_t ranks_elems(int64_t NB, int u) { return pad_elems((NB * u + 3) / 4, u); }
-// Work-area elements a chunk of vb vectors of one term needs: the term's
-// compact indices, the gathered basis tensor X (and the slice accumulator Y
-// when the term is sliced), and two buffers of the largest grid stage when the
-// term has a grid (a term without a grid has a second basis-sized buffer
-// instead, for the staged compress-add); every buffer padded to 16 bytes (u
-// elements).
-__host__ __device__ inline int64_t chunk_need(int64_t NB, int64_t stage, bool sliced, bool grid, int vb, int u)
-{
-    return ranks_elems(NB, u) + (sliced || !grid ? 2 : 1) * pad_elems(NB * vb, u) +
-           (grid ? 2 * pad_elems(stage * vb, u) : 0);
-}
-// Byte offset, inside a work area of `work_bytes`, of the scratch copy of a
-// term record (at most desccap 16-byte units) taken during the prologue: the
-// end of the area, 16-byte aligned.  The term's compact indices, copied at the
-// same time, occupy the start; the planner keeps the two apart.
-__host__ __device__ inline int64_t record_scratch_offset(int64_t work_bytes, int desccap)
-{
-    return ((work_bytes - 16 * (int64_t)desccap) / 16) * 16;
-}
-// Inner-block table per outer grid point: the upper triangle of the NBI x NBI
-// symmetric block (NBI (NBI+1)/2 values, row by row) in units of mt_unit
-// elements (16 bytes, or one element when NBI = 1).
-__host__ __device__ inline int mt_unit(int NBI, int u) { return NBI == 1 ? 1 : u; }
-__host__ __device__ inline int mt_units(int NBI, int u)
-{
-    const int ue = mt_unit(NBI, u);
-    return (NBI * (NBI + 1) / 2 + ue - 1) / ue;
-}
+__host__ __device__ inline int xs_stride(int nvec) { return nvec <= 2 ? nvec : (nvec + 3) & ~3; }
 
-// Per-term record of the fast kernel, in processing order, 16-byte units:
-// header | positions[m] | active pairs[npair] | induced matrices[nind] (padded).
-// Positions: the inner slots (mode order) first, then the outer slots in the
-// order of fewest multiply-adds (ascending 1/nb - 1/nq, ties in mode order).
-// Induced matrices: the two-mode monomials whose partner mode is collapsed,
-// per position (summed into the term image's H1; listed for the inner-block
-// tables).
-struct alignas(16) FDescHdr {
-    int m, R, NB, coef;          // positions, inner positions, basis size, D_l
-    int s, npair, nind, gsize;   // slicing depth, active pairs, induced matrices, G-table words
-    double c0;                   // constant of the term (collapsed modes)
-    long long rank_off;          // start of the term's compact indices (layout order)
-};
-struct FDescPos { unsigned char mode, lev, nb, nq; int offB, offBW, offH1; };
-struct FDescPair { unsigned char pa, pb, r0, r1; int goff, gsm, r2; };  // gsm: shared-memory offset of G
-struct FDescInd { unsigned char pos, r0, r1, r2; int ioff; };
-static_assert(sizeof(FDescHdr) == 48 && sizeof(FDescPos) == 16 && sizeof(FDescPair) == 16 &&
-              sizeof(FDescInd) == 8, "descriptor layout");
-
-// Fast-path tables (potentials whose monomials touch at most two modes).
-// All offsets are element offsets into FastParams::tab (T precision) or
-// ::sc (FP64 scalars); -1 marks an absent entry.
-struct FastParams {
-    int enabled;
-    int nb1, nq1;          // uniform sizes of level 1 (0 if modes differ)
-    int npairs;            // coupled mode pairs (i < i')
-    const int *pair_modes; // [npairs][2]
-    const int *h1off;      // [D][L+1]: single-mode matrix (nb x nb) of an active level
-    const int *goff;       // [npairs][L+1][L+1]: coupling table G[u_i][u_i'] (active levels)
-    const int *ioff;       // [npairs][2][L+1][L+1]: induced matrix on side s's mode at
-                           //   level l_s when the partner is collapsed at level l_o
-    const int *soff;       // [D][L+1]: scalar of a collapsed mode (into sc)
-    const int *spoff;      // [npairs][L+1][L+1]: scalar of a pair with both modes collapsed
-    const double *sc;      // scalars
-    const double *tabd;    // FP64 fast tables
-    const float *tabf;     // FP32 copies
-    double c0const;        // constant monomials
-    const int4 *desc;      // term records (processing order)
-    const unsigned *desc_off;  // [n_terms+1] record starts, in 16-byte units
-    const int *ranks;      // compact index of every basis function of every term (layout order)
-    const long long *rank_start;  // [n_terms + 1] start of each term's indices in ranks (processing order)
-    int desccap;           // largest record, in 16-byte units
-    int gcap;              // largest set of a term's G tables, in words
-    int nbocap;            // largest sliced outer block (slice weights)
-    int n_big;             // terms [0, n_big) run one per block, the rest one per warp
-    int work_cta, work_warp;   // work-area capacities (elements) of the two kernels
-    // per-term shared-memory images (processing order): the term's B, B^T W and
-    // H1 (base + induced, summed on the host) per position, then its G tables
-    const double *imgd;        // FP64 contexts
-    const float *imgf;         // FP32 contexts
-    const long long *img_off;  // [n_terms + 1] image starts, in elements
-    // inner-block tables: per term with coupled pairs, the action of its inner
-    // positions at every outer grid point (symmetric NBI x NBI, upper triangle),
-    // formed once per context; layout [slice][unit][outer grid point][unit elements]
-    const double *mtabd;       // FP64 contexts
-    const float *mtabf;        // FP32 contexts
-    const long long *mt_off;   // [n_terms + 1] starts, in elements (16-byte aligned; 0-size without a grid)
-    // double-float contexts (SG_DF64): contractions in pairs of FP32 numbers
-    // (hi, lo), FP64 accumulation; images and inner-block tables as (hi, lo)
-    int df;
-    const float2 *imgx;
-    const float2 *mtabx;
-};
-
-// Everything a kernel needs, passed by value (a multiple of 16 bytes, so
-// that a kernel can copy it in 16-byte units).
+// Everything the set-up kernels and the term-by-term kernel need.
 struct alignas(16) KParams {
     int D, L, Dpad;
     int nmono, pmax, kw;
@@ -212,13 +137,6 @@ struct alignas(16) KParams {
     const int *harm_mono;    // [D] monomial holding the harmonic part of mode i (-1: not split)
     const double *esplit;    // [n_cs] sum over split modes of omega_i s_i^2 (k_i + 1/2)
     unsigned long long *acc; // [n_cs][nvec][acc_words] fixed-point accumulators (entry-major)
-    // Entry-major copy of the input vectors in the contraction type, made at
-    // the start of each apply: xs[r * xs_stride(xs_nvec) + v] = x_v[r] (the
-    // vectors of one compact entry adjacent).  Holds up to xs_nvec vectors;
-    // nullptr: the term kernels read x itself.
-    const void *xs;
-    int xs_nvec;
-    FastParams fast;
     // capacities of the per-CTA shared-memory areas (elements)
     int cap;       // each of the two grid ping-pong buffers
     int maxnb;     // term basis tensor
@@ -227,6 +145,18 @@ struct alignas(16) KParams {
     int *err;      // device error word (0 = fine)
     // term-sharded applies: only processing positions p with p % nparts == part
     int part, nparts;
+};
+
+// Shift tables of the row form (device copies of the HostTables arrays).
+struct RowShifts {
+    int nshift;
+    const int *off;        // [nshift + 1] into mode / d
+    const int *mode, *d;   // the modes a shift moves, and by how much
+    const int *src_off;    // [nshift + 1] into src
+    const int *src;        // products that contribute to the shift
+    const int *prod_off;   // [nprod + 1] into fmode / fop
+    const int *fmode, *fop;  // factors of a product: mode, power (0: the kinetic matrix)
+    const double *coef;    // [nprod]
 };
 
 // Host-side description of a problem (after validation).
@@ -254,24 +184,18 @@ struct HostTables {
     std::vector<double> tabd;
     std::vector<int> harm_mono;      // [D]
     std::vector<double> esplit;      // [n_cs]
-    // fast path
+    // pair form: every monomial touches at most two modes, in at most kMaxPairs pairs
     bool fast = false;
-    int nb1 = 0, nq1 = 0;
-    std::vector<int> pair_modes, h1off, goff, ioff, soff, spoff;
-    std::vector<double> ftab, fsc;
-    double c0const = 0.0;
-    int fast_cap = 0, fast_maxnb = 0, fast_matcap = 0;
-    std::vector<double> fimg;         // per-term shared-memory images (see FastParams)
-    std::vector<long long> fimg_off;  // [n_terms + 1]
-    std::vector<long long> fvt_off;   // [n_terms + 1] inner-block table starts (see FastParams::mt_off)
-    std::vector<int4> fdesc;          // term records
-    std::vector<unsigned> fdesc_off;  // [n_terms+1]
-    int64_t franks = 0;               // total compact indices (N_s)
-    std::vector<long long> frank_start;  // [n_terms + 1] start of each term's indices
-    int fdesccap = 0, fgcap = 0, fnbocap = 1, fn_big = 0, fwork_cta = 0, fwork_warp = 0;
-    int slice_vt = 0;                 // slicing target the records were planned with (0: default)
-    int warp_vt = 0;                  // warp-form threshold the records were planned with (0: default)
-    int fbudget = 0;                  // shared-memory budget the records were planned with
+    int nb1 = 0, nq1 = 0;            // uniform sizes of level 1 (0 if modes differ)
+    std::vector<int> pair_modes;     // [npairs][2]
+    // row form (see RowShifts); rows = false: the term-by-term kernel applies H_S
+    bool rows = false;
+    int64_t row_nnz = 0;             // entries of the row operator
+    std::vector<int> sh_off, sh_mode, sh_d, sh_src_off, sh_src, pr_off, pr_mode, pr_op;
+    std::vector<double> pr_coef;
+    // plan of the row kernels (0: default): vectors per lane, rows per window
+    // in units of 64, shared-memory budget of a block (bytes)
+    int slice_vt = 0, warp_vt = 0, fbudget = 0;
     int cap = 0, maxnb = 0, matcap = 0, vtabcap = 0;
     int64_t flops_per_vec = 0;       // FMA-counted work of one real apply (2 flops per FMA)
 };
@@ -282,45 +206,68 @@ std::string build_tables(const Problem &p, int smem_budget_bytes, int real_bytes
 // One-mode Gauss-Hermite rule with Hermite-function-normalised weights.
 std::string gauss_hermite(int n, std::vector<double> *x, std::vector<double> *wf);
 
-// Kernel launchers (sg_apply.cu).  Return cudaSuccess or the launch error.
+// Term-by-term kernel (sg_apply.cu).  Return cudaSuccess or the launch error.
 cudaError_t launch_apply(const KParams &kp, bool fp32, const double *x, double *y, int nvec,
-                         long long *maxbits, int *lsb_exp, cudaStream_t stream);
+                         long long *maxbits, cudaStream_t stream);
 cudaError_t launch_index_map(const KParams &kp, int64_t t0, int64_t nt, const int64_t *offsets_dev,
                              int64_t *cs_index, cudaStream_t stream);
 size_t apply_smem_bytes(const KParams &kp, bool fp32);
 cudaError_t configure_kernels(size_t smem_bytes, bool fp32);
-
-// Fast path (sg_apply_fast.cu, sg_setup.cpp)
-std::string build_fast_tables(const Problem &p, HostTables *T);
-std::string build_fast_descs(const Problem &p, bool fp32, HostTables *T, int fbudget, int rb);
-cudaError_t launch_build_ranks(const KParams &kp, int *ranks, cudaStream_t stream);
-// Fills the inner-block tables (FastParams::mtab*) from the records and the FP64 tables.
-cudaError_t launch_build_mtab(const KParams &kp, bool fp32, cudaStream_t stream);
-size_t fast_smem_bytes(const KParams &kp, bool fp32);
-cudaError_t configure_fast_kernels(const KParams &kp, bool fp32);
-cudaError_t launch_apply_fast(const KParams &kp, bool fp32, const double *x, int nvec,
-                              const long long *maxbits, cudaStream_t stream);
-
-// Many problems per apply (sg_batch.cpp): the term kernels of one problem
-// without the max|x| and finalisation passes; those two over all problems.
+// The passes of launch_apply: per-vector max|x| bits (zeroed first), the terms,
+// and y = (accumulated integer) * 2^E + esplit * x, which also clears kp.acc.
+cudaError_t launch_maxabs(const KParams &kp, const double *x, int nvec, long long *maxbits, cudaStream_t stream);
 cudaError_t launch_apply_terms(const KParams &kp, bool fp32, const double *x, const long long *maxbits, int nvec,
                                cudaStream_t stream);
-// The passes around the term kernels of one problem: per-vector max|x| bits
-// (zeroed first), and y = (accumulated integer) * 2^E + esplit * x, which also
-// clears kp.acc.
-cudaError_t launch_maxabs(const KParams &kp, const double *x, int nvec, long long *maxbits, cudaStream_t stream);
-// kp.xs = the input vectors entry-major in the contraction type (kp.xs set, nvec <= kp.xs_nvec; rows of
-// xs_stride(kp.xs_nvec) elements); for a batch, every problem's rows from cs_prefix[j].
-cudaError_t launch_stage_x(const KParams &kp, bool fp32, const double *x, int nvec, cudaStream_t stream);
-cudaError_t launch_stage_x_batch(bool fp32, const double *x, const long long *cs_prefix, int nprob, int64_t max_ncs,
-                                 int nvec, int xs_nvec, void *xs, cudaStream_t stream);
 cudaError_t launch_finalize(const KParams &kp, bool fp32, const double *x, double *y, int nvec,
                             const long long *maxbits, cudaStream_t stream);
-cudaError_t launch_maxabs_batch(const double *x, const long long *cs_prefix, int nprob, int64_t max_ncs, int nvec,
-                                long long *maxbits, cudaStream_t stream);
-cudaError_t launch_finalize_batch(const KParams *kps, const long long *cs_prefix, int nprob, int64_t max_ncs,
-                                  const double *x, double *y, unsigned long long *acc, const long long *maxbits,
-                                  int nvec, bool fp32, cudaStream_t stream);
+
+// Size of the problem in its term-by-term form (sg_setup.cpp).
+struct TermForm {
+    bool fits;      // every term fits the shared memory of its form
+    int64_t bytes;  // M^B, inner-block tables, records, images
+};
+TermForm term_form(const Problem &p, const HostTables &T);
+
+// Row form, host half (sg_rows_setup.cpp).
+void build_row_shifts(const Problem &p, HostTables *T);
+int row_vt(const HostTables &T, sg_precision prec);      // vectors per lane of the plan
+int row_window_units(const HostTables &T);               // rows per window / 64 of the plan
+int row_budget(const HostTables &T, sg_precision prec);  // shared memory per block (bytes) of the plan
+int row_value_bytes(sg_precision prec);                  // bytes of a stored element
+// Upper bound of the device bytes of the row operator.
+int64_t row_form_bytes(const HostTables &T, sg_precision prec);
+struct RowWindows {
+    std::vector<RowWin> wins;
+    std::vector<uint2> meta;
+    std::vector<long long> start;  // first entry of each row
+    int64_t entries = 0;           // with the padding of the windows
+    int cap = 0, wrows = 0;
+};
+// Cuts the rows (cnt[r] entries each) into windows of at most `wrows` rows and
+// `budget` bytes, and orders the rows of each by decreasing length.
+RowWindows cut_rows(const std::vector<int> &cnt, int wrows, int budget, int value_bytes);
+int row_window_rows(int64_t n, int units);
+
+// Row form, device half (sg_rows.cu).  prec selects the element type.
+cudaError_t launch_row_count(const KParams &kp, const RowShifts &sh, int *cnt, cudaStream_t stream);
+cudaError_t launch_row_fill(const KParams &kp, const RowShifts &sh, sg_precision prec, const long long *start,
+                            int *cols, void *vals, cudaStream_t stream);
+cudaError_t configure_rows();
+// y = H_S x (io.y), or the sums of the windows of io.part into io.acc; vt: vectors per lane.
+cudaError_t launch_rows(const RowOp &R, const RowIO &io, sg_precision prec, int vt, cudaStream_t stream);
+// io.xs = the vectors entry-major in the contraction type; a batch: every problem's rows from cs_prefix[j] * stride.
+cudaError_t launch_row_stage(const RowOp &R, const RowIO &io, sg_precision prec, cudaStream_t stream);
+cudaError_t launch_row_stage_batch(const RowIO &io, sg_precision prec, const long long *cs_prefix, const int2 *items,
+                                   int nitems, cudaStream_t stream);
+// Vectors with a non-finite input become NaN; clears the flags.
+cudaError_t launch_row_settle(const RowIO &io, int n, cudaStream_t stream);
+cudaError_t launch_row_settle_batch(const RowIO &io, const long long *cs_prefix, int nprob, cudaStream_t stream);
+// y from the summed accumulators of all parts; clears them.
+cudaError_t launch_row_finish(const RowOp &R, const RowIO &io, cudaStream_t stream);
+// Many problems: item = (problem, window); RowIO holds the batch's buffers.
+cudaError_t launch_rows_batch(const RowOp *ops, const int2 *items, int nitems, int cap, int wrows, const RowIO &io,
+                              sg_precision prec, int vt, const long long *cs_prefix, cudaStream_t stream);
+
 // Propagation server (sg_server_api.cpp, sg_server.cu): device state of one
 // active request's Chebyshev recurrence.  One iteration after Y = H X logs
 // norm and energy for requests at k = 0, forms T_{k+1} (T_1 from T_0 when
@@ -349,21 +296,6 @@ std::vector<double> bessel_j(int kmax, double x);
 // Device bytes sg_create would allocate for a planned context (tables, records, M^B).
 int64_t planned_device_bytes(const sg_ctx *ctx);
 
-// Shared-memory partition of one term group of the fast kernels (block form or warp form).
-size_t fast_part_bytes(const KParams &kp, bool fp32, bool warp_form);
-// Fast-path kernels over many problems of one kernel variant; items are
-// (problem, processing position) pairs in cost order.
-struct FastBatchGroup {
-    const KParams *kps;       // device, one per problem of the batch
-    const int2 *items[2];     // device: [0] block form, [1] warp form
-    int count[2];
-    int part[2];              // bytes per term group
-};
-cudaError_t configure_fast_batch(const KParams &kp_any, bool fp32, const FastBatchGroup &g);
-cudaError_t launch_fast_batch(const KParams &kp_any, bool fp32, const FastBatchGroup &g, const double *x,
-                              unsigned long long *acc, const long long *maxbits, const long long *cs_prefix,
-                              int nvec, cudaStream_t stream);
-
 }  // namespace sg
 
 struct sg_ctx {
@@ -378,10 +310,17 @@ struct sg_ctx {
     std::vector<void *> allocations;
     double *stage_x = nullptr, *stage_y = nullptr;  // host-API staging (device)
     int64_t stage_elems = 0;
-    // apply workspace: fixed-point accumulators and per-vector scale exponents
+    // row operator: its buffers, and the plan's vectors per lane
+    sg::RowOp rop{};
+    std::vector<void *> row_allocs;
+    std::vector<int> win_entries;  // entries of each window
+    int64_t row_bytes = 0;
+    // apply workspace.  Row form: per-vector flags and the entry-major input
+    // copy; term-by-term kernel: fixed-point accumulators and scale exponents
+    unsigned *flags = nullptr;
+    void *xs = nullptr;
     unsigned long long *acc = nullptr;
     long long *maxbits = nullptr;
-    void *xs = nullptr;       // entry-major input copy (fast path), acc_nvec vectors
     int acc_nvec = 0;
     int plan_version = 0;     // incremented whenever sg_tune installs a plan
     std::string last_error;
@@ -394,3 +333,13 @@ inline bool sg_on_ctx_device(const sg_ctx *ctx)
     int cur = -1;
     return cudaGetDevice(&cur) == cudaSuccess && cur == ctx->device;
 }
+
+namespace sg {
+
+// Row operator of a context (sg_api.cpp): forms it with the context's plan
+// (replacing an earlier one), releases it, and enqueues one apply or part.
+cudaError_t build_rows(sg_ctx *ctx);
+void free_rows(sg_ctx *ctx);
+cudaError_t apply_rows(sg_ctx *ctx, RowIO io, cudaStream_t s);
+
+}  // namespace sg

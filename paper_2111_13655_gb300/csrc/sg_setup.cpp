@@ -97,6 +97,40 @@ std::string gauss_hermite(int n, std::vector<double> *x, std::vector<double> *wf
     return "";
 }
 
+// Pair form: every monomial touches at most two modes, in at most kMaxPairs
+// mode pairs; the pairs, and the sizes of level 1 where all modes share them.
+static void find_pairs(const Problem &p, HostTables *Tp)
+{
+    HostTables &T = *Tp;
+    const int D = p.D, Lp = p.L + 1;
+    T.fast = false;
+    T.pair_modes.clear();
+    for (int m = 0; m < (int)p.mcoef.size(); m++) {
+        int a = -1, b = -1;
+        for (int f = p.mfoff[m]; f < p.mfoff[m + 1]; f++) {
+            const int i = p.mfmode[f];
+            if (i == a || i == b) continue;
+            if (a < 0) a = i;
+            else if (b < 0) b = i;
+            else return;
+        }
+        if (b < 0) continue;
+        if (a > b) std::swap(a, b);
+        bool seen = false;
+        for (size_t q = 0; q < T.pair_modes.size(); q += 2)
+            seen |= T.pair_modes[q] == a && T.pair_modes[q + 1] == b;
+        if (!seen) { T.pair_modes.push_back(a); T.pair_modes.push_back(b); }
+    }
+    if (T.pair_modes.size() / 2 > (size_t)kMaxPairs) return;
+    T.nb1 = T.nq1 = 0;
+    if (p.L >= 1) {
+        T.nb1 = T.lvl[1].nb; T.nq1 = T.lvl[1].nq;
+        for (int i = 1; i < D; i++)
+            if (T.lvl[(size_t)i * Lp + 1].nb != T.nb1 || T.lvl[(size_t)i * Lp + 1].nq != T.nq1) { T.nb1 = T.nq1 = 0; break; }
+    }
+    T.fast = true;
+}
+
 std::string build_tables(const Problem &p, int smem_budget, int rb, HostTables *out)
 {
     HostTables &T = *out;
@@ -357,10 +391,6 @@ std::string build_tables(const Problem &p, int smem_budget, int rb, HostTables *
     T.cap = (int)(((size_t)smem_budget - fixed) / (2 * (size_t)rb));
     T.cap = std::max(T.cap, stage_min_max);
 
-    // fast path (potentials with at most two-mode monomials)
-    std::string fe = build_fast_tables(p, &T);
-    if (!fe.empty()) return fe;
-
     // processing order: most expensive terms first (longest-processing-time first)
     T.order.resize(T.n_terms);
     std::iota(T.order.begin(), T.order.end(), 0);
@@ -369,14 +399,8 @@ std::string build_tables(const Problem &p, int smem_budget, int rb, HostTables *
     T.pcost.resize(T.n_terms);
     for (int64_t q = 0; q < T.n_terms; q++) T.pcost[q] = cost[T.order[q]];
 
-    if (T.fast) {
-        // fast kernel: matrices, G tables, slice weights and ranks, then a work
-        // area for X, Y and two grid buffers (sized per term and vector chunk)
-        const int fbudget = std::min(smem_budget, rb == 4 ? SG_F32_SMEM_KB * 1024 : SG_F64_SMEM_KB * 1024);
-        T.fbudget = fbudget;
-        std::string de = build_fast_descs(p, rb == 4, &T, fbudget, rb);
-        if (!de.empty()) return de;
-    }
+    find_pairs(p, &T);
+    build_row_shifts(p, &T);
     return "";
 }
 
@@ -384,414 +408,108 @@ std::string build_tables(const Problem &p, int smem_budget, int rb, HostTables *
 
 namespace sg {
 
-// Fast-path tables.  Valid when every monomial of V touches at most two
-// distinct modes.  A term's operator then splits exactly into
-//   c0 I + sum_{slots j} H1_j + (x_j B_j^T W_j) diag(sum_{active pairs p} G_p) (x_j B_j),
-// where the single-mode matrices H1_j and the scalar c0 collect, for the
-// term's levels, the kinetic part, the one-mode monomials and the two-mode
-// monomials whose partner mode holds one basis function (folded through
-// that mode's quadrature moments), and G_p tabulates the two-mode monomials
-// on the grids of the pair's levels.  Everything here depends only on
-// (mode, level) combinations, so it is computed once.
-std::string build_fast_tables(const Problem &p, HostTables *Tp)
+// Size of the problem term by term: per term its compact indices (M^B), its
+// record, its 1D matrices and pair tables, and the table of its inner blocks
+// (up to three level-1 modes of a term with coupled modes, one symmetric block
+// per grid point of its other modes).  It is what sg_size reports for a planned
+// context and what the request server admits by: an upper bound of the row
+// operator that sg_create allocates, and independent of its layout.
+// `fits` tells whether every term fits a block's shared memory (slicing its
+// leading outer modes, at most 64 functions per slice): pair potentials where
+// one does not are outside the double-float mode and the tuner.
+TermForm term_form(const Problem &p, const HostTables &T)
 {
-    HostTables &T = *Tp;
-    const int D = p.D, L = p.L, Lp = L + 1;
-    T.fast = false;
-    const int nmono = (int)p.mcoef.size();
-    // distinct modes (and summed powers) of every monomial
-    std::vector<std::vector<std::pair<int, int>>> facs(nmono);
-    for (int m = 0; m < nmono; m++) {
-        for (int f = p.mfoff[m]; f < p.mfoff[m + 1]; f++) {
-            bool found = false;
-            for (auto &pr : facs[m])
-                if (pr.first == p.mfmode[f]) { pr.second += p.mfpow[f]; found = true; }
-            if (!found) facs[m].push_back({p.mfmode[f], p.mfpow[f]});
-        }
-        if (facs[m].size() > 2) return "";  // not eligible: the generic kernel handles it
-        if (facs[m].size() == 2 && facs[m][0].first > facs[m][1].first) std::swap(facs[m][0], facs[m][1]);
-    }
-    auto split = [&](int m) {
-        for (int i = 0; i < D; i++) if (T.harm_mono[i] == m) return true;
-        return false;
-    };
-    auto LI = [&](int i, int l) -> const LevelInfo & { return T.lvl[(size_t)i * Lp + l]; };
-    const double *td = T.tabd.data();
-    auto mu = [&](int i, int l, int pw) { return td[LI(i, l).offMu + pw]; };
-    auto Mp = [&](int i, int l, int pw) { return td + LI(i, l).offM + (size_t)(pw - 1) * LI(i, l).nb * LI(i, l).nb; };
-
-    // uniform level-1 sizes (for the register block)
-    T.nb1 = T.nq1 = 0;
-    if (L >= 1) {
-        T.nb1 = LI(0, 1).nb; T.nq1 = LI(0, 1).nq;
-        for (int i = 1; i < D; i++)
-            if (LI(i, 1).nb != T.nb1 || LI(i, 1).nq != T.nq1) { T.nb1 = T.nq1 = 0; break; }
-    }
-    // coupled pairs
-    std::vector<int> pidx((size_t)D * D, -1);
-    T.pair_modes.clear();
-    for (int m = 0; m < nmono; m++)
-        if (facs[m].size() == 2) {
-            int a = facs[m][0].first, b = facs[m][1].first;
-            if (pidx[(size_t)a * D + b] < 0) {
-                pidx[(size_t)a * D + b] = (int)T.pair_modes.size() / 2;
-                T.pair_modes.push_back(a);
-                T.pair_modes.push_back(b);
-            }
-        }
-    const int np = (int)T.pair_modes.size() / 2;
-    if (np > kMaxPairs) return "";
-    T.ftab.clear();
-    T.fsc.clear();
-    T.c0const = 0.0;
-    for (int m = 0; m < nmono; m++)
-        if (facs[m].empty()) T.c0const += p.mcoef[m];
-    // single-mode matrices (active levels) and scalars (collapsed levels)
-    T.h1off.assign((size_t)D * Lp, -1);
-    T.soff.assign((size_t)D * Lp, -1);
-    for (int i = 0; i < D; i++)
-        for (int l = 0; l <= L; l++) {
-            const LevelInfo &li = LI(i, l);
-            const int nb = li.nb;
-            const bool sp = T.harm_mono[i] >= 0;
-            if (nb > 1) {
-                T.h1off[(size_t)i * Lp + l] = (int)T.ftab.size();
-                for (int e = 0; e < nb * nb; e++) {
-                    double h = sp ? 0.0 : td[li.offK + e];
-                    for (int m = 0; m < nmono; m++)
-                        if (facs[m].size() == 1 && facs[m][0].first == i && !split(m))
-                            h += p.mcoef[m] * Mp(i, l, facs[m][0].second)[e];
-                    T.ftab.push_back(h);
-                }
-            } else {
-                T.soff[(size_t)i * Lp + l] = (int)T.fsc.size();
-                double sc = sp ? 0.0 : td[li.offK];
-                for (int m = 0; m < nmono; m++)
-                    if (facs[m].size() == 1 && facs[m][0].first == i && !split(m))
-                        sc += p.mcoef[m] * mu(i, l, facs[m][0].second);
-                T.fsc.push_back(sc);
-            }
-        }
-    // pair tables, induced matrices, pair scalars
-    T.goff.assign((size_t)np * Lp * Lp, -1);
-    T.ioff.assign((size_t)np * 2 * Lp * Lp, -1);
-    T.spoff.assign((size_t)np * Lp * Lp, -1);
-    for (int P = 0; P < np; P++) {
-        const int a = T.pair_modes[2 * P], b = T.pair_modes[2 * P + 1];
-        for (int la = 0; la <= L; la++)
-            for (int lb = 0; la + lb <= L; lb++) {
-                const LevelInfo &A = LI(a, la), &B = LI(b, lb);
-                const size_t key = ((size_t)P * Lp + la) * Lp + lb;
-                if (A.nb > 1 && B.nb > 1) {
-                    T.goff[key] = (int)T.ftab.size();
-                    for (int ua = 0; ua < A.nq; ua++)
-                        for (int ub = 0; ub < B.nq; ub++) {
-                            double g = 0.0;
-                            for (int m = 0; m < nmono; m++)
-                                if (facs[m].size() == 2 && facs[m][0].first == a && facs[m][1].first == b)
-                                    g += p.mcoef[m] * std::pow(td[A.offQ + ua], facs[m][0].second) *
-                                         std::pow(td[B.offQ + ub], facs[m][1].second);
-                            T.ftab.push_back(g);
-                        }
-                } else if (A.nb > 1 || B.nb > 1) {
-                    // one side active: induced single-mode matrix on that side
-                    const int side = A.nb > 1 ? 0 : 1;
-                    const int act = side == 0 ? a : b, lact = side == 0 ? la : lb;
-                    const int col = side == 0 ? b : a, lcol = side == 0 ? lb : la;
-                    const int nb = LI(act, lact).nb;
-                    T.ioff[(((size_t)P * 2 + side) * Lp + lact) * Lp + lcol] = (int)T.ftab.size();
-                    for (int e = 0; e < nb * nb; e++) {
-                        double h = 0.0;
-                        for (int m = 0; m < nmono; m++)
-                            if (facs[m].size() == 2 && facs[m][0].first == a && facs[m][1].first == b) {
-                                const int pact = side == 0 ? facs[m][0].second : facs[m][1].second;
-                                const int pcol = side == 0 ? facs[m][1].second : facs[m][0].second;
-                                h += p.mcoef[m] * mu(col, lcol, pcol) * Mp(act, lact, pact)[e];
-                            }
-                        T.ftab.push_back(h);
-                    }
-                } else {
-                    T.spoff[key] = (int)T.fsc.size();
-                    double sc = 0.0;
-                    for (int m = 0; m < nmono; m++)
-                        if (facs[m].size() == 2 && facs[m][0].first == a && facs[m][1].first == b)
-                            sc += p.mcoef[m] * mu(a, la, facs[m][0].second) * mu(b, lb, facs[m][1].second);
-                    T.fsc.push_back(sc);
-                }
-            }
-    }
-    if (T.ftab.size() >= ((size_t)1 << 30)) return "fast tables too large";
-    if (T.fsc.empty()) T.fsc.push_back(0.0);
-    if (T.ftab.empty()) T.ftab.push_back(0.0);
-    T.fast = true;
-    return "";
-}
-
-}  // namespace sg
-
-namespace sg {
-
-namespace {
-
-template <typename S>
-void put(std::vector<int4> &v, size_t unit, size_t byte, const S &x)
-{
-    std::memcpy(reinterpret_cast<char *>(v.data() + unit) + byte, &x, sizeof(S));
-}
-
-}  // namespace
-
-// Per-term records of the fast kernel (processing order).  For every term:
-// the transformed modes ("positions": for a term with coupled pairs, the last
-// fast_rmax level-1 modes first as inner positions, whose action is tabulated
-// per outer grid point; then the outer positions in the order of fewest
-// multiply-adds) with the offsets of their tables, the term constant c0, the
-// active coupled pairs with the offsets of their G tables, the induced
-// single-mode matrices, and the slicing depth for its kernel.  The most expensive terms (a prefix of the
-// processing order) run one per thread block; the small ones at its tail run
-// one per warp, four per block, in a quarter of the block's shared memory
-// each (a term goes to the warp form when a chunk of 4 vectors fits that
-// quarter without slicing).
-std::string build_fast_descs(const Problem &p, bool fp32, HostTables *Tp, int fbudget, int rb)
-{
-    HostTables &T = *Tp;
-    const int D = p.D, L = p.L, Lp = L + 1;
-    const int RMAX = fast_rmax(T.nb1);
-    const int U = 16 / rb;  // elements per 16 bytes
+    TermForm F{T.fast, 0};
+    if (!T.fast) return F;
+    const int D = p.D, Lp = p.L + 1;
+    const int rb = p.prec == SG_MIXED ? 4 : 8, U = 16 / rb;
+    const int rmax = T.nb1 == 2 ? 3 : T.nb1 == 3 ? 2 : 0, slice_max = 64;
     const int np = (int)T.pair_modes.size() / 2;
     auto LI = [&](int i, int l) -> const LevelInfo & { return T.lvl[(size_t)i * Lp + l]; };
+    auto pad = [U](int64_t n) { return (n + U - 1) / U * U; };
 
-    struct TermPlan {
-        int na, R, posmode[kMaxD];
-        int64_t NB, NBIn;
-        bool grid;
-        int gsize;
-        double c0;
-        std::vector<FDescPair> prs;
-        std::vector<FDescInd> inds;
+    struct Plan {
+        int na, R, mode[kMaxD], nprs, ninds;
+        int64_t NB, NBin, gsize, mat;
     };
-    auto plan_term = [&](int t, TermPlan &tp) {
+    auto plan = [&](int64_t t, Plan &P) {
         const uint8_t *lt = &T.levels[(size_t)t * T.Dpad];
-        int act[kMaxD], na = 0, pos_of_mode[kMaxD];
-        bool l1[kMaxD], inner[kMaxD];
-        double c0 = T.c0const;
-        for (int i = 0; i < D; i++) {
-            pos_of_mode[i] = -1;
-            const LevelInfo &li = LI(i, lt[i]);
-            if (li.nb > 1) { act[na] = i; l1[na] = li.nb == T.nb1 && li.nq == T.nq1; inner[na] = false; na++; }
-            else c0 += T.fsc[T.soff[(size_t)i * Lp + lt[i]]];
+        bool inner[kMaxD] = {false};
+        P.nprs = P.ninds = 0;
+        P.gsize = 0;
+        for (int q = 0; q < np; q++) {
+            const int a = T.pair_modes[2 * q], b = T.pair_modes[2 * q + 1];
+            const bool aa = LI(a, lt[a]).nb > 1, ab = LI(b, lt[b]).nb > 1;
+            if (aa && ab) { P.nprs++; P.gsize += LI(a, lt[a]).nq * LI(b, lt[b]).nq; }
+            else if (aa || ab) P.ninds++;
         }
-        // the term has a grid when some coupled pair has both modes transformed;
-        // only then are level-1 modes made inner positions
-        bool has_grid = false;
-        for (int P = 0; P < np && !has_grid; P++)
-            has_grid = LI(T.pair_modes[2 * P], lt[T.pair_modes[2 * P]]).nb > 1 &&
-                       LI(T.pair_modes[2 * P + 1], lt[T.pair_modes[2 * P + 1]]).nb > 1;
-        int R = 0;
-        for (int a = na - 1; a >= 0 && R < (has_grid ? RMAX : 0); a--)
-            if (l1[a]) { inner[a] = true; R++; }
-        int pos = 0;
-        for (int a = 0; a < na; a++) if (inner[a]) { pos_of_mode[act[a]] = pos; tp.posmode[pos++] = act[a]; }
-        // Outer slots in the order of the forward (basis -> grid) chain that needs
-        // the fewest multiply-adds.  A contraction costs (current size) x nq and
-        // multiplies the size by nq/nb, so swapping neighbours j, k shows that j
-        // goes first iff 1/nb_j - 1/nq_j < 1/nb_k - 1/nq_k (for nb = l+1,
-        // nq = l+2: higher levels first).  Compared exactly in integers; ties
-        // keep mode order.  The backward chain runs in reverse.
-        int outer[kMaxD], no = 0;
-        for (int a = 0; a < na; a++) if (!inner[a]) outer[no++] = a;
-        std::stable_sort(outer, outer + no, [&](int x, int y) {
-            const LevelInfo &u = LI(act[x], lt[act[x]]), &w = LI(act[y], lt[act[y]]);
+        P.R = P.na = 0;
+        for (int i = D - 1; i >= 0 && P.R < (P.nprs ? rmax : 0); i--) {
+            const LevelInfo &li = LI(i, lt[i]);
+            if (li.nb > 1 && li.nb == T.nb1 && li.nq == T.nq1) { inner[i] = true; P.R++; }
+        }
+        P.NB = P.NBin = 1;
+        P.mat = 0;
+        for (int i = 0; i < D; i++) {
+            const LevelInfo &li = LI(i, lt[i]);
+            if (li.nb <= 1) continue;
+            P.NB *= li.nb;
+            P.mat += 2 * li.nb * li.nq + li.nb * li.nb;
+            if (inner[i]) P.NBin *= li.nb;
+            else P.mode[P.na++] = i;
+        }
+        std::stable_sort(P.mode, P.mode + P.na, [&](int x, int y) {  // by 1/nb - 1/nq
+            const LevelInfo &u = LI(x, lt[x]), &w = LI(y, lt[y]);
             return (int64_t)(u.nq - u.nb) * w.nb * w.nq < (int64_t)(w.nq - w.nb) * u.nb * u.nq;
         });
-        for (int k = 0; k < no; k++) { pos_of_mode[act[outer[k]]] = pos; tp.posmode[pos++] = act[outer[k]]; }
-        tp.na = na; tp.R = R; tp.NB = 1; tp.NBIn = 1;
-        for (int j = 0; j < na; j++) {
-            tp.NB *= LI(tp.posmode[j], lt[tp.posmode[j]]).nb;
-            if (j < R) tp.NBIn *= LI(tp.posmode[j], lt[tp.posmode[j]]).nb;
+    };
+    auto need = [&](const Plan &P, int64_t stage, bool sliced) {
+        return pad((P.NB * U + 3) / 4) + (sliced || !P.nprs ? 2 : 1) * pad(P.NB) + (P.nprs ? 2 * pad(stage) : 0);
+    };
+    Plan P;
+    int64_t gcap = 1, mcap = 1, units = 1;
+    for (int64_t t = 0; t < T.n_terms; t++) {
+        plan(t, P);
+        const int m = P.na + P.R;
+        const int64_t u = 3 + m + P.nprs + (P.ninds + 1) / 2;
+        gcap = std::max(gcap, P.gsize);
+        mcap = std::max(mcap, P.mat);
+        units = std::max(units, u);
+        int64_t blocks = 0;
+        if (P.nprs) {
+            int64_t grid = 1;
+            for (int j = 0; j < P.na; j++) grid *= LI(P.mode[j], T.levels[(size_t)t * T.Dpad + P.mode[j]]).nq;
+            const int64_t tri = P.NBin * (P.NBin + 1) / 2;
+            blocks = pad((P.NBin == 1 ? 1 : pad(tri)) * grid);
         }
-        tp.prs.clear(); tp.inds.clear();
-        tp.gsize = 0;
-        for (int P = 0; P < np; P++) {
-            const int a = T.pair_modes[2 * P], b = T.pair_modes[2 * P + 1];
-            const int pa = pos_of_mode[a], pb = pos_of_mode[b];
-            const size_t key = ((size_t)P * Lp + lt[a]) * Lp + lt[b];
-            if (pa >= 0 && pb >= 0) {
-                tp.prs.push_back(FDescPair{(unsigned char)pa, (unsigned char)pb, 0, 0, T.goff[key], tp.gsize, 0});
-                tp.gsize += LI(a, lt[a]).nq * LI(b, lt[b]).nq;
-            } else if (pa >= 0 || pb >= 0) {
-                const int side = pa >= 0 ? 0 : 1;
-                const int lact = side == 0 ? lt[a] : lt[b], lcol = side == 0 ? lt[b] : lt[a];
-                tp.inds.push_back(FDescInd{(unsigned char)(side == 0 ? pa : pb), 0, 0, 0,
-                                           T.ioff[(((size_t)P * 2 + side) * Lp + lact) * Lp + lcol]});
-            } else {
-                c0 += T.fsc[T.spoff[key]];
-            }
-        }
-        tp.grid = !tp.prs.empty();
-        tp.c0 = c0;
-    };
-    auto stage_of = [&](int t, const TermPlan &tp, int s) {
+        F.bytes += 4 * P.NB + 16 * u + rb * (P.mat + P.gsize + blocks);
+    }
+    F.bytes += (T.n_terms + 1) * (3 * (int64_t)sizeof(long long) + sizeof(unsigned));
+    const int64_t budget = 1024 * (int64_t)(rb == 4 ? 52 : 70);
+    const int64_t head = (rb * (mcap + gcap + 2 * slice_max) + 15) & ~(int64_t)15;
+    const int64_t work = (budget - head - 1024) / rb;
+    const int64_t record = (work * rb - 16 * units) / 16 * 16;  // scratch of a record at the end of the work area
+    if (work < 2 * T.maxnb + 64 || work * rb < 16 * (3 + (int64_t)kMaxD + 2 * np)) { F.fits = false; return F; }
+    for (int64_t t = 0; t < T.n_terms && F.fits; t++) {
+        plan(t, P);
         const uint8_t *lt = &T.levels[(size_t)t * T.Dpad];
-        int64_t sz = tp.NBIn;
-        for (int j = tp.R + s; j < tp.na; j++) sz *= LI(tp.posmode[j], lt[tp.posmode[j]]).nq;
-        return sz;
-    };
-    // slicing depth for a work area: the smallest leaving room for the slicing
-    // target's vectors per chunk (else half as many, ...)
-    const int vt0 = T.slice_vt > 0 ? T.slice_vt : fp32 ? SG_F32_SLICE_VT : SG_F64_SLICE_VT;
-    // (sliced blocks larger than nbocap functions are not used: their slice
-    // weights would not fit the group's head)
-    const int nbocap = 64;
-    // the term's compact indices (start of the work area) and the record's
-    // scratch copy (its end) are written at the same time in the prologue
-    int rec_units = 1;  // largest record, in 16-byte units (pass 1)
-    auto ranks_fit = [&](const TermPlan &tp, int64_t work) {
-        return 4 * tp.NB <= record_scratch_offset(work * rb, rec_units);
-    };
-    auto depth_for = [&](int t, const TermPlan &tp, int64_t work, int smax) {
-        if (!ranks_fit(tp, work)) return -1;
-        if (!tp.grid) return chunk_need(tp.NB, 0, false, false, 1, U) <= work ? 0 : -1;
-        const uint8_t *lt = &T.levels[(size_t)t * T.Dpad];
-        for (int vt = vt0; vt >= 1; vt /= 2) {
+        bool ok = 4 * P.NB <= record;
+        if (ok && P.nprs) {
+            ok = false;
             int64_t nbo = 1;
-            for (int s = 0; s <= std::min(smax, tp.na - tp.R); s++) {
-                if (s > 0) nbo *= LI(tp.posmode[tp.R + s - 1], lt[tp.posmode[tp.R + s - 1]]).nb;
-                if (nbo > nbocap) break;
-                if (chunk_need(tp.NB, stage_of(t, tp, s), s > 0, true, vt, U) <= work) return s;
+            for (int s = 0; s <= P.na && !ok; s++) {
+                if (s > 0) nbo *= LI(P.mode[s - 1], lt[P.mode[s - 1]]).nb;
+                if (nbo > slice_max) break;
+                int64_t stage = P.NBin;
+                for (int j = s; j < P.na; j++) stage *= LI(P.mode[j], lt[P.mode[j]]).nq;
+                ok = need(P, stage, s > 0) <= work;
             }
+        } else if (ok) {
+            ok = need(P, 0, false) <= work;
         }
-        return -1;
-    };
-
-    // pass 1: capacities
-    int gcap = 1, mcap = 1;
-    size_t img_total = 0;
-    TermPlan tp;
-    for (int64_t q = 0; q < T.n_terms; q++) {
-        plan_term(T.order[q], tp);
-        gcap = std::max(gcap, tp.gsize);
-        rec_units = std::max(rec_units, 3 + tp.na + (int)tp.prs.size() + ((int)tp.inds.size() + 1) / 2);
-        const uint8_t *lt = &T.levels[(size_t)T.order[q] * T.Dpad];
-        int mat = 0;
-        for (int j = 0; j < tp.na; j++) {
-            const LevelInfo &li = LI(tp.posmode[j], lt[tp.posmode[j]]);
-            mat += 2 * li.nb * li.nq + li.nb * li.nb;
-        }
-        mcap = std::max(mcap, mat);
-        img_total += (size_t)mat + tp.gsize;
+        F.fits = ok;
     }
-    const size_t head = ((size_t)rb * (mcap + gcap + 2 * nbocap) + 15) & ~(size_t)15;
-    const size_t hdr_static = 4 * 1024;  // per-group header in static shared memory (kHdrBytes)
-    const int64_t work_cta = ((int64_t)fbudget - (int64_t)head - 1024) / rb;
-    const int64_t work_warp = (((int64_t)fbudget - 4 * (int64_t)hdr_static) / 4 - (int64_t)head - 16) / rb;
-    if (work_cta < 2 * T.maxnb + 64 || (size_t)work_cta * rb < 16 * (3 + (size_t)kMaxD + 2 * (size_t)np)) {
-        T.fast = false;
-        return "";
-    }
-    T.matcap = std::max(T.matcap, mcap);
-    T.fgcap = gcap;
-    T.fnbocap = nbocap;
-    T.fwork_cta = (int)work_cta;
-    T.fwork_warp = (int)std::max<int64_t>(work_warp, 0);
-    T.fast_cap = T.fwork_cta;
-    // split: terms that fit a warp's quarter with a chunk of warp_vt vectors
-    // (unsliced, or sliced when warp-form slicing is on) run one per warp; the
-    // last term that does not ends the block-form prefix
-    const int warp_vt = T.warp_vt > 0 ? T.warp_vt : SG_WARP_VT;
-    const int warp_smax = SG_WARP_SLICE ? kMaxD : 0;
-    auto fits_warp = [&](int t, const TermPlan &tp) {
-        if (work_warp <= 0 || !ranks_fit(tp, work_warp)) return false;
-        if (!tp.grid) return chunk_need(tp.NB, 0, false, false, warp_vt, U) <= work_warp;
-        for (int s = 0; s <= std::min(warp_smax, tp.na - tp.R); s++)
-            if (chunk_need(tp.NB, stage_of(t, tp, s), s > 0, true, warp_vt, U) <= work_warp) return true;
-        return false;
-    };
-    int64_t n_big = 0;
-    for (int64_t q = 0; q < T.n_terms; q++) {
-        plan_term(T.order[q], tp);
-        if (!fits_warp(T.order[q], tp)) n_big = q + 1;
-    }
-    T.fn_big = (int)n_big;
-    // pass 2: records
-    T.fdesc.clear();
-    T.fdesc_off.assign(T.n_terms + 1, 0);
-    T.fdesccap = 0;
-    T.fimg.clear();
-    T.fimg.reserve(img_total);
-    T.fimg_off.assign(T.n_terms + 1, 0);
-    T.fvt_off.assign(T.n_terms + 1, 0);
-    T.frank_start.assign(T.n_terms + 1, 0);
-    int64_t rank_off = 0;
-    for (int64_t q = 0; q < T.n_terms; q++) {
-        const int t = T.order[q];
-        const uint8_t *lt = &T.levels[(size_t)t * T.Dpad];
-        plan_term(t, tp);
-        const bool big = q < n_big;
-        int sv = depth_for(t, tp, big ? work_cta : work_warp, big ? kMaxD : warp_smax);
-        if (sv < 0) { T.fast = false; T.fdesc.clear(); return ""; }  // generic kernel instead
-        int64_t nbo = 1;
-        for (int j = tp.R; j < tp.R + sv; j++) nbo *= LI(tp.posmode[j], lt[tp.posmode[j]]).nb;
-        if (nbo > nbocap) { T.fast = false; T.fdesc.clear(); return ""; }
-        const int na = tp.na;
-        // the term's shared-memory image: per position B, B^T W, H1 (+ induced), then G tables
-        for (int j = 0; j < na; j++) {
-            const int i = tp.posmode[j];
-            const LevelInfo &li = LI(i, lt[i]);
-            const size_t nbq = (size_t)li.nb * li.nq, nbb = (size_t)li.nb * li.nb;
-            T.fimg.insert(T.fimg.end(), T.tabd.begin() + li.offB, T.tabd.begin() + li.offB + nbq);
-            T.fimg.insert(T.fimg.end(), T.tabd.begin() + li.offBW, T.tabd.begin() + li.offBW + nbq);
-            const size_t h0 = T.fimg.size();
-            const int hb = T.h1off[(size_t)i * Lp + lt[i]];
-            T.fimg.insert(T.fimg.end(), T.ftab.begin() + hb, T.ftab.begin() + hb + nbb);
-            for (const FDescInd &d : tp.inds)
-                if (d.pos == j)
-                    for (size_t e = 0; e < nbb; e++) T.fimg[h0 + e] += T.ftab[d.ioff + e];
-        }
-        for (const FDescPair &pr : tp.prs) {
-            const size_t sz = (size_t)LI(tp.posmode[pr.pa], lt[tp.posmode[pr.pa]]).nq *
-                              LI(tp.posmode[pr.pb], lt[tp.posmode[pr.pb]]).nq;
-            T.fimg.insert(T.fimg.end(), T.ftab.begin() + pr.goff, T.ftab.begin() + pr.goff + sz);
-        }
-        T.fimg_off[q + 1] = (long long)T.fimg.size();
-        {
-            // inner-block table: its units per outer grid point, over every
-            // outer grid point (all slices), padded to 16 bytes
-            long long sz = 0;
-            if (tp.grid) {
-                long long ngo = 1;
-                for (int j = tp.R; j < na; j++) ngo *= LI(tp.posmode[j], lt[tp.posmode[j]]).nq;
-                const int nbi = (int)tp.NBIn;
-                sz = pad_elems((int64_t)mt_units(nbi, U) * mt_unit(nbi, U) * ngo, U);
-            }
-            T.fvt_off[q + 1] = T.fvt_off[q] + sz;
-        }
-        const int units = 3 + na + (int)tp.prs.size() + ((int)tp.inds.size() + 1) / 2;
-        const size_t u0 = T.fdesc.size();
-        T.fdesc.resize(u0 + units, int4{0, 0, 0, 0});
-        FDescHdr h{};
-        h.m = na; h.R = tp.R; h.NB = (int)tp.NB; h.coef = T.coefs[t];
-        h.s = sv; h.npair = (int)tp.prs.size(); h.nind = (int)tp.inds.size(); h.gsize = tp.gsize;
-        h.c0 = tp.c0; h.rank_off = rank_off;
-        put(T.fdesc, u0, 0, h);
-        for (int j = 0; j < na; j++) {
-            const int i = tp.posmode[j];
-            const LevelInfo &li = LI(i, lt[i]);
-            FDescPos e{(unsigned char)i, (unsigned char)lt[i], (unsigned char)li.nb, (unsigned char)li.nq,
-                       li.offB, li.offBW, T.h1off[(size_t)i * Lp + lt[i]]};
-            put(T.fdesc, u0 + 3 + j, 0, e);
-        }
-        for (size_t q2 = 0; q2 < tp.prs.size(); q2++) put(T.fdesc, u0 + 3 + na + q2, 0, tp.prs[q2]);
-        for (size_t q2 = 0; q2 < tp.inds.size(); q2++)
-            put(T.fdesc, u0 + 3 + na + tp.prs.size() + q2 / 2, 8 * (q2 % 2), tp.inds[q2]);
-        T.fdesc_off[q + 1] = (unsigned)(u0 + units);
-        T.fdesccap = std::max(T.fdesccap, units);
-        rank_off += tp.NB;
-        T.frank_start[q + 1] = rank_off;
-    }
-    if (T.fdesc.size() >= ((size_t)1 << 32)) return "fast-path records too large";
-    T.franks = rank_off;
-    return "";
+    return F;
 }
 
 }  // namespace sg

@@ -132,8 +132,13 @@ struct Solver {
     }
     // Davidson start: unit vectors of the r lowest harmonic energies (the
     // preconditioner's diagonal; ties by index), so the subspace overlaps the
-    // low-lying states from the first step.  False when no mode is split.
-    bool lowest_diagonal_block(double *X, int r)
+    // low-lying states from the first step; then, when `extra`, one vector with
+    // random components of every function, weighted towards the low energies.
+    // Symmetries of H leave sectors that no unit vector of the block lies in
+    // (chained Henon-Heiles: the parity of mode 0), and the row operator keeps
+    // them apart exactly: without that vector their states are never found.
+    // False when no mode is split.
+    bool lowest_diagonal_block(double *X, int r, bool extra)
     {
         const std::vector<double> &d = ctx->host.esplit;
         if ((int64_t)d.size() != n) return false;
@@ -144,8 +149,13 @@ struct Solver {
         for (int64_t i = 0; i < n; i++) idx[i] = i;
         std::partial_sort(idx.begin(), idx.begin() + r, idx.end(),
                           [&](int64_t a, int64_t b) { return d[a] < d[b] || (d[a] == d[b] && a < b); });
-        std::vector<double> h((size_t)r * n, 0.0);
+        std::vector<double> h((size_t)(r + extra) * n, 0.0);
         for (int j = 0; j < r; j++) h[(size_t)j * n + idx[j]] = 1.0;
+        uint64_t st = 0x5eed4321ull;
+        for (int64_t i = 0; extra && i < n; i++) {
+            const double w = 1.0 + (d[i] - d[idx[0]]);
+            h[(size_t)r * n + i] = ((double)(splitmix(st) >> 11) * 0x1.0p-53 - 0.5) / (w * w);
+        }
         ck(cudaMemcpyAsync(X, h.data(), sizeof(double) * h.size(), cudaMemcpyHostToDevice, s), "start copy");
         ck(cudaStreamSynchronize(s), "start sync");
         return true;
@@ -173,6 +183,11 @@ struct Solver {
 // Lanczos-type Krylov method with full reorthogonalisation and Rayleigh-Ritz).
 // Returns the number of converged eigenpairs; evals/resid on the host, the
 // Ritz vectors in evecs (device, nev x n) when not null.
+// Davidson carries b Ritz pairs beyond the nev wanted ones (its start block
+// and what it keeps at a restart hold them too), and expands once more along
+// their residuals when the nev have converged: a state that the basis has
+// missed so far, in a sector of its own or in a cluster closer than tol, then
+// takes its place among the nev and the iteration goes on.
 int block_eigs(Solver &S, int nev, int b, bool davidson, double tol, int max_it, const double *X0, int nx0,
                double *evals, double *evecs, double *resid)
 {
@@ -181,16 +196,19 @@ int block_eigs(Solver &S, int nev, int b, bool davidson, double tol, int max_it,
     // form keeps at most 320 vectors (its projected problem is solved densely)
     const int kmax = (int)std::min<int64_t>(n, davidson ? std::max(3 * nev, nev + 6 * b)
                                                         : std::min<int64_t>((int64_t)max_it * b + b, 320));
-    DBuf V((size_t)kmax * n), W((size_t)kmax * n), X((size_t)std::max(nev, b) * n), HX((size_t)std::max(nev, b) * n),
-        T((size_t)b * n), dd(kBlk + 8);
+    const int guard = davidson ? b : 0;
+    const size_t nx = (size_t)std::max(nev + guard, b);
+    DBuf V((size_t)kmax * n), W((size_t)kmax * n), X(nx * n), HX(nx * n), T((size_t)b * n), dd(kBlk + 8);
     std::vector<double> Tm;  // projected matrix, k x k
     int k = 0;
     // initial block
-    int r0 = std::min<int64_t>(b, n);
+    int r0 = davidson ? std::min(nev + b, kmax) : (int)std::min<int64_t>(b, n);
     if (X0 && nx0 > 0) {
         r0 = std::min(nx0, kmax);
         ck(cudaMemcpyAsync(V.p, X0, sizeof(double) * n * r0, cudaMemcpyDeviceToDevice, S.s), "x0 copy");
-    } else if (!davidson || !S.lowest_diagonal_block(V.p, r0)) {
+    } else if (const bool extra = r0 < kmax; davidson && S.lowest_diagonal_block(V.p, r0, extra)) {
+        r0 += extra;
+    } else {
         S.random_block(V.p, r0, 0x5eed1234ull);
     }
     r0 = S.orthonormalise(V.p, r0);
@@ -220,10 +238,11 @@ int block_eigs(Solver &S, int nev, int b, bool davidson, double tol, int max_it,
     extend(r0);
     std::vector<double> theta, Z;
     int nconv = 0;
+    bool checked = !davidson;  // the expansion after convergence has been made
     const int ne = std::min<int64_t>(nev, n);
     for (int it = 0; it < max_it; it++) {
         sym_eig(k, Tm, theta, Z);
-        const int nr = std::min(ne, k);
+        const int nr = std::min(ne + guard, k);
         // Ritz vectors and their images, residuals
         std::vector<double> Zr((size_t)k * nr);
         for (int i = 0; i < k; i++)
@@ -234,10 +253,12 @@ int block_eigs(Solver &S, int nev, int b, bool davidson, double tol, int max_it,
         std::vector<double> rn = S.norms(HX.p, nr);
         nconv = 0;
         while (nconv < nr && rn[nconv] <= tol * std::max(1.0, std::fabs(theta[nconv]))) nconv++;
-        for (int j = 0; j < nr; j++) { evals[j] = theta[j]; if (resid) resid[j] = rn[j]; }
-        if (nconv >= ne || k >= n) break;
+        for (int j = 0; j < std::min(nr, ne); j++) { evals[j] = theta[j]; if (resid) resid[j] = rn[j]; }
+        if (k >= n || (nconv >= ne && (checked || nconv >= nr))) break;
+        checked = nconv >= ne || !davidson;
         // new directions: the residuals of the first unconverged Ritz pairs
-        int r = std::min(b, nr - nconv);
+        // (of the wanted ones, or of those beyond them when these have converged)
+        int r = std::min(b, (nconv >= ne ? nr : std::min(ne, k)) - nconv);
         if (r <= 0) r = 1;
         if (!davidson && k + r > kmax) break;
         const int first = std::min(nconv, nr - r);
@@ -272,7 +293,7 @@ int block_eigs(Solver &S, int nev, int b, bool davidson, double tol, int max_it,
     }
     if (evecs) ck(cudaMemcpyAsync(evecs, X.p, sizeof(double) * n * std::min(ne, k), cudaMemcpyDeviceToDevice, S.s), "evecs");
     ck(cudaStreamSynchronize(S.s), "eigs sync");
-    return nconv;
+    return std::min(nconv, ne);
 }
 
 // Spectral interval of H_S for the Chebyshev propagator: a 40-vector Krylov

@@ -1,22 +1,16 @@
-// sg_tune (declared in include/smolyak.h): measured choice of the fast path's
-// term schedule for one context.
+// sg_tune (declared in include/smolyak.h): measured choice of the row kernels'
+// plan for one context.
 //
-// Three knobs of the host plan, searched one after another (coordinate
-// descent: each in turn over its candidates with the others at their best so
-// far), every candidate timed on real applies of the caller's block size:
-//   1. the slicing target: a term whose grid leaves room for fewer than that
-//      many vectors per chunk is sliced over its leading outer positions
-//      (smaller slices, fewer chunks), else it runs unsliced in more, smaller
-//      chunks;
-//   2. the block/warp split: terms that fit a quarter of a block's shared
-//      memory with that many vectors per chunk run one per warp (no block
-//      barriers, four terms per block), the larger ones one per block;
-//   3. the shared-memory budget of a block (the group size in memory): more
-//      per block means more vectors per chunk and fewer resident blocks.
-// Only the term records (slicing depths), the split point and the work-area
-// capacities change; M^B, the term images and the sizes of the inner-block
-// tables do not (the tables' layout follows the slicing and is rebuilt for
-// each candidate).
+// Three knobs, searched one after another (coordinate descent: each in turn
+// over its candidates with the others at their best so far), every candidate
+// timed on real applies of the caller's block size:
+//   1. vectors per lane (1, 2, 4): wider loads of the input copy and fewer
+//      lanes per row, against more rows in flight;
+//   2. rows per window, in units of 64 (1, 2, 4): how many rows a block takes,
+//      and how well it can pair long rows with short ones;
+//   3. the shared-memory budget of a block: a window ends early where its
+//      entries would exceed it.
+// A row's sum does not depend on the plan, so results do not either.
 #include <algorithm>
 #include <cmath>
 #include <limits>
@@ -40,31 +34,15 @@ struct Tuner {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t err = cudaSuccess;
 
-    // Re-plans the records for p and installs them (records, split, capacities,
-    // inner-block tables).  False when the plan cannot hold every term.
-    bool install(const Plan &p, size_t rec_bytes)
+    // Cuts the row operator into the windows of p.  False on a CUDA error.
+    bool install(const Plan &p)
     {
         sg::HostTables &T = ctx->host;
         T.slice_vt = p.slice_vt;
+        const bool same = ctx->rop.nwin > 0 && T.warp_vt == p.warp_vt && T.fbudget == p.smem_kb * 1024;
         T.warp_vt = p.warp_vt;
-        const int rb = ctx->fp32 ? 4 : 8;
-        const int budget = p.smem_kb * 1024;
-        const std::string e = sg::build_fast_descs(ctx->prob, ctx->fp32, &T, budget, rb);
-        if (!e.empty() || !T.fast || T.fdesc.size() * sizeof(int4) != rec_bytes) {
-            T.fast = true;
-            return false;
-        }
-        sg::FastParams &F = ctx->kp.fast;
-        T.fbudget = budget;
-        F.n_big = T.fn_big;
-        F.work_cta = T.fwork_cta;
-        F.work_warp = T.fwork_warp;
-        ctx->smem_bytes = sg::fast_smem_bytes(ctx->kp, ctx->fp32);
-        if ((err = cudaMemcpy(const_cast<int4 *>(F.desc), T.fdesc.data(), rec_bytes, cudaMemcpyHostToDevice)) !=
-                cudaSuccess ||
-            (err = sg::launch_build_mtab(ctx->kp, ctx->fp32, s)) != cudaSuccess ||
-            (err = cudaStreamSynchronize(s)) != cudaSuccess)
-            return false;
+        T.fbudget = p.smem_kb * 1024;
+        if (!same && (err = sg::build_rows(ctx)) != cudaSuccess) return false;
         ctx->plan_version++;
         return true;
     }
@@ -97,7 +75,7 @@ extern "C" sg_status sg_tune(sg_ctx *ctx, int nvec, int *slice_vt, double *ms_ou
     if (!sg_on_ctx_device(ctx)) { ctx->last_error = std::string("sg_tune: ") + "the current CUDA device is not the one the context was made on"; return SG_EINVAL; }
     if (nvec < 1 || nvec > 64) { ctx->last_error = "sg_tune: need 1 <= nvec <= 64"; return SG_EINVAL; }
     sg::HostTables &T = ctx->host;
-    if (!ctx->kp.fast.enabled) {  // generic kernel: no schedule to choose
+    if (!T.rows || !sg::term_form(ctx->prob, T).fits) {  // not a pair potential: the default plan
         if (slice_vt) *slice_vt = 0;
         if (ms_out) *ms_out = 0.0;
         return SG_OK;
@@ -121,9 +99,8 @@ extern "C" sg_status sg_tune(sg_ctx *ctx, int nvec, int *slice_vt, double *ms_ou
     if (e == cudaSuccess) e = cudaEventCreate(&tu.e0);
     if (e == cudaSuccess) e = cudaEventCreate(&tu.e1);
     sg_status st = e == cudaSuccess ? SG_OK : SG_ECUDA;
-    const size_t rec_bytes = T.fdesc.size() * sizeof(int4);
-    const Plan original{T.slice_vt > 0 ? T.slice_vt : (ctx->fp32 ? SG_F32_SLICE_VT : SG_F64_SLICE_VT),
-                        T.warp_vt > 0 ? T.warp_vt : SG_WARP_VT, T.fbudget / 1024};
+    const sg_precision prec = ctx->prob.prec;
+    const Plan original{sg::row_vt(T, prec), sg::row_window_units(T), sg::row_budget(T, prec) / 1024};
     Plan best = original;
     double best_ms = std::numeric_limits<double>::infinity();
     std::vector<Plan> tried;
@@ -131,7 +108,7 @@ extern "C" sg_status sg_tune(sg_ctx *ctx, int nvec, int *slice_vt, double *ms_ou
         for (const Plan &q : tried)
             if (q.slice_vt == p.slice_vt && q.warp_vt == p.warp_vt && q.smem_kb == p.smem_kb) return;
         tried.push_back(p);
-        if (st != SG_OK || !tu.install(p, rec_bytes)) {
+        if (st != SG_OK || !tu.install(p)) {
             if (tu.err != cudaSuccess) st = SG_ECUDA;
             return;
         }
@@ -147,7 +124,7 @@ extern "C" sg_status sg_tune(sg_ctx *ctx, int nvec, int *slice_vt, double *ms_ou
     const bool ok = std::isfinite(best_ms);
     const cudaError_t keep_err = tu.err;
     tu.err = cudaSuccess;
-    if (!tu.install(ok ? best : original, rec_bytes) && st == SG_OK) {
+    if (!tu.install(ok ? best : original) && st == SG_OK) {
         st = tu.err != cudaSuccess ? SG_ECUDA : SG_EINVAL;
         if (st == SG_EINVAL) ctx->last_error = "sg_tune: the kept plan could not be installed";
     }
@@ -170,9 +147,9 @@ extern "C" sg_status sg_tune_plan(const sg_ctx *ctx, int *slice_vt, int *warp_vt
 {
     if (!ctx) return SG_EINVAL;
     const sg::HostTables &T = ctx->host;
-    const bool fast = ctx->kp.fast.enabled || (!ctx->has_device && T.fast);
-    if (slice_vt) *slice_vt = fast ? (T.slice_vt > 0 ? T.slice_vt : (ctx->fp32 ? SG_F32_SLICE_VT : SG_F64_SLICE_VT)) : 0;
-    if (warp_vt) *warp_vt = fast ? (T.warp_vt > 0 ? T.warp_vt : SG_WARP_VT) : 0;
-    if (smem_kb) *smem_kb = fast ? T.fbudget / 1024 : 0;
+    const bool plan = T.rows && sg::term_form(ctx->prob, T).fits;
+    if (slice_vt) *slice_vt = plan ? sg::row_vt(T, ctx->prob.prec) : 0;
+    if (warp_vt) *warp_vt = plan ? sg::row_window_units(T) : 0;
+    if (smem_kb) *smem_kb = plan ? sg::row_budget(T, ctx->prob.prec) / 1024 : 0;
     return SG_OK;
 }
