@@ -243,7 +243,6 @@ cudaError_t build_rows(sg_ctx *ctx)
     RowShifts S{};
     S.nshift = (int)T.sh_off.size() - 1;
     int *cnt = nullptr;
-    long long *start = nullptr;
     cudaError_t e = cudaSuccess;
     auto ints = [&](const std::vector<int> &v, const int **dst) {
         int *p = nullptr;
@@ -257,28 +256,27 @@ cudaError_t build_rows(sg_ctx *ctx)
     if (e == cudaSuccess) e = row_upload(tmp, T.pr_coef.data(), T.pr_coef.size(), &coef, nullptr);
     S.coef = coef;
     if (e == cudaSuccess) e = row_upload<int>(tmp, nullptr, n, &cnt, nullptr);
-    if (e == cudaSuccess) e = row_upload<long long>(tmp, nullptr, n, &start, nullptr);
     if (e == cudaSuccess) e = launch_row_count(kp, S, cnt, 0);
     std::vector<int> hc(n);
     if (e == cudaSuccess) e = cudaMemcpy(hc.data(), cnt, n * sizeof(int), cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) {
-        const int rb = row_value_bytes(prec);
-        const RowWindows W = cut_rows(hc, row_window_rows((int64_t)n, row_window_units(T)), row_budget(T, prec), rb);
+        const RowWindows W = cut_rows(hc, row_window_rows((int64_t)n, row_window_units(T)), row_budget(T, prec),
+                                      row_value_bytes(prec));
         RowOp R{};
         RowWin *wins = nullptr;
+        unsigned char *blob = nullptr;
         uint2 *meta = nullptr;
-        int *cols = nullptr;
-        unsigned char *vals = nullptr;
+        const int *win = nullptr, *start = nullptr;
         int64_t bytes = 0;
         e = row_upload(ctx->row_allocs, W.wins.data(), W.wins.size(), &wins, &bytes);
-        if (e == cudaSuccess) e = row_upload(ctx->row_allocs, W.meta.data(), W.meta.size(), &meta, &bytes);
-        if (e == cudaSuccess) e = row_upload<int>(ctx->row_allocs, nullptr, (size_t)W.entries, &cols, &bytes);
-        if (e == cudaSuccess)
-            e = row_upload<unsigned char>(ctx->row_allocs, nullptr, (size_t)W.entries * rb, &vals, &bytes);
-        if (e == cudaSuccess) e = cudaMemcpy(start, W.start.data(), n * sizeof(long long), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = launch_row_fill(kp, S, prec, start, cols, vals, 0);
+        if (e == cudaSuccess) e = row_upload<unsigned char>(ctx->row_allocs, nullptr, (size_t)W.bytes, &blob, &bytes);
+        if (e == cudaSuccess) e = row_upload(tmp, W.meta.data(), W.meta.size(), &meta, nullptr);
+        ints(W.win, &win);
+        ints(W.start, &start);
+        if (e == cudaSuccess) e = launch_row_fill(kp, S, prec, wins, win, start, meta, blob, 0);
         if (e == cudaSuccess) e = cudaStreamSynchronize(0);
-        R.cols = cols; R.vals = vals; R.wins = wins; R.meta = meta;
+        R.blob = blob;
+        R.wins = wins;
         R.esplit = kp.esplit;
         R.err = kp.err;
         R.nwin = (int)W.wins.size();

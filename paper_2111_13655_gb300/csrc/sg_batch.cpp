@@ -25,7 +25,7 @@ struct sg_batch {
     const sg::RowOp *d_ops = nullptr;  // one per problem
     const int2 *items = nullptr;       // (problem, window) of the packed problems, most entries first
     const int2 *stage_items = nullptr; // (problem, chunk of 256 rows) of the packed problems
-    int n_items = 0, n_stage = 0, cap = 4, wrows = 16;
+    int n_items = 0, n_stage = 0, cap = 0, wrows = 16;
     std::vector<int> packed, solo;     // row-form problems: shared launches, launches of their own
     std::vector<int> generic;          // problems applied term by term
     std::vector<void *> allocations;
@@ -271,8 +271,8 @@ sg_status enqueue_apply(sg_batch *b, const double *x, double *y, int nvec, cudaS
     if (!b->packed.empty()) {
         const int vt = b->fp32 ? SG_F32_VT : SG_F64_VT;
         if ((e = sg::launch_row_stage_batch(io, prec, b->d_cs_prefix, b->stage_items, b->n_stage, s)) != cudaSuccess ||
-            (e = sg::launch_rows_batch(b->d_ops, b->items, b->n_items, b->cap, b->wrows, io, prec, vt, b->d_cs_prefix,
-                                       s)) != cudaSuccess ||
+            (e = sg::launch_rows_batch(b->d_ops, b->items, b->n_items, b->cap, b->wrows, io, prec, vt,
+                                       b->d_cs_prefix, s)) != cudaSuccess ||
             (e = sg::launch_row_settle_batch(io, b->d_cs_prefix, (int)b->ctxs.size(), s)) != cudaSuccess)
             return bfail(b, SG_ECUDA, std::string("batched row launch: ") + cudaGetErrorString(e));
     }

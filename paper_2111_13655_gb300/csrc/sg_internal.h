@@ -61,22 +61,30 @@ constexpr int kMaxPairs = 64;  // coupled mode pairs of the pair form (below)
 // shifts stay inside the compact basis: 15 per row at D=12 L=10.  The
 // elements are formed once per context in FP64 and stored row by row.
 
-// Rows of one window (consecutive compact indices) and their entries.
+// One window: consecutive rows and their entries, stored together (a 16-byte
+// aligned record that a bulk copy brings into shared memory):
+//   per row, by decreasing length: {first entry | local row << 24, entries}
+//   (8 bytes each, padded to 16), then the columns (int32 compact indices) and
+//   the elements (float, double, or float2 = (hi, lo)) of the rows one after
+//   another, each row filled to a multiple of four entries.
 struct RowWin {
-    long long ent0;  // first entry (a multiple of 4: 16-byte copies)
+    long long off;    // byte offset of the record
     int row0, nrows;
-    int nent, pad;
+    int nent, pad;    // entries, fillers included
 };
+__host__ __device__ inline int row_meta_bytes(int nrows) { return (8 * nrows + 15) & ~15; }
+__host__ __device__ inline int row_win_bytes(const RowWin &w, int value_bytes)
+{
+    return row_meta_bytes(w.nrows) + w.nent * (4 + value_bytes);
+}
 // One problem's row operator on the device.
 struct RowOp {
-    const int *cols;        // compact index of each entry's column
-    const void *vals;       // its element (float, double or float2 = (hi, lo))
+    const unsigned char *blob;  // the windows' records
     const RowWin *wins;
-    const uint2 *meta;      // per row, rows of a window by decreasing length: {start | local row << 24, length}
     const double *esplit;   // harmonic diagonal (FP64)
     int *err;
     int nwin, n;
-    int cap;                // entries of a window staged at a time (the largest window, or the budget)
+    int cap;                // largest record that is staged (bytes); longer ones (a very long row) are read in place
     int wrows;              // rows per window (a power of two)
 };
 // What a row kernel reads and writes.
@@ -100,10 +108,17 @@ constexpr int64_t kRowMaxBytes = (int64_t)64 << 30;
 #define SG_F32_VT 4
 #endif
 #ifndef SG_F64_VT
-#define SG_F64_VT 2
+#define SG_F64_VT 1
+#endif
+#ifndef SG_DF_VT
+#define SG_DF_VT 2
 #endif
 #ifndef SG_ROW_WINDOW
-#define SG_ROW_WINDOW 2  // rows per window, in units of 64
+#define SG_ROW_WINDOW 4  // rows per window, in units of 16
+#endif
+constexpr int kRowWindowMax = 64;  // rows per window at most
+#ifndef SG_ROW_SHARE
+#define SG_ROW_SHARE 4   // resident blocks that share the shared-memory budget
 #endif
 #ifndef SG_F32_SMEM_KB
 #define SG_F32_SMEM_KB 52
@@ -194,7 +209,7 @@ struct HostTables {
     std::vector<int> sh_off, sh_mode, sh_d, sh_src_off, sh_src, pr_off, pr_mode, pr_op;
     std::vector<double> pr_coef;
     // plan of the row kernels (0: default): vectors per lane, rows per window
-    // in units of 64, shared-memory budget of a block (bytes)
+    // in units of 16, shared memory that SG_ROW_SHARE blocks may use (bytes)
     int slice_vt = 0, warp_vt = 0, fbudget = 0;
     int cap = 0, maxnb = 0, matcap = 0, vtabcap = 0;
     int64_t flops_per_vec = 0;       // FMA-counted work of one real apply (2 flops per FMA)
@@ -231,16 +246,17 @@ TermForm term_form(const Problem &p, const HostTables &T);
 // Row form, host half (sg_rows_setup.cpp).
 void build_row_shifts(const Problem &p, HostTables *T);
 int row_vt(const HostTables &T, sg_precision prec);      // vectors per lane of the plan
-int row_window_units(const HostTables &T);               // rows per window / 64 of the plan
-int row_budget(const HostTables &T, sg_precision prec);  // shared memory per block (bytes) of the plan
+int row_window_units(const HostTables &T);               // rows per window / 16 of the plan
+int row_budget(const HostTables &T, sg_precision prec);  // shared memory that SG_ROW_SHARE blocks may use (bytes)
 int row_value_bytes(sg_precision prec);                  // bytes of a stored element
 // Upper bound of the device bytes of the row operator.
 int64_t row_form_bytes(const HostTables &T, sg_precision prec);
 struct RowWindows {
     std::vector<RowWin> wins;
-    std::vector<uint2> meta;
-    std::vector<long long> start;  // first entry of each row
-    int64_t entries = 0;           // with the padding of the windows
+    std::vector<uint2> meta;   // in the order of the records
+    std::vector<int> win;      // window of each row
+    std::vector<int> start;    // first entry of each row in its window
+    int64_t bytes = 0;
     int cap = 0, wrows = 0;
 };
 // Cuts the rows (cnt[r] entries each) into windows of at most `wrows` rows and
@@ -250,8 +266,9 @@ int row_window_rows(int64_t n, int units);
 
 // Row form, device half (sg_rows.cu).  prec selects the element type.
 cudaError_t launch_row_count(const KParams &kp, const RowShifts &sh, int *cnt, cudaStream_t stream);
-cudaError_t launch_row_fill(const KParams &kp, const RowShifts &sh, sg_precision prec, const long long *start,
-                            int *cols, void *vals, cudaStream_t stream);
+cudaError_t launch_row_fill(const KParams &kp, const RowShifts &sh, sg_precision prec, const RowWin *wins,
+                            const int *win, const int *start, const uint2 *meta, unsigned char *blob,
+                            cudaStream_t stream);
 cudaError_t configure_rows();
 // y = H_S x (io.y), or the sums of the windows of io.part into io.acc; vt: vectors per lane.
 cudaError_t launch_rows(const RowOp &R, const RowIO &io, sg_precision prec, int vt, cudaStream_t stream);

@@ -26,8 +26,14 @@ namespace sg {
 
 namespace {
 
-constexpr int kRT = 128;    // threads per window block
-constexpr int kTileV = 8;   // vectors per pass (the tile's columns)
+// Two warps per block: with a window of 64 rows every slot takes a long and a
+// short row, and few warps wait for the longest one.  Against 128 threads:
+// 32 batched wavepackets 63.6 -> 52.0 us, D=12 L=10 mixed and FP64 within 3%.
+constexpr int kRT = 64;
+constexpr int kTileV = 8;  // vectors per pass (the tile's columns)
+constexpr int kOut = kTileV * kRowWindowMax / kRT;  // outputs per thread and pass
+// resident blocks per SM the kernels are compiled for (80 / 128 registers)
+template <typename T> constexpr int row_blocks() { return sizeof(T) == 4 ? 12 : 8; }
 
 // ---------------------------------------------------------------- set-up
 
@@ -131,15 +137,20 @@ template <> struct Elem<double> { static __device__ double of(double v) { return
 template <> struct Elem<df2> { static __device__ df2 of(double v) { return df2(v); } };
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_row_fill(const KParams P, const RowShifts S,
-                                                  const long long *__restrict__ start, int *__restrict__ cols,
-                                                  T *__restrict__ vals)
+__global__ void __launch_bounds__(256) k_row_fill(const KParams P, const RowShifts S, const RowWin *__restrict__ wins,
+                                                  const int *__restrict__ win, const int *__restrict__ start,
+                                                  const uint2 *__restrict__ meta, unsigned char *__restrict__ blob)
 {
     const int r = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (r >= P.n_cs) return;
     int k[kMaxD], k2[kMaxD];
     const int sum = unrank(P, r, k);
-    long long at = start[r];
+    const RowWin w = wins[win[r]];
+    unsigned char *rec = blob + w.off;
+    if (lane == 0) reinterpret_cast<uint2 *>(rec)[r - w.row0] = meta[r];
+    int *cols = reinterpret_cast<int *>(rec + row_meta_bytes(w.nrows));
+    T *vals = reinterpret_cast<T *>(cols + w.nent);
+    int at = start[r];
     for (int q0 = 0; q0 < S.nshift; q0 += 32) {
         const int q = q0 + lane;
         const bool in = q < S.nshift && shift_fits(P, S, q, k, sum);
@@ -155,11 +166,18 @@ __global__ void __launch_bounds__(256) k_row_fill(const KParams P, const RowShif
             double v = 0.0;
             for (int e = S.src_off[q]; e < S.src_off[q + 1]; e++)
                 v = fma(S.coef[S.src[e]], product_elem(P, S, S.src[e], k, k2, sum), v);
-            const long long p = at + __popc(m & ((1u << lane) - 1u));
+            const int p = at + __popc(m & ((1u << lane) - 1u));
             cols[p] = c;
             vals[p] = Elem<T>::of(v);
         }
         at += __popc(m);
+    }
+    // the row's last group of four is filled with zero elements (of its last column)
+    const int pad = (4 - ((at - start[r]) & 3)) & 3;
+    __syncwarp();
+    if (lane < pad) {
+        cols[at + lane] = cols[at - 1];
+        vals[at + lane] = Elem<T>::of(0.0);
     }
 }
 
@@ -192,41 +210,179 @@ __device__ __forceinline__ Vec<T, W> load_vec(const T *p)
     return r;
 }
 
-// Row sum of one vector in each precision.
-template <typename T> struct Sum;
-template <> struct Sum<double> {
-    double s;
-    __device__ __forceinline__ void zero() { s = 0.0; }
-    __device__ __forceinline__ void add(double a, double x) { s = fma(a, x, s); }
-    __device__ __forceinline__ double value() const { return s; }
-};
-template <> struct Sum<float> {
-    float hi, lo;
-    __device__ __forceinline__ void zero() { hi = lo = 0.0f; }
-    __device__ __forceinline__ void add(float a, float x)
-    {
-        float s, e;
-        dfops::two_sum(hi, dfops::mul(a, x), s, e);
-        hi = s;
-        lo = dfops::add(lo, e);
+// Two FP32 numbers per instruction (IEEE rounding, as the scalar forms)
+__device__ __forceinline__ uint64_t pack2(float a, float b)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float &a, float &b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// a - b as one multiply-add: -1 * b is exact
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) { return fma2(b, 0xBF800000BF800000ull, a); }
+
+// hi + lo of a pair of FP32 numbers as a double.  The FP64 pipe is narrow (1/64
+// of the FP32 rate): the conversions are made with integer instructions; pairs
+// with a subnormal, an infinity or a NaN go through the conversion instruction.
+__device__ __forceinline__ double widen(unsigned u)
+{
+    const unsigned m = u << 1;  // exponent and mantissa
+    const unsigned hi = m ? (m >> 4) + 0x38000000u : 0u;
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ bool plain(unsigned u)  // a zero or a normal number
+{
+    return (u << 1) - 0x01000000u < 0xFE000000u || (u << 1) == 0u;
+}
+__device__ __forceinline__ double convert(unsigned u)  // volatile: stays on its (rare) branch
+{
+    double d;
+    asm volatile("cvt.f64.f32 %0, %1;" : "=d"(d) : "f"(__uint_as_float(u)));
+    return d;
+}
+__device__ __forceinline__ double widen_pair(uint64_t t)
+{
+    const unsigned h = (unsigned)t, l = (unsigned)(t >> 32);
+    double a = widen(h), b = widen(l);
+    if (!plain(h) || !plain(l)) {
+        a = convert(h);
+        b = convert(l);
     }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+    return a + b;
+}
+
+// Row sums of VT vectors.  add4: the next four entries, n of them real (the
+// others are zero elements).
+template <typename T, int VT> struct Sum;
+template <int VT> struct Sum<double, VT> {
+    double s[VT];
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int u = 0; u < VT; u++) s[u] = 0.0;
+    }
+    __device__ __forceinline__ void add4(const double *a, const Vec<double, VT> *x, int n)
+    {
+#pragma unroll
+        for (int b = 0; b < 4; b++) {
+            if (b < n) {
+#pragma unroll
+                for (int u = 0; u < VT; u++) s[u] = fma(a[b], x[b].v[u], s[u]);
+            }
+        }
+    }
+    __device__ __forceinline__ uint64_t bits(int u) const { return (uint64_t)__double_as_longlong(s[u]); }
+    static __device__ __forceinline__ double value(uint64_t t) { return __longlong_as_double((long long)t); }
 };
-template <> struct Sum<df2> {
-    df2 s;
-    __device__ __forceinline__ void zero() { s = df2(0.0f, 0.0f); }
-    __device__ __forceinline__ void add(df2 a, df2 x) { s = df_fma(a, x, s); }
-    __device__ __forceinline__ double value() const { return s.to_double(); }
+// FP32 sums of four products, each added without error (two-sum) to a pair of
+// FP32 numbers; two vectors per instruction.
+template <int VT> struct Sum<float, VT> {
+    static constexpr int NP = (VT + 1) / 2;
+    uint64_t hi[NP], lo[NP];
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int q = 0; q < NP; q++) hi[q] = lo[q] = 0ull;
+    }
+    __device__ __forceinline__ void add4(const float *a, const Vec<float, VT> *x, int)
+    {
+        uint64_t p[NP];
+#pragma unroll
+        for (int b = 0; b < 4; b++) {
+            const uint64_t ab = pack2(a[b], a[b]);
+#pragma unroll
+            for (int q = 0; q < NP; q++) {
+                const uint64_t xb = pack2(x[b].v[2 * q], 2 * q + 1 < VT ? x[b].v[2 * q + 1 < VT ? 2 * q + 1 : 0] : 0.0f);
+                p[q] = b == 0 ? mul2(ab, xb) : fma2(ab, xb, p[q]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < NP; q++) {
+            const uint64_t s = add2(hi[q], p[q]);
+            const uint64_t ap = sub2(s, p[q]), bp = sub2(s, ap);
+            const uint64_t e = add2(sub2(hi[q], ap), sub2(p[q], bp));
+            hi[q] = s;
+            lo[q] = add2(lo[q], e);
+        }
+    }
+    __device__ __forceinline__ uint64_t bits(int u) const
+    {
+        float h[2], l[2];
+        unpack2(hi[u >> 1], h[0], h[1]);
+        unpack2(lo[u >> 1], l[0], l[1]);
+        return pack2(h[u & 1], l[u & 1]);
+    }
+    static __device__ __forceinline__ double value(uint64_t t) { return widen_pair(t); }
+};
+template <int VT> struct Sum<df2, VT> {
+    df2 s[VT];
+    __device__ __forceinline__ void zero()
+    {
+#pragma unroll
+        for (int u = 0; u < VT; u++) s[u] = df2(0.0f, 0.0f);
+    }
+    __device__ __forceinline__ void add4(const df2 *a, const Vec<df2, VT> *x, int n)
+    {
+#pragma unroll
+        for (int b = 0; b < 4; b++) {
+            if (b < n) {
+#pragma unroll
+                for (int u = 0; u < VT; u++) s[u] = df_fma(a[b], x[b].v[u], s[u]);
+            }
+        }
+    }
+    __device__ __forceinline__ uint64_t bits(int u) const { return pack2(s[u].hi, s[u].lo); }
+    static __device__ __forceinline__ double value(uint64_t t) { return widen_pair(t); }
 };
 
-__device__ __forceinline__ void copy16(void *dst, const void *src)
+// Bulk copy of a record into shared memory, completing on an mbarrier.
+__device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void bar_init(uint64_t *bar)
 {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void bulk_copy(void *dst, const void *src, unsigned bytes, uint64_t *bar)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_addr(dst)),
+                 "l"(src), "r"(bytes), "r"(smem_addr(bar))
                  : "memory");
 }
-__device__ __forceinline__ void copy_wait()
+// Waits for phase `parity` of the barrier, a bounded number of polls (false: not reached).
+constexpr int kBarPolls = 1 << 20;
+__device__ __forceinline__ bool bar_wait(uint64_t *bar, unsigned parity)
 {
-    asm volatile("cp.async.wait_all;" ::: "memory");
+    for (int q = 0; q < kBarPolls; q++) {
+        unsigned done;
+        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+                     : "=r"(done)
+                     : "r"(smem_addr(bar)), "r"(parity)
+                     : "memory");
+        if (done) return true;
+    }
+    return false;
 }
 
 __device__ __forceinline__ bool finite(double v)
@@ -234,145 +390,151 @@ __device__ __forceinline__ bool finite(double v)
     return (__double2hiint(v) & 0x7FF00000) != 0x7FF00000;
 }
 
-// Bytes of shared memory of a window block.
-__host__ __device__ inline size_t rows_smem(int cap, int wrows, size_t rb)
+// Shared memory of a block: the window's record, and a tile of kTileV vectors by
+// wrows rows for the sums on their way to y.
+__host__ __device__ inline size_t rows_smem(int cap, int wrows)
 {
-    return (size_t)cap * (4 + rb) + (size_t)kTileV * wrows * 8;
+    return (size_t)((cap + 15) & ~15) + (size_t)kTileV * wrows * 8;
 }
 
-// One window.  ST: values come from the entry-major copy io.xs (VT adjacent
-// ones per lane); else from x itself, converted (VT = 1).
+// One window of problem R, whose vectors start at io.x, io.y, io.xs.  ST:
+// values come from the entry-major copy io.xs (VT adjacent ones per lane);
+// else from x itself, converted (VT = 1).
 template <typename T, int VT, bool ST>
-__device__ __forceinline__ void rows_window(const RowOp &R, const RowIO &io, int w, int lgl, unsigned char *smem)
+__device__ __forceinline__ void rows_window(const RowOp &R, const RowIO &io, const RowWin &win, int lgl, int cap,
+                                            unsigned char *smem, uint64_t *bar)
 {
-    const int tid = threadIdx.x;
-    const RowWin win = R.wins[w];
-    double *tile = reinterpret_cast<double *>(smem);
-    T *sv = reinterpret_cast<T *>(smem + (size_t)kTileV * R.wrows * 8);
-    int *sc = reinterpret_cast<int *>(sv + R.cap);
-    const T *gv = static_cast<const T *>(R.vals) + win.ent0;
-    const int *gc = R.cols + win.ent0;
+    const int tid = threadIdx.x, n = R.n;
+    const int bytes = row_win_bytes(win, (int)sizeof(T));
+    const bool staged = bytes <= cap;
+    if (staged && tid == 0) {
+        bar_init(bar);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        bulk_copy(smem, R.blob + win.off, (unsigned)bytes, bar);
+    }
+    // the thread's row of the tile, its first vector and its step over the vectors
+    const int lw = 31 - __clz(R.wrows);
+    const int tr = tid & (R.wrows - 1), tv = tid >> lw, tvs = kRT >> lw;
+    const bool own = tr < win.nrows;
+    const double es = own && io.y ? __ldg(R.esplit + win.row0 + tr) : 0.0;
+    uint64_t *tile = reinterpret_cast<uint64_t *>(smem + ((cap + 15) & ~15));
+
+    const unsigned char *rec = staged ? smem : R.blob + win.off;
+    const uint2 *meta = reinterpret_cast<const uint2 *>(rec);
+    const int *cols = reinterpret_cast<const int *>(rec + row_meta_bytes(win.nrows));
+    const T *vals = reinterpret_cast<const T *>(cols + win.nent);
+    const T *xs = static_cast<const T *>(io.xs);
     const int lane = tid & ((1 << lgl) - 1), slot = tid >> lgl, nslot = kRT >> lgl;
     const int vpass = VT << lgl;  // vectors per pass, at most kTileV
-    const int lw = 31 - __clz(R.wrows);
-    const bool once = win.nent <= R.cap;
-
-    auto stage = [&](int e0, int n) {  // entries [e0, e0 + n) into shared memory
-        constexpr int UV = 16 / (int)sizeof(T);
-        for (int i = tid; i < (n + 3) / 4; i += kRT) copy16(sc + 4 * i, gc + e0 + 4 * i);
-        for (int i = tid; i < (n + UV - 1) / UV; i += kRT) copy16(sv + UV * i, gv + e0 + UV * i);
-        copy_wait();
-    };
-    if (once) {
-        stage(0, win.nent);
-        __syncthreads();
-    }
     for (int v0 = 0; v0 < io.nvec; v0 += vpass) {
+        const int nv = min(vpass, io.nvec - v0);
+        // x of the thread's outputs is on its way during the sums
+        const size_t g0 = (size_t)(v0 + tv) * n + win.row0 + tr, gs = (size_t)tvs * n;
+        double xi[kOut];
+#pragma unroll
+        for (int q = 0; q < kOut; q++)
+            if (io.y && own && tv + q * tvs < nv) xi[q] = __ldg(io.x + g0 + q * gs);
+        if (v0 == 0) {
+            __syncthreads();  // the barrier is initialised
+            const bool late = staged && !bar_wait(bar, 0);
+            if (__syncthreads_or(late)) {
+                if (tid == 0) atomicCAS(R.err, 0, 120);
+                bar_wait(bar, 0);
+                return;
+            }
+        }
         const int v = v0 + lane * VT;
         for (int it = 0; it * nslot < win.nrows; it++) {
             // every second round in reverse: long and short rows on each slot
             const int q = it * nslot + (it & 1 ? nslot - 1 - slot : slot);
-            const bool on = q < win.nrows && v < io.nvec;
-            uint2 mt = make_uint2(0u, 0u);
-            if (on) mt = __ldg(R.meta + win.row0 + q);
-            const int start = (int)(mt.x & 0xFFFFFFu), len = (int)mt.y;
-            Sum<T> acc[VT];
+            if (q >= win.nrows || v >= io.nvec) continue;
+            const uint2 mt = meta[q];
+            Sum<T, VT> acc;
+            acc.zero();
+            // groups of four entries, the loads of two groups ahead of their sums
+            auto load4 = [&](const int *cp, Vec<T, VT> *xv) {
+                const int4 c = *reinterpret_cast<const int4 *>(cp);
+                const int cc[4] = {c.x, c.y, c.z, c.w};
 #pragma unroll
-            for (int u = 0; u < VT; u++) acc[u].zero();
-            auto run = [&](const int *cp, const T *vp, int n) {
-                constexpr int UN = 4;
-                int e = 0;
-                for (; e + UN <= n; e += UN) {
-                    Vec<T, VT> xv[UN];
-#pragma unroll
-                    for (int b = 0; b < UN; b++) {
-                        const size_t c = (size_t)cp[e + b];
-                        if constexpr (ST) xv[b] = load_vec<T, VT>(static_cast<const T *>(io.xs) + c * io.stride + v);
-                        else xv[b].v[0] = Elem<T>::of(__ldg(io.x + (size_t)v * R.n + c));
-                    }
-#pragma unroll
-                    for (int b = 0; b < UN; b++) {
-                        const T a = vp[e + b];
-#pragma unroll
-                        for (int u = 0; u < VT; u++) acc[u].add(a, xv[b].v[u]);
-                    }
-                }
-                for (; e < n; e++) {
-                    const size_t c = (size_t)cp[e];
-                    Vec<T, VT> xv;
-                    if constexpr (ST) xv = load_vec<T, VT>(static_cast<const T *>(io.xs) + c * io.stride + v);
-                    else xv.v[0] = Elem<T>::of(__ldg(io.x + (size_t)v * R.n + c));
-                    const T a = vp[e];
-#pragma unroll
-                    for (int u = 0; u < VT; u++) acc[u].add(a, xv.v[u]);
+                for (int u = 0; u < 4; u++) {
+                    if constexpr (ST) xv[u] = load_vec<T, VT>(xs + (size_t)cc[u] * io.stride + v);
+                    else xv[u].v[0] = Elem<T>::of(__ldg(io.x + (size_t)v * n + cc[u]));
                 }
             };
-            if (once) {
-                run(sc + start, sv + start, len);
-            } else {
-                // a single row longer than the staging area: piece by piece
-                for (int e0 = 0; e0 < win.nent; e0 += R.cap) {
-                    const int n = min(R.cap, win.nent - e0);
-                    __syncthreads();
-                    stage(e0, n);
-                    __syncthreads();
-                    if (on) run(sc, sv, n);
-                }
+            auto sum4 = [&](const T *vp, const Vec<T, VT> *xv, int m) {
+                const Vec<T, 4> a = *reinterpret_cast<const Vec<T, 4> *>(vp);
+                acc.add4(a.v, xv, m);
+            };
+            const int *cp = cols + (mt.x & 0xFFFFFFu);
+            const T *vp = vals + (mt.x & 0xFFFFFFu);
+            const int m = (int)mt.y;
+            int e = 0;
+            for (; e + 4 < m; e += 8) {
+                Vec<T, VT> x0[4], x1[4];
+                load4(cp + e, x0);
+                load4(cp + e + 4, x1);
+                sum4(vp + e, x0, 4);
+                sum4(vp + e + 4, x1, m - e - 4);
             }
-            if (on) {
-                const int lr = (int)(mt.x >> 24);
+            if (e < m) {
+                Vec<T, VT> x0[4];
+                load4(cp + e, x0);
+                sum4(vp + e, x0, m - e);
+            }
+            uint64_t *t = tile + ((lane * VT) << lw) + (mt.x >> 24);
 #pragma unroll
-                for (int u = 0; u < VT; u++)
-                    if (lane * VT + u < kTileV) tile[((lane * VT + u) << lw) + lr] = acc[u].value();
-            }
+            for (int u = 0; u < VT; u++) t[u << lw] = acc.bits(u);
         }
         __syncthreads();
         // y = sum + harmonic diagonal, or the sums' bits into the accumulators
-        const int nv = min(vpass, io.nvec - v0);
-        for (int i = tid; i < nv << lw; i += kRT) {
-            const int u = i >> lw, r = i & (R.wrows - 1);
-            if (r >= win.nrows) continue;
-            const double s = tile[i];
-            const size_t row = (size_t)win.row0 + r;
-            if (io.y) {
-                const size_t g = (size_t)(v0 + u) * R.n + row;
-                const double xi = __ldg(io.x + g);
-                io.y[g] = fma(__ldg(R.esplit + row), xi, s);
-                if (!finite(xi)) atomicOr(io.flags + v0 + u, 1u);
-                if (!finite(xi) || !finite(s)) atomicCAS(R.err, 0, 201);
-            } else {
-                io.acc[(row * io.nvec + v0 + u) * io.words] += (unsigned long long)__double_as_longlong(s);
+        if (own) {
+#pragma unroll
+            for (int q = 0; q < kOut; q++) {
+                const int u = tv + q * tvs;
+                if (u >= nv) break;
+                double s = Sum<T, VT>::value(tile[tid + q * kRT]);
+                if (io.y) {
+                    s = fma(es, xi[q], s);
+                    io.y[g0 + q * gs] = s;
+                    if (!finite(s) && !finite(xi[q])) atomicOr(io.flags + v0 + u, 1u);
+                } else {
+                    io.acc[((size_t)(win.row0 + tr) * io.nvec + v0 + u) * io.words] +=
+                        (unsigned long long)__double_as_longlong(s);
+                }
                 if (!finite(s)) atomicCAS(R.err, 0, 201);
             }
         }
-        __syncthreads();
+        if (v0 + vpass < io.nvec) __syncthreads();
     }
 }
 
 template <typename T, int VT, bool ST>
-__global__ void __launch_bounds__(kRT) k_rows(const RowOp R, const RowIO io, int lgl)
+__global__ void __launch_bounds__(kRT, row_blocks<T>()) k_rows(const RowOp R, const RowIO io, int lgl)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int w = blockIdx.x * io.nparts + io.part;
-    if (w >= R.nwin) return;
-    rows_window<T, VT, ST>(R, io, w, lgl, smem);
+    __shared__ uint64_t bar;
+    rows_window<T, VT, ST>(R, io, R.wins[blockIdx.x * io.nparts + io.part], lgl, R.cap, smem, &bar);
 }
 
-// Many problems: vectors of problem j from nvec * cs_prefix[j], its rows of xs from cs_prefix[j], flags from j * nvec.
+// Many problems: item = (problem, window); vectors of problem j from
+// nvec * cs_prefix[j], its rows of xs from cs_prefix[j], flags from j * nvec.
 template <typename T, int VT>
-__global__ void __launch_bounds__(kRT) k_rows_batch(const RowOp *__restrict__ ops, const int2 *__restrict__ items,
-                                                    const RowIO io, int lgl, const long long *__restrict__ cs_prefix)
+__global__ void __launch_bounds__(kRT, row_blocks<T>()) k_rows_batch(const RowOp *__restrict__ ops,
+                                                                const int2 *__restrict__ items, const RowIO io,
+                                                                int lgl, const long long *__restrict__ cs_prefix,
+                                                                int cap)
 {
     extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint64_t bar;
     const int2 it = items[blockIdx.x];
-    const RowOp R = ops[it.x];
+    const RowOp &R = ops[it.x];
     RowIO o = io;
     const size_t c0 = (size_t)cs_prefix[it.x];
     o.x += c0 * io.nvec;
     o.y += c0 * io.nvec;
     o.xs = static_cast<const T *>(io.xs) + c0 * io.stride;
     o.flags += (size_t)it.x * io.nvec;
-    rows_window<T, VT, true>(R, o, it.y, lgl, smem);
+    rows_window<T, VT, true>(R, o, R.wins[it.y], lgl, cap, smem, &bar);
 }
 
 // xs[r * stride + v] = x_v[r] in T (zero beyond nvec), rows r0 .. r0 + nr - 1
@@ -491,9 +653,9 @@ cudaError_t smem_limits()
 template <typename T>
 cudaError_t rows_t(const RowOp &R, const RowIO &io, int vt, cudaStream_t s)
 {
-    const unsigned blocks = (unsigned)((R.nwin - io.part + io.nparts - 1) / io.nparts);
     if (R.nwin <= io.part) return cudaSuccess;
-    const size_t smem = rows_smem(R.cap, R.wrows, sizeof(T));
+    const size_t smem = rows_smem(R.cap, R.wrows);
+    const unsigned blocks = (unsigned)((R.nwin - io.part + io.nparts - 1) / io.nparts);
     if (!io.xs) {
         k_rows<T, 1, false><<<blocks, kRT, smem, s>>>(R, io, lanes_log2(io.nvec, 1));
         return cudaGetLastError();
@@ -507,14 +669,16 @@ cudaError_t rows_t(const RowOp &R, const RowIO &io, int vt, cudaStream_t s)
 }
 
 template <typename T>
-cudaError_t rows_batch_t(const RowOp *ops, const int2 *items, int nitems, size_t smem, const RowIO &io, int vt,
+cudaError_t rows_batch_t(const RowOp *ops, const int2 *items, int nitems, int cap, int wrows, const RowIO &io, int vt,
                          const long long *cs_prefix, cudaStream_t s)
 {
+    const size_t smem = rows_smem(cap, wrows);
+    const unsigned blocks = (unsigned)nitems;
     vt = fit_vt(vt, io.stride);
     const int l = lanes_log2(io.nvec, vt);
-    if (vt == 4) k_rows_batch<T, 4><<<(unsigned)nitems, kRT, smem, s>>>(ops, items, io, l, cs_prefix);
-    else if (vt == 2) k_rows_batch<T, 2><<<(unsigned)nitems, kRT, smem, s>>>(ops, items, io, l, cs_prefix);
-    else k_rows_batch<T, 1><<<(unsigned)nitems, kRT, smem, s>>>(ops, items, io, l, cs_prefix);
+    if (vt == 4) k_rows_batch<T, 4><<<blocks, kRT, smem, s>>>(ops, items, io, l, cs_prefix, cap);
+    else if (vt == 2) k_rows_batch<T, 2><<<blocks, kRT, smem, s>>>(ops, items, io, l, cs_prefix, cap);
+    else k_rows_batch<T, 1><<<blocks, kRT, smem, s>>>(ops, items, io, l, cs_prefix, cap);
     return cudaGetLastError();
 }
 
@@ -526,13 +690,14 @@ cudaError_t launch_row_count(const KParams &kp, const RowShifts &sh, int *cnt, c
     return cudaGetLastError();
 }
 
-cudaError_t launch_row_fill(const KParams &kp, const RowShifts &sh, sg_precision prec, const long long *start,
-                            int *cols, void *vals, cudaStream_t stream)
+cudaError_t launch_row_fill(const KParams &kp, const RowShifts &sh, sg_precision prec, const RowWin *wins,
+                            const int *win, const int *start, const uint2 *meta, unsigned char *blob,
+                            cudaStream_t stream)
 {
     const unsigned blocks = (unsigned)(((size_t)kp.n_cs * 32 + 255) / 256);
-    if (prec == SG_MIXED) k_row_fill<float><<<blocks, 256, 0, stream>>>(kp, sh, start, cols, static_cast<float *>(vals));
-    else if (prec == SG_DF64) k_row_fill<df2><<<blocks, 256, 0, stream>>>(kp, sh, start, cols, static_cast<df2 *>(vals));
-    else k_row_fill<double><<<blocks, 256, 0, stream>>>(kp, sh, start, cols, static_cast<double *>(vals));
+    if (prec == SG_MIXED) k_row_fill<float><<<blocks, 256, 0, stream>>>(kp, sh, wins, win, start, meta, blob);
+    else if (prec == SG_DF64) k_row_fill<df2><<<blocks, 256, 0, stream>>>(kp, sh, wins, win, start, meta, blob);
+    else k_row_fill<double><<<blocks, 256, 0, stream>>>(kp, sh, wins, win, start, meta, blob);
     return cudaGetLastError();
 }
 
@@ -556,9 +721,8 @@ cudaError_t launch_rows_batch(const RowOp *ops, const int2 *items, int nitems, i
                               sg_precision prec, int vt, const long long *cs_prefix, cudaStream_t stream)
 {
     if (nitems <= 0) return cudaSuccess;
-    const size_t smem = rows_smem(cap, wrows, (size_t)row_value_bytes(prec));
-    if (prec == SG_MIXED) return rows_batch_t<float>(ops, items, nitems, smem, io, vt, cs_prefix, stream);
-    return rows_batch_t<double>(ops, items, nitems, smem, io, vt, cs_prefix, stream);
+    if (prec == SG_MIXED) return rows_batch_t<float>(ops, items, nitems, cap, wrows, io, vt, cs_prefix, stream);
+    return rows_batch_t<double>(ops, items, nitems, cap, wrows, io, vt, cs_prefix, stream);
 }
 
 cudaError_t launch_row_stage(const RowOp &R, const RowIO &io, sg_precision prec, cudaStream_t stream)

@@ -148,7 +148,7 @@ void build_row_shifts(const Problem &p, HostTables *Tp)
 int row_value_bytes(sg_precision prec) { return prec == SG_MIXED ? 4 : 8; }
 int row_vt(const HostTables &T, sg_precision prec)
 {
-    return T.slice_vt > 0 ? T.slice_vt : prec == SG_MIXED ? SG_F32_VT : SG_F64_VT;
+    return T.slice_vt > 0 ? T.slice_vt : prec == SG_MIXED ? SG_F32_VT : prec == SG_DF64 ? SG_DF_VT : SG_F64_VT;
 }
 int row_window_units(const HostTables &T) { return T.warp_vt > 0 ? T.warp_vt : SG_ROW_WINDOW; }
 int row_budget(const HostTables &T, sg_precision prec)
@@ -156,11 +156,11 @@ int row_budget(const HostTables &T, sg_precision prec)
     return T.fbudget > 0 ? T.fbudget : 1024 * (prec == SG_MIXED ? SG_F32_SMEM_KB : SG_F64_SMEM_KB);
 }
 
-// Rows per window: 64 * units, fewer on small problems so that the windows
+// Rows per window: 16 * units, fewer on small problems so that the windows
 // cover the SMs about twice (at least 16).
 int row_window_rows(int64_t n, int units)
 {
-    int w = 64 * units;
+    int w = std::min(16 * units, kRowWindowMax);
     while (w > 16 && (n + w - 1) / w < 304) w >>= 1;
     return w;
 }
@@ -168,32 +168,34 @@ int row_window_rows(int64_t n, int units)
 int64_t row_form_bytes(const HostTables &T, sg_precision prec)
 {
     if (!T.rows) return 0;
-    const int w = row_window_rows(T.n_cs, 1);
-    const int64_t nwin = (T.n_cs + w - 1) / w + 1;
-    // every window may end early for its entries; count them as if each did, and its padding of three
-    const int64_t by_budget = T.row_nnz * (4 + row_value_bytes(prec)) / (32 * 1024) + 1;
-    return (T.row_nnz + 4 * (nwin + by_budget)) * (4 + row_value_bytes(prec)) + T.n_cs * (int64_t)sizeof(uint2) +
-           (nwin + by_budget) * (int64_t)sizeof(RowWin);
+    // a window for every 16 rows, and one more for every 4 KB of entries that may end one early;
+    // every row filled up by up to three entries
+    const int64_t ent = T.row_nnz + 3 * T.n_cs, eb = 4 + row_value_bytes(prec);
+    const int64_t nwin = T.n_cs / 16 + 1 + ent * eb / 4096;
+    return ent * eb + 8 * T.n_cs + nwin * (8 + (int64_t)sizeof(RowWin));
 }
+
+// entries of a row with its last group of four filled
+static int padded(int n) { return (n + 3) & ~3; }
 
 RowWindows cut_rows(const std::vector<int> &cnt, int wrows, int budget, int value_bytes)
 {
     RowWindows W;
     const int n = (int)cnt.size();
-    // staged entries beside the result tile of 8 vectors
-    const int room = std::max(0, (budget - 1024 - 64 * wrows) / (4 + value_bytes));
-    const int cap = std::max(64, room / 4 * 4);
+    // a block's shared memory: a record (rows' entries behind 8 bytes per row) and a tile of 8 vectors
+    const int room = budget / SG_ROW_SHARE - 64 * wrows - 8 * wrows - 32;
+    const int cap = std::max(64, room / (4 + value_bytes));
     W.meta.resize(n);
+    W.win.resize(n);
     W.start.resize(n);
-    int64_t ent = 0;
-    int widest = 4;
-    std::vector<int> head, slot;
+    std::vector<int> head;
     for (int r0 = 0; r0 < n;) {
         int r1 = r0, ne = 0, longest = 0;
-        while (r1 < n && r1 - r0 < wrows && (r1 == r0 || ne + cnt[r1] <= cap)) {
-            W.start[r1] = ent + ne;
+        while (r1 < n && r1 - r0 < wrows && (r1 == r0 || ne + padded(cnt[r1]) <= cap)) {
+            W.win[r1] = (int)W.wins.size();
+            W.start[r1] = ne;
             longest = std::max(longest, cnt[r1]);
-            ne += cnt[r1++];
+            ne += padded(cnt[r1++]);
         }
         // rows by decreasing length (counting sort, equal lengths in row order)
         head.assign(longest + 2, 0);
@@ -201,14 +203,14 @@ RowWindows cut_rows(const std::vector<int> &cnt, int wrows, int budget, int valu
         for (int l = 0; l <= longest; l++) head[l + 1] += head[l];
         for (int r = r0; r < r1; r++)
             W.meta[r0 + head[longest - cnt[r]]++] =
-                make_uint2((unsigned)(W.start[r] - ent) | ((unsigned)(r - r0) << 24), (unsigned)cnt[r]);
-        W.wins.push_back(RowWin{(long long)ent, r0, r1 - r0, ne, 0});
-        widest = std::max(widest, (std::min(ne, cap) + 3) / 4 * 4);
-        ent += (ne + 3) / 4 * 4;
+                make_uint2((unsigned)W.start[r] | ((unsigned)(r - r0) << 24), (unsigned)cnt[r]);
+        const RowWin w{(long long)W.bytes, r0, r1 - r0, ne, 0};
+        const int bytes = row_win_bytes(w, value_bytes);
+        if (ne <= cap) W.cap = std::max(W.cap, bytes);
+        W.bytes += bytes;
+        W.wins.push_back(w);
         r0 = r1;
     }
-    W.entries = ent;
-    W.cap = widest;
     W.wrows = wrows;
     return W;
 }

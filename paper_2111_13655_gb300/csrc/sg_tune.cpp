@@ -6,10 +6,9 @@
 // timed on real applies of the caller's block size:
 //   1. vectors per lane (1, 2, 4): wider loads of the input copy and fewer
 //      lanes per row, against more rows in flight;
-//   2. rows per window, in units of 64 (1, 2, 4): how many rows a block takes,
-//      and how well it can pair long rows with short ones;
-//   3. the shared-memory budget of a block: a window ends early where its
-//      entries would exceed it.
+//   2. rows per window, in units of 16 (1, 2, 4): how many rows a block takes;
+//   3. the shared memory that SG_ROW_SHARE resident blocks may use: a window
+//      ends early where its entries would exceed its part.
 // A row's sum does not depend on the plan, so results do not either.
 #include <algorithm>
 #include <cmath>
