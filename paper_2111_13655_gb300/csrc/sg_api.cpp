@@ -61,6 +61,8 @@ void free_all(sg_ctx *ctx)
     if (ctx->stage_x) cudaFree(ctx->stage_x);
     if (ctx->stage_y) cudaFree(ctx->stage_y);
     ctx->stage_x = ctx->stage_y = nullptr;
+    if (ctx->pin) cudaFreeHost(ctx->pin);
+    ctx->pin = nullptr;
     free_workspace(ctx);
 }
 

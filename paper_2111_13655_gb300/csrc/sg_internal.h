@@ -339,6 +339,8 @@ struct sg_ctx {
     unsigned long long *acc = nullptr;
     long long *maxbits = nullptr;
     int acc_nvec = 0;
+    double *pin = nullptr;    // pinned host memory of the solvers' small matrices
+    size_t pin_doubles = 0;
     int plan_version = 0;     // incremented whenever sg_tune installs a plan
     std::string last_error;
 };

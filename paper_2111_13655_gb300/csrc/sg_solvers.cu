@@ -74,10 +74,56 @@ __global__ void k_gram_final(const double *__restrict__ partial, int nchunk, int
     C[q] = v;
 }
 
-// out[j][e] = beta * out[j][e] + alpha * sum_i V[i][e] S[i][j]   (S: k x r, row-major, device)
-__global__ void __launch_bounds__(256) k_combine(const double *__restrict__ V, int k, const double *__restrict__ S,
-                                                 int r, double alpha, double beta, double *__restrict__ out,
-                                                 int64_t n)
+// Vectors of at most kSmallN entries: the kernels above would put the whole
+// product on a few SMs, whose FP64 pipe (1/64 of the FP32 rate) then sets the
+// time (n = 1,001, 34 x 8: 20 us).  One block per inner product, and one column
+// per block of 64 entries, spread it over all SMs.
+constexpr int64_t kSmallN = 8192;
+constexpr int kDotThreads = 128;
+
+// Sum over the block, in a fixed order; the result in every thread.
+template <int THREADS>
+__device__ __forceinline__ double block_sum(double v)
+{
+    __shared__ double red[THREADS / 32];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double t = red[0];
+#pragma unroll
+    for (int w = 1; w < THREADS / 32; w++) t += red[w];
+    return t;
+}
+
+// C[i][j] = sum_e A_i[e] B_j[e], block (i, j)
+__global__ void __launch_bounds__(kDotThreads) k_gram_small(const double *__restrict__ A, const double *__restrict__ B,
+                                                            int n, double *__restrict__ C)
+{
+    const double *a = A + (size_t)blockIdx.x * n, *b = B + (size_t)blockIdx.y * n;
+    double v = 0.0;
+#pragma unroll 4
+    for (int e = threadIdx.x; e < n; e += kDotThreads) v = fma(a[e], b[e], v);
+    v = block_sum<kDotThreads>(v);
+    if (threadIdx.x == 0) C[blockIdx.x * gridDim.y + blockIdx.y] = v;
+}
+
+// out[j][e] = base[j][e] + alpha * sum_i V[i][e] S[i][j] (base nullptr: 0), column j = blockIdx.y
+__global__ void __launch_bounds__(64) k_combine_small(const double *__restrict__ V, int k, const double *__restrict__ S,
+                                                      int r, double alpha, const double *base, double *out, int n)
+{
+    const int e = blockIdx.x * 64 + threadIdx.x, j = blockIdx.y;
+    if (e >= n) return;
+    double acc = 0.0;
+#pragma unroll 4
+    for (int i = 0; i < k; i++) acc = fma(V[(size_t)i * n + e], __ldg(S + i * r + j), acc);
+    const size_t o = (size_t)j * n + e;
+    out[o] = (base ? base[o] : 0.0) + alpha * acc;
+}
+
+// out = base + alpha * V S for longer vectors (one block column of up to kMaxCols outputs)
+__global__ void __launch_bounds__(256) k_combine_base(const double *__restrict__ V, int k, const double *__restrict__ S,
+                                                      int r, double alpha, const double *base, double *out, int64_t n)
 {
     extern __shared__ double Ss[];
     for (int q = threadIdx.x; q < k * r; q += blockDim.x) Ss[q] = S[q];
@@ -93,10 +139,117 @@ __global__ void __launch_bounds__(256) k_combine(const double *__restrict__ V, i
                 if (j < r) acc[j] = fma(v, Ss[i * r + j], acc[j]);
         }
         for (int j = 0; j < r; j++) {
-            double *o = out + (size_t)j * n + e;
-            *o = (beta == 0.0 ? 0.0 : beta * *o) + alpha * acc[j];
+            const size_t o = (size_t)j * n + e;
+            out[o] = (base ? base[o] : 0.0) + alpha * acc[j];
         }
     }
+}
+
+// Cholesky G = R^T R (b x b, row-major, b <= kMaxChol) to Ri = R^{-1}; columns
+// after the first dependent one are zero, *rank the leading independent ones.
+constexpr int kMaxChol = 16;
+__global__ void __launch_bounds__(32) k_chol_inverse(const double *__restrict__ G, int b, double *__restrict__ Ri, int *rank)
+{
+    __shared__ double R[kMaxChol][kMaxChol + 1], I[kMaxChol][kMaxChol + 1];
+    const int i = threadIdx.x;
+    for (int q = i; q < b * b; q += 32) { R[q / b][q % b] = 0.0; I[q / b][q % b] = 0.0; }
+    __syncwarp();
+    int rk = b;
+    for (int j = 0; j < b; j++) {
+        double v = 0.0;  // lane i >= j: entry (j, i) before the division
+        if (i >= j && i < b) {
+            v = G[j * b + i];
+            for (int k = 0; k < j; k++) v = fma(-R[k][j], R[k][i], v);
+        }
+        const double d = __shfl_sync(0xffffffffu, v, j);
+        if (!(d > 1e-24 * fmax(1.0, fabs(G[j * b + j])))) { rk = j; break; }
+        const double s = sqrt(d);
+        if (i == j) R[j][j] = s;
+        else if (i > j && i < b) R[j][i] = v / s;
+        __syncwarp();
+    }
+    // column i of the inverse of the leading rk x rk block
+    if (i < rk) {
+        I[i][i] = 1.0 / R[i][i];
+        for (int r = i - 1; r >= 0; r--) {
+            double v = 0.0;
+            for (int k = r + 1; k <= i; k++) v = fma(R[r][k], I[k][i], v);
+            I[r][i] = -v / R[r][r];
+        }
+    }
+    __syncwarp();
+    for (int q = i; q < b * b; q += 32) Ri[q] = I[q / b][q % b];
+    if (i == 0) *rank = rk;
+}
+
+// Residuals: HX_j -= theta_j X_j, and their squared norms (partial[j][chunk], chunk = blockIdx.x)
+__global__ void __launch_bounds__(256) k_residual(const double *__restrict__ X, const double *__restrict__ theta,
+                                                  double *__restrict__ HX, int64_t n, int64_t chunk,
+                                                  double *__restrict__ partial)
+{
+    const int j = blockIdx.y;
+    const int64_t e0 = blockIdx.x * chunk, e1 = min(n, e0 + chunk);
+    const double *x = X + (size_t)j * n;
+    double *h = HX + (size_t)j * n;
+    const double th = theta[j];
+    double v = 0.0;
+    for (int64_t e = e0 + threadIdx.x; e < e1; e += 256) {
+        const double r = fma(-th, x[e], h[e]);
+        h[e] = r;
+        v = fma(r, r, v);
+    }
+    v = block_sum<256>(v);
+    if (threadIdx.x == 0) partial[j * gridDim.x + blockIdx.x] = v;
+}
+__global__ void k_sum_rows(const double *__restrict__ partial, int nchunk, int rows, double *__restrict__ out)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= rows) return;
+    double v = 0.0;
+    for (int c = 0; c < nchunk; c++) v += partial[j * nchunk + c];
+    out[j] = v;
+}
+
+// Directions: T_q = R_q / (d - theta_q) (guarded), or T_q = R_q without d
+__global__ void __launch_bounds__(256) k_direction(const double *__restrict__ R, const double *__restrict__ d,
+                                                   const double *__restrict__ theta, int64_t n, double *__restrict__ T)
+{
+    const int q = blockIdx.y;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+        double v = R[(size_t)q * n + e];
+        if (d) {
+            const double den = d[e] - theta[q];
+            v /= (fabs(den) < 1e-3 ? (den < 0 ? -1e-3 : 1e-3) : den);
+        }
+        T[(size_t)q * n + e] = v;
+    }
+}
+
+// X_j = the unit vector of entry at[j]
+__global__ void k_unit_vectors(double *__restrict__ X, int64_t n, const double *__restrict__ at, int r)
+{
+    const int64_t total = n * r;
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t j = q / n;
+        X[q] = q - j * n == (int64_t)at[j] ? 1.0 : 0.0;
+    }
+}
+
+// x <- x / ||x|| by one block (0 when ||x||^2 <= 1e-24), the squared norm in *nn
+__global__ void __launch_bounds__(1024) k_normalise(double *x, int64_t n, double *nn)
+{
+    double v = 0.0;
+    for (int64_t e = threadIdx.x; e < n; e += 1024) v = fma(x[e], x[e], v);
+    v = block_sum<1024>(v);
+    const double f = v > 1e-24 ? 1.0 / sqrt(v) : 0.0;
+    for (int64_t e = threadIdx.x; e < n; e += 1024) x[e] *= f;
+    if (threadIdx.x == 0) *nn = v;
+}
+// the same for longer vectors, from the squared norm
+__global__ void k_scale_norm(double *x, int64_t n, const double *nn)
+{
+    const double v = *nn, f = v > 1e-24 ? 1.0 / sqrt(v) : 0.0;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) x[e] *= f;
 }
 
 // y[j] = a * x[j] + b * y[j] over several vectors laid out contiguously
@@ -104,17 +257,6 @@ __global__ void k_axpby(int64_t len, double a, const double *__restrict__ x, dou
 {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < len; e += (int64_t)gridDim.x * blockDim.x)
         y[e] = a * x[e] + (b == 0.0 ? 0.0 : b * y[e]);
-}
-
-// element-wise preconditioner: r[j][e] /= (d[e] - theta[j]) (guarded)
-__global__ void k_precond(const double *__restrict__ d, const double *__restrict__ theta, int r, int64_t n,
-                          double *__restrict__ x)
-{
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n * r; e += (int64_t)gridDim.x * blockDim.x) {
-        const int j = (int)(e / n);
-        const double den = d[e - (int64_t)j * n] - theta[j];
-        x[e] /= (fabs(den) < 1e-3 ? (den < 0 ? -1e-3 : 1e-3) : den);
-    }
 }
 
 }  // namespace
@@ -126,6 +268,10 @@ cudaError_t dev_gram(const double *A, int ka, const double *B, int kb, int64_t n
                      double *partial, cudaStream_t s)
 {
     if (kb > kMaxCols || kb < 1 || ka < 1) return cudaErrorInvalidValue;
+    if (n <= kSmallN) {
+        k_gram_small<<<dim3(ka, kb), kDotThreads, 0, s>>>(A, B, (int)n, C_dev);
+        return cudaGetLastError();
+    }
     dim3 grid(kGramChunks, (ka + kGramRows - 1) / kGramRows);
     k_gram_partial<<<grid, 256, 0, s>>>(A, ka, B, kb, n, partial);
     k_gram_final<<<(ka * kb + 255) / 256, 256, 0, s>>>(partial, kGramChunks, ka, kb, C_dev);
@@ -134,23 +280,68 @@ cudaError_t dev_gram(const double *A, int ka, const double *B, int kb, int64_t n
 
 size_t gram_partial_doubles(int ka) { return (size_t)kGramChunks * ka * kMaxCols; }
 
-cudaError_t dev_combine(const double *V, int k, const double *S_dev, int r, double alpha, double beta, double *out,
-                        int64_t n, cudaStream_t s)
+// out (r x n) = base (r x n, or nullptr: zero; may be out) + alpha * V (k x n)^T-combination with S (k x r, device)
+cudaError_t dev_combine(const double *V, int k, const double *S_dev, int r, double alpha, const double *base,
+                        double *out, int64_t n, cudaStream_t s)
 {
     if (r > kMaxCols || r < 1 || k < 1) return cudaErrorInvalidValue;
-    k_combine<<<608, 256, sizeof(double) * k * r, s>>>(V, k, S_dev, r, alpha, beta, out, n);
+    if (n <= kSmallN)
+        k_combine_small<<<dim3((unsigned)((n + 63) / 64), r), 64, 0, s>>>(V, k, S_dev, r, alpha, base, out, (int)n);
+    else
+        k_combine_base<<<608, 256, sizeof(double) * k * r, s>>>(V, k, S_dev, r, alpha, base, out, n);
+    return cudaGetLastError();
+}
+
+cudaError_t dev_chol_inverse(const double *G, int b, double *Ri, int *rank, cudaStream_t s)
+{
+    if (b < 1 || b > kMaxChol) return cudaErrorInvalidValue;
+    k_chol_inverse<<<1, 32, 0, s>>>(G, b, Ri, rank);
+    return cudaGetLastError();
+}
+
+// HX_j -= theta_j X_j; norms2[j] = ||HX_j||^2 (device or pinned host).  partial: 304 doubles per row.
+cudaError_t dev_residual(const double *X, const double *theta, double *HX, int rows, int64_t n, double *norms2,
+                         double *partial, cudaStream_t s)
+{
+    if (rows < 1) return cudaErrorInvalidValue;
+    const int nchunk = (int)std::max<int64_t>(1, std::min<int64_t>(kGramChunks, (n + 2047) / 2048));
+    const int64_t chunk = (n + nchunk - 1) / nchunk;
+    k_residual<<<dim3(nchunk, rows), 256, 0, s>>>(X, theta, HX, n, chunk, nchunk == 1 ? norms2 : partial);
+    if (nchunk > 1) k_sum_rows<<<(rows + 31) / 32, 32, 0, s>>>(partial, nchunk, rows, norms2);
+    return cudaGetLastError();
+}
+
+cudaError_t dev_direction(const double *R, const double *d, const double *theta, int rows, int64_t n, double *T,
+                          cudaStream_t s)
+{
+    const unsigned bx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(608, (n + 255) / 256));
+    k_direction<<<dim3(bx, rows), 256, 0, s>>>(R, d, theta, n, T);
+    return cudaGetLastError();
+}
+
+cudaError_t dev_unit_vectors(double *X, int64_t n, const double *at, int r, cudaStream_t s)
+{
+    const unsigned bx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(1216, (n * r + 255) / 256));
+    k_unit_vectors<<<bx, 256, 0, s>>>(X, n, at, r);
+    return cudaGetLastError();
+}
+
+// x <- x / ||x|| (zero when ||x||^2 <= 1e-24); nn: the squared norm (device)
+cudaError_t dev_normalise(double *x, int64_t n, double *nn, double *partial, cudaStream_t s)
+{
+    if (n <= kSmallN) {
+        k_normalise<<<1, 1024, 0, s>>>(x, n, nn);
+        return cudaGetLastError();
+    }
+    cudaError_t e = dev_gram(x, 1, x, 1, n, nn, partial, s);
+    if (e != cudaSuccess) return e;
+    k_scale_norm<<<608, 256, 0, s>>>(x, n, nn);
     return cudaGetLastError();
 }
 
 cudaError_t dev_axpby(int64_t len, double a, const double *x, double b, double *y, cudaStream_t s)
 {
     k_axpby<<<608, 256, 0, s>>>(len, a, x, b, y);
-    return cudaGetLastError();
-}
-
-cudaError_t dev_precond(const double *d, const double *theta_dev, int r, int64_t n, double *x, cudaStream_t s)
-{
-    k_precond<<<608, 256, 0, s>>>(d, theta_dev, r, n, x);
     return cudaGetLastError();
 }
 

@@ -12,10 +12,16 @@ namespace sg {
 cudaError_t dev_gram(const double *A, int ka, const double *B, int kb, int64_t n, double *C_dev, double *partial,
                      cudaStream_t s);
 size_t gram_partial_doubles(int ka);
-cudaError_t dev_combine(const double *V, int k, const double *S_dev, int r, double alpha, double beta, double *out,
-                        int64_t n, cudaStream_t s);
+cudaError_t dev_combine(const double *V, int k, const double *S_dev, int r, double alpha, const double *base,
+                        double *out, int64_t n, cudaStream_t s);
+cudaError_t dev_chol_inverse(const double *G, int b, double *Ri, int *rank, cudaStream_t s);
+cudaError_t dev_residual(const double *X, const double *theta, double *HX, int rows, int64_t n, double *norms2,
+                         double *partial, cudaStream_t s);
+cudaError_t dev_direction(const double *R, const double *d, const double *theta, int rows, int64_t n, double *T,
+                          cudaStream_t s);
+cudaError_t dev_unit_vectors(double *X, int64_t n, const double *at, int r, cudaStream_t s);
+cudaError_t dev_normalise(double *x, int64_t n, double *nn, double *partial, cudaStream_t s);
 cudaError_t dev_axpby(int64_t len, double a, const double *x, double b, double *y, cudaStream_t s);
-cudaError_t dev_precond(const double *d, const double *theta_dev, int r, int64_t n, double *x, cudaStream_t s);
 void sym_eig(int n, std::vector<double> A, std::vector<double> &w, std::vector<double> &Z);
 int chol_inverse(int b, std::vector<double> &G);
 std::vector<double> bessel_j(int kmax, double x);
@@ -59,16 +65,46 @@ uint64_t splitmix(uint64_t &s)
     return z ^ (z >> 31);
 }
 
-// Solver context: the apply, scratch, and small dense helpers.
+// Solver context: the apply, scratch, and small dense helpers.  Small matrices
+// go to the device, and results come back, through the context's pinned host
+// memory: the kernels write inner products there, and one stream
+// synchronisation makes several of them readable.
 struct Solver {
     sg_ctx *ctx;
     cudaStream_t s;
     int64_t n;
-    DBuf partial, smalls;  // Gram scratch; small device matrices
+    DBuf partial, small;  // Gram scratch; small device matrices
+    double *pin = nullptr;
+    size_t cap, used = 0;  // doubles of pin and small; handed out since the last synchronisation
     const ApplyFn *apply_fn = nullptr;  // when set, applications of H_S go through it
-    Solver(sg_ctx *c, cudaStream_t st, int kmax)
-        : ctx(c), s(st), n(c->host.n_cs), partial(gram_partial_doubles(std::max(kmax, 1))),
-          smalls((size_t)std::max(kmax, 1) * kBlk * 2 + 64) {}
+    // kmax: largest basis; cols: largest number of columns combined at once
+    Solver(sg_ctx *c, cudaStream_t st, int kmax, int cols)
+        : ctx(c), s(st), n(c->host.n_cs), partial(gram_partial_doubles(std::max({kmax, cols, 2 * kBlk}))),
+          small(capacity(kmax, cols)), cap(capacity(kmax, cols))
+    {
+        if (ctx->pin_doubles < cap) {
+            if (ctx->pin) cudaFreeHost(ctx->pin);
+            ctx->pin = nullptr;
+            ctx->pin_doubles = 0;
+            ck(cudaMallocHost(&ctx->pin, cap * sizeof(double)), "solver cudaMallocHost");
+            ctx->pin_doubles = cap;
+        }
+        pin = ctx->pin;
+    }
+    static size_t capacity(int kmax, int cols) { return (size_t)(kmax + 16) * (2 * cols + 6 * kBlk) + 1024; }
+
+    // a range of pin and of small, free until the next synchronisation
+    size_t take(size_t k)
+    {
+        if (used + k > cap) throw SolverError{SG_ECUDA, "solver scratch too small"};
+        used += k;
+        return used - k;
+    }
+    void sync(const char *where)
+    {
+        ck(cudaStreamSynchronize(s), where);
+        used = 0;
+    }
 
     void apply(const double *x, double *y, int r)
     {
@@ -78,55 +114,100 @@ struct Solver {
         const sg_status st = (*apply_fn)(x, y, r);
         if (st != SG_OK) throw SolverError{st, "routed apply failed"};
     }
-    // C (ka x kb host, row-major) = A^T B
-    std::vector<double> gram(const double *A, int ka, const double *B, int kb)
+    // Small matrix with its columns in groups of at most kBlk (each k x group, row-major).
+    struct Mat {
+        const double *d;
+        int k, r;
+    };
+    Mat upload(const std::vector<double> &S, int k, int r)  // S: k x r row-major
     {
-        std::vector<double> C((size_t)ka * kb);
-        for (int j0 = 0; j0 < kb; j0 += kBlk) {
-            const int r = std::min(kBlk, kb - j0);
-            ck(dev_gram(A, ka, B + (size_t)j0 * n, r, n, smalls.p, partial.p, s), "gram");
-            std::vector<double> tmp((size_t)ka * r);
-            ck(cudaMemcpyAsync(tmp.data(), smalls.p, sizeof(double) * ka * r, cudaMemcpyDeviceToHost, s), "gram copy");
-            ck(cudaStreamSynchronize(s), "gram sync");
-            for (int i = 0; i < ka; i++)
-                for (int j = 0; j < r; j++) C[(size_t)i * kb + j0 + j] = tmp[(size_t)i * r + j];
-        }
-        return C;
-    }
-    // out (r x n) = beta out + alpha * V (k x n)^T-combination with S (k x r host, row-major)
-    void combine(const double *V, int k, const std::vector<double> &S, int r, double alpha, double beta, double *out)
-    {
+        const size_t o = take((size_t)k * r);
+        double *q = pin + o;
         for (int j0 = 0; j0 < r; j0 += kBlk) {
             const int rr = std::min(kBlk, r - j0);
-            std::vector<double> Sj((size_t)k * rr);
             for (int i = 0; i < k; i++)
-                for (int j = 0; j < rr; j++) Sj[(size_t)i * rr + j] = S[(size_t)i * r + j0 + j];
-            ck(cudaMemcpyAsync(smalls.p, Sj.data(), sizeof(double) * Sj.size(), cudaMemcpyHostToDevice, s), "S copy");
-            ck(dev_combine(V, k, smalls.p, rr, alpha, beta, out + (size_t)j0 * n, n, s), "combine");
+                for (int j = 0; j < rr; j++) *q++ = S[(size_t)i * r + j0 + j];
+        }
+        ck(cudaMemcpyAsync(small.p + o, pin + o, sizeof(double) * k * r, cudaMemcpyHostToDevice, s), "small copy");
+        return {small.p + o, k, r};
+    }
+    const double *upload(const double *v, int k)
+    {
+        const size_t o = take(k);
+        std::copy(v, v + k, pin + o);
+        ck(cudaMemcpyAsync(small.p + o, pin + o, sizeof(double) * k, cudaMemcpyHostToDevice, s), "small copy");
+        return small.p + o;
+    }
+    // A^T B (A: ka vectors, B: kb) into C, columns in groups; C on the device or pinned
+    void gram_to(const double *A, int ka, const double *B, int kb, double *C)
+    {
+        for (int j0 = 0; j0 < kb; j0 += kBlk) {
+            const int r = std::min(kBlk, kb - j0);
+            ck(dev_gram(A, ka, B + (size_t)j0 * n, r, n, C + (size_t)ka * j0, partial.p, s), "gram");
         }
     }
-    // X (r x n) <- X - V V^T X, twice (V: k x n orthonormal)
+    static std::vector<double> ungroup(const double *C, int ka, int kb)
+    {
+        std::vector<double> out((size_t)ka * kb);
+        for (int j0 = 0; j0 < kb; j0 += kBlk) {
+            const int r = std::min(kBlk, kb - j0);
+            const double *c = C + (size_t)ka * j0;
+            for (int i = 0; i < ka; i++)
+                for (int j = 0; j < r; j++) out[(size_t)i * kb + j0 + j] = c[(size_t)i * r + j];
+        }
+        return out;
+    }
+    // the same on the host (ka x kb, row-major)
+    std::vector<double> gram(const double *A, int ka, const double *B, int kb)
+    {
+        double *C = pin + take((size_t)ka * kb);
+        gram_to(A, ka, B, kb, C);
+        sync("gram sync");
+        return ungroup(C, ka, kb);
+    }
+    // out (S.r vectors) = base (or 0) + alpha * V S
+    void combine(const double *V, const Mat &S, double alpha, const double *base, double *out)
+    {
+        for (int j0 = 0; j0 < S.r; j0 += kBlk) {
+            const int rr = std::min(kBlk, S.r - j0);
+            ck(dev_combine(V, S.k, S.d + (size_t)S.k * j0, rr, alpha, base ? base + (size_t)j0 * n : nullptr,
+                           out + (size_t)j0 * n, n, s), "combine");
+        }
+    }
+    // X (r vectors) <- X - V V^T X, twice (V: k orthonormal vectors)
     void orth_against(const double *V, int k, double *X, int r)
     {
         if (k <= 0) return;
         for (int pass = 0; pass < 2; pass++) {
-            std::vector<double> C = gram(V, k, X, r);
-            combine(V, k, C, r, -1.0, 1.0, X);
+            double *C = small.p + take((size_t)k * r);
+            gram_to(V, k, X, r, C);
+            combine(V, {C, k, r}, -1.0, X, X);
         }
     }
-    // orthonormalise the r columns of X (Cholesky QR twice); returns the rank kept
-    int orthonormalise(double *X, int r)
+    // One pass of Cholesky QR: out = X R^{-1} (r <= kBlk vectors), the rank to *rank (pinned)
+    void chol_pass(const double *X, int r, double *out, int *rank)
+    {
+        double *G = small.p + take((size_t)r * r), *Ri = small.p + take((size_t)r * r);
+        ck(dev_gram(X, r, X, r, n, G, partial.p, s), "gram");
+        ck(dev_chol_inverse(G, r, Ri, rank, s), "cholesky");
+        combine(X, {Ri, r, r}, 1.0, nullptr, out);
+    }
+    // orthonormalise the r vectors of X (Cholesky QR twice, tmp: r vectors of
+    // scratch); returns the rank kept
+    int orthonormalise(double *X, int r, double *tmp)
     {
         int rank = r;
         for (int pass = 0; pass < 2; pass++) {
             std::vector<double> G = gram(X, rank, X, rank);
-            const int rk = chol_inverse(rank, G);
-            DBuf tmp((size_t)rank * n);
-            // X <- X R^{-1} (first rk columns)
-            combine(X, rank, G, rk, 1.0, 0.0, tmp.p);
-            ck(cudaMemcpyAsync(X, tmp.p, sizeof(double) * n * rk, cudaMemcpyDeviceToDevice, s), "orth copy");
+            const int rk = chol_inverse(rank, G), was = rank;
             rank = rk;
             if (rank == 0) break;
+            // X <- X R^{-1} (first rk columns)
+            std::vector<double> Gk((size_t)was * rk);
+            for (int i = 0; i < was; i++)
+                for (int j = 0; j < rk; j++) Gk[(size_t)i * rk + j] = G[(size_t)i * was + j];
+            combine(X, upload(Gk, was, rk), 1.0, nullptr, tmp);
+            ck(cudaMemcpyAsync(X, tmp, sizeof(double) * n * rk, cudaMemcpyDeviceToDevice, s), "orth copy");
         }
         return rank;
     }
@@ -149,14 +230,17 @@ struct Solver {
         for (int64_t i = 0; i < n; i++) idx[i] = i;
         std::partial_sort(idx.begin(), idx.begin() + r, idx.end(),
                           [&](int64_t a, int64_t b) { return d[a] < d[b] || (d[a] == d[b] && a < b); });
-        std::vector<double> h((size_t)(r + extra) * n, 0.0);
-        for (int j = 0; j < r; j++) h[(size_t)j * n + idx[j]] = 1.0;
+        std::vector<double> at(r);  // positions, exact as doubles (N_cs < 2^31)
+        for (int j = 0; j < r; j++) at[j] = (double)idx[j];
+        ck(dev_unit_vectors(X, n, upload(at.data(), r), r, s), "start block");
+        std::vector<double> h(extra ? n : 0);
         uint64_t st = 0x5eed4321ull;
         for (int64_t i = 0; extra && i < n; i++) {
             const double w = 1.0 + (d[i] - d[idx[0]]);
-            h[(size_t)r * n + i] = ((double)(splitmix(st) >> 11) * 0x1.0p-53 - 0.5) / (w * w);
+            h[i] = ((double)(splitmix(st) >> 11) * 0x1.0p-53 - 0.5) / (w * w);
         }
-        ck(cudaMemcpyAsync(X, h.data(), sizeof(double) * h.size(), cudaMemcpyHostToDevice, s), "start copy");
+        if (extra)
+            ck(cudaMemcpyAsync(X + (size_t)r * n, h.data(), sizeof(double) * n, cudaMemcpyHostToDevice, s), "start copy");
         ck(cudaStreamSynchronize(s), "start sync");
         return true;
     }
@@ -167,15 +251,6 @@ struct Solver {
         for (auto &v : h) v = (double)(splitmix(st) >> 11) * 0x1.0p-53 - 0.5;
         ck(cudaMemcpyAsync(X, h.data(), sizeof(double) * h.size(), cudaMemcpyHostToDevice, s), "random copy");
         ck(cudaStreamSynchronize(s), "random sync");
-    }
-    std::vector<double> norms(const double *X, int r)
-    {
-        std::vector<double> out(r);
-        for (int j = 0; j < r; j++) {
-            std::vector<double> g = gram(X + (size_t)j * n, 1, X + (size_t)j * n, 1);
-            out[j] = std::sqrt(std::max(0.0, g[0]));
-        }
-        return out;
     }
 };
 
@@ -198,26 +273,29 @@ int block_eigs(Solver &S, int nev, int b, bool davidson, double tol, int max_it,
                                                         : std::min<int64_t>((int64_t)max_it * b + b, 320));
     const int guard = davidson ? b : 0;
     const size_t nx = (size_t)std::max(nev + guard, b);
-    DBuf V((size_t)kmax * n), W((size_t)kmax * n), X(nx * n), HX(nx * n), T((size_t)b * n), dd(kBlk + 8);
+    const int rmax = std::min(kmax, std::max(nev + b, nx0) + 1);  // largest block orthonormalised at once
+    // one allocation: basis V, images W = H V, Ritz vectors X, their images and residuals HX, directions T, scratch Q
+    DBuf mem((2 * (size_t)kmax + 2 * nx + b + rmax) * n);
+    double *const V = mem.p, *const W = V + (size_t)kmax * n, *const X = W + (size_t)kmax * n,
+                 *const HX = X + nx * n, *const T = HX + nx * n, *const Q = T + (size_t)b * n;
     std::vector<double> Tm;  // projected matrix, k x k
     int k = 0;
     // initial block
     int r0 = davidson ? std::min(nev + b, kmax) : (int)std::min<int64_t>(b, n);
     if (X0 && nx0 > 0) {
         r0 = std::min(nx0, kmax);
-        ck(cudaMemcpyAsync(V.p, X0, sizeof(double) * n * r0, cudaMemcpyDeviceToDevice, S.s), "x0 copy");
-    } else if (const bool extra = r0 < kmax; davidson && S.lowest_diagonal_block(V.p, r0, extra)) {
+        ck(cudaMemcpyAsync(V, X0, sizeof(double) * n * r0, cudaMemcpyDeviceToDevice, S.s), "x0 copy");
+    } else if (const bool extra = r0 < kmax; davidson && S.lowest_diagonal_block(V, r0, extra)) {
         r0 += extra;
     } else {
-        S.random_block(V.p, r0, 0x5eed1234ull);
+        S.random_block(V, r0, 0x5eed1234ull);
     }
-    r0 = S.orthonormalise(V.p, r0);
-    auto extend = [&](int r) {  // V[k..k+r) are new orthonormal vectors: W = H V, grow Tm
-        for (int j0 = 0; j0 < r; j0 += kBlk) {
-            const int rr = std::min(kBlk, r - j0);
-            S.apply(V.p + (size_t)(k + j0) * n, W.p + (size_t)(k + j0) * n, rr);
-        }
-        std::vector<double> C = S.gram(V.p, k + r, W.p + (size_t)k * n, r);  // (k+r) x r
+    r0 = S.orthonormalise(V, r0, Q);
+    auto images = [&](int r) {  // W = H V for the new vectors V[k..k+r)
+        for (int j0 = 0; j0 < r; j0 += kBlk)
+            S.apply(V + (size_t)(k + j0) * n, W + (size_t)(k + j0) * n, std::min(kBlk, r - j0));
+    };
+    auto grow = [&](int r, const std::vector<double> &C) {  // C = V^T W of the new columns, (k+r) x r
         std::vector<double> Tn((size_t)(k + r) * (k + r));
         for (int i = 0; i < k; i++)
             for (int j = 0; j < k; j++) Tn[(size_t)i * (k + r) + j] = Tm[(size_t)i * k + j];
@@ -235,10 +313,16 @@ int block_eigs(Solver &S, int nev, int b, bool davidson, double tol, int max_it,
         Tm.swap(Tn);
         k += r;
     };
+    auto extend = [&](int r) {  // V[k..k+r) are new orthonormal vectors
+        images(r);
+        grow(r, S.gram(V, k + r, W + (size_t)k * n, r));
+    };
     extend(r0);
     std::vector<double> theta, Z;
     int nconv = 0;
     bool checked = !davidson;  // the expansion after convergence has been made
+    bool any = false;          // harmonic energies: a diagonal preconditioner
+    for (int i = 0; davidson && i < S.ctx->prob.D; i++) any |= S.ctx->host.harm_mono[i] >= 0;
     const int ne = std::min<int64_t>(nev, n);
     for (int it = 0; it < max_it; it++) {
         sym_eig(k, Tm, theta, Z);
@@ -247,10 +331,15 @@ int block_eigs(Solver &S, int nev, int b, bool davidson, double tol, int max_it,
         std::vector<double> Zr((size_t)k * nr);
         for (int i = 0; i < k; i++)
             for (int j = 0; j < nr; j++) Zr[(size_t)i * nr + j] = Z[(size_t)i * k + j];
-        S.combine(V.p, k, Zr, nr, 1.0, 0.0, X.p);
-        S.combine(W.p, k, Zr, nr, 1.0, 0.0, HX.p);
-        for (int j = 0; j < nr; j++) ck(dev_axpby(n, -theta[j], X.p + (size_t)j * n, 1.0, HX.p + (size_t)j * n, S.s), "resid");
-        std::vector<double> rn = S.norms(HX.p, nr);
+        const Solver::Mat Zd = S.upload(Zr, k, nr);
+        const double *th = S.upload(theta.data(), nr);
+        S.combine(V, Zd, 1.0, nullptr, X);
+        S.combine(W, Zd, 1.0, nullptr, HX);
+        double *rn2 = S.pin + S.take(nr);
+        ck(dev_residual(X, th, HX, nr, n, rn2, S.partial.p, S.s), "resid");
+        S.sync("residual sync");
+        std::vector<double> rn(rn2, rn2 + nr);
+        for (double &v : rn) v = std::sqrt(v);
         nconv = 0;
         while (nconv < nr && rn[nconv] <= tol * std::max(1.0, std::fabs(theta[nconv]))) nconv++;
         for (int j = 0; j < std::min(nr, ne); j++) { evals[j] = theta[j]; if (resid) resid[j] = rn[j]; }
@@ -262,85 +351,94 @@ int block_eigs(Solver &S, int nev, int b, bool davidson, double tol, int max_it,
         if (r <= 0) r = 1;
         if (!davidson && k + r > kmax) break;
         const int first = std::min(nconv, nr - r);
-        ck(cudaMemcpyAsync(T.p, HX.p + (size_t)first * n, sizeof(double) * n * r, cudaMemcpyDeviceToDevice, S.s), "dir copy");
-        if (davidson) {
-            const double *d = S.ctx->kp.esplit;  // harmonic energies: a diagonal preconditioner
-            bool any = false;
-            for (int i = 0; i < S.ctx->prob.D; i++) any |= S.ctx->host.harm_mono[i] >= 0;
-            if (any) {
-                std::vector<double> th(theta.begin() + first, theta.begin() + first + r);
-                ck(cudaMemcpyAsync(dd.p, th.data(), sizeof(double) * r, cudaMemcpyHostToDevice, S.s), "theta copy");
-                ck(dev_precond(d, dd.p, r, n, T.p, S.s), "precond");
-            }
-            if (k + r > kmax) {  // restart with the current Ritz vectors
-                const int keep = std::min(nr, kmax - r);
-                ck(cudaMemcpyAsync(V.p, X.p, sizeof(double) * n * keep, cudaMemcpyDeviceToDevice, S.s), "restart V");
-                k = 0;
-                Tm.clear();
-                extend(S.orthonormalise(V.p, keep));  // recomputes W = H V
-            }
+        const double *thf = S.upload(theta.data() + first, r);
+        ck(dev_direction(HX + (size_t)first * n, any ? S.ctx->kp.esplit : nullptr, thf, r, n, T, S.s), "directions");
+        if (davidson && k + r > kmax) {  // restart with the current Ritz vectors
+            const int keep = std::min(nr, kmax - r);
+            ck(cudaMemcpyAsync(V, X, sizeof(double) * n * keep, cudaMemcpyDeviceToDevice, S.s), "restart V");
+            k = 0;
+            Tm.clear();
+            extend(S.orthonormalise(V, keep, Q));  // recomputes W = H V
         }
-        S.orth_against(V.p, k, T.p, r);
-        int rk = S.orthonormalise(T.p, r);
+        S.orth_against(V, k, T, r);
+        // The new vectors, their images and inner products on the assumption
+        // that the r directions are independent; the ranks come with the results.
+        int *rank = reinterpret_cast<int *>(S.pin + S.take(1));
+        S.chol_pass(T, r, Q, rank);
+        S.chol_pass(Q, r, V + (size_t)k * n, rank + 1);
+        images(r);
+        double *C = S.pin + S.take((size_t)(k + r) * r);
+        S.gram_to(V, k + r, W + (size_t)k * n, r, C);
+        S.sync("extend sync");
+        if (rank[0] == r && rank[1] == r) {
+            grow(r, Solver::ungroup(C, k + r, r));
+            continue;
+        }
+        int rk = S.orthonormalise(T, r, Q);
         if (rk == 0) {  // the directions lie in the basis: add random ones
-            S.random_block(T.p, r, 0x5eed0000ull + (uint64_t)it);
-            S.orth_against(V.p, k, T.p, r);
-            rk = S.orthonormalise(T.p, r);
+            S.random_block(T, r, 0x5eed0000ull + (uint64_t)it);
+            S.orth_against(V, k, T, r);
+            rk = S.orthonormalise(T, r, Q);
             if (rk == 0) break;
         }
-        ck(cudaMemcpyAsync(V.p + (size_t)k * n, T.p, sizeof(double) * n * rk, cudaMemcpyDeviceToDevice, S.s), "append");
+        ck(cudaMemcpyAsync(V + (size_t)k * n, T, sizeof(double) * n * rk, cudaMemcpyDeviceToDevice, S.s), "append");
         extend(rk);
     }
-    if (evecs) ck(cudaMemcpyAsync(evecs, X.p, sizeof(double) * n * std::min(ne, k), cudaMemcpyDeviceToDevice, S.s), "evecs");
-    ck(cudaStreamSynchronize(S.s), "eigs sync");
+    if (evecs) ck(cudaMemcpyAsync(evecs, X, sizeof(double) * n * std::min(ne, k), cudaMemcpyDeviceToDevice, S.s), "evecs");
+    S.sync("eigs sync");
     return std::min(nconv, ne);
 }
 
 // Spectral interval of H_S for the Chebyshev propagator: a 40-vector Krylov
 // run (Rayleigh-Ritz), the extreme Ritz values widened by their residual norms
 // and by 5% of the range.  Deterministic (fixed start vector, ordered sums).
+// The run stays on the device: a vector that vanishes against the basis
+// becomes zero there, and the host ends the basis at it afterwards.
+constexpr int kBoundVectors = 40;
 void spectral_bounds(Solver &S, double &emin, double &emax)
 {
     const int64_t n = S.n;
-    const int ks = (int)std::min<int64_t>(n, 40);
-    {
-        DBuf V((size_t)(ks + 1) * n), W((size_t)(ks + 1) * n), Xr(2 * (size_t)n), HXr(2 * (size_t)n);
-        S.random_block(V.p, 1, 0xc4eb00ull);
-        S.orthonormalise(V.p, 1);
-        std::vector<double> Tm;
-        int k = 0;
-        for (int it = 0; it < ks; it++) {
-            S.apply(V.p + (size_t)k * n, W.p + (size_t)k * n, 1);
-            std::vector<double> C = S.gram(V.p, k + 1, W.p + (size_t)k * n, 1);
-            std::vector<double> Tn((size_t)(k + 1) * (k + 1));
-            for (int i = 0; i < k; i++)
-                for (int j = 0; j < k; j++) Tn[(size_t)i * (k + 1) + j] = Tm[(size_t)i * k + j];
-            for (int i = 0; i <= k; i++) Tn[(size_t)i * (k + 1) + k] = Tn[(size_t)k * (k + 1) + i] = C[i];
-            Tm.swap(Tn);
-            k++;
-            if (k >= ks) break;
-            ck(cudaMemcpyAsync(V.p + (size_t)k * n, W.p + (size_t)(k - 1) * n, sizeof(double) * n,
-                               cudaMemcpyDeviceToDevice, S.s), "krylov copy");
-            S.orth_against(V.p, k, V.p + (size_t)k * n, 1);
-            if (S.orthonormalise(V.p + (size_t)k * n, 1) == 0) break;
-        }
-        std::vector<double> th, Z;
-        sym_eig(k, Tm, th, Z);
-        double rlo = 0, rhi = 0;
-        for (int end = 0; end < 2; end++) {
-            const int j = end == 0 ? 0 : k - 1;
-            std::vector<double> z(k);
-            for (int i = 0; i < k; i++) z[i] = Z[(size_t)i * k + j];
-            S.combine(V.p, k, z, 1, 1.0, 0.0, Xr.p);
-            S.combine(W.p, k, z, 1, 1.0, 0.0, HXr.p);
-            ck(dev_axpby(n, -th[j], Xr.p, 1.0, HXr.p, S.s), "bound resid");
-            const double rr = S.norms(HXr.p, 1)[0];
-            (end == 0 ? rlo : rhi) = rr;
-        }
-        const double range = th[k - 1] - th[0];
-        emin = th[0] - rlo - 0.05 * range;
-        emax = th[k - 1] + rhi + 0.05 * range;
+    const int ks = (int)std::min<int64_t>(n, kBoundVectors);
+    DBuf mem((2 * (size_t)ks + 5) * n + (size_t)ks * (ks + 2));
+    double *const V = mem.p, *const W = V + (size_t)(ks + 1) * n, *const X = W + (size_t)ks * n, *const HX = X + 2 * n,
+                 *const cols = HX + 2 * n, *const nn = cols + (size_t)ks * (ks + 1);
+    S.random_block(V, 1, 0xc4eb00ull);
+    ck(dev_normalise(V, n, nn, S.partial.p, S.s), "krylov start");
+    for (int k = 0; k < ks; k++) {
+        S.apply(V + (size_t)k * n, W + (size_t)k * n, 1);
+        // column k of the projected matrix, which is also the first projection of the next vector
+        double *c = cols + (size_t)k * ks;
+        ck(dev_gram(V, k + 1, W + (size_t)k * n, 1, n, c, S.partial.p, S.s), "krylov gram");
+        if (k + 1 == ks) break;
+        double *next = V + (size_t)(k + 1) * n, *c2 = S.small.p;
+        ck(dev_combine(V, k + 1, c, 1, -1.0, W + (size_t)k * n, next, n, S.s), "krylov step");
+        ck(dev_gram(V, k + 1, next, 1, n, c2, S.partial.p, S.s), "krylov gram");
+        ck(dev_combine(V, k + 1, c2, 1, -1.0, next, next, n, S.s), "krylov step");
+        ck(dev_normalise(next, n, nn + k + 1, S.partial.p, S.s), "krylov norm");
     }
+    S.sync("krylov sync");
+    std::vector<double> hc((size_t)ks * ks), hn(ks);
+    ck(cudaMemcpy(hc.data(), cols, sizeof(double) * hc.size(), cudaMemcpyDeviceToHost), "krylov copy");
+    ck(cudaMemcpy(hn.data(), nn, sizeof(double) * ks, cudaMemcpyDeviceToHost), "krylov copy");
+    int k = 1;
+    while (k < ks && hn[k] > 1e-24) k++;
+    std::vector<double> Tm((size_t)k * k), th, Z;
+    for (int j = 0; j < k; j++)
+        for (int i = 0; i <= j; i++) Tm[(size_t)i * k + j] = Tm[(size_t)j * k + i] = hc[(size_t)j * ks + i];
+    sym_eig(k, Tm, th, Z);
+    std::vector<double> z((size_t)k * 2);
+    for (int i = 0; i < k; i++) { z[2 * i] = Z[(size_t)i * k]; z[2 * i + 1] = Z[(size_t)i * k + k - 1]; }
+    const double ends[2] = {th[0], th[k - 1]};
+    const Solver::Mat zd = S.upload(z, k, 2);
+    const double *te = S.upload(ends, 2);
+    S.combine(V, zd, 1.0, nullptr, X);
+    S.combine(W, zd, 1.0, nullptr, HX);
+    double *rn2 = S.pin + S.take(2);
+    ck(dev_residual(X, te, HX, 2, n, rn2, S.partial.p, S.s), "bound resid");
+    S.sync("bounds sync");
+    const double range = th[k - 1] - th[0];
+    emin = th[0] - std::sqrt(rn2[0]) - 0.05 * range;
+    emax = th[k - 1] + std::sqrt(rn2[1]) + 0.05 * range;
 }
 
 }  // namespace
@@ -360,7 +458,7 @@ sg_status sg_eigs(sg_ctx *ctx, int nev, int method, int block, double tol, int m
     }
     const int b = block <= 0 ? std::min(nev, kBlk) : std::min(block, kBlk);
     try {
-        Solver S(ctx, (cudaStream_t)stream, std::max(3 * nev, nev + 6 * b) + 328);
+        Solver S(ctx, (cudaStream_t)stream, std::max({3 * nev, nev + 6 * b, 328}), nev + b + 1);
         const int nconv = block_eigs(S, nev, b, method == SG_DAVIDSON, tol, max_it, nullptr, 0, evals, evecs, resid);
         if (nconv < std::min<int64_t>(nev, ctx->host.n_cs)) {
             ctx->last_error = "sg_eigs: " + std::to_string(nconv) + " of " + std::to_string(nev) + " eigenpairs converged";
@@ -384,7 +482,7 @@ sg_status sg_eigs_refine(sg_ctx *ctx, int nev, double *evecs, double *evals, dou
     if (!sg_on_ctx_device(ctx)) { ctx->last_error = "the current CUDA device is not the one the context was made on"; return SG_EINVAL; }
     const int b = std::min(nev, kBlk);
     try {
-        Solver S(ctx, (cudaStream_t)stream, std::max(3 * nev, nev + 6 * b) + 8);
+        Solver S(ctx, (cudaStream_t)stream, std::max(3 * nev, nev + 6 * b), nev + b + 1);
         const int nconv = block_eigs(S, nev, b, true, tol, max_it, evecs, nev, evals, evecs, resid);
         if (nconv < nev) {
             ctx->last_error = "sg_eigs_refine: " + std::to_string(nconv) + " of " + std::to_string(nev) + " converged";
@@ -431,7 +529,7 @@ sg_status sg_propagate(sg_ctx *ctx, double *psi, double dt, int nsteps, int orde
     }
     if (!sg_on_ctx_device(ctx)) { ctx->last_error = "the current CUDA device is not the one the context was made on"; return SG_EINVAL; }
     try {
-        Solver S(ctx, (cudaStream_t)stream, 48);
+        Solver S(ctx, (cudaStream_t)stream, kBoundVectors, 2);
         const int64_t n = S.n;
         double emin, emax;
         spectral_bounds(S, emin, emax);
@@ -502,7 +600,7 @@ sg_status davidson_routed(sg_ctx *ctx, cudaStream_t stream, const ApplyFn &apply
 {
     const int b = block <= 0 ? std::min(nev, kBlk) : std::min(block, kBlk);
     try {
-        Solver S(ctx, stream, std::max(3 * nev, nev + 6 * b) + 328);
+        Solver S(ctx, stream, std::max(3 * nev, nev + 6 * b), nev + b + 1);
         S.apply_fn = &apply;
         *nconv = block_eigs(S, nev, b, true, tol, max_it, nullptr, 0, evals, evecs, resid);
     } catch (const SolverError &e) {
@@ -515,7 +613,7 @@ sg_status davidson_routed(sg_ctx *ctx, cudaStream_t stream, const ApplyFn &apply
 sg_status chebyshev_bounds(sg_ctx *ctx, cudaStream_t stream, double *emin, double *emax)
 {
     try {
-        Solver S(ctx, stream, 48);
+        Solver S(ctx, stream, kBoundVectors, 2);
         spectral_bounds(S, *emin, *emax);
         ck(cudaStreamSynchronize(S.s), "bounds sync");
     } catch (const SolverError &e) {
