@@ -26,6 +26,8 @@ struct sg_batch {
     const int2 *items = nullptr;       // (problem, window) of the packed problems, most entries first
     const int2 *stage_items = nullptr; // (problem, chunk of 256 rows) of the packed problems
     int n_items = 0, n_stage = 0, cap = 0, wrows = 16;
+    const int2 *all_items = nullptr, *all_stage = nullptr;  // the same over every row-form problem
+    int n_all = 0, n_all_stage = 0, all_cap = 0;
     std::vector<int> packed, solo;     // row-form problems: shared launches, launches of their own
     std::vector<int> generic;          // problems applied term by term
     std::vector<void *> allocations;
@@ -124,14 +126,17 @@ extern "C" sg_status sg_batch_create(sg_ctx *const *ctxs, int n, sg_batch **out)
     b->cs_prefix.assign(n + 1, 0);
     std::vector<sg::RowOp> ops(n);
     struct Item { int nent, j, w; };
-    std::vector<Item> it;
-    std::vector<int2> stage;
+    std::vector<Item> it, all;
+    std::vector<int2> stage, all_stage;
     for (int j = 0; j < n; j++) {
         const sg_ctx *c = ctxs[j];
         b->cs_prefix[j + 1] = b->cs_prefix[j] + c->host.n_cs;
         b->n_terms += c->host.n_terms;
         ops[j] = c->rop;
         if (!c->host.rows) { b->generic.push_back(j); continue; }
+        b->all_cap = std::max(b->all_cap, c->rop.cap);
+        for (int w = 0; w < c->rop.nwin; w++) all.push_back({c->win_entries[w], j, w});
+        for (int q = 0; q * (int64_t)256 < c->host.n_cs; q++) all_stage.push_back(make_int2(j, q));
         if (c->host.n_cs >= kSoloRows) { b->solo.push_back(j); continue; }
         b->packed.push_back(j);
         b->cap = std::max(b->cap, c->rop.cap);
@@ -139,15 +144,22 @@ extern "C" sg_status sg_batch_create(sg_ctx *const *ctxs, int n, sg_batch **out)
         for (int w = 0; w < c->rop.nwin; w++) it.push_back({c->win_entries[w], j, w});
         for (int q = 0; q * (int64_t)256 < c->host.n_cs; q++) stage.push_back(make_int2(j, q));
     }
-    if (it.size() > (size_t)0x7FFFFFFF) { delete b; return SG_EUNSUPPORTED; }
-    std::stable_sort(it.begin(), it.end(), [](const Item &a, const Item &c) { return a.nent > c.nent; });
-    std::vector<int2> items(it.size());
-    for (size_t q = 0; q < it.size(); q++) items[q] = make_int2(it[q].j, it[q].w);
+    if (all.size() > (size_t)0x7FFFFFFF) { delete b; return SG_EUNSUPPORTED; }
+    auto largest_first = [](std::vector<Item> &v) {
+        std::stable_sort(v.begin(), v.end(), [](const Item &a, const Item &c) { return a.nent > c.nent; });
+        std::vector<int2> out(v.size());
+        for (size_t q = 0; q < v.size(); q++) out[q] = make_int2(v[q].j, v[q].w);
+        return out;
+    };
+    const std::vector<int2> items = largest_first(it), all_items = largest_first(all);
     b->n_items = (int)items.size();
     b->n_stage = (int)stage.size();
+    b->n_all = (int)all_items.size();
+    b->n_all_stage = (int)all_stage.size();
     sg_status st;
     if ((st = bupload(b, ops, &b->d_ops)) != SG_OK || (st = bupload(b, b->cs_prefix, &b->d_cs_prefix)) != SG_OK ||
-        (st = bupload(b, items, &b->items)) != SG_OK || (st = bupload(b, stage, &b->stage_items)) != SG_OK) {
+        (st = bupload(b, items, &b->items)) != SG_OK || (st = bupload(b, stage, &b->stage_items)) != SG_OK ||
+        (st = bupload(b, all_items, &b->all_items)) != SG_OK || (st = bupload(b, all_stage, &b->all_stage)) != SG_OK) {
         free_all(b);
         delete b;
         return st;
@@ -285,6 +297,28 @@ sg_status enqueue_apply(sg_batch *b, const double *x, double *y, int nvec, cudaS
     }
     return SG_OK;
 }
+
+namespace sg {
+
+sg_status batch_cheb(sg_batch *b, const ChebIO &io, const ChebState *st, bool restage, cudaStream_t s)
+{
+    if (!b->generic.empty()) return SG_EUNSUPPORTED;
+    const sg_precision prec = b->fp32 ? SG_MIXED : SG_FP64;
+    cudaError_t e = cudaSuccess;
+    if (restage) {
+        RowIO r{};
+        r.x = io.X;
+        r.xs = io.xs;
+        r.nvec = 2;
+        r.stride = xs_stride(2);
+        e = launch_row_stage_batch(r, prec, b->d_cs_prefix, b->all_stage, b->n_all_stage, s);
+    }
+    if (e == cudaSuccess)
+        e = launch_cheb_rows_batch(b->d_ops, b->all_items, b->n_all, b->all_cap, io, st, prec, b->d_cs_prefix, s);
+    return e == cudaSuccess ? SG_OK : bfail(b, SG_ECUDA, std::string("recurrence launch: ") + cudaGetErrorString(e));
+}
+
+}  // namespace sg
 
 extern "C" const char *sg_batch_last_error(const sg_batch *b)
 {

@@ -299,6 +299,32 @@ struct ChebState {
 };
 cudaError_t launch_cheb_iteration(ChebState *st, const long long *prefix, int nitems, int64_t total,
                                   const double *X, const double *Y, double *P, double *A, cudaStream_t s);
+// Logs the requests at the start of a step, then moves every request to its next term.
+cudaError_t launch_cheb_log_advance(ChebState *st, const long long *prefix, int nitems, const double *X,
+                                    const double *Y, cudaStream_t s);
+// One recurrence term in one launch (sg_rows.cu): y = H T_k row by row, and the
+// update of launch_cheb_iteration where the row sum ends.  Vectors as there
+// (real parts, then imaginary parts); xs, xs_next: T_k and T_{k+1} entry-major
+// in the contraction type; y is stored only at the start of a step (when not
+// nullptr).  The term comes from `one` (host values) or, for a batch, from the
+// requests' device states.
+struct ChebTerm {
+    int kn, K;             // forms T_kn; K: the step's last term
+    double ebar, inv_de, cph, sph;
+    double c0, cn;         // weights of T_0 (used when kn = 1) and of T_kn
+};
+struct ChebIO {
+    const double *X;
+    double *Y, *P, *A;
+    const void *xs;
+    void *xs_next;
+    unsigned *flags;       // two words, set when X holds a non-finite value (nullptr: not kept)
+};
+cudaError_t launch_cheb_rows(const RowOp &R, const ChebIO &io, const ChebTerm &one, sg_precision prec,
+                             cudaStream_t stream);
+cudaError_t launch_cheb_rows_batch(const RowOp *ops, const int2 *items, int nitems, int cap, const ChebIO &io,
+                                   const ChebState *st, sg_precision prec, const long long *cs_prefix,
+                                   cudaStream_t stream);
 // Chebyshev spectral interval of a context's H_S (Krylov, as sg_propagate); synchronous.
 sg_status chebyshev_bounds(sg_ctx *ctx, cudaStream_t stream, double *emin, double *emax);
 // Block Davidson of sg_eigs (method SG_DAVIDSON, same start block and
@@ -360,5 +386,9 @@ namespace sg {
 cudaError_t build_rows(sg_ctx *ctx);
 void free_rows(sg_ctx *ctx);
 cudaError_t apply_rows(sg_ctx *ctx, RowIO io, cudaStream_t s);
+
+// One recurrence term of every problem of a batch, two vectors each (sg_batch.cpp);
+// `restage`: xs is made from X first.  SG_EUNSUPPORTED when a problem is applied term by term.
+sg_status batch_cheb(sg_batch *b, const ChebIO &io, const ChebState *st, bool restage, cudaStream_t s);
 
 }  // namespace sg

@@ -19,8 +19,8 @@
 #include <algorithm>
 #include <cstring>
 
+#include "sg_cheb.cuh"
 #include "sg_df.cuh"
-#include "sg_internal.h"
 
 namespace sg {
 
@@ -206,6 +206,21 @@ __device__ __forceinline__ Vec<T, W> load_vec(const T *p)
             const uint4 t = __ldg(reinterpret_cast<const uint4 *>(p) + i);
             memcpy(reinterpret_cast<char *>(&r) + 16 * i, &t, 16);
         }
+    }
+    return r;
+}
+
+// Two adjacent values written by an earlier launch that this one may overlap (not the read-only path)
+template <typename T>
+__device__ __forceinline__ Vec<T, 2> load_pair(const T *p)
+{
+    Vec<T, 2> r;
+    if constexpr (sizeof(T) == 4) {
+        const uint2 t = __ldcg(reinterpret_cast<const uint2 *>(p));
+        memcpy(&r, &t, 8);
+    } else {
+        const uint4 t = __ldcg(reinterpret_cast<const uint4 *>(p));
+        memcpy(&r, &t, 16);
     }
     return r;
 }
@@ -537,6 +552,134 @@ __global__ void __launch_bounds__(kRT, row_blocks<T>()) k_rows_batch(const RowOp
     rows_window<T, VT, true>(R, o, R.wins[it.y], lgl, cap, smem, &bar);
 }
 
+// One Chebyshev term of a window: a thread takes a row, both vectors (the real
+// and the imaginary part), and updates the row's entry where its sum ends.
+// The record does not depend on the previous term: with programmatic launches
+// it is fetched while that term still runs (`chained`).
+template <typename T>
+__device__ __forceinline__ void cheb_window(const RowOp &R, const ChebIO &io, const ChebTerm &term, bool done,
+                                            const RowWin &win, int cap, bool chained, unsigned char *smem,
+                                            uint64_t *bar)
+{
+    const int tid = threadIdx.x;
+    const size_t n = (size_t)R.n;
+    const int bytes = row_win_bytes(win, (int)sizeof(T));
+    const bool staged = bytes <= cap;
+    if (staged && tid == 0) {
+        bar_init(bar);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        bulk_copy(smem, R.blob + win.off, (unsigned)bytes, bar);
+    }
+    __syncthreads();  // the barrier is initialised
+    const bool late = staged && !bar_wait(bar, 0);
+    if (chained) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (__syncthreads_or(late)) {
+        if (tid == 0) atomicCAS(R.err, 0, 120);
+        bar_wait(bar, 0);
+        return;
+    }
+    if (tid >= win.nrows) return;
+    const unsigned char *rec = staged ? smem : R.blob + win.off;
+    const uint2 mt = reinterpret_cast<const uint2 *>(rec)[tid];
+    const int *cols = reinterpret_cast<const int *>(rec + row_meta_bytes(win.nrows));
+    const T *vals = reinterpret_cast<const T *>(cols + win.nent);
+    const T *xs = static_cast<const T *>(io.xs);
+    const size_t re = (size_t)win.row0 + (mt.x >> 24), im = re + n;
+    // (state of an earlier launch that this one may overlap: read past the L1 cache)
+    const double xr = __ldcg(io.X + re), xi = __ldcg(io.X + im);
+    double pr = 0.0, pi = 0.0, ar = 0.0, ai = 0.0;
+    if (!done && term.kn > 1) {
+        pr = __ldcg(io.P + re);
+        pi = __ldcg(io.P + im);
+        ar = __ldcg(io.A + re);
+        ai = __ldcg(io.A + im);
+    }
+    Sum<T, 2> acc;
+    acc.zero();
+    auto load4 = [&](const int *cp, Vec<T, 2> *xv) {
+        const int4 c = *reinterpret_cast<const int4 *>(cp);
+        const int cc[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+        for (int u = 0; u < 4; u++) xv[u] = load_pair<T>(xs + 2 * (size_t)cc[u]);
+    };
+    auto sum4 = [&](const T *vp, const Vec<T, 2> *xv, int m) {
+        const Vec<T, 4> a = *reinterpret_cast<const Vec<T, 4> *>(vp);
+        acc.add4(a.v, xv, m);
+    };
+    const int *cp = cols + (mt.x & 0xFFFFFFu);
+    const T *vp = vals + (mt.x & 0xFFFFFFu);
+    const int m = (int)mt.y;
+    int e = 0;
+    for (; e + 4 < m; e += 8) {
+        Vec<T, 2> x0[4], x1[4];
+        load4(cp + e, x0);
+        load4(cp + e + 4, x1);
+        sum4(vp + e, x0, 4);
+        sum4(vp + e + 4, x1, m - e - 4);
+    }
+    if (e < m) {
+        Vec<T, 2> x0[4];
+        load4(cp + e, x0);
+        sum4(vp + e, x0, m - e);
+    }
+    const double es = __ldg(R.esplit + re);
+    const double yr = fma(es, xr, Sum<T, 2>::value(acc.bits(0))), yi = fma(es, xi, Sum<T, 2>::value(acc.bits(1)));
+    if (!finite(yr) || !finite(yi)) {
+        if (io.flags && (!finite(xr) || !finite(xi))) {  // one non-finite value makes both parts NaN at the end
+            atomicOr(io.flags, 1u);
+            atomicOr(io.flags + 1, 1u);
+        }
+        atomicCAS(R.err, 0, 201);
+    }
+    if (done) {  // past its last step: psi passes through
+        pr = xr;
+        pi = xi;
+    } else {
+        if (term.kn == 1 && io.Y) {
+            io.Y[re] = yr;
+            io.Y[im] = yi;
+        }
+        if (!cheb_entry(term, xr, xi, yr, yi, pr, pi, ar, ai)) {
+            io.A[re] = ar;
+            io.A[im] = ai;
+        }
+    }
+    io.P[re] = pr;
+    io.P[im] = pi;
+    Vec<T, 2> o;
+    o.v[0] = Elem<T>::of(pr);
+    o.v[1] = Elem<T>::of(pi);
+    *reinterpret_cast<Vec<T, 2> *>(static_cast<T *>(io.xs_next) + 2 * re) = o;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kRT) k_cheb_rows(const RowOp R, const ChebIO io, const ChebTerm term)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint64_t bar;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    cheb_window<T>(R, io, term, false, R.wins[blockIdx.x], R.cap, true, smem, &bar);
+}
+
+// Many problems: item = (problem, window); problem j's vectors from 2 * cs_prefix[j], its term from its state.
+template <typename T>
+__global__ void __launch_bounds__(kRT) k_cheb_rows_batch(const RowOp *__restrict__ ops,
+                                                         const int2 *__restrict__ items, const ChebIO io,
+                                                         const ChebState *__restrict__ st,
+                                                         const long long *__restrict__ cs_prefix, int cap)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint64_t bar;
+    const int2 it = items[blockIdx.x];
+    const RowOp &R = ops[it.x];
+    const ChebState &s = st[it.x];
+    const size_t c0 = 2 * (size_t)cs_prefix[it.x];
+    const ChebIO o{io.X + c0, io.Y + c0, io.P + c0, io.A + c0, static_cast<const T *>(io.xs) + c0,
+                   static_cast<T *>(io.xs_next) + c0, nullptr};
+    const bool done = s.step >= s.nsteps;
+    cheb_window<T>(R, o, done ? ChebTerm{} : cheb_term(s), done, R.wins[it.y], cap, false, smem, &bar);
+}
+
 // xs[r * stride + v] = x_v[r] in T (zero beyond nvec), rows r0 .. r0 + nr - 1
 template <typename T>
 __device__ __forceinline__ void stage_row(const double *__restrict__ x, size_t n, int nvec, int stride,
@@ -647,6 +790,8 @@ cudaError_t smem_limits()
     if (e == cudaSuccess) e = smem_limit(k_rows_batch<T, 1>);
     if (e == cudaSuccess) e = smem_limit(k_rows_batch<T, 2>);
     if (e == cudaSuccess) e = smem_limit(k_rows_batch<T, 4>);
+    if (e == cudaSuccess) e = smem_limit(k_cheb_rows<T>);
+    if (e == cudaSuccess) e = smem_limit(k_cheb_rows_batch<T>);
     return e;
 }
 
@@ -723,6 +868,49 @@ cudaError_t launch_rows_batch(const RowOp *ops, const int2 *items, int nitems, i
     if (nitems <= 0) return cudaSuccess;
     if (prec == SG_MIXED) return rows_batch_t<float>(ops, items, nitems, cap, wrows, io, vt, cs_prefix, stream);
     return rows_batch_t<double>(ops, items, nitems, cap, wrows, io, vt, cs_prefix, stream);
+}
+
+namespace {
+
+template <typename T>
+cudaError_t cheb_rows_t(const RowOp &R, const ChebIO &io, const ChebTerm &term, cudaStream_t s)
+{
+    if (R.nwin <= 0) return cudaSuccess;
+    // the next term's blocks may start, and fetch their records, before this one's have ended
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3((unsigned)R.nwin);
+    c.blockDim = dim3(kRT);
+    c.dynamicSmemBytes = (size_t)((R.cap + 15) & ~15);
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, k_cheb_rows<T>, R, io, term);
+}
+
+}  // namespace
+
+cudaError_t launch_cheb_rows(const RowOp &R, const ChebIO &io, const ChebTerm &one, sg_precision prec,
+                             cudaStream_t stream)
+{
+    if (prec == SG_MIXED) return cheb_rows_t<float>(R, io, one, stream);
+    if (prec == SG_DF64) return cheb_rows_t<df2>(R, io, one, stream);
+    return cheb_rows_t<double>(R, io, one, stream);
+}
+
+cudaError_t launch_cheb_rows_batch(const RowOp *ops, const int2 *items, int nitems, int cap, const ChebIO &io,
+                                   const ChebState *st, sg_precision prec, const long long *cs_prefix,
+                                   cudaStream_t stream)
+{
+    if (nitems <= 0) return cudaSuccess;
+    const size_t smem = (size_t)((cap + 15) & ~15);
+    if (prec == SG_MIXED)
+        k_cheb_rows_batch<float><<<(unsigned)nitems, kRT, smem, stream>>>(ops, items, io, st, cs_prefix, cap);
+    else
+        k_cheb_rows_batch<double><<<(unsigned)nitems, kRT, smem, stream>>>(ops, items, io, st, cs_prefix, cap);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_row_stage(const RowOp &R, const RowIO &io, sg_precision prec, cudaStream_t stream)

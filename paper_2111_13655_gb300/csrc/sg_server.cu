@@ -11,7 +11,7 @@
 // part) per request, requests one after another (the batch layout, nvec = 2).
 #include <algorithm>
 
-#include "sg_internal.h"
+#include "sg_cheb.cuh"
 
 namespace sg {
 
@@ -26,17 +26,6 @@ __device__ __forceinline__ int owner(const long long *__restrict__ prefix, int n
         if (prefix[mid] <= g) lo = mid; else hi = mid - 1;
     }
     return lo;
-}
-
-// (-i)^q (tr + i ti)
-__device__ __forceinline__ void rot(int q, double tr, double ti, double &outr, double &outi)
-{
-    switch (q & 3) {
-        case 0: outr = tr; outi = ti; break;
-        case 1: outr = ti; outi = -tr; break;
-        case 2: outr = -tr; outi = -ti; break;
-        default: outr = -ti; outi = tr; break;
-    }
 }
 
 // X = T_k, Y = H T_k, P = T_{k-1} (unused when forming T_1), A = partial sum;
@@ -61,59 +50,45 @@ __global__ void k_cheb_update(const ChebState *__restrict__ st, const long long 
             P[im] = xi;
             continue;
         }
-        const int kn = it.k + 1;
-        const double hr = (Y[re] - it.ebar * xr) * it.inv_de, hi = (Y[im] - it.ebar * xi) * it.inv_de;
-        double tr, ti, ar, ai;
-        if (it.k == 0) {
-            tr = hr;
-            ti = hi;
-            ar = it.c[0] * xr;
-            ai = it.c[0] * xi;
-        } else {
-            tr = 2.0 * hr - P[re];
-            ti = 2.0 * hi - P[im];
+        const ChebTerm t = cheb_term(it);
+        double pr = 0.0, pi = 0.0, ar = 0.0, ai = 0.0;
+        if (t.kn > 1) {
+            pr = P[re];
+            pi = P[im];
             ar = A[re];
             ai = A[im];
         }
-        double qr, qi;
-        rot(kn, tr, ti, qr, qi);
-        const double cn = it.c[kn];
-        ar = fma(cn, qr, ar);
-        ai = fma(cn, qi, ai);
-        if (kn == it.K) {
-            P[re] = it.cph * ar - it.sph * ai;
-            P[im] = it.sph * ar + it.cph * ai;
-        } else {
-            P[re] = tr;
-            P[im] = ti;
+        const bool last = cheb_entry(t, xr, xi, Y[re], Y[im], pr, pi, ar, ai);
+        P[re] = pr;
+        P[im] = pi;
+        if (!last) {
             A[re] = ar;
             A[im] = ai;
         }
     }
 }
 
-// Moves every request to its next recurrence term (after k_cheb_update).
-__global__ void k_cheb_advance(ChebState *st, int nitems)
-{
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= nitems) return;
-    ChebState &s = st[j];
-    if (s.step >= s.nsteps) return;
-    if (s.k + 1 == s.K) { s.k = 0; s.step++; }
-    else s.k++;
-}
-
-// One block per request; requests at the start of a step (k = 0) log
-// <psi|psi> and <psi|H psi>/<psi|psi> over their own entries, summed in an
-// order that depends on their size only.
+// One block per request, after the update: requests at the start of a step
+// (k = 0) log <psi|psi> and <psi|H psi>/<psi|psi> over their own entries,
+// summed in an order that depends on their size only; then every request moves
+// to its next recurrence term.
 constexpr int kLogThreads = 256;
-__global__ void __launch_bounds__(kLogThreads) k_cheb_log(const ChebState *__restrict__ st,
-                                                          const long long *__restrict__ prefix,
-                                                          const double *__restrict__ X,
-                                                          const double *__restrict__ Y)
+__global__ void __launch_bounds__(kLogThreads) k_cheb_log_advance(ChebState *st,
+                                                                  const long long *__restrict__ prefix,
+                                                                  const double *__restrict__ X,
+                                                                  const double *__restrict__ Y)
 {
-    const ChebState &S = st[blockIdx.x];
-    if (S.k != 0 || S.step >= S.nsteps) return;
+    ChebState &S = st[blockIdx.x];
+    const int k = S.k, step = S.step, K = S.K;
+    __syncthreads();  // every thread has read the state that thread 0 moves on
+    if (step >= S.nsteps) return;
+    if (k != 0) {
+        if (threadIdx.x == 0) {
+            S.k = k + 1 == K ? 0 : k + 1;
+            if (k + 1 == K) S.step = step + 1;
+        }
+        return;
+    }
     const long long off = prefix[blockIdx.x], n = prefix[blockIdx.x + 1] - off;
     const double *xr = X + 2 * off, *xi = xr + n, *yr = Y + 2 * off, *yi = yr + n;
     double nn = 0.0, ee = 0.0;
@@ -133,8 +108,10 @@ __global__ void __launch_bounds__(kLogThreads) k_cheb_log(const ChebState *__res
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        S.log[2 * S.step] = sn[0];
-        S.log[2 * S.step + 1] = se[0] / sn[0];
+        S.log[2 * step] = sn[0];
+        S.log[2 * step + 1] = se[0] / sn[0];
+        if (K == 1) S.step = step + 1;
+        else S.k = 1;
     }
 }
 
@@ -144,10 +121,17 @@ cudaError_t launch_cheb_iteration(ChebState *st, const long long *prefix, int ni
                                   const double *X, const double *Y, double *P, double *A, cudaStream_t s)
 {
     if (nitems <= 0 || total <= 0) return cudaSuccess;
-    k_cheb_log<<<(unsigned)nitems, kLogThreads, 0, s>>>(st, prefix, X, Y);
     const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 152 * 8));
     k_cheb_update<<<blocks, 256, 0, s>>>(st, prefix, nitems, X, Y, P, A);
-    k_cheb_advance<<<(unsigned)((nitems + 127) / 128), 128, 0, s>>>(st, nitems);
+    k_cheb_log_advance<<<(unsigned)nitems, kLogThreads, 0, s>>>(st, prefix, X, Y);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_cheb_log_advance(ChebState *st, const long long *prefix, int nitems, const double *X,
+                                    const double *Y, cudaStream_t s)
+{
+    if (nitems <= 0) return cudaSuccess;
+    k_cheb_log_advance<<<(unsigned)nitems, kLogThreads, 0, s>>>(st, prefix, X, Y);
     return cudaGetLastError();
 }
 

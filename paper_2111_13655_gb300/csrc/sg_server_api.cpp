@@ -109,6 +109,11 @@ struct sg_server {
     bool dirty = false;
     // state buffers over the active requests (batch layout, nvec = 2)
     double *X = nullptr, *Y = nullptr, *P = nullptr, *A = nullptr;
+    // entry-major copies (contraction type) of the two state buffers, and the
+    // buffer that the first belongs to; valid: the copy of X is up to date
+    void *xs[2] = {nullptr, nullptr};
+    const double *xs_of = nullptr;
+    bool xs_valid = false;
     int64_t total = 0;
     int nslots = 0;
     sg::ChebState *d_state = nullptr;
@@ -138,6 +143,11 @@ void free_state(sg_server *s)
 {
     for (double **p : {&s->X, &s->Y, &s->P, &s->A})
         if (*p) { cudaFree(*p); *p = nullptr; }
+    for (void *&p : s->xs) {
+        if (p) cudaFree(p);
+        p = nullptr;
+    }
+    s->xs_valid = false;
     if (s->d_state) cudaFree(s->d_state);
     if (s->d_prefix) cudaFree(s->d_prefix);
     s->d_state = nullptr;
@@ -249,6 +259,10 @@ sg_status relayout(sg_server *s)
         return sfail(s, SG_ECUDA, std::string("relayout sync: ") + cudaGetErrorString(e));
     free_state(s);
     s->X = nb[0]; s->Y = nb[1]; s->P = nb[2]; s->A = nb[3];
+    s->xs_of = s->X;
+    for (void *&p : s->xs)
+        if (total > 0 && (e = cudaMalloc(&p, 2 * (size_t)total * sg::row_value_bytes(s->prec))) != cudaSuccess)
+            return sfail(s, SG_ENOMEM, std::string("server state cudaMalloc: ") + cudaGetErrorString(e));
     s->total = total;
     s->nslots = (int)state.size();
     const size_t na = std::max<size_t>(1, state.size());
@@ -429,11 +443,36 @@ sg_status admit(sg_server *s)
     return SG_OK;
 }
 
+bool has_eig(const sg_server *s)
+{
+    for (const Req *r : s->active)
+        if (r->kind == kEig) return true;
+    return false;
+}
+
 // One engine iteration with the current roles of X and P: Y = H X over all
-// active requests, then logs, recurrence update (into P) and state advance,
-// over every two-vector slot (an eigen request holds several).
+// active requests, recurrence update (into P), logs and state advance, over
+// every two-vector slot (an eigen request holds several).  With propagation
+// requests alone the first two are one launch; an eigen block needs all of Y.
+// Both ways give the same bits.
 sg_status enqueue_iteration(sg_server *s, double *X, double *P)
 {
+    if (!has_eig(s)) {
+        // application, update and the next term's entry-major copy in one launch
+        const int c = X == s->xs_of ? 0 : 1;
+        const sg::ChebIO io{X, s->Y, P, s->A, s->xs[c], s->xs[1 - c], nullptr};
+        const sg_status sr = sg::batch_cheb(s->batch, io, s->d_state, !s->xs_valid, s->stream);
+        if (sr == SG_OK) {
+            s->xs_valid = true;
+            const cudaError_t el =
+                sg::launch_cheb_log_advance(s->d_state, s->d_prefix, s->nslots, X, s->Y, s->stream);
+            if (el != cudaSuccess) return sfail(s, SG_ECUDA, std::string("log launch: ") + cudaGetErrorString(el));
+            return SG_OK;
+        }
+        if (sr != SG_EUNSUPPORTED)
+            return sfail(s, sr, std::string("batched recurrence: ") + sg_batch_last_error(s->batch));
+    }
+    s->xs_valid = false;
     sg_status st = sg_apply_H_batch(s->batch, X, s->Y, 2, s->stream);
     if (st != SG_OK) return sfail(s, st, std::string("batched apply: ") + sg_batch_last_error(s->batch));
     cudaError_t e = sg::launch_cheb_iteration(s->d_state, s->d_prefix, s->nslots, s->total, X, s->Y, P, s->A,
@@ -451,13 +490,15 @@ sg_status iterate(sg_server *s, int64_t n)
     sg_status st;
     int64_t done = 0;
     int slot = s->graph_x[0] == s->X ? 0 : (s->graph_x[1] == s->X ? 1 : -1);
+    // the first iteration of a layout, outside any capture, sizes the batch
+    // workspace or makes the entry-major copy of X that a captured pair starts from
+    if (n >= 3 && ((!s->graph_x[0] && !s->graph_x[1]) || !s->xs_valid)) {
+        if ((st = enqueue_iteration(s, s->X, s->P)) != SG_OK) return st;
+        std::swap(s->X, s->P);
+        done = 1;
+        slot = s->graph_x[0] == s->X ? 0 : (s->graph_x[1] == s->X ? 1 : -1);
+    }
     if (slot < 0 && n >= 3) {
-        if (!s->graph_x[0] && !s->graph_x[1]) {
-            // the first iteration sizes the batch workspace outside any capture
-            if ((st = enqueue_iteration(s, s->X, s->P)) != SG_OK) return st;
-            std::swap(s->X, s->P);
-            done = 1;
-        }
         slot = s->graph_x[0] ? 1 : 0;
         if ((e = cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
             return sfail(s, SG_ECUDA, std::string("begin capture: ") + cudaGetErrorString(e));
@@ -494,13 +535,6 @@ int64_t until_first_finish(const sg_server *s)
     for (const Req *r : s->active)
         if (r->kind == kProp) m = std::min<int64_t>(m, (int64_t)(r->nsteps - r->step - 1) * r->K + (r->K - r->k));
     return m;
-}
-
-bool has_eig(const sg_server *s)
-{
-    for (const Req *r : s->active)
-        if (r->kind == kEig) return true;
-    return false;
 }
 
 // Waits (at most 600 s) until every active eigen request has handed over a

@@ -441,6 +441,60 @@ void spectral_bounds(Solver &S, double &emin, double &emax)
     emax = th[k - 1] + std::sqrt(rn2[1]) + 0.05 * range;
 }
 
+// The steps of sg_propagate on the row form: one launch per Chebyshev term.
+void propagate_rows(Solver &S, double *psi, double Ebar, double dE, double dt, const std::vector<double> &J, int kend,
+                    int nsteps, double *norm_log, double *energy_log)
+{
+    if (nsteps == 0) return;
+    const size_t n = (size_t)S.n;
+    const sg_precision prec = S.ctx->prob.prec;
+    const size_t rb = (size_t)row_value_bytes(prec);
+    const bool logs = norm_log || energy_log;
+    // T_k and T_{k-1}, the partial sum, H psi, the two entry-major copies, inner products of every step, flags
+    DBuf mem(8 * n + 2 * (2 * n * rb + 7) / 8 + 8 * (size_t)nsteps + 4);
+    double *x = mem.p, *p = x + 2 * n, *acc = p + 2 * n, *y = acc + 2 * n, *c0 = y + 2 * n;
+    unsigned char *xs = reinterpret_cast<unsigned char *>(c0), *xn = xs + 2 * n * rb;
+    double *dots = c0 + 2 * (2 * n * rb + 7) / 8;
+    unsigned *flags = reinterpret_cast<unsigned *>(dots + 8 * (size_t)nsteps);
+    ck(cudaMemsetAsync(flags, 0, 2 * sizeof(unsigned), S.s), "flags");
+    ck(cudaMemcpyAsync(x, psi, sizeof(double) * 2 * n, cudaMemcpyDeviceToDevice, S.s), "psi copy");
+    RowIO r{};
+    r.x = x;
+    r.xs = xs;
+    r.nvec = 2;
+    r.stride = xs_stride(2);
+    ck(launch_row_stage(S.ctx->rop, r, prec, S.s), "psi stage");
+    for (int step = 0; step < nsteps; step++) {
+        for (int kn = 1; kn <= kend; kn++) {
+            const ChebIO io{x, logs ? y : nullptr, p, acc, xs, xn, flags};
+            const ChebTerm t{kn, kend, Ebar, 1.0 / dE, std::cos(Ebar * dt), -std::sin(Ebar * dt), J[0], 2.0 * J[kn]};
+            ck(launch_cheb_rows(S.ctx->rop, io, t, prec, S.s), "chebyshev term");
+            if (kn == 1 && logs) {  // <psi|psi> and <psi|H psi> of the parts: the diagonals of 2 x 2 products
+                ck(dev_gram(x, 2, x, 2, (int64_t)n, dots + 8 * step, S.partial.p, S.s), "norm");
+                ck(dev_gram(x, 2, y, 2, (int64_t)n, dots + 8 * step + 4, S.partial.p, S.s), "energy");
+            }
+            std::swap(x, p);
+            std::swap(xs, xn);
+        }
+    }
+    ck(cudaMemcpyAsync(psi, x, sizeof(double) * 2 * n, cudaMemcpyDeviceToDevice, S.s), "psi copy");
+    RowIO f{};
+    f.y = psi;
+    f.flags = flags;
+    f.nvec = 2;
+    ck(launch_row_settle(f, (int)n, S.s), "settle");
+    S.sync("propagate sync");
+    if (!logs) return;
+    std::vector<double> h(8 * (size_t)nsteps);
+    ck(cudaMemcpy(h.data(), dots, sizeof(double) * h.size(), cudaMemcpyDeviceToHost), "logs");
+    for (int step = 0; step < nsteps; step++) {
+        const double *q = &h[8 * (size_t)step];
+        const double nn = q[0] + q[3];
+        if (norm_log) norm_log[step] = nn;
+        if (energy_log) energy_log[step] = (q[4] + q[7]) / nn;
+    }
+}
+
 }  // namespace
 
 extern "C" {
@@ -537,6 +591,10 @@ sg_status sg_propagate(sg_ctx *ctx, double *psi, double dt, int nsteps, int orde
         const std::vector<double> J = bessel_j(order, dE * dt);
         int kend = order;  // skip terms whose Bessel weight is below double precision
         while (kend > 1 && kend > dE * dt && std::fabs(J[kend]) < 1e-17) kend--;
+        if (ctx->host.rows) {
+            propagate_rows(S, psi, Ebar, dE, dt, J, kend, nsteps, norm_log, energy_log);
+            return SG_OK;
+        }
         // phi buffers: 2 real vectors (re, im) each
         DBuf p0(2 * (size_t)n), p1(2 * (size_t)n), hp(2 * (size_t)n), acc(2 * (size_t)n);
         const double cph = std::cos(Ebar * dt), sph = -std::sin(Ebar * dt);  // e^{-i Ebar dt}
