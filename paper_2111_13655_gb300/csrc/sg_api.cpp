@@ -5,7 +5,9 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <vector>
 
+#include "sg_arena.h"
 #include "sg_internal.h"
 
 namespace {
@@ -45,7 +47,6 @@ void free_workspace(sg_ctx *ctx)
     if (ctx->acc) cudaFree(ctx->acc);
     if (ctx->maxbits) cudaFree(ctx->maxbits);
     if (ctx->xs) cudaFree(ctx->xs);
-    if (ctx->flags) cudaFree(ctx->flags);
     ctx->acc = nullptr;
     ctx->maxbits = nullptr;
     ctx->xs = nullptr;
@@ -77,10 +78,11 @@ sg_status ensure_workspace(sg_ctx *ctx, int nvec, cudaStream_t s)
     if (e != cudaSuccess) return cuda_fail(ctx, e, "stream synchronize");
     free_workspace(ctx);
     if (ctx->host.rows) {
-        const size_t xs_bytes = (size_t)ctx->host.n_cs * sg::xs_stride(nvec) * sg::row_value_bytes(ctx->prob.prec);
-        if ((e = cudaMalloc(&ctx->flags, sizeof(unsigned) * nvec)) != cudaSuccess ||
-            (e = cudaMalloc(&ctx->xs, xs_bytes)) != cudaSuccess)
+        const size_t xs_bytes =
+            (((size_t)ctx->host.n_cs * sg::xs_stride(nvec) * sg::row_value_bytes(ctx->prob.prec)) + 15) & ~(size_t)15;
+        if ((e = cudaMalloc(&ctx->xs, xs_bytes + sizeof(unsigned) * nvec)) != cudaSuccess)
             return fail(ctx, SG_ENOMEM, std::string("workspace cudaMalloc: ") + cudaGetErrorString(e));
+        ctx->flags = reinterpret_cast<unsigned *>(static_cast<unsigned char *>(ctx->xs) + xs_bytes);
         if ((e = cudaMemsetAsync(ctx->flags, 0, sizeof(unsigned) * nvec, s)) != cudaSuccess)
             return cuda_fail(ctx, e, "workspace memset");
     } else {
@@ -218,22 +220,6 @@ void free_rows(sg_ctx *ctx)
     ctx->rop = RowOp{};
 }
 
-namespace {
-
-template <typename T>
-cudaError_t row_upload(std::vector<void *> &own, const T *src, size_t n, T **dst, int64_t *bytes)
-{
-    *dst = nullptr;
-    const size_t b = std::max<size_t>(1, n) * sizeof(T);
-    cudaError_t e = cudaMalloc(reinterpret_cast<void **>(dst), b);
-    if (e != cudaSuccess) return e;
-    own.push_back(*dst);
-    if (bytes) *bytes += (int64_t)b;
-    return src && n ? cudaMemcpy(*dst, src, n * sizeof(T), cudaMemcpyHostToDevice) : cudaSuccess;
-}
-
-}  // namespace
-
 cudaError_t build_rows(sg_ctx *ctx)
 {
     free_rows(ctx);
@@ -241,44 +227,43 @@ cudaError_t build_rows(sg_ctx *ctx)
     const KParams &kp = ctx->kp;
     const sg_precision prec = ctx->prob.prec;
     const size_t n = (size_t)T.n_cs;
-    std::vector<void *> tmp;  // set-up tables, released below
+    // set-up tables (released below) and the row lengths
+    Arena A;
+    const size_t o[9] = {A.add(T.sh_off), A.add(T.sh_mode), A.add(T.sh_d), A.add(T.sh_src_off), A.add(T.sh_src),
+                         A.add(T.pr_off), A.add(T.pr_mode), A.add(T.pr_op), A.add(T.pr_coef)};
+    unsigned char *set = nullptr, *plan = nullptr, *own = nullptr;
+    size_t at = 0;
+    cudaError_t e = A.put(&set, n * sizeof(int), &at);
     RowShifts S{};
     S.nshift = (int)T.sh_off.size() - 1;
-    int *cnt = nullptr;
-    cudaError_t e = cudaSuccess;
-    auto ints = [&](const std::vector<int> &v, const int **dst) {
-        int *p = nullptr;
-        if (e == cudaSuccess) e = row_upload(tmp, v.data(), v.size(), &p, nullptr);
-        *dst = p;
-    };
-    ints(T.sh_off, &S.off); ints(T.sh_mode, &S.mode); ints(T.sh_d, &S.d);
-    ints(T.sh_src_off, &S.src_off); ints(T.sh_src, &S.src);
-    ints(T.pr_off, &S.prod_off); ints(T.pr_mode, &S.fmode); ints(T.pr_op, &S.fop);
-    double *coef = nullptr;
-    if (e == cudaSuccess) e = row_upload(tmp, T.pr_coef.data(), T.pr_coef.size(), &coef, nullptr);
-    S.coef = coef;
-    if (e == cudaSuccess) e = row_upload<int>(tmp, nullptr, n, &cnt, nullptr);
-    if (e == cudaSuccess) e = launch_row_count(kp, S, cnt, 0);
+    auto ints = [&](int q) { return reinterpret_cast<const int *>(set + o[q]); };
+    if (e == cudaSuccess) {
+        S.off = ints(0); S.mode = ints(1); S.d = ints(2); S.src_off = ints(3); S.src = ints(4);
+        S.prod_off = ints(5); S.fmode = ints(6); S.fop = ints(7);
+        S.coef = reinterpret_cast<const double *>(set + o[8]);
+        e = launch_row_count(kp, S, reinterpret_cast<int *>(set + at), 0);
+    }
     std::vector<int> hc(n);
-    if (e == cudaSuccess) e = cudaMemcpy(hc.data(), cnt, n * sizeof(int), cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(hc.data(), set + at, n * sizeof(int), cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) {
         const RowWindows W = cut_rows(hc, row_window_rows((int64_t)n, row_window_units(T)), row_budget(T, prec),
                                       row_value_bytes(prec));
+        Arena B, C;  // for the fill kernel; kept: the windows and their records
+        const size_t meta = B.add(W.meta), win = B.add(W.win), start = B.add(W.start);
+        size_t rec = 0;
+        C.add(W.wins);
+        e = B.put(&plan);
+        if (e == cudaSuccess) e = C.put(&own, (size_t)W.bytes, &rec);
+        if (own) ctx->row_allocs.push_back(own);
         RowOp R{};
-        RowWin *wins = nullptr;
-        unsigned char *blob = nullptr;
-        uint2 *meta = nullptr;
-        const int *win = nullptr, *start = nullptr;
-        int64_t bytes = 0;
-        e = row_upload(ctx->row_allocs, W.wins.data(), W.wins.size(), &wins, &bytes);
-        if (e == cudaSuccess) e = row_upload<unsigned char>(ctx->row_allocs, nullptr, (size_t)W.bytes, &blob, &bytes);
-        if (e == cudaSuccess) e = row_upload(tmp, W.meta.data(), W.meta.size(), &meta, nullptr);
-        ints(W.win, &win);
-        ints(W.start, &start);
-        if (e == cudaSuccess) e = launch_row_fill(kp, S, prec, wins, win, start, meta, blob, 0);
+        if (e == cudaSuccess) {
+            R.wins = reinterpret_cast<const RowWin *>(own);
+            R.blob = own + rec;
+            e = launch_row_fill(kp, S, prec, R.wins, reinterpret_cast<const int *>(plan + win),
+                                reinterpret_cast<const int *>(plan + start), reinterpret_cast<const uint2 *>(plan + meta),
+                                own + rec, 0);
+        }
         if (e == cudaSuccess) e = cudaStreamSynchronize(0);
-        R.blob = blob;
-        R.wins = wins;
         R.esplit = kp.esplit;
         R.err = kp.err;
         R.nwin = (int)W.wins.size();
@@ -288,10 +273,11 @@ cudaError_t build_rows(sg_ctx *ctx)
         ctx->rop = R;
         ctx->win_entries.resize(W.wins.size());
         for (size_t w = 0; w < W.wins.size(); w++) ctx->win_entries[w] = W.wins[w].nent;
-        ctx->row_bytes = bytes;
-        ctx->bytes_device += bytes;
+        ctx->row_bytes = (int64_t)(rec + W.bytes);
+        ctx->bytes_device += ctx->row_bytes;
     }
-    for (void *p : tmp) cudaFree(p);
+    if (set) cudaFree(set);
+    if (plan) cudaFree(plan);
     if (e != cudaSuccess) {
         free_rows(ctx);
         (void)cudaGetLastError();  // reported here; not by a later launch
@@ -338,32 +324,57 @@ sg_status sg_create(int D, int L, const sg_basis *basis, const sg_grid *grids,
     Problem &p = ctx->prob;
     HostTables &T = ctx->host;
     KParams &kp = ctx->kp;
-    std::vector<float> tabf(T.tabd.begin(), T.tabd.end());
-    std::vector<int> zero(1, 0);
     sg_status st = SG_OK;
-    const int *errp = nullptr;
-    if ((st = upload(ctx, T.levels, &kp.levels)) != SG_OK ||
-        (st = upload(ctx, T.coefs, &kp.coefs)) != SG_OK ||
-        (st = upload(ctx, T.order, &kp.order)) != SG_OK ||
-        (st = upload(ctx, T.rank_tab, &kp.rank_tab)) != SG_OK ||
-        (st = upload(ctx, T.lmin_tab, &kp.lmin_tab)) != SG_OK ||
-        (st = upload(ctx, T.lvl, &kp.lvl)) != SG_OK ||
-        (st = upload(ctx, T.tabd, &kp.tabd)) != SG_OK ||
-        (st = upload(ctx, tabf, &kp.tabf)) != SG_OK ||
-        (st = upload(ctx, p.mcoef, &kp.mcoef)) != SG_OK ||
-        (st = upload(ctx, p.mnfac, &kp.mnfac)) != SG_OK ||
-        (st = upload(ctx, p.mfoff, &kp.mfoff)) != SG_OK ||
-        (st = upload(ctx, p.mfmode, &kp.mfmode)) != SG_OK ||
-        (st = upload(ctx, p.mfpow, &kp.mfpow)) != SG_OK ||
-        (st = upload(ctx, T.harm_mono, &kp.harm_mono)) != SG_OK ||
-        (st = upload(ctx, T.esplit, &kp.esplit)) != SG_OK ||
-        (st = upload(ctx, zero, &errp)) != SG_OK) {
-        g_create_error = ctx->last_error;
-        free_all(ctx);
-        delete ctx;
-        return st;
+    if (T.rows) {
+        // what the row form's set-up kernels and the index map read, and the harmonic energies
+        sg::Arena A;
+        const int zero = 0;
+        const size_t rank = A.add(T.rank_tab), lmin = A.add(T.lmin_tab), lvl = A.add(T.lvl), tab = A.add(T.tabd),
+                     es = A.add(T.esplit), err = A.add(&zero, 1);
+        unsigned char *base = nullptr;
+        e = A.put(&base);
+        if (base) ctx->allocations.push_back(base);
+        if (e != cudaSuccess) {
+            st = fail(nullptr, e == cudaErrorMemoryAllocation ? SG_ENOMEM : SG_ECUDA,
+                      std::string("cudaMalloc: ") + cudaGetErrorString(e));
+            free_all(ctx);
+            delete ctx;
+            return st;
+        }
+        ctx->bytes_device += (int64_t)A.host.size();
+        kp.rank_tab = reinterpret_cast<const int *>(base + rank);
+        kp.lmin_tab = base + lmin;
+        kp.lvl = reinterpret_cast<const LevelInfo *>(base + lvl);
+        kp.tabd = reinterpret_cast<const double *>(base + tab);
+        kp.esplit = reinterpret_cast<const double *>(base + es);
+        kp.err = reinterpret_cast<int *>(base + err);
+    } else {
+        const std::vector<float> tabf(T.tabd.begin(), T.tabd.end());
+        const std::vector<int> zero(1, 0);
+        const int *errp = nullptr;
+        if ((st = upload(ctx, T.levels, &kp.levels)) != SG_OK ||
+            (st = upload(ctx, T.coefs, &kp.coefs)) != SG_OK ||
+            (st = upload(ctx, T.order, &kp.order)) != SG_OK ||
+            (st = upload(ctx, T.rank_tab, &kp.rank_tab)) != SG_OK ||
+            (st = upload(ctx, T.lmin_tab, &kp.lmin_tab)) != SG_OK ||
+            (st = upload(ctx, T.lvl, &kp.lvl)) != SG_OK ||
+            (st = upload(ctx, T.tabd, &kp.tabd)) != SG_OK ||
+            (st = upload(ctx, tabf, &kp.tabf)) != SG_OK ||
+            (st = upload(ctx, p.mcoef, &kp.mcoef)) != SG_OK ||
+            (st = upload(ctx, p.mnfac, &kp.mnfac)) != SG_OK ||
+            (st = upload(ctx, p.mfoff, &kp.mfoff)) != SG_OK ||
+            (st = upload(ctx, p.mfmode, &kp.mfmode)) != SG_OK ||
+            (st = upload(ctx, p.mfpow, &kp.mfpow)) != SG_OK ||
+            (st = upload(ctx, T.harm_mono, &kp.harm_mono)) != SG_OK ||
+            (st = upload(ctx, T.esplit, &kp.esplit)) != SG_OK ||
+            (st = upload(ctx, zero, &errp)) != SG_OK) {
+            g_create_error = ctx->last_error;
+            free_all(ctx);
+            delete ctx;
+            return st;
+        }
+        kp.err = const_cast<int *>(errp);
     }
-    kp.err = const_cast<int *>(errp);
     ctx->has_device = true;
     if (p.prec == SG_DF64 && (!T.rows || !term_form(p, T).fits)) {
         st = fail(nullptr, SG_EUNSUPPORTED,
@@ -557,14 +568,20 @@ sg_status sg_index_map(sg_ctx *ctx, int64_t t0, int64_t nt, int64_t *offsets_hos
     if (!cs_index_dev || nt == 0) return SG_OK;
     if (!ctx->has_device) return fail(ctx, SG_EINVAL, "context was made by sg_plan (no device state)");
     if (!sg_on_ctx_device(ctx)) return fail(ctx, SG_EINVAL, "the current CUDA device is not the one the context was made on");
-    int64_t *offs_dev = nullptr;
+    // the offsets and the levels of the range
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = cudaMalloc(&offs_dev, sizeof(int64_t) * (nt + 1));
-    if (e != cudaSuccess) return fail(ctx, SG_ENOMEM, "cudaMalloc offsets");
-    e = cudaMemcpyAsync(offs_dev, offsets_host, sizeof(int64_t) * (nt + 1), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = sg::launch_index_map(ctx->kp, t0, nt, offs_dev, cs_index_dev, s);
+    sg::Arena A;
+    const size_t off = A.add(offsets_host, (size_t)nt + 1);
+    const size_t lev = A.add(T.levels.data() + (size_t)t0 * T.Dpad, (size_t)nt * T.Dpad);
+    unsigned char *base = nullptr;
+    cudaError_t e = A.put(&base);
+    if (!base) return fail(ctx, SG_ENOMEM, "cudaMalloc offsets");
+    sg::KParams kp = ctx->kp;
+    kp.levels = base + lev;
+    if (e == cudaSuccess)
+        e = sg::launch_index_map(kp, 0, nt, reinterpret_cast<const int64_t *>(base + off), cs_index_dev, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(offs_dev);
+    cudaFree(base);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "index map");
     return SG_OK;
 }

@@ -6,6 +6,7 @@
 #include <string>
 #include <vector>
 
+#include "sg_arena.h"
 #include "sg_internal.h"
 
 // A problem with at least this many rows fills the GPU for several waves by
@@ -54,20 +55,6 @@ sg_status bfail(sg_batch *b, sg_status st, const std::string &msg)
 {
     if (b) b->last_error = msg;
     return st;
-}
-
-template <typename T>
-sg_status bupload(sg_batch *b, const std::vector<T> &v, const T **dst)
-{
-    void *p = nullptr;
-    const size_t bytes = std::max<size_t>(1, v.size()) * sizeof(T);
-    cudaError_t e = cudaMalloc(&p, bytes);
-    if (e != cudaSuccess) return bfail(b, SG_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
-    b->allocations.push_back(p);
-    if (!v.empty() && (e = cudaMemcpy(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice)) != cudaSuccess)
-        return bfail(b, SG_ECUDA, std::string("cudaMemcpy: ") + cudaGetErrorString(e));
-    *dst = static_cast<const T *>(p);
-    return SG_OK;
 }
 
 void drop_graph(sg_batch *b)
@@ -156,14 +143,23 @@ extern "C" sg_status sg_batch_create(sg_ctx *const *ctxs, int n, sg_batch **out)
     b->n_stage = (int)stage.size();
     b->n_all = (int)all_items.size();
     b->n_all_stage = (int)all_stage.size();
-    sg_status st;
-    if ((st = bupload(b, ops, &b->d_ops)) != SG_OK || (st = bupload(b, b->cs_prefix, &b->d_cs_prefix)) != SG_OK ||
-        (st = bupload(b, items, &b->items)) != SG_OK || (st = bupload(b, stage, &b->stage_items)) != SG_OK ||
-        (st = bupload(b, all_items, &b->all_items)) != SG_OK || (st = bupload(b, all_stage, &b->all_stage)) != SG_OK) {
+    sg::Arena A;
+    const size_t o[6] = {A.add(ops), A.add(b->cs_prefix), A.add(items), A.add(stage), A.add(all_items), A.add(all_stage)};
+    unsigned char *base = nullptr;
+    const cudaError_t e = A.put(&base);
+    if (base) b->allocations.push_back(base);
+    if (e != cudaSuccess) {
+        const sg_status st = e == cudaErrorMemoryAllocation ? SG_ENOMEM : SG_ECUDA;
         free_all(b);
         delete b;
         return st;
     }
+    b->d_ops = reinterpret_cast<const sg::RowOp *>(base + o[0]);
+    b->d_cs_prefix = reinterpret_cast<const long long *>(base + o[1]);
+    b->items = reinterpret_cast<const int2 *>(base + o[2]);
+    b->stage_items = reinterpret_cast<const int2 *>(base + o[3]);
+    b->all_items = reinterpret_cast<const int2 *>(base + o[4]);
+    b->all_stage = reinterpret_cast<const int2 *>(base + o[5]);
     *out = b;
     return SG_OK;
 }

@@ -360,8 +360,8 @@ struct sg_ctx {
     int64_t row_bytes = 0;
     // apply workspace.  Row form: per-vector flags and the entry-major input
     // copy; term-by-term kernel: fixed-point accumulators and scale exponents
-    unsigned *flags = nullptr;
     void *xs = nullptr;
+    unsigned *flags = nullptr;  // behind xs, in its allocation
     unsigned long long *acc = nullptr;
     long long *maxbits = nullptr;
     int acc_nvec = 0;

@@ -39,6 +39,7 @@
 #include <thread>
 #include <vector>
 
+#include "sg_arena.h"
 #include "sg_internal.h"
 
 namespace {
@@ -108,6 +109,8 @@ struct sg_server {
     sg_batch *batch = nullptr;
     bool dirty = false;
     // state buffers over the active requests (batch layout, nvec = 2)
+    // (one allocation, with the copies and tables below)
+    unsigned char *state_mem = nullptr;
     double *X = nullptr, *Y = nullptr, *P = nullptr, *A = nullptr;
     // entry-major copies (contraction type) of the two state buffers, and the
     // buffer that the first belongs to; valid: the copy of X is up to date
@@ -141,15 +144,11 @@ sg_status sfail(sg_server *s, sg_status st, const std::string &m)
 
 void free_state(sg_server *s)
 {
-    for (double **p : {&s->X, &s->Y, &s->P, &s->A})
-        if (*p) { cudaFree(*p); *p = nullptr; }
-    for (void *&p : s->xs) {
-        if (p) cudaFree(p);
-        p = nullptr;
-    }
+    if (s->state_mem) cudaFree(s->state_mem);
+    s->state_mem = nullptr;
+    s->X = s->Y = s->P = s->A = nullptr;
+    s->xs[0] = s->xs[1] = nullptr;
     s->xs_valid = false;
-    if (s->d_state) cudaFree(s->d_state);
-    if (s->d_prefix) cudaFree(s->d_prefix);
     s->d_state = nullptr;
     s->d_prefix = nullptr;
     s->total = 0;
@@ -226,14 +225,19 @@ sg_status relayout(sg_server *s)
         }
     }
     const int64_t total = prefix.back();
-    double *nb[4] = {nullptr, nullptr, nullptr, nullptr};
-    if (total > 0) {
-        for (double *&p : nb)
-            if ((e = cudaMalloc(&p, sizeof(double) * 2 * (size_t)total)) != cudaSuccess) {
-                for (double *q : nb) if (q) cudaFree(q);
-                return sfail(s, SG_ENOMEM, std::string("server state cudaMalloc: ") + cudaGetErrorString(e));
-            }
+    // the recurrence states and the layout, then the state vectors and their entry-major copies
+    sg::Arena T;
+    const size_t at_state = T.add(state), at_prefix = T.add(prefix);
+    const size_t vec = sizeof(double) * 2 * (size_t)total, copy = 2 * (size_t)total * sg::row_value_bytes(s->prec);
+    unsigned char *mem = nullptr;
+    size_t at = 0;
+    if ((e = T.put(&mem, 4 * vec + 2 * copy, &at)) != cudaSuccess) {
+        if (mem) cudaFree(mem);
+        return sfail(s, e == cudaErrorMemoryAllocation ? SG_ENOMEM : SG_ECUDA,
+                     std::string("server state cudaMalloc: ") + cudaGetErrorString(e));
     }
+    double *nb[4];
+    for (int q = 0; q < 4; q++) nb[q] = reinterpret_cast<double *>(mem + at + q * vec);
     double *old[4] = {s->X, s->Y, s->P, s->A};
     for (size_t j = 0; j < s->active.size(); j++) {
         Req *r = s->active[j];
@@ -258,22 +262,14 @@ sg_status relayout(sg_server *s)
     if ((e = cudaStreamSynchronize(s->stream)) != cudaSuccess)
         return sfail(s, SG_ECUDA, std::string("relayout sync: ") + cudaGetErrorString(e));
     free_state(s);
+    s->state_mem = mem;
     s->X = nb[0]; s->Y = nb[1]; s->P = nb[2]; s->A = nb[3];
     s->xs_of = s->X;
-    for (void *&p : s->xs)
-        if (total > 0 && (e = cudaMalloc(&p, 2 * (size_t)total * sg::row_value_bytes(s->prec))) != cudaSuccess)
-            return sfail(s, SG_ENOMEM, std::string("server state cudaMalloc: ") + cudaGetErrorString(e));
+    for (int q = 0; q < 2; q++) s->xs[q] = mem + at + 4 * vec + q * copy;
+    s->d_state = reinterpret_cast<sg::ChebState *>(mem + at_state);
+    s->d_prefix = reinterpret_cast<long long *>(mem + at_prefix);
     s->total = total;
     s->nslots = (int)state.size();
-    const size_t na = std::max<size_t>(1, state.size());
-    if ((e = cudaMalloc(&s->d_state, sizeof(sg::ChebState) * na)) != cudaSuccess ||
-        (e = cudaMalloc(&s->d_prefix, sizeof(long long) * (na + 1))) != cudaSuccess)
-        return sfail(s, SG_ENOMEM, std::string("server tables cudaMalloc: ") + cudaGetErrorString(e));
-    if ((e = cudaMemcpy(s->d_prefix, prefix.data(), sizeof(long long) * prefix.size(), cudaMemcpyHostToDevice)) !=
-            cudaSuccess ||
-        (!state.empty() && (e = cudaMemcpy(s->d_state, state.data(), sizeof(sg::ChebState) * state.size(),
-                                           cudaMemcpyHostToDevice)) != cudaSuccess))
-        return sfail(s, SG_ECUDA, std::string("server tables upload: ") + cudaGetErrorString(e));
     if (!ctxs.empty()) {
         sg_status st = sg_batch_create(ctxs.data(), (int)ctxs.size(), &s->batch);
         if (st != SG_OK) return sfail(s, st, "sg_batch_create over the active requests failed");

@@ -147,16 +147,29 @@ std::string build_tables(const Problem &p, int smem_budget, int rb, HostTables *
     }
     T.lvl.assign((size_t)D * (L + 1), LevelInfo{});
     T.tabd.clear();
+    std::vector<std::vector<double>> rule_x(kMaxLevelSize + 1), rule_w(kMaxLevelSize + 1);  // by number of nodes
     for (int i = 0; i < D; i++) {
         const double q0 = p.basis[i].q0, s = p.basis[i].scale;
+        // an earlier mode with the same basis, grid and kinetic prefactor has the same tables
+        int same = 0;
+        while (same < i && !(p.basis[same].q0 == q0 && p.basis[same].scale == s && p.omega[same] == p.omega[i] &&
+                             p.basis[same].nb_A == p.basis[i].nb_A && p.basis[same].nb_B == p.basis[i].nb_B &&
+                             p.grids[same].nq_A == p.grids[i].nq_A && p.grids[same].nq_B == p.grids[i].nq_B))
+            same++;
         for (int l = 0; l <= L; l++) {
             LevelInfo &li = T.lvl[(size_t)i * (L + 1) + l];
+            if (same < i) {
+                li = T.lvl[(size_t)same * (L + 1) + l];
+                continue;
+            }
             li.nb = nsz(p.basis[i].nb_A, p.basis[i].nb_B, l);
             li.nq = nsz(p.grids[i].nq_A, p.grids[i].nq_B, l);
             const int nb = li.nb, nq = li.nq;
-            std::vector<double> xg, wf;
-            std::string e = gauss_hermite(nq, &xg, &wf);
-            if (!e.empty()) return e;
+            if (rule_x[nq].empty()) {
+                const std::string e = gauss_hermite(nq, &rule_x[nq], &rule_w[nq]);
+                if (!e.empty()) return e;
+            }
+            const std::vector<double> &xg = rule_x[nq], &wf = rule_w[nq];
             std::vector<double> h(nb + 2), B(nq * nb), BW(nb * nq), D2(nq * nb), Q(nq), W(nq);
             for (int u = 0; u < nq; u++) {
                 hermite_fns(nb + 2, xg[u], h.data());
@@ -194,13 +207,16 @@ std::string build_tables(const Problem &p, int smem_budget, int rb, HostTables *
             }
             // single-mode potential factors in the basis: M_p = B^T W diag(Q^p) B
             li.offM = (int)T.tabd.size();
-            for (int pw = 1; pw <= std::max(T.pmax, 1); pw++)
+            for (int pw = 1; pw <= std::max(T.pmax, 1); pw++) {
+                std::vector<double> Qp(nq);
+                for (int u = 0; u < nq; u++) Qp[u] = std::pow(Q[u], pw);
                 for (int k = 0; k < nb; k++)
                     for (int kp = 0; kp < nb; kp++) {
                         double acc = 0.0;
-                        for (int u = 0; u < nq; u++) acc += BW[k * nq + u] * std::pow(Q[u], pw) * B[u * nb + kp];
+                        for (int u = 0; u < nq; u++) acc += BW[k * nq + u] * Qp[u] * B[u * nb + kp];
                         T.tabd.push_back(acc);
                     }
+            }
         }
     }
     // Harmonic split.  For a mode centred at q0 = 0 with scale s, the basis

@@ -147,7 +147,10 @@ __global__ void __launch_bounds__(256) k_combine_base(const double *__restrict__
 
 // Cholesky G = R^T R (b x b, row-major, b <= kMaxChol) to Ri = R^{-1}; columns
 // after the first dependent one are zero, *rank the leading independent ones.
+// A column is dependent when what the earlier ones leave of its squared norm is
+// rounding: below 1e-13 of it (a Gram matrix resolves no more), or 1e-24.
 constexpr int kMaxChol = 16;
+constexpr double kDependent = 1e-13;
 __global__ void __launch_bounds__(32) k_chol_inverse(const double *__restrict__ G, int b, double *__restrict__ Ri, int *rank)
 {
     __shared__ double R[kMaxChol][kMaxChol + 1], I[kMaxChol][kMaxChol + 1];
@@ -162,7 +165,7 @@ __global__ void __launch_bounds__(32) k_chol_inverse(const double *__restrict__ 
             for (int k = 0; k < j; k++) v = fma(-R[k][j], R[k][i], v);
         }
         const double d = __shfl_sync(0xffffffffu, v, j);
-        if (!(d > 1e-24 * fmax(1.0, fabs(G[j * b + j])))) { rk = j; break; }
+        if (!(d > fmax(1e-24, kDependent * G[j * b + j]))) { rk = j; break; }
         const double s = sqrt(d);
         if (i == j) R[j][j] = s;
         else if (i > j && i < b) R[j][i] = v / s;
@@ -210,15 +213,17 @@ __global__ void k_sum_rows(const double *__restrict__ partial, int nchunk, int r
     out[j] = v;
 }
 
-// Directions: T_q = R_q / (d - theta_q) (guarded), or T_q = R_q without d
+// Directions: T_q = R_p / (d - theta_q) (guarded), or T_q = R_p without d; sel[2q] = p, sel[2q + 1] = theta_q
 __global__ void __launch_bounds__(256) k_direction(const double *__restrict__ R, const double *__restrict__ d,
-                                                   const double *__restrict__ theta, int64_t n, double *__restrict__ T)
+                                                   const double *__restrict__ sel, int64_t n, double *__restrict__ T)
 {
     const int q = blockIdx.y;
+    const double *r = R + (size_t)sel[2 * q] * n;
+    const double theta = sel[2 * q + 1];
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        double v = R[(size_t)q * n + e];
+        double v = r[e];
         if (d) {
-            const double den = d[e] - theta[q];
+            const double den = d[e] - theta;
             v /= (fabs(den) < 1e-3 ? (den < 0 ? -1e-3 : 1e-3) : den);
         }
         T[(size_t)q * n + e] = v;
@@ -263,7 +268,7 @@ __global__ void k_axpby(int64_t len, double a, const double *__restrict__ x, dou
 
 // ---------------------------------------------------------------- device helpers
 // C (ka x kb, row-major, device) = A^T B for column vectors A (ka x n), B (kb x n), kb <= kMaxCols.
-// partial: gram_partial_doubles(ka) doubles of device scratch.  Deterministic.
+// partial: gram_partial_doubles(n, ka) doubles of device scratch.  Deterministic.
 cudaError_t dev_gram(const double *A, int ka, const double *B, int kb, int64_t n, double *C_dev,
                      double *partial, cudaStream_t s)
 {
@@ -278,7 +283,7 @@ cudaError_t dev_gram(const double *A, int ka, const double *B, int kb, int64_t n
     return cudaGetLastError();
 }
 
-size_t gram_partial_doubles(int ka) { return (size_t)kGramChunks * ka * kMaxCols; }
+size_t gram_partial_doubles(int64_t n, int ka) { return n <= kSmallN ? (size_t)8 * ka : (size_t)kGramChunks * ka * kMaxCols; }
 
 // out (r x n) = base (r x n, or nullptr: zero; may be out) + alpha * V (k x n)^T-combination with S (k x r, device)
 cudaError_t dev_combine(const double *V, int k, const double *S_dev, int r, double alpha, const double *base,
@@ -311,11 +316,11 @@ cudaError_t dev_residual(const double *X, const double *theta, double *HX, int r
     return cudaGetLastError();
 }
 
-cudaError_t dev_direction(const double *R, const double *d, const double *theta, int rows, int64_t n, double *T,
+cudaError_t dev_direction(const double *R, const double *d, const double *sel, int rows, int64_t n, double *T,
                           cudaStream_t s)
 {
     const unsigned bx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(608, (n + 255) / 256));
-    k_direction<<<dim3(bx, rows), 256, 0, s>>>(R, d, theta, n, T);
+    k_direction<<<dim3(bx, rows), 256, 0, s>>>(R, d, sel, n, T);
     return cudaGetLastError();
 }
 
@@ -346,56 +351,99 @@ cudaError_t dev_axpby(int64_t len, double a, const double *x, double b, double *
 }
 
 // ---------------------------------------------------------------- host dense algebra
-// Symmetric eigenproblem (cyclic Jacobi): A (n x n, row-major) destroyed;
-// eigenvalues ascending in w, eigenvectors as columns of Z (row-major n x n).
+// Symmetric eigenproblem: Householder reduction to tridiagonal form, then
+// implicit QR steps with the Wilkinson shift (Golub & Van Loan, Matrix
+// Computations, 8.3).  A: n x n, row-major; eigenvalues ascending in w,
+// eigenvectors as columns of Z (row-major n x n).
 void sym_eig(int n, std::vector<double> A, std::vector<double> &w, std::vector<double> &Z)
 {
-    Z.assign((size_t)n * n, 0.0);
-    for (int i = 0; i < n; i++) Z[(size_t)i * n + i] = 1.0;
-    for (int sweep = 0; sweep < 60; sweep++) {
-        double off = 0.0, tot = 0.0;
-        for (int i = 0; i < n; i++)
-            for (int j = 0; j < n; j++) {
-                const double v = A[(size_t)i * n + j] * A[(size_t)i * n + j];
-                tot += v;
-                if (i != j) off += v;
+    std::vector<double> d(n), e(n, 0.0), p(n);
+    std::vector<double> Q((size_t)n * n, 0.0);  // row i: the i-th column of the orthogonal factor
+    auto a = [&](int i, int j) -> double & { return A[(size_t)i * n + j]; };
+    std::vector<std::vector<double>> refl(n > 2 ? n - 2 : 0);
+    for (int k = 0; k + 2 < n; k++) {
+        // reflector v (unit) that takes column k below the diagonal to alpha e_1
+        std::vector<double> &v = refl[k];
+        v.assign(n - k - 1, 0.0);
+        double nrm = 0.0;
+        for (int i = k + 1; i < n; i++) { v[i - k - 1] = a(i, k); nrm = std::hypot(nrm, a(i, k)); }
+        const double alpha = v[0] > 0.0 ? -nrm : nrm;
+        e[k] = alpha;
+        v[0] -= alpha;
+        double vn = 0.0;
+        for (double t : v) vn = std::hypot(vn, t);
+        if (vn == 0.0) { v.clear(); continue; }
+        for (double &t : v) t /= vn;
+        // trailing block B <- B - 2 v q^T - 2 q v^T, q = B v - (v^T B v) v
+        const int m = n - k - 1, o = k + 1;
+        double vbv = 0.0;
+        for (int i = 0; i < m; i++) {
+            double t = 0.0;
+            for (int j = 0; j < m; j++) t += a(o + i, o + j) * v[j];
+            p[i] = t;
+            vbv += v[i] * t;
+        }
+        for (int i = 0; i < m; i++) p[i] -= vbv * v[i];
+        for (int i = 0; i < m; i++)
+            for (int j = 0; j < m; j++) a(o + i, o + j) -= 2.0 * (v[i] * p[j] + p[i] * v[j]);
+    }
+    for (int i = 0; i < n; i++) { d[i] = a(i, i); Q[(size_t)i * n + i] = 1.0; }
+    if (n > 1) e[n - 2] = a(n - 1, n - 2);
+    // Q = H_0 H_1 ... : applied to the columns (rows of the array) from the last reflector on
+    for (int k = n - 3; k >= 0; k--) {
+        const std::vector<double> &v = refl[k];
+        if (v.empty()) continue;
+        const int o = k + 1, m = n - o;
+        for (int c = 0; c < n; c++) {
+            double *q = &Q[(size_t)c * n + o], t = 0.0;
+            for (int i = 0; i < m; i++) t += v[i] * q[i];
+            for (int i = 0; i < m; i++) q[i] -= 2.0 * t * v[i];
+        }
+    }
+    // implicit QR on the unreduced block that ends at hi
+    const double eps = 2.220446049250313e-16;
+    int hi = n - 1, steps = 0;
+    while (hi > 0 && steps < 60 * n) {
+        for (int i = 0; i < hi; i++)
+            if (std::fabs(e[i]) <= eps * (std::fabs(d[i]) + std::fabs(d[i + 1]))) e[i] = 0.0;
+        if (e[hi - 1] == 0.0) { hi--; continue; }
+        int lo = hi - 1;
+        while (lo > 0 && e[lo - 1] != 0.0) lo--;
+        steps++;
+        const double half = 0.5 * (d[hi - 1] - d[hi]), b = e[hi - 1];
+        const double shift = d[hi] - b * b / (half + std::copysign(std::hypot(half, b), half));
+        double x = d[lo] - shift, z = e[lo];
+        for (int k = lo; k < hi; k++) {
+            // rotation of rows and columns k, k+1 that clears z against x
+            const double r = std::hypot(x, z);
+            const double c = r == 0.0 ? 1.0 : x / r, s = r == 0.0 ? 0.0 : z / r;
+            if (k > lo) e[k - 1] = r;
+            const double dk = d[k], dn = d[k + 1], ek = e[k];
+            d[k] = c * c * dk + 2.0 * c * s * ek + s * s * dn;
+            d[k + 1] = s * s * dk - 2.0 * c * s * ek + c * c * dn;
+            e[k] = c * s * (dn - dk) + (c * c - s * s) * ek;
+            if (k + 1 < hi) {
+                x = e[k];
+                z = s * e[k + 1];
+                e[k + 1] *= c;
             }
-        if (off <= 1e-30 * tot || off == 0.0) break;
-        for (int p = 0; p < n - 1; p++)
-            for (int q = p + 1; q < n; q++) {
-                const double apq = A[(size_t)p * n + q];
-                if (std::fabs(apq) < 1e-300) continue;
-                const double app = A[(size_t)p * n + p], aqq = A[(size_t)q * n + q];
-                const double tau = (aqq - app) / (2.0 * apq);
-                const double t = (tau >= 0 ? 1.0 : -1.0) / (std::fabs(tau) + std::sqrt(1.0 + tau * tau));
-                const double c = 1.0 / std::sqrt(1.0 + t * t), s = t * c;
-                for (int k = 0; k < n; k++) {  // A <- A G (columns p, q)
-                    const double akp = A[(size_t)k * n + p], akq = A[(size_t)k * n + q];
-                    A[(size_t)k * n + p] = c * akp - s * akq;
-                    A[(size_t)k * n + q] = s * akp + c * akq;
-                }
-                for (int k = 0; k < n; k++) {  // A <- G^T A (rows p, q)
-                    const double apk = A[(size_t)p * n + k], aqk = A[(size_t)q * n + k];
-                    A[(size_t)p * n + k] = c * apk - s * aqk;
-                    A[(size_t)q * n + k] = s * apk + c * aqk;
-                }
-                for (int k = 0; k < n; k++) {
-                    const double zkp = Z[(size_t)k * n + p], zkq = Z[(size_t)k * n + q];
-                    Z[(size_t)k * n + p] = c * zkp - s * zkq;
-                    Z[(size_t)k * n + q] = s * zkp + c * zkq;
-                }
+            double *q0 = &Q[(size_t)k * n], *q1 = q0 + n;
+            for (int i = 0; i < n; i++) {
+                const double t0 = q0[i], t1 = q1[i];
+                q0[i] = c * t0 + s * t1;
+                q1[i] = c * t1 - s * t0;
             }
+        }
     }
     std::vector<int> idx(n);
     for (int i = 0; i < n; i++) idx[i] = i;
-    std::sort(idx.begin(), idx.end(), [&](int a, int b) { return A[(size_t)a * n + a] < A[(size_t)b * n + b]; });
-    std::vector<double> Zs((size_t)n * n);
+    std::sort(idx.begin(), idx.end(), [&](int i, int j) { return d[i] < d[j]; });
     w.assign(n, 0.0);
-    for (int c2 = 0; c2 < n; c2++) {
-        w[c2] = A[(size_t)idx[c2] * n + idx[c2]];
-        for (int k = 0; k < n; k++) Zs[(size_t)k * n + c2] = Z[(size_t)k * n + idx[c2]];
+    Z.assign((size_t)n * n, 0.0);
+    for (int c = 0; c < n; c++) {
+        w[c] = d[idx[c]];
+        for (int i = 0; i < n; i++) Z[(size_t)i * n + c] = Q[(size_t)idx[c] * n + i];
     }
-    Z.swap(Zs);
 }
 
 // Cholesky G = R^T R (G: b x b row-major, overwritten by R^{-1}, upper triangular).
@@ -407,7 +455,7 @@ int chol_inverse(int b, std::vector<double> &G)
     for (int j = 0; j < b; j++) {
         double d = G[(size_t)j * b + j];
         for (int k = 0; k < j; k++) d -= R[(size_t)k * b + j] * R[(size_t)k * b + j];
-        if (!(d > 1e-24 * std::max(1.0, std::fabs(G[(size_t)j * b + j])))) { rank = j; break; }
+        if (!(d > std::max(1e-24, kDependent * G[(size_t)j * b + j]))) { rank = j; break; }
         R[(size_t)j * b + j] = std::sqrt(d);
         for (int i = j + 1; i < b; i++) {
             double v = G[(size_t)j * b + i];

@@ -11,13 +11,13 @@
 namespace sg {
 cudaError_t dev_gram(const double *A, int ka, const double *B, int kb, int64_t n, double *C_dev, double *partial,
                      cudaStream_t s);
-size_t gram_partial_doubles(int ka);
+size_t gram_partial_doubles(int64_t n, int ka);
 cudaError_t dev_combine(const double *V, int k, const double *S_dev, int r, double alpha, const double *base,
                         double *out, int64_t n, cudaStream_t s);
 cudaError_t dev_chol_inverse(const double *G, int b, double *Ri, int *rank, cudaStream_t s);
 cudaError_t dev_residual(const double *X, const double *theta, double *HX, int rows, int64_t n, double *norms2,
                          double *partial, cudaStream_t s);
-cudaError_t dev_direction(const double *R, const double *d, const double *theta, int rows, int64_t n, double *T,
+cudaError_t dev_direction(const double *R, const double *d, const double *sel, int rows, int64_t n, double *T,
                           cudaStream_t s);
 cudaError_t dev_unit_vectors(double *X, int64_t n, const double *at, int r, cudaStream_t s);
 cudaError_t dev_normalise(double *x, int64_t n, double *nn, double *partial, cudaStream_t s);
@@ -73,15 +73,26 @@ struct Solver {
     sg_ctx *ctx;
     cudaStream_t s;
     int64_t n;
-    DBuf partial, small;  // Gram scratch; small device matrices
+    DBuf mem;  // Gram scratch, then the small device matrices
+    struct { double *p; } partial, small;
     double *pin = nullptr;
     size_t cap, used = 0;  // doubles of pin and small; handed out since the last synchronisation
+    std::vector<double> pageable;
     const ApplyFn *apply_fn = nullptr;  // when set, applications of H_S go through it
-    // kmax: largest basis; cols: largest number of columns combined at once
-    Solver(sg_ctx *c, cudaStream_t st, int kmax, int cols)
-        : ctx(c), s(st), n(c->host.n_cs), partial(gram_partial_doubles(std::max({kmax, cols, 2 * kBlk}))),
-          small(capacity(kmax, cols)), cap(capacity(kmax, cols))
+    // kmax: largest basis; cols: largest number of columns combined at once.
+    // pinned: results may be written to pin (a solver with many round trips);
+    // without, pin only stages uploads.
+    Solver(sg_ctx *c, cudaStream_t st, int kmax, int cols, bool pinned = true)
+        : ctx(c), s(st), n(c->host.n_cs), mem(scratch(c->host.n_cs, kmax, cols) + capacity(kmax, cols)),
+          cap(capacity(kmax, cols))
     {
+        partial.p = mem.p;
+        small.p = mem.p + scratch(n, kmax, cols);
+        if (!pinned) {
+            pageable.resize(cap);
+            pin = pageable.data();
+            return;
+        }
         if (ctx->pin_doubles < cap) {
             if (ctx->pin) cudaFreeHost(ctx->pin);
             ctx->pin = nullptr;
@@ -90,6 +101,10 @@ struct Solver {
             ctx->pin_doubles = cap;
         }
         pin = ctx->pin;
+    }
+    static size_t scratch(int64_t n, int kmax, int cols)
+    {
+        return gram_partial_doubles(n, std::max({kmax, cols, 2 * kBlk}));
     }
     static size_t capacity(int kmax, int cols) { return (size_t)(kmax + 16) * (2 * cols + 6 * kBlk) + 1024; }
 
@@ -345,14 +360,17 @@ int block_eigs(Solver &S, int nev, int b, bool davidson, double tol, int max_it,
         for (int j = 0; j < std::min(nr, ne); j++) { evals[j] = theta[j]; if (resid) resid[j] = rn[j]; }
         if (k >= n || (nconv >= ne && (checked || nconv >= nr))) break;
         checked = nconv >= ne || !davidson;
-        // new directions: the residuals of the first unconverged Ritz pairs
-        // (of the wanted ones, or of those beyond them when these have converged)
-        int r = std::min(b, (nconv >= ne ? nr : std::min(ne, k)) - nconv);
-        if (r <= 0) r = 1;
+        // new directions: the residuals of the first unconverged Ritz pairs (of
+        // the wanted ones, or of those beyond them when these have converged);
+        // a converged pair among them would only add rounding noise
+        std::vector<double> sel;
+        const int upto = nconv >= ne ? nr : std::min(ne, k);
+        for (int j = nconv; j < upto && (int)sel.size() < 2 * b; j++)
+            if (rn[j] > tol * std::max(1.0, std::fabs(theta[j]))) { sel.push_back(j); sel.push_back(theta[j]); }
+        if (sel.empty()) { sel.push_back(nr - 1); sel.push_back(theta[nr - 1]); }
+        const int r = (int)sel.size() / 2;
         if (!davidson && k + r > kmax) break;
-        const int first = std::min(nconv, nr - r);
-        const double *thf = S.upload(theta.data() + first, r);
-        ck(dev_direction(HX + (size_t)first * n, any ? S.ctx->kp.esplit : nullptr, thf, r, n, T, S.s), "directions");
+        ck(dev_direction(HX, any ? S.ctx->kp.esplit : nullptr, S.upload(sel.data(), 2 * r), r, n, T, S.s), "directions");
         if (davidson && k + r > kmax) {  // restart with the current Ritz vectors
             const int keep = std::min(nr, kmax - r);
             ck(cudaMemcpyAsync(V, X, sizeof(double) * n * keep, cudaMemcpyDeviceToDevice, S.s), "restart V");
@@ -417,9 +435,9 @@ void spectral_bounds(Solver &S, double &emin, double &emax)
         ck(dev_normalise(next, n, nn + k + 1, S.partial.p, S.s), "krylov norm");
     }
     S.sync("krylov sync");
-    std::vector<double> hc((size_t)ks * ks), hn(ks);
+    std::vector<double> hc((size_t)ks * (ks + 2));
     ck(cudaMemcpy(hc.data(), cols, sizeof(double) * hc.size(), cudaMemcpyDeviceToHost), "krylov copy");
-    ck(cudaMemcpy(hn.data(), nn, sizeof(double) * ks, cudaMemcpyDeviceToHost), "krylov copy");
+    const double *hn = &hc[(size_t)ks * (ks + 1)];
     int k = 1;
     while (k < ks && hn[k] > 1e-24) k++;
     std::vector<double> Tm((size_t)k * k), th, Z;
@@ -433,9 +451,10 @@ void spectral_bounds(Solver &S, double &emin, double &emax)
     const double *te = S.upload(ends, 2);
     S.combine(V, zd, 1.0, nullptr, X);
     S.combine(W, zd, 1.0, nullptr, HX);
-    double *rn2 = S.pin + S.take(2);
-    ck(dev_residual(X, te, HX, 2, n, rn2, S.partial.p, S.s), "bound resid");
+    double *rn2d = S.small.p + S.take(2), rn2[2];
+    ck(dev_residual(X, te, HX, 2, n, rn2d, S.partial.p, S.s), "bound resid");
     S.sync("bounds sync");
+    ck(cudaMemcpy(rn2, rn2d, sizeof rn2, cudaMemcpyDeviceToHost), "bound copy");
     const double range = th[k - 1] - th[0];
     emin = th[0] - std::sqrt(rn2[0]) - 0.05 * range;
     emax = th[k - 1] + std::sqrt(rn2[1]) + 0.05 * range;
@@ -583,7 +602,7 @@ sg_status sg_propagate(sg_ctx *ctx, double *psi, double dt, int nsteps, int orde
     }
     if (!sg_on_ctx_device(ctx)) { ctx->last_error = "the current CUDA device is not the one the context was made on"; return SG_EINVAL; }
     try {
-        Solver S(ctx, (cudaStream_t)stream, kBoundVectors, 2);
+        Solver S(ctx, (cudaStream_t)stream, kBoundVectors, 2, !ctx->host.rows);
         const int64_t n = S.n;
         double emin, emax;
         spectral_bounds(S, emin, emax);
@@ -671,7 +690,7 @@ sg_status davidson_routed(sg_ctx *ctx, cudaStream_t stream, const ApplyFn &apply
 sg_status chebyshev_bounds(sg_ctx *ctx, cudaStream_t stream, double *emin, double *emax)
 {
     try {
-        Solver S(ctx, stream, kBoundVectors, 2);
+        Solver S(ctx, stream, kBoundVectors, 2, false);
         spectral_bounds(S, *emin, *emax);
         ck(cudaStreamSynchronize(S.s), "bounds sync");
     } catch (const SolverError &e) {
