@@ -80,10 +80,10 @@ sg_status ensure_workspace(sg_ctx *ctx, int nvec, cudaStream_t s)
     if (ctx->host.rows) {
         const size_t xs_bytes =
             (((size_t)ctx->host.n_cs * sg::xs_stride(nvec) * sg::row_value_bytes(ctx->prob.prec)) + 15) & ~(size_t)15;
-        if ((e = cudaMalloc(&ctx->xs, xs_bytes + sizeof(unsigned) * nvec)) != cudaSuccess)
+        if ((e = cudaMalloc(&ctx->xs, xs_bytes + sizeof(unsigned) * (nvec + 1))) != cudaSuccess)
             return fail(ctx, SG_ENOMEM, std::string("workspace cudaMalloc: ") + cudaGetErrorString(e));
         ctx->flags = reinterpret_cast<unsigned *>(static_cast<unsigned char *>(ctx->xs) + xs_bytes);
-        if ((e = cudaMemsetAsync(ctx->flags, 0, sizeof(unsigned) * nvec, s)) != cudaSuccess)
+        if ((e = cudaMemsetAsync(ctx->flags, 0, sizeof(unsigned) * (nvec + 1), s)) != cudaSuccess)
             return cuda_fail(ctx, e, "workspace memset");
     } else {
         const size_t words = (size_t)ctx->host.n_cs * nvec * sg::acc_words(ctx->fp32);
@@ -105,6 +105,7 @@ sg::RowIO row_io(const sg_ctx *ctx, const double *x, double *y, int nvec)
     io.xs = ctx->xs;
     io.y = y;
     io.flags = ctx->flags;
+    io.ticket = ctx->flags + ctx->acc_nvec;
     io.nvec = nvec;
     io.stride = sg::xs_stride(nvec);
     io.words = sg::acc_words(ctx->fp32);
@@ -198,6 +199,7 @@ namespace sg {
 // Input copies small enough to stay in the caches are not made: the row
 // kernel then gathers from x itself.
 constexpr int64_t kDirectElems = 65536;
+constexpr int kTicketBlocks = 1024;
 
 cudaError_t apply_rows(sg_ctx *ctx, RowIO io, cudaStream_t s)
 {
@@ -206,8 +208,11 @@ cudaError_t apply_rows(sg_ctx *ctx, RowIO io, cudaStream_t s)
     if (prec == SG_FP64 && io.nvec == 1) io.xs = io.x;  // x is its own entry-major copy
     else if (!io.xs || ctx->host.n_cs * (int64_t)io.nvec <= kDirectElems) io.xs = nullptr;
     else e = launch_row_stage(ctx->rop, io, prec, s);
+    // few blocks: the last one settles the vectors; many: the counter would be
+    // a point of contention, and a launch is short beside them
+    if (!io.y || ctx->rop.nwin > kTicketBlocks) io.ticket = nullptr;
     if (e == cudaSuccess) e = launch_rows(ctx->rop, io, prec, row_vt(ctx->host, prec), s);
-    if (e == cudaSuccess && io.y) e = launch_row_settle(io, ctx->rop.n, s);
+    if (e == cudaSuccess && io.y && !io.ticket) e = launch_row_settle(io, ctx->rop.n, s);
     return e;
 }
 

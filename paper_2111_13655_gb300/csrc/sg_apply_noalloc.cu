@@ -110,6 +110,7 @@ extern "C" sg_status sg_apply_H_noalloc(sg_ctx *ctx, const double *x, double *y,
         io.y = y;
         io.xs = scratch + kNoAllocMaxVec;
         io.flags = reinterpret_cast<unsigned *>(scratch);
+        io.ticket = io.flags + kNoAllocMaxVec;
         io.nvec = nvec;
         io.stride = sg::xs_stride(nvec);
         io.nparts = 1;

@@ -94,6 +94,7 @@ struct RowIO {
     double *y;              // result, or nullptr: the sums go to acc
     unsigned long long *acc;
     unsigned *flags;        // per vector: set when x holds a non-finite value
+    unsigned *ticket;       // zero between launches; nullptr: launch_row_settle follows
     int nvec, stride, words;
     int part, nparts;       // windows w with w % nparts == part
 };
@@ -276,7 +277,7 @@ cudaError_t launch_rows(const RowOp &R, const RowIO &io, sg_precision prec, int 
 cudaError_t launch_row_stage(const RowOp &R, const RowIO &io, sg_precision prec, cudaStream_t stream);
 cudaError_t launch_row_stage_batch(const RowIO &io, sg_precision prec, const long long *cs_prefix, const int2 *items,
                                    int nitems, cudaStream_t stream);
-// Vectors with a non-finite input become NaN; clears the flags.
+// Vectors with a non-finite input become NaN; clears the flags (after launch_rows without a ticket).
 cudaError_t launch_row_settle(const RowIO &io, int n, cudaStream_t stream);
 cudaError_t launch_row_settle_batch(const RowIO &io, const long long *cs_prefix, int nprob, cudaStream_t stream);
 // y from the summed accumulators of all parts; clears them.
@@ -361,7 +362,7 @@ struct sg_ctx {
     // apply workspace.  Row form: per-vector flags and the entry-major input
     // copy; term-by-term kernel: fixed-point accumulators and scale exponents
     void *xs = nullptr;
-    unsigned *flags = nullptr;  // behind xs, in its allocation
+    unsigned *flags = nullptr;  // behind xs, in its allocation; after acc_nvec flags, the ticket
     unsigned long long *acc = nullptr;
     long long *maxbits = nullptr;
     int acc_nvec = 0;

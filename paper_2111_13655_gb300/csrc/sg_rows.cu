@@ -523,12 +523,36 @@ __device__ __forceinline__ void rows_window(const RowOp &R, const RowIO &io, con
     }
 }
 
+// A vector of n entries that holds a non-finite value gives NaN everywhere;
+// clears its flag.  By a whole block.
+__device__ __forceinline__ void settle_vectors(unsigned *flags, int nvec, double *y, size_t n)
+{
+    for (int v = 0; v < nvec; v++) {
+        if (__ldcg(flags + v) == 0u) continue;
+        for (size_t i = threadIdx.x; i < n; i += blockDim.x) y[(size_t)v * n + i] = __longlong_as_double(0x7FF8000000000000ll);
+    }
+    __syncthreads();
+    for (int v = threadIdx.x; v < nvec; v += blockDim.x)
+        if (__ldcg(flags + v)) flags[v] = 0u;
+}
+
 template <typename T, int VT, bool ST>
 __global__ void __launch_bounds__(kRT, row_blocks<T>()) k_rows(const RowOp R, const RowIO io, int lgl)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint64_t bar;
     rows_window<T, VT, ST>(R, io, R.wins[blockIdx.x * io.nparts + io.part], lgl, R.cap, smem, &bar);
+    if (!io.ticket) return;
+    // the block that ends last settles the vectors (instead of a launch of its own)
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(io.ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    settle_vectors(io.flags, io.nvec, io.y, (size_t)R.n);
+    if (threadIdx.x == 0) *io.ticket = 0u;
 }
 
 // Many problems: item = (problem, window); vectors of problem j from
@@ -721,23 +745,13 @@ __global__ void __launch_bounds__(256) k_row_stage_batch(const int2 *__restrict_
                      const_cast<T *>(static_cast<const T *>(io.xs)) + c0 * io.stride, r);
 }
 
-// A vector that holds a non-finite value gives NaN everywhere; clears the
-// flags.  Block j: problem j (its vectors from nvec * cs_prefix[j]).
+// Block j: problem j (its vectors from nvec * cs_prefix[j]).
 __global__ void __launch_bounds__(1024) k_row_settle(const RowIO io, int n_one, const long long *__restrict__ cs_prefix)
 {
     const int j = blockIdx.x;
     const size_t c0 = cs_prefix ? (size_t)cs_prefix[j] : 0;
     const size_t n = cs_prefix ? (size_t)cs_prefix[j + 1] - c0 : (size_t)n_one;
-    unsigned *flags = io.flags + (size_t)j * io.nvec;
-    for (int v = 0; v < io.nvec; v++) {
-        const bool bad = flags[v] != 0u;  // the same for the whole block: written by earlier launches only
-        if (!bad) continue;
-        double *y = io.y + (c0 * io.nvec + (size_t)v * n);
-        for (size_t i = threadIdx.x; i < n; i += blockDim.x) y[i] = __longlong_as_double(0x7FF8000000000000ll);
-    }
-    __syncthreads();
-    for (int v = threadIdx.x; v < io.nvec; v += blockDim.x)
-        if (flags[v]) flags[v] = 0u;
+    settle_vectors(io.flags + (size_t)j * io.nvec, io.nvec, io.y + c0 * io.nvec, n);
 }
 
 // y = the double whose bits the parts summed to, plus the harmonic diagonal; clears the accumulators.

@@ -79,21 +79,26 @@ __global__ void k_gram_final(const double *__restrict__ partial, int nchunk, int
 // time (n = 1,001, 34 x 8: 20 us).  One block per inner product, and one column
 // per block of 64 entries, spread it over all SMs.
 constexpr int64_t kSmallN = 8192;
-constexpr int kDotThreads = 128;
+constexpr int kDotThreads = 256;
 
-// Sum over the block, in a fixed order; the result in every thread.
+// Sum over the block, in a fixed order, to every thread.  The last step is made
+// by one warp: the FP64 pipe serves one warp instruction in about 19 cycles, and
+// letting every thread add the warps' sums took 10 us of a 1,024-thread block.
 template <int THREADS>
 __device__ __forceinline__ double block_sum(double v)
 {
-    __shared__ double red[THREADS / 32];
+    constexpr int NW = THREADS / 32;
+    __shared__ double red[NW];
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
-    double t = red[0];
-#pragma unroll
-    for (int w = 1; w < THREADS / 32; w++) t += red[w];
-    return t;
+    if (threadIdx.x < 32) {
+        double t = threadIdx.x < NW ? red[threadIdx.x] : 0.0;
+        for (int o = NW / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (threadIdx.x == 0) red[0] = t;
+    }
+    __syncthreads();
+    return red[0];
 }
 
 // C[i][j] = sum_e A_i[e] B_j[e], block (i, j)
@@ -102,8 +107,8 @@ __global__ void __launch_bounds__(kDotThreads) k_gram_small(const double *__rest
 {
     const double *a = A + (size_t)blockIdx.x * n, *b = B + (size_t)blockIdx.y * n;
     double v = 0.0;
-#pragma unroll 4
-    for (int e = threadIdx.x; e < n; e += kDotThreads) v = fma(a[e], b[e], v);
+#pragma unroll 8
+    for (int e = threadIdx.x; e < n; e += kDotThreads) v = fma(__ldg(a + e), __ldg(b + e), v);
     v = block_sum<kDotThreads>(v);
     if (threadIdx.x == 0) C[blockIdx.x * gridDim.y + blockIdx.y] = v;
 }
@@ -115,10 +120,37 @@ __global__ void __launch_bounds__(64) k_combine_small(const double *__restrict__
     const int e = blockIdx.x * 64 + threadIdx.x, j = blockIdx.y;
     if (e >= n) return;
     double acc = 0.0;
-#pragma unroll 4
-    for (int i = 0; i < k; i++) acc = fma(V[(size_t)i * n + e], __ldg(S + i * r + j), acc);
+#pragma unroll 16
+    for (int i = 0; i < k; i++) acc = fma(__ldg(V + (size_t)i * n + e), __ldg(S + i * r + j), acc);
     const size_t o = (size_t)j * n + e;
     out[o] = (base ? base[o] : 0.0) + alpha * acc;
+}
+
+// x <- (x - sum_i V_i c_i) / norm, norm^2 = c_k - sum_i c_i^2 (V orthonormal, c_i = V_i . x, c_k = x . x); x <- 0 when
+// norm^2 <= 1e-24.  *nn = norm^2.
+__global__ void __launch_bounds__(64) k_project_normalise(const double *__restrict__ V, int k,
+                                                          const double *__restrict__ c, double *x, int n,
+                                                          double *__restrict__ nn)
+{
+    __shared__ double scale;
+    if (threadIdx.x < 32) {
+        double q = 0.0;
+        for (int i = threadIdx.x; i < k; i += 32) q = fma(c[i], c[i], q);
+        for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        if (threadIdx.x == 0) {
+            const double v = c[k] - q;
+            scale = v > 1e-24 ? rsqrt(v) : 0.0;
+            if (blockIdx.x == 0) *nn = v;
+        }
+    }
+    const int e = blockIdx.x * 64 + threadIdx.x;
+    double acc = 0.0;
+    if (e < n) {
+#pragma unroll 16
+        for (int i = 0; i < k; i++) acc = fma(__ldg(V + (size_t)i * n + e), __ldg(c + i), acc);
+    }
+    __syncthreads();
+    if (e < n) x[e] = (x[e] - acc) * scale;
 }
 
 // out = base + alpha * V S for longer vectors (one block column of up to kMaxCols outputs)
@@ -166,18 +198,18 @@ __global__ void __launch_bounds__(32) k_chol_inverse(const double *__restrict__ 
         }
         const double d = __shfl_sync(0xffffffffu, v, j);
         if (!(d > fmax(1e-24, kDependent * G[j * b + j]))) { rk = j; break; }
-        const double s = sqrt(d);
+        const double s = rsqrt(d);  // R[j][j] holds its reciprocal
         if (i == j) R[j][j] = s;
-        else if (i > j && i < b) R[j][i] = v / s;
+        else if (i > j && i < b) R[j][i] = v * s;
         __syncwarp();
     }
     // column i of the inverse of the leading rk x rk block
     if (i < rk) {
-        I[i][i] = 1.0 / R[i][i];
+        I[i][i] = R[i][i];
         for (int r = i - 1; r >= 0; r--) {
             double v = 0.0;
             for (int k = r + 1; k <= i; k++) v = fma(R[r][k], I[k][i], v);
-            I[r][i] = -v / R[r][r];
+            I[r][i] = -v * R[r][r];
         }
     }
     __syncwarp();
@@ -246,14 +278,23 @@ __global__ void __launch_bounds__(1024) k_normalise(double *x, int64_t n, double
     double v = 0.0;
     for (int64_t e = threadIdx.x; e < n; e += 1024) v = fma(x[e], x[e], v);
     v = block_sum<1024>(v);
-    const double f = v > 1e-24 ? 1.0 / sqrt(v) : 0.0;
+    __shared__ double f;
+    if (threadIdx.x == 0) f = v > 1e-24 ? 1.0 / sqrt(v) : 0.0;
+    __syncthreads();
     for (int64_t e = threadIdx.x; e < n; e += 1024) x[e] *= f;
     if (threadIdx.x == 0) *nn = v;
 }
-// the same for longer vectors, from the squared norm
-__global__ void k_scale_norm(double *x, int64_t n, const double *nn)
+// the same for longer vectors, from the squared norm (less the squares of k projections c_i already taken out)
+__global__ void k_scale_norm(double *x, int64_t n, const double *xx, const double *c, int k, double *nn)
 {
-    const double v = *nn, f = v > 1e-24 ? 1.0 / sqrt(v) : 0.0;
+    __shared__ double f;
+    if (threadIdx.x == 0) {
+        double v = *xx;
+        for (int i = 0; i < k; i++) v = fma(-c[i], c[i], v);
+        f = v > 1e-24 ? 1.0 / sqrt(v) : 0.0;
+        if (blockIdx.x == 0) *nn = v;
+    }
+    __syncthreads();
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) x[e] *= f;
 }
 
@@ -338,9 +379,24 @@ cudaError_t dev_normalise(double *x, int64_t n, double *nn, double *partial, cud
         k_normalise<<<1, 1024, 0, s>>>(x, n, nn);
         return cudaGetLastError();
     }
-    cudaError_t e = dev_gram(x, 1, x, 1, n, nn, partial, s);
+    double *xx = partial + gram_partial_doubles(n, 1);
+    cudaError_t e = dev_gram(x, 1, x, 1, n, xx, partial, s);
     if (e != cudaSuccess) return e;
-    k_scale_norm<<<608, 256, 0, s>>>(x, n, nn);
+    k_scale_norm<<<608, 256, 0, s>>>(x, n, xx, nullptr, 0, nn);
+    return cudaGetLastError();
+}
+
+// x <- (x - sum_{i<k} V_i c_i) / its norm, with c_i = V_i . x and c_k = x . x (device); nn: the squared norm
+cudaError_t dev_project_normalise(const double *V, int k, const double *c, double *x, int64_t n, double *nn,
+                                  cudaStream_t s)
+{
+    if (n <= kSmallN) {
+        k_project_normalise<<<(unsigned)((n + 63) / 64), 64, 0, s>>>(V, k, c, x, (int)n, nn);
+        return cudaGetLastError();
+    }
+    cudaError_t e = dev_combine(V, k, c, 1, -1.0, x, x, n, s);
+    if (e != cudaSuccess) return e;
+    k_scale_norm<<<608, 256, 0, s>>>(x, n, c + k, c, k, nn);
     return cudaGetLastError();
 }
 

@@ -21,6 +21,8 @@ cudaError_t dev_direction(const double *R, const double *d, const double *sel, i
                           cudaStream_t s);
 cudaError_t dev_unit_vectors(double *X, int64_t n, const double *at, int r, cudaStream_t s);
 cudaError_t dev_normalise(double *x, int64_t n, double *nn, double *partial, cudaStream_t s);
+cudaError_t dev_project_normalise(const double *V, int k, const double *c, double *x, int64_t n, double *nn,
+                                  cudaStream_t s);
 cudaError_t dev_axpby(int64_t len, double a, const double *x, double b, double *y, cudaStream_t s);
 void sym_eig(int n, std::vector<double> A, std::vector<double> &w, std::vector<double> &Z);
 int chol_inverse(int b, std::vector<double> &G);
@@ -430,9 +432,9 @@ void spectral_bounds(Solver &S, double &emin, double &emax)
         if (k + 1 == ks) break;
         double *next = V + (size_t)(k + 1) * n, *c2 = S.small.p;
         ck(dev_combine(V, k + 1, c, 1, -1.0, W + (size_t)k * n, next, n, S.s), "krylov step");
-        ck(dev_gram(V, k + 1, next, 1, n, c2, S.partial.p, S.s), "krylov gram");
-        ck(dev_combine(V, k + 1, c2, 1, -1.0, next, next, n, S.s), "krylov step");
-        ck(dev_normalise(next, n, nn + k + 1, S.partial.p, S.s), "krylov norm");
+        // the second projection, with next . next as its last product (next follows the basis)
+        ck(dev_gram(V, k + 2, next, 1, n, c2, S.partial.p, S.s), "krylov gram");
+        ck(dev_project_normalise(V, k + 1, c2, next, n, nn + k + 1, S.s), "krylov norm");
     }
     S.sync("krylov sync");
     std::vector<double> hc((size_t)ks * (ks + 2));
