@@ -21,6 +21,7 @@
 
 #include "sg_cheb.cuh"
 #include "sg_df.cuh"
+#include "sg_launch.cuh"
 
 namespace sg {
 
@@ -402,11 +403,6 @@ __device__ __forceinline__ bool bar_wait(uint64_t *bar, unsigned parity)
     return false;
 }
 
-// Programmatic launches: a kernel lets its successor's blocks start, and waits
-// for its predecessor (whose writes it then sees); both are no-ops otherwise.
-__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 __device__ __forceinline__ bool finite(double v)
 {
     return (__double2hiint(v) & 0x7FF00000) != 0x7FF00000;
@@ -597,11 +593,11 @@ __global__ void __launch_bounds__(kRT, row_blocks<T>()) k_rows_batch(const RowOp
 
 // One Chebyshev term of a window: a thread takes a row, both vectors (the real
 // and the imaginary part), and updates the row's entry where its sum ends.
-// The record does not depend on the previous term: with programmatic launches
-// it is fetched while that term still runs.
-template <typename T>
-__device__ __forceinline__ void cheb_window(const RowOp &R, const ChebIO &io, const ChebTerm &term, bool done,
-                                            const RowWin &win, int cap, unsigned char *smem, uint64_t *bar)
+// The record does not depend on the previous term: it is fetched while that
+// term still runs.  term_of(done): the term, asked for after the wait.
+template <typename T, typename F>
+__device__ __forceinline__ void cheb_window(const RowOp &R, const ChebIO &io, const F &term_of, const RowWin &win,
+                                            int cap, unsigned char *smem, uint64_t *bar)
 {
     const int tid = threadIdx.x;
     const size_t n = (size_t)R.n;
@@ -621,6 +617,8 @@ __device__ __forceinline__ void cheb_window(const RowOp &R, const ChebIO &io, co
         return;
     }
     if (tid >= win.nrows) return;
+    bool done = false;
+    const ChebTerm term = term_of(done);
     const unsigned char *rec = staged ? smem : R.blob + win.off;
     const uint2 mt = reinterpret_cast<const uint2 *>(rec)[tid];
     const int *cols = reinterpret_cast<const int *>(rec + row_meta_bytes(win.nrows));
@@ -700,26 +698,32 @@ __global__ void __launch_bounds__(kRT) k_cheb_rows(const RowOp R, const ChebIO i
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint64_t bar;
     grid_trigger();
-    cheb_window<T>(R, io, term, false, R.wins[blockIdx.x], R.cap, smem, &bar);
+    cheb_window<T>(R, io, [&](bool &) { return term; }, R.wins[blockIdx.x], R.cap, smem, &bar);
 }
 
 // Many problems: item = (problem, window); problem j's vectors from 2 * cs_prefix[j], its term from its state.
 template <typename T>
 __global__ void __launch_bounds__(kRT) k_cheb_rows_batch(const RowOp *__restrict__ ops,
                                                          const int2 *__restrict__ items, const ChebIO io,
-                                                         const ChebState *__restrict__ st,
+                                                         const ChebState *st,
                                                          const long long *__restrict__ cs_prefix, int cap)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint64_t bar;
+    grid_trigger();
     const int2 it = items[blockIdx.x];
     const RowOp &R = ops[it.x];
-    const ChebState &s = st[it.x];
     const size_t c0 = 2 * (size_t)cs_prefix[it.x];
     const ChebIO o{io.X + c0, io.Y + c0, io.P + c0, io.A + c0, static_cast<const T *>(io.xs) + c0,
                    static_cast<T *>(io.xs_next) + c0, nullptr};
-    const bool done = s.step >= s.nsteps;
-    cheb_window<T>(R, o, done ? ChebTerm{} : cheb_term(s), done, R.wins[it.y], cap, smem, &bar);
+    const ChebState *s = st + it.x;  // moved on by the launch before
+    cheb_window<T>(
+        R, o,
+        [&](bool &done) {
+            done = s->step >= s->nsteps;
+            return done ? ChebTerm{} : cheb_term(*s);
+        },
+        R.wins[it.y], cap, smem, &bar);
 }
 
 // xs[r * stride + v] = x_v[r] in T (zero beyond nvec), rows r0 .. r0 + nr - 1
@@ -828,25 +832,9 @@ cudaError_t smem_limits()
     return e;
 }
 
-// A launch whose blocks may start before the preceding kernel of the stream has
-// ended: they fetch their records, which nothing writes after set-up, then wait
-// for it.  D=12 L=10, 5 vectors: 99.1 us with plain launches, 93.2 with these.
-template <typename... P, typename... A>
-cudaError_t launch_early(void (*k)(P...), dim3 grid, size_t smem, cudaStream_t s, A... args)
-{
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t c{};
-    c.gridDim = grid;
-    c.blockDim = dim3(kRT);
-    c.dynamicSmemBytes = smem;
-    c.stream = s;
-    c.attrs = &at;
-    c.numAttrs = 1;
-    return cudaLaunchKernelEx(&c, k, args...);
-}
-
+// Launched early: the blocks fetch their records, which nothing writes after
+// set-up, while the preceding kernel runs (D=12 L=10, 5 vectors: 99.1 us with
+// plain launches, 93.2 with these).
 template <typename T>
 cudaError_t rows_t(const RowOp &R, const RowIO &io, int vt, cudaStream_t s)
 {
@@ -859,10 +847,10 @@ cudaError_t rows_t(const RowOp &R, const RowIO &io, int vt, cudaStream_t s)
     // most two blocks per SM and leave SMs idle (D=2, 28 functions, 16 vectors:
     // 10.8 us one after another, 10.0 side by side, the rest is the call)
     const dim3 grid(blocks, blocks <= 304 ? std::min(16, (io.nvec + vpass - 1) / vpass) : 1);
-    if (!io.xs) return launch_early(k_rows<T, 1, false>, grid, smem, s, R, io, l);
-    if (vt == 4) return launch_early(k_rows<T, 4, true>, grid, smem, s, R, io, l);
-    if (vt == 2) return launch_early(k_rows<T, 2, true>, grid, smem, s, R, io, l);
-    return launch_early(k_rows<T, 1, true>, grid, smem, s, R, io, l);
+    if (!io.xs) return launch_early(k_rows<T, 1, false>, grid, kRT, smem, s, R, io, l);
+    if (vt == 4) return launch_early(k_rows<T, 4, true>, grid, kRT, smem, s, R, io, l);
+    if (vt == 2) return launch_early(k_rows<T, 2, true>, grid, kRT, smem, s, R, io, l);
+    return launch_early(k_rows<T, 1, true>, grid, kRT, smem, s, R, io, l);
 }
 
 template <typename T>
@@ -928,7 +916,7 @@ template <typename T>
 cudaError_t cheb_rows_t(const RowOp &R, const ChebIO &io, const ChebTerm &term, cudaStream_t s)
 {
     if (R.nwin <= 0) return cudaSuccess;
-    return launch_early(k_cheb_rows<T>, dim3((unsigned)R.nwin), (size_t)((R.cap + 15) & ~15), s, R, io, term);
+    return launch_early(k_cheb_rows<T>, dim3((unsigned)R.nwin), kRT, (size_t)((R.cap + 15) & ~15), s, R, io, term);
 }
 
 }  // namespace
@@ -948,10 +936,10 @@ cudaError_t launch_cheb_rows_batch(const RowOp *ops, const int2 *items, int nite
     if (nitems <= 0) return cudaSuccess;
     const size_t smem = (size_t)((cap + 15) & ~15);
     if (prec == SG_MIXED)
-        k_cheb_rows_batch<float><<<(unsigned)nitems, kRT, smem, stream>>>(ops, items, io, st, cs_prefix, cap);
-    else
-        k_cheb_rows_batch<double><<<(unsigned)nitems, kRT, smem, stream>>>(ops, items, io, st, cs_prefix, cap);
-    return cudaGetLastError();
+        return launch_early(k_cheb_rows_batch<float>, dim3((unsigned)nitems), kRT, smem, stream, ops, items, io, st,
+                            cs_prefix, cap);
+    return launch_early(k_cheb_rows_batch<double>, dim3((unsigned)nitems), kRT, smem, stream, ops, items, io, st,
+                        cs_prefix, cap);
 }
 
 cudaError_t launch_row_stage(const RowOp &R, const RowIO &io, sg_precision prec, cudaStream_t stream)

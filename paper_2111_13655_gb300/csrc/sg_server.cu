@@ -12,6 +12,7 @@
 #include <algorithm>
 
 #include "sg_cheb.cuh"
+#include "sg_launch.cuh"
 
 namespace sg {
 
@@ -75,9 +76,10 @@ __global__ void k_cheb_update(const ChebState *__restrict__ st, const long long 
 constexpr int kLogThreads = 256;
 __global__ void __launch_bounds__(kLogThreads) k_cheb_log_advance(ChebState *st,
                                                                   const long long *__restrict__ prefix,
-                                                                  const double *__restrict__ X,
-                                                                  const double *__restrict__ Y)
+                                                                  const double *X, const double *Y)
 {
+    grid_trigger();
+    grid_wait();
     ChebState &S = st[blockIdx.x];
     const int k = S.k, step = S.step, K = S.K;
     __syncthreads();  // every thread has read the state that thread 0 moves on
@@ -123,16 +125,14 @@ cudaError_t launch_cheb_iteration(ChebState *st, const long long *prefix, int ni
     if (nitems <= 0 || total <= 0) return cudaSuccess;
     const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 152 * 8));
     k_cheb_update<<<blocks, 256, 0, s>>>(st, prefix, nitems, X, Y, P, A);
-    k_cheb_log_advance<<<(unsigned)nitems, kLogThreads, 0, s>>>(st, prefix, X, Y);
-    return cudaGetLastError();
+    return launch_early(k_cheb_log_advance, dim3((unsigned)nitems), kLogThreads, 0, s, st, prefix, X, Y);
 }
 
 cudaError_t launch_cheb_log_advance(ChebState *st, const long long *prefix, int nitems, const double *X,
                                     const double *Y, cudaStream_t s)
 {
     if (nitems <= 0) return cudaSuccess;
-    k_cheb_log_advance<<<(unsigned)nitems, kLogThreads, 0, s>>>(st, prefix, X, Y);
-    return cudaGetLastError();
+    return launch_early(k_cheb_log_advance, dim3((unsigned)nitems), kLogThreads, 0, s, st, prefix, X, Y);
 }
 
 }  // namespace sg

@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "sg_internal.h"
+#include "sg_launch.cuh"
 
 namespace sg {
 
@@ -102,36 +103,40 @@ __device__ __forceinline__ double block_sum(double v)
 }
 
 // C[i][j] = sum_e A_i[e] B_j[e], block (i, j)
-__global__ void __launch_bounds__(kDotThreads) k_gram_small(const double *__restrict__ A, const double *__restrict__ B,
-                                                            int n, double *__restrict__ C)
+__global__ void __launch_bounds__(kDotThreads) k_gram_small(const double *A, const double *B, int n, double *C)
 {
+    grid_trigger();
+    grid_wait();
     const double *a = A + (size_t)blockIdx.x * n, *b = B + (size_t)blockIdx.y * n;
     double v = 0.0;
 #pragma unroll 8
-    for (int e = threadIdx.x; e < n; e += kDotThreads) v = fma(__ldg(a + e), __ldg(b + e), v);
+    for (int e = threadIdx.x; e < n; e += kDotThreads) v = fma(a[e], b[e], v);
     v = block_sum<kDotThreads>(v);
     if (threadIdx.x == 0) C[blockIdx.x * gridDim.y + blockIdx.y] = v;
 }
 
 // out[j][e] = base[j][e] + alpha * sum_i V[i][e] S[i][j] (base nullptr: 0), column j = blockIdx.y
-__global__ void __launch_bounds__(64) k_combine_small(const double *__restrict__ V, int k, const double *__restrict__ S,
-                                                      int r, double alpha, const double *base, double *out, int n)
+__global__ void __launch_bounds__(64) k_combine_small(const double *V, int k, const double *S, int r, double alpha,
+                                                      const double *base, double *out, int n)
 {
+    grid_trigger();
+    grid_wait();
     const int e = blockIdx.x * 64 + threadIdx.x, j = blockIdx.y;
     if (e >= n) return;
     double acc = 0.0;
 #pragma unroll 16
-    for (int i = 0; i < k; i++) acc = fma(__ldg(V + (size_t)i * n + e), __ldg(S + i * r + j), acc);
+    for (int i = 0; i < k; i++) acc = fma(V[(size_t)i * n + e], S[i * r + j], acc);
     const size_t o = (size_t)j * n + e;
     out[o] = (base ? base[o] : 0.0) + alpha * acc;
 }
 
 // x <- (x - sum_i V_i c_i) / norm, norm^2 = c_k - sum_i c_i^2 (V orthonormal, c_i = V_i . x, c_k = x . x); x <- 0 when
 // norm^2 <= 1e-24.  *nn = norm^2.
-__global__ void __launch_bounds__(64) k_project_normalise(const double *__restrict__ V, int k,
-                                                          const double *__restrict__ c, double *x, int n,
-                                                          double *__restrict__ nn)
+__global__ void __launch_bounds__(64) k_project_normalise(const double *V, int k, const double *c, double *x, int n,
+                                                          double *nn)
 {
+    grid_trigger();
+    grid_wait();
     __shared__ double scale;
     if (threadIdx.x < 32) {
         double q = 0.0;
@@ -147,7 +152,7 @@ __global__ void __launch_bounds__(64) k_project_normalise(const double *__restri
     double acc = 0.0;
     if (e < n) {
 #pragma unroll 16
-        for (int i = 0; i < k; i++) acc = fma(__ldg(V + (size_t)i * n + e), __ldg(c + i), acc);
+        for (int i = 0; i < k; i++) acc = fma(V[(size_t)i * n + e], c[i], acc);
     }
     __syncthreads();
     if (e < n) x[e] = (x[e] - acc) * scale;
@@ -183,8 +188,10 @@ __global__ void __launch_bounds__(256) k_combine_base(const double *__restrict__
 // rounding: below 1e-13 of it (a Gram matrix resolves no more), or 1e-24.
 constexpr int kMaxChol = 16;
 constexpr double kDependent = 1e-13;
-__global__ void __launch_bounds__(32) k_chol_inverse(const double *__restrict__ G, int b, double *__restrict__ Ri, int *rank)
+__global__ void __launch_bounds__(32) k_chol_inverse(const double *G, int b, double *Ri, int *rank)
 {
+    grid_trigger();
+    grid_wait();
     __shared__ double R[kMaxChol][kMaxChol + 1], I[kMaxChol][kMaxChol + 1];
     const int i = threadIdx.x;
     for (int q = i; q < b * b; q += 32) { R[q / b][q % b] = 0.0; I[q / b][q % b] = 0.0; }
@@ -218,10 +225,11 @@ __global__ void __launch_bounds__(32) k_chol_inverse(const double *__restrict__ 
 }
 
 // Residuals: HX_j -= theta_j X_j, and their squared norms (partial[j][chunk], chunk = blockIdx.x)
-__global__ void __launch_bounds__(256) k_residual(const double *__restrict__ X, const double *__restrict__ theta,
-                                                  double *__restrict__ HX, int64_t n, int64_t chunk,
-                                                  double *__restrict__ partial)
+__global__ void __launch_bounds__(256) k_residual(const double *X, const double *theta, double *HX, int64_t n,
+                                                  int64_t chunk, double *partial)
 {
+    grid_trigger();
+    grid_wait();
     const int j = blockIdx.y;
     const int64_t e0 = blockIdx.x * chunk, e1 = min(n, e0 + chunk);
     const double *x = X + (size_t)j * n;
@@ -246,9 +254,11 @@ __global__ void k_sum_rows(const double *__restrict__ partial, int nchunk, int r
 }
 
 // Directions: T_q = R_p / (d - theta_q) (guarded), or T_q = R_p without d; sel[2q] = p, sel[2q + 1] = theta_q
-__global__ void __launch_bounds__(256) k_direction(const double *__restrict__ R, const double *__restrict__ d,
-                                                   const double *__restrict__ sel, int64_t n, double *__restrict__ T)
+__global__ void __launch_bounds__(256) k_direction(const double *R, const double *d, const double *sel, int64_t n,
+                                                   double *T)
 {
+    grid_trigger();
+    grid_wait();
     const int q = blockIdx.y;
     const double *r = R + (size_t)sel[2 * q] * n;
     const double theta = sel[2 * q + 1];
@@ -275,6 +285,8 @@ __global__ void k_unit_vectors(double *__restrict__ X, int64_t n, const double *
 // x <- x / ||x|| by one block (0 when ||x||^2 <= 1e-24), the squared norm in *nn
 __global__ void __launch_bounds__(1024) k_normalise(double *x, int64_t n, double *nn)
 {
+    grid_trigger();
+    grid_wait();
     double v = 0.0;
     for (int64_t e = threadIdx.x; e < n; e += 1024) v = fma(x[e], x[e], v);
     v = block_sum<1024>(v);
@@ -315,8 +327,7 @@ cudaError_t dev_gram(const double *A, int ka, const double *B, int kb, int64_t n
 {
     if (kb > kMaxCols || kb < 1 || ka < 1) return cudaErrorInvalidValue;
     if (n <= kSmallN) {
-        k_gram_small<<<dim3(ka, kb), kDotThreads, 0, s>>>(A, B, (int)n, C_dev);
-        return cudaGetLastError();
+        return launch_early(k_gram_small, dim3(ka, kb), kDotThreads, 0, s, A, B, (int)n, C_dev);
     }
     dim3 grid(kGramChunks, (ka + kGramRows - 1) / kGramRows);
     k_gram_partial<<<grid, 256, 0, s>>>(A, ka, B, kb, n, partial);
@@ -332,17 +343,16 @@ cudaError_t dev_combine(const double *V, int k, const double *S_dev, int r, doub
 {
     if (r > kMaxCols || r < 1 || k < 1) return cudaErrorInvalidValue;
     if (n <= kSmallN)
-        k_combine_small<<<dim3((unsigned)((n + 63) / 64), r), 64, 0, s>>>(V, k, S_dev, r, alpha, base, out, (int)n);
-    else
-        k_combine_base<<<608, 256, sizeof(double) * k * r, s>>>(V, k, S_dev, r, alpha, base, out, n);
+        return launch_early(k_combine_small, dim3((unsigned)((n + 63) / 64), r), 64, 0, s, V, k, S_dev, r, alpha, base,
+                            out, (int)n);
+    k_combine_base<<<608, 256, sizeof(double) * k * r, s>>>(V, k, S_dev, r, alpha, base, out, n);
     return cudaGetLastError();
 }
 
 cudaError_t dev_chol_inverse(const double *G, int b, double *Ri, int *rank, cudaStream_t s)
 {
     if (b < 1 || b > kMaxChol) return cudaErrorInvalidValue;
-    k_chol_inverse<<<1, 32, 0, s>>>(G, b, Ri, rank);
-    return cudaGetLastError();
+    return launch_early(k_chol_inverse, dim3(1), 32, 0, s, G, b, Ri, rank);
 }
 
 // HX_j -= theta_j X_j; norms2[j] = ||HX_j||^2 (device or pinned host).  partial: 304 doubles per row.
@@ -352,7 +362,9 @@ cudaError_t dev_residual(const double *X, const double *theta, double *HX, int r
     if (rows < 1) return cudaErrorInvalidValue;
     const int nchunk = (int)std::max<int64_t>(1, std::min<int64_t>(kGramChunks, (n + 2047) / 2048));
     const int64_t chunk = (n + nchunk - 1) / nchunk;
-    k_residual<<<dim3(nchunk, rows), 256, 0, s>>>(X, theta, HX, n, chunk, nchunk == 1 ? norms2 : partial);
+    const cudaError_t e =
+        launch_early(k_residual, dim3(nchunk, rows), 256, 0, s, X, theta, HX, n, chunk, nchunk == 1 ? norms2 : partial);
+    if (e != cudaSuccess) return e;
     if (nchunk > 1) k_sum_rows<<<(rows + 31) / 32, 32, 0, s>>>(partial, nchunk, rows, norms2);
     return cudaGetLastError();
 }
@@ -361,8 +373,7 @@ cudaError_t dev_direction(const double *R, const double *d, const double *sel, i
                           cudaStream_t s)
 {
     const unsigned bx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(608, (n + 255) / 256));
-    k_direction<<<dim3(bx, rows), 256, 0, s>>>(R, d, sel, n, T);
-    return cudaGetLastError();
+    return launch_early(k_direction, dim3(bx, rows), 256, 0, s, R, d, sel, n, T);
 }
 
 cudaError_t dev_unit_vectors(double *X, int64_t n, const double *at, int r, cudaStream_t s)
@@ -376,8 +387,7 @@ cudaError_t dev_unit_vectors(double *X, int64_t n, const double *at, int r, cuda
 cudaError_t dev_normalise(double *x, int64_t n, double *nn, double *partial, cudaStream_t s)
 {
     if (n <= kSmallN) {
-        k_normalise<<<1, 1024, 0, s>>>(x, n, nn);
-        return cudaGetLastError();
+        return launch_early(k_normalise, dim3(1), 1024, 0, s, x, n, nn);
     }
     double *xx = partial + gram_partial_doubles(n, 1);
     cudaError_t e = dev_gram(x, 1, x, 1, n, xx, partial, s);
@@ -391,8 +401,7 @@ cudaError_t dev_project_normalise(const double *V, int k, const double *c, doubl
                                   cudaStream_t s)
 {
     if (n <= kSmallN) {
-        k_project_normalise<<<(unsigned)((n + 63) / 64), 64, 0, s>>>(V, k, c, x, (int)n, nn);
-        return cudaGetLastError();
+        return launch_early(k_project_normalise, dim3((unsigned)((n + 63) / 64)), 64, 0, s, V, k, c, x, (int)n, nn);
     }
     cudaError_t e = dev_combine(V, k, c, 1, -1.0, x, x, n, s);
     if (e != cudaSuccess) return e;
