@@ -580,6 +580,7 @@ __global__ void __launch_bounds__(kRT, row_blocks<T>()) k_rows_batch(const RowOp
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint64_t bar;
+    grid_trigger();
     const int2 it = items[blockIdx.x];
     const RowOp &R = ops[it.x];
     RowIO o = io;
@@ -728,19 +729,18 @@ __global__ void __launch_bounds__(kRT) k_cheb_rows_batch(const RowOp *__restrict
 
 // xs[r * stride + v] = x_v[r] in T (zero beyond nvec), rows r0 .. r0 + nr - 1
 template <typename T>
-__device__ __forceinline__ void stage_row(const double *__restrict__ x, size_t n, int nvec, int stride,
-                                          T *__restrict__ xs, size_t r)
+__device__ __forceinline__ void stage_row(const double *x, size_t n, int nvec, int stride, T *xs, size_t r)
 {
     T *row = xs + r * stride;
     if (stride < 4) {
-        for (int v = 0; v < stride; v++) row[v] = Elem<T>::of(__ldg(x + (size_t)v * n + r));
+        for (int v = 0; v < stride; v++) row[v] = Elem<T>::of(x[(size_t)v * n + r]);
         return;
     }
     constexpr int U = 16 / (int)sizeof(T);
     for (int v0 = 0; v0 < stride; v0 += 4) {
         Vec<T, 4> t;
 #pragma unroll
-        for (int u = 0; u < 4; u++) t.v[u] = v0 + u < nvec ? Elem<T>::of(__ldg(x + (size_t)(v0 + u) * n + r)) : Elem<T>::of(0.0);
+        for (int u = 0; u < 4; u++) t.v[u] = v0 + u < nvec ? Elem<T>::of(x[(size_t)(v0 + u) * n + r]) : Elem<T>::of(0.0);
 #pragma unroll
         for (int u = 0; u < 4; u += U)
             *reinterpret_cast<Vec<T, U> *>(row + v0 + u) = *reinterpret_cast<const Vec<T, U> *>(t.v + u);
@@ -751,6 +751,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_row_stage(const RowOp R, const RowIO io)
 {
     grid_trigger();
+    grid_wait();
     T *xs = const_cast<T *>(static_cast<const T *>(io.xs));
     for (size_t r = blockIdx.x * (size_t)blockDim.x + threadIdx.x; r < (size_t)R.n; r += (size_t)gridDim.x * blockDim.x)
         stage_row<T>(io.x, R.n, io.nvec, io.stride, xs, r);
@@ -760,6 +761,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_row_stage_batch(const int2 *__restrict__ items, const RowIO io,
                                                          const long long *__restrict__ cs_prefix)
 {
+    grid_trigger();
+    grid_wait();
     const int2 it = items[blockIdx.x];  // (problem, chunk of 256 rows)
     const size_t c0 = (size_t)cs_prefix[it.x], n = (size_t)cs_prefix[it.x + 1] - c0;
     const size_t r = (size_t)it.y * 256 + threadIdx.x;
@@ -771,6 +774,7 @@ __global__ void __launch_bounds__(256) k_row_stage_batch(const int2 *__restrict_
 // Block j: problem j (its vectors from nvec * cs_prefix[j]).
 __global__ void __launch_bounds__(1024) k_row_settle(const RowIO io, int n_one, const long long *__restrict__ cs_prefix)
 {
+    grid_wait();
     const int j = blockIdx.x;
     const size_t c0 = cs_prefix ? (size_t)cs_prefix[j] : 0;
     const size_t n = cs_prefix ? (size_t)cs_prefix[j + 1] - c0 : (size_t)n_one;
@@ -858,13 +862,12 @@ cudaError_t rows_batch_t(const RowOp *ops, const int2 *items, int nitems, int ca
                          const long long *cs_prefix, cudaStream_t s)
 {
     const size_t smem = rows_smem(cap, wrows);
-    const unsigned blocks = (unsigned)nitems;
+    const dim3 grid((unsigned)nitems);
     vt = fit_vt(vt, io.stride);
     const int l = lanes_log2(io.nvec, vt);
-    if (vt == 4) k_rows_batch<T, 4><<<blocks, kRT, smem, s>>>(ops, items, io, l, cs_prefix, cap);
-    else if (vt == 2) k_rows_batch<T, 2><<<blocks, kRT, smem, s>>>(ops, items, io, l, cs_prefix, cap);
-    else k_rows_batch<T, 1><<<blocks, kRT, smem, s>>>(ops, items, io, l, cs_prefix, cap);
-    return cudaGetLastError();
+    if (vt == 4) return launch_early(k_rows_batch<T, 4>, grid, kRT, smem, s, ops, items, io, l, cs_prefix, cap);
+    if (vt == 2) return launch_early(k_rows_batch<T, 2>, grid, kRT, smem, s, ops, items, io, l, cs_prefix, cap);
+    return launch_early(k_rows_batch<T, 1>, grid, kRT, smem, s, ops, items, io, l, cs_prefix, cap);
 }
 
 }  // namespace
@@ -945,31 +948,28 @@ cudaError_t launch_cheb_rows_batch(const RowOp *ops, const int2 *items, int nite
 cudaError_t launch_row_stage(const RowOp &R, const RowIO &io, sg_precision prec, cudaStream_t stream)
 {
     const unsigned blocks = (unsigned)std::max(1, std::min((R.n + 255) / 256, 152 * 16));
-    if (prec == SG_MIXED) k_row_stage<float><<<blocks, 256, 0, stream>>>(R, io);
-    else if (prec == SG_DF64) k_row_stage<df2><<<blocks, 256, 0, stream>>>(R, io);
-    else k_row_stage<double><<<blocks, 256, 0, stream>>>(R, io);
-    return cudaGetLastError();
+    if (prec == SG_MIXED) return launch_early(k_row_stage<float>, dim3(blocks), 256, 0, stream, R, io);
+    if (prec == SG_DF64) return launch_early(k_row_stage<df2>, dim3(blocks), 256, 0, stream, R, io);
+    return launch_early(k_row_stage<double>, dim3(blocks), 256, 0, stream, R, io);
 }
 
 cudaError_t launch_row_stage_batch(const RowIO &io, sg_precision prec, const long long *cs_prefix, const int2 *items,
                                    int nitems, cudaStream_t stream)
 {
     if (nitems <= 0) return cudaSuccess;
-    if (prec == SG_MIXED) k_row_stage_batch<float><<<(unsigned)nitems, 256, 0, stream>>>(items, io, cs_prefix);
-    else k_row_stage_batch<double><<<(unsigned)nitems, 256, 0, stream>>>(items, io, cs_prefix);
-    return cudaGetLastError();
+    const dim3 grid((unsigned)nitems);
+    if (prec == SG_MIXED) return launch_early(k_row_stage_batch<float>, grid, 256, 0, stream, items, io, cs_prefix);
+    return launch_early(k_row_stage_batch<double>, grid, 256, 0, stream, items, io, cs_prefix);
 }
 
 cudaError_t launch_row_settle(const RowIO &io, int n, cudaStream_t stream)
 {
-    k_row_settle<<<1, 1024, 0, stream>>>(io, n, nullptr);
-    return cudaGetLastError();
+    return launch_early(k_row_settle, dim3(1), 1024, 0, stream, io, n, nullptr);
 }
 
 cudaError_t launch_row_settle_batch(const RowIO &io, const long long *cs_prefix, int nprob, cudaStream_t stream)
 {
-    k_row_settle<<<(unsigned)nprob, 1024, 0, stream>>>(io, 0, cs_prefix);
-    return cudaGetLastError();
+    return launch_early(k_row_settle, dim3((unsigned)nprob), 1024, 0, stream, io, 0, cs_prefix);
 }
 
 cudaError_t launch_row_finish(const RowOp &R, const RowIO &io, cudaStream_t stream)
