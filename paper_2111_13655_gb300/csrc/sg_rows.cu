@@ -420,7 +420,7 @@ __host__ __device__ inline size_t rows_smem(int cap, int wrows)
 // else from x itself, converted (VT = 1).  True in a thread that found a
 // non-finite input value.
 template <typename T, int VT, bool ST>
-__device__ __forceinline__ bool rows_window(const RowOp &R, const RowIO &io, const RowWin &win, int lgl, int cap,
+__device__ __forceinline__ bool rows_window(const RowOp &R, const RowIO &io, const RowWin &win, int lanes, int cap,
                                             unsigned char *smem, uint64_t *bar)
 {
     const int tid = threadIdx.x, n = R.n;
@@ -443,8 +443,8 @@ __device__ __forceinline__ bool rows_window(const RowOp &R, const RowIO &io, con
     const int *cols = reinterpret_cast<const int *>(rec + row_meta_bytes(win.nrows));
     const T *vals = reinterpret_cast<const T *>(cols + win.nent);
     const T *xs = static_cast<const T *>(io.xs);
-    const int lane = tid & ((1 << lgl) - 1), slot = tid >> lgl, nslot = kRT >> lgl;
-    const int vpass = VT << lgl;  // vectors per pass, at most kTileV
+    const int slot = tid / lanes, lane = tid - slot * lanes, nslot = kRT / lanes;  // slots from nslot on are idle
+    const int vpass = VT * lanes;  // vectors per pass, at most kTileV
     __syncthreads();  // the barrier is initialised
     const bool late = staged && !bar_wait(bar, 0);
     // everything above reads the operator only; x, y and the flags belong to earlier launches until here
@@ -468,7 +468,7 @@ __device__ __forceinline__ bool rows_window(const RowOp &R, const RowIO &io, con
         for (int it = 0; it * nslot < win.nrows; it++) {
             // every second round in reverse: long and short rows on each slot
             const int q = it * nslot + (it & 1 ? nslot - 1 - slot : slot);
-            if (q >= win.nrows || v >= io.nvec) continue;
+            if (slot >= nslot || q >= win.nrows || v >= io.nvec) continue;
             const uint2 mt = meta[q];
             Sum<T, VT> acc;
             acc.zero();
@@ -547,13 +547,13 @@ __device__ __forceinline__ void settle_vectors(unsigned *flags, int nvec, double
 }
 
 template <typename T, int VT, bool ST>
-__global__ void __launch_bounds__(kRT, row_blocks<T>()) k_rows(const RowOp R, const RowIO io, int lgl)
+__global__ void __launch_bounds__(kRT, row_blocks<T>()) k_rows(const RowOp R, const RowIO io, int lanes)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint64_t bar;
     grid_trigger();
     const bool odd =
-        rows_window<T, VT, ST>(R, io, R.wins[blockIdx.x * io.nparts + io.part], lgl, R.cap, smem, &bar);
+        rows_window<T, VT, ST>(R, io, R.wins[blockIdx.x * io.nparts + io.part], lanes, R.cap, smem, &bar);
     if (!io.ticket) return;
     // the block that ends last settles the vectors (instead of a launch of its
     // own) if any block found one: the high half of the ticket counts those
@@ -575,7 +575,7 @@ __global__ void __launch_bounds__(kRT, row_blocks<T>()) k_rows(const RowOp R, co
 template <typename T, int VT>
 __global__ void __launch_bounds__(kRT, row_blocks<T>()) k_rows_batch(const RowOp *__restrict__ ops,
                                                                 const int2 *__restrict__ items, const RowIO io,
-                                                                int lgl, const long long *__restrict__ cs_prefix,
+                                                                int lanes, const long long *__restrict__ cs_prefix,
                                                                 int cap)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -589,7 +589,7 @@ __global__ void __launch_bounds__(kRT, row_blocks<T>()) k_rows_batch(const RowOp
     o.y += c0 * io.nvec;
     o.xs = static_cast<const T *>(io.xs) + c0 * io.stride;
     o.flags += (size_t)it.x * io.nvec;
-    rows_window<T, VT, true>(R, o, R.wins[it.y], lgl, cap, smem, &bar);
+    rows_window<T, VT, true>(R, o, R.wins[it.y], lanes, cap, smem, &bar);
 }
 
 // One Chebyshev term of a window: a thread takes a row, both vectors (the real
@@ -796,12 +796,15 @@ __global__ void __launch_bounds__(256) k_row_finish(const RowOp R, const RowIO i
     }
 }
 
-// lanes per row (log2): as many as cover the vectors of a pass
-int lanes_log2(int nvec, int vt)
+// Lanes per row, of vt vectors each: the vectors are dealt out evenly over the
+// fewest passes of at most kTileV.  An idle lane costs as much as a busy one, so
+// the count is not rounded up to a power of two (D=12 L=9 FP64: 3, 5, 12 and 17
+// vectors 52.5, 88.0, 166.9 and 249.4 us with powers of two, 45.8, 68.7, 144.9
+// and 216.4 so; D=12 L=8 double-float, 5 vectors: 34.6 and 32.4).
+int row_lanes(int nvec, int vt)
 {
-    int l = 0;
-    while ((vt << (l + 1)) <= kTileV && (vt << l) < nvec) l++;
-    return l;
+    const int need = (nvec + vt - 1) / vt, most = kTileV / vt, passes = (need + most - 1) / most;
+    return (need + passes - 1) / passes;
 }
 // vectors per lane: the plan's, within the row length of the copy
 int fit_vt(int vt, int stride)
@@ -846,7 +849,7 @@ cudaError_t rows_t(const RowOp &R, const RowIO &io, int vt, cudaStream_t s)
     const size_t smem = rows_smem(R.cap, R.wrows);
     const unsigned blocks = (unsigned)((R.nwin - io.part + io.nparts - 1) / io.nparts);
     vt = io.xs ? fit_vt(vt, io.stride) : 1;
-    const int l = lanes_log2(io.nvec, vt), vpass = vt << l;
+    const int l = row_lanes(io.nvec, vt), vpass = vt * l;
     // several passes over the vectors: side by side while the windows are at
     // most two blocks per SM and leave SMs idle (D=2, 28 functions, 16 vectors:
     // 10.8 us one after another, 10.0 side by side, the rest is the call)
@@ -864,7 +867,7 @@ cudaError_t rows_batch_t(const RowOp *ops, const int2 *items, int nitems, int ca
     const size_t smem = rows_smem(cap, wrows);
     const dim3 grid((unsigned)nitems);
     vt = fit_vt(vt, io.stride);
-    const int l = lanes_log2(io.nvec, vt);
+    const int l = row_lanes(io.nvec, vt);
     if (vt == 4) return launch_early(k_rows_batch<T, 4>, grid, kRT, smem, s, ops, items, io, l, cs_prefix, cap);
     if (vt == 2) return launch_early(k_rows_batch<T, 2>, grid, kRT, smem, s, ops, items, io, l, cs_prefix, cap);
     return launch_early(k_rows_batch<T, 1>, grid, kRT, smem, s, ops, items, io, l, cs_prefix, cap);
