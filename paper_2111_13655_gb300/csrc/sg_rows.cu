@@ -33,8 +33,12 @@ namespace {
 constexpr int kRT = 64;
 constexpr int kTileV = 8;  // vectors per pass (the tile's columns)
 constexpr int kOut = kTileV * kRowWindowMax / kRT;  // outputs per thread and pass
-// resident blocks per SM the kernels are compiled for (80 / 128 registers)
+// Resident blocks per SM the kernels are compiled for (80 / 128 registers).
+// Sixteen FP32 blocks spill: D=12 L=10 83 -> 102 us.  Twelve FP64 blocks cost
+// D=12 L=9 3% but are worth it for batches, whose windows are few and wait on
+// memory: 12 FP64 wavepackets 22.9 -> 20.9 us.
 template <typename T> constexpr int row_blocks() { return sizeof(T) == 4 ? 12 : 8; }
+constexpr int kBatchBlocks = 12;
 
 // ---------------------------------------------------------------- set-up
 
@@ -458,12 +462,19 @@ __device__ __forceinline__ bool rows_window(const RowOp &R, const RowIO &io, con
     // (the passes of few windows go to blocks of their own: gridDim.y)
     for (int v0 = blockIdx.y * vpass; v0 < io.nvec; v0 += gridDim.y * vpass) {
         const int nv = min(vpass, io.nvec - v0);
-        // x of the thread's outputs is on its way during the sums
+        // x of the thread's outputs is on its way during the sums, unless these
+        // take all registers (FP32, four vectors per lane; D=12 L=10, 8 vectors:
+        // 88.8 us with the loads up front, 82.9 after the sums; one or two
+        // vectors per lane: batches 46.2 and 46.6, FP64 91.7 and 92.7)
         const size_t g0 = (size_t)(v0 + tv) * n + win.row0 + tr, gs = (size_t)tvs * n;
         double xi[kOut];
+        auto fetch = [&] {
 #pragma unroll
-        for (int q = 0; q < kOut; q++)
-            if (io.y && own && tv + q * tvs < nv) xi[q] = io.x[g0 + q * gs];
+            for (int q = 0; q < kOut; q++)
+                if (io.y && own && tv + q * tvs < nv) xi[q] = io.x[g0 + q * gs];
+        };
+        constexpr bool early = !(sizeof(T) == 4 && VT == 4);
+        if (early) fetch();
         const int v = v0 + lane * VT;
         for (int it = 0; it * nslot < win.nrows; it++) {
             // every second round in reverse: long and short rows on each slot
@@ -506,6 +517,7 @@ __device__ __forceinline__ bool rows_window(const RowOp &R, const RowIO &io, con
 #pragma unroll
             for (int u = 0; u < VT; u++) t[u << lw] = acc.bits(u);
         }
+        if (!early) fetch();
         __syncthreads();
         // y = sum + harmonic diagonal, or the sums' bits into the accumulators
         if (own) {
@@ -573,7 +585,7 @@ __global__ void __launch_bounds__(kRT, row_blocks<T>()) k_rows(const RowOp R, co
 // Many problems: item = (problem, window); vectors of problem j from
 // nvec * cs_prefix[j], its rows of xs from cs_prefix[j], flags from j * nvec.
 template <typename T, int VT>
-__global__ void __launch_bounds__(kRT, row_blocks<T>()) k_rows_batch(const RowOp *__restrict__ ops,
+__global__ void __launch_bounds__(kRT, kBatchBlocks) k_rows_batch(const RowOp *__restrict__ ops,
                                                                 const int2 *__restrict__ items, const RowIO io,
                                                                 int lanes, const long long *__restrict__ cs_prefix,
                                                                 int cap)
