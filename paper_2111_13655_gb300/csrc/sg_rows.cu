@@ -549,6 +549,10 @@ __device__ __forceinline__ bool rows_window(const RowOp &R, const RowIO &io, con
 // clears its flag.  By a whole block.
 __device__ __forceinline__ void settle_vectors(unsigned *flags, int nvec, double *y, size_t n)
 {
+    // the flags all at once: one after another their latencies made 5 us of a launch that finds none
+    bool any = false;
+    for (int v = threadIdx.x; v < nvec; v += blockDim.x) any |= __ldcg(flags + v) != 0u;
+    if (!__syncthreads_or(any)) return;
     for (int v = 0; v < nvec; v++) {
         if (__ldcg(flags + v) == 0u) continue;
         for (size_t i = threadIdx.x; i < n; i += blockDim.x) y[(size_t)v * n + i] = __longlong_as_double(0x7FF8000000000000ll);
