@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(256) k_row_count(const KParams P, const RowShi
 template <typename T> struct Elem;
 template <> struct Elem<float> { static __device__ float of(double v) { return (float)v; } };
 template <> struct Elem<double> { static __device__ double of(double v) { return v; } };
-template <> struct Elem<df2> { static __device__ df2 of(double v) { return df2(v); } };
+template <> struct Elem<df2> { static __device__ df2 of(double v) { return df_split(v); } };
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_row_fill(const KParams P, const RowShifts S, const RowWin *__restrict__ wins,
