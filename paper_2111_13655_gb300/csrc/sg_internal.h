@@ -213,7 +213,6 @@ struct HostTables {
     // in units of 16, shared memory that SG_ROW_SHARE blocks may use (bytes)
     int slice_vt = 0, warp_vt = 0, fbudget = 0;
     int cap = 0, maxnb = 0, matcap = 0, vtabcap = 0;
-    int64_t flops_per_vec = 0;       // FMA-counted work of one real apply (2 flops per FMA)
 };
 
 // Host setup (sg_setup.cpp).  Returns an empty string on success, else the error text.

@@ -5,14 +5,15 @@
 // Each engine iteration
 //   1. retires requests whose last step has ended (psi and logs to the host),
 //   2. admits queued requests, first come first served, while their planned
-//      device memory fits the budget (context tables, M^B, state vectors,
-//      batch workspace): builds the context, the spectral interval and the
+//      device memory fits the budget (context tables, state vectors, batch
+//      workspace): builds the context, the spectral interval and the
 //      Chebyshev weights,
 //   3. on any change of the active set, rebuilds the batch over the active
 //      contexts and moves the surviving states to the new layout,
-//   4. applies H_S to every active request's current Chebyshev vector in one
-//      sg_apply_H_batch (all requests' terms in one launch per kernel form),
-//   5. advances every request's recurrence by one term in one fused kernel.
+//   4. sums every row of every active request's current Chebyshev vector and
+//      advances its recurrence at the row's entry, in one launch (batch_cheb),
+//   5. logs and moves the recurrence states on.  With eigen requests active, or
+//      problems outside the row form: a batched apply, then an update kernel.
 // A request's arithmetic is the same whatever else is in the batch (batched
 // applies are bitwise those of the request's own context, the update is
 // elementwise, the logged sums run over the request's own entries in a fixed

@@ -359,7 +359,6 @@ std::string build_tables(const Problem &p, int smem_budget, int rb, HostTables *
     int fsum_max = 1, stage_min_max = 1;
     T.n_s = 0;
     T.n_grid = 0;
-    T.flops_per_vec = 0;
     for (int64_t t = 0; t < T.n_terms; t++) {
         const uint8_t *lt = &T.levels[(size_t)t * T.Dpad];
         int nb[kMaxD], nq[kMaxD], m = 0;
@@ -381,7 +380,7 @@ std::string build_tables(const Problem &p, int smem_budget, int rb, HostTables *
         T.matcap = std::max(T.matcap, mats);
         fsum_max = std::max(fsum_max, fsum);
         if (m > 0) stage_min_max = std::max(stage_min_max, nb[m - 1]);
-        // FMA count of the collapsed route: forward and backward chains + kinetic
+        // cost of the term: multiply-adds of the forward and backward chains and the kinetic matrices
         int64_t fma = 0;
         for (int tt = 0; tt < m; tt++) {
             int64_t sz = (int64_t)nb[tt] * nq[tt];
@@ -390,7 +389,6 @@ std::string build_tables(const Problem &p, int smem_budget, int rb, HostTables *
             fma += 2 * sz;
         }
         for (int j = 0; j < m; j++) fma += NB * nb[j];
-        T.flops_per_vec += 2 * fma + NG + 2 * NB;
         cost[t] = 2 * fma + 8 * NG + 16 * NB + 256;
     }
     T.vtabcap = fsum_max + (int)std::min<int64_t>(pair_entries, 1 << 24);
