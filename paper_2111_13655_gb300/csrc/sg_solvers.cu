@@ -16,70 +16,19 @@ namespace sg {
 
 namespace {
 
-constexpr int kGramRows = 8;   // rows of A per block in the Gram kernel
 constexpr int kMaxCols = 8;    // columns of B (block size) per call
-constexpr int kGramChunks = 304;
 
-// partial[c][i][j] = sum over chunk c of A[i][e] * B[j][e]  (A: ka x n, B: kb x n, column vectors)
-__global__ void __launch_bounds__(256) k_gram_partial(const double *__restrict__ A, int ka,
-                                                      const double *__restrict__ B, int kb, int64_t n,
-                                                      double *__restrict__ partial)
-{
-    __shared__ double red[kGramRows * kMaxCols][8];
-    const int c = blockIdx.x, i0 = blockIdx.y * kGramRows;
-    const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
-    const int64_t e0 = c * chunk, e1 = min(n, e0 + chunk);
-    double acc[kGramRows][kMaxCols];
-#pragma unroll
-    for (int r = 0; r < kGramRows; r++)
-#pragma unroll
-        for (int j = 0; j < kMaxCols; j++) acc[r][j] = 0.0;
-    for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-        double b[kMaxCols];
-#pragma unroll
-        for (int j = 0; j < kMaxCols; j++) b[j] = j < kb ? B[(size_t)j * n + e] : 0.0;
-#pragma unroll
-        for (int r = 0; r < kGramRows; r++) {
-            if (i0 + r >= ka) break;
-            const double a = A[(size_t)(i0 + r) * n + e];
-#pragma unroll
-            for (int j = 0; j < kMaxCols; j++) acc[r][j] = fma(a, b[j], acc[r][j]);
-        }
-    }
-    // block reduction: warp shuffles, then the 8 warps in fixed order
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int r = 0; r < kGramRows; r++)
-#pragma unroll
-        for (int j = 0; j < kMaxCols; j++) {
-            double v = acc[r][j];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-            if (lane == 0) red[r * kMaxCols + j][warp] = v;
-        }
-    __syncthreads();
-    for (int q = threadIdx.x; q < kGramRows * kMaxCols; q += blockDim.x) {
-        double v = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) v += red[q][w];
-        const int r = q / kMaxCols, j = q % kMaxCols;
-        if (i0 + r < ka && j < kb) partial[((size_t)c * ka + i0 + r) * kb + j] = v;
-    }
-}
-
-// C[i][j] = sum_c partial[c][i][j], in chunk order (deterministic)
-__global__ void k_gram_final(const double *__restrict__ partial, int nchunk, int ka, int kb, double *__restrict__ C)
-{
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= ka * kb) return;
-    double v = 0.0;
-    for (int c = 0; c < nchunk; c++) v += partial[(size_t)c * ka * kb + q];
-    C[q] = v;
-}
-
-// Vectors of at most kSmallN entries: the kernels above would put the whole
-// product on a few SMs, whose FP64 pipe (1/64 of the FP32 rate) then sets the
-// time (n = 1,001, 34 x 8: 20 us).  One block per inner product, and one column
-// per block of 64 entries, spread it over all SMs.
-constexpr int64_t kSmallN = 8192;
+// One block per inner product and chunk, one column per block of 64 entries:
+// the products go to as many SMs as there are, since the narrow FP64 pipe (1/64
+// of the FP32 rate) sets the time and sharing loads between products saves
+// none of it.  Blocks that made 8 x 8 products over 304 chunks reduced 64 sums
+// each through that pipe, and the 304 partial sums one after another: six
+// Davidson pairs at n = 12,870 22.2 ms, now 4.0; eight at n = 646,646 85.9 and
+// 40.9, and two propagation steps there 55.5 and 10.2 ms (most of it bounds).
+// A product of n = 646,646 in one block instead of 40: 78.6 and 38.6 ms.
+constexpr int64_t kChunk = 16384;  // entries per block; a product of more is summed in chunk order
+constexpr int kMaxChunks = 64;
+int chunks(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>(kMaxChunks, (n + kChunk - 1) / kChunk)); }
 constexpr int kDotThreads = 256;
 
 // Sum over the block, in a fixed order, to every thread.  The last step is made
@@ -102,26 +51,40 @@ __device__ __forceinline__ double block_sum(double v)
     return red[0];
 }
 
-// C[i][j] = sum_e A_i[e] B_j[e], block (i, j)
-__global__ void __launch_bounds__(kDotThreads) k_gram_small(const double *A, const double *B, int n, double *C)
+// C[z][i][j] = sum over chunk z of A_i[e] B_j[e], block (i, j, z)
+__global__ void __launch_bounds__(kDotThreads) k_gram(const double *A, const double *B, int n, int chunk, double *C)
 {
     grid_trigger();
     grid_wait();
-    const double *a = A + (size_t)blockIdx.x * n, *b = B + (size_t)blockIdx.y * n;
+    const size_t e0 = (size_t)blockIdx.z * chunk;
+    const double *a = A + (size_t)blockIdx.x * n + e0, *b = B + (size_t)blockIdx.y * n + e0;
+    const int len = min(chunk, n - (int)e0);
     double v = 0.0;
 #pragma unroll 8
-    for (int e = threadIdx.x; e < n; e += kDotThreads) v = fma(a[e], b[e], v);
+    for (int e = threadIdx.x; e < len; e += kDotThreads) v = fma(a[e], b[e], v);
     v = block_sum<kDotThreads>(v);
-    if (threadIdx.x == 0) C[blockIdx.x * gridDim.y + blockIdx.y] = v;
+    if (threadIdx.x == 0) C[((size_t)blockIdx.z * gridDim.x + blockIdx.x) * gridDim.y + blockIdx.y] = v;
+}
+// C[q] = sum_z partial[z][q], in chunk order
+__global__ void __launch_bounds__(64) k_sum_chunks(const double *partial, int nchunk, int count, double *C)
+{
+    grid_trigger();
+    grid_wait();
+    const int q = blockIdx.x * 64 + threadIdx.x;
+    if (q >= count) return;
+    double v = 0.0;
+#pragma unroll 16
+    for (int z = 0; z < nchunk; z++) v += partial[(size_t)z * count + q];
+    C[q] = v;
 }
 
 // out[j][e] = base[j][e] + alpha * sum_i V[i][e] S[i][j] (base nullptr: 0), column j = blockIdx.y
-__global__ void __launch_bounds__(64) k_combine_small(const double *V, int k, const double *S, int r, double alpha,
-                                                      const double *base, double *out, int n)
+__global__ void __launch_bounds__(64) k_combine(const double *V, int k, const double *S, int r, double alpha,
+                                                const double *base, double *out, unsigned n)
 {
     grid_trigger();
     grid_wait();
-    const int e = blockIdx.x * 64 + threadIdx.x, j = blockIdx.y;
+    const unsigned e = blockIdx.x * 64 + threadIdx.x, j = blockIdx.y;
     if (e >= n) return;
     double acc = 0.0;
 #pragma unroll 16
@@ -132,8 +95,8 @@ __global__ void __launch_bounds__(64) k_combine_small(const double *V, int k, co
 
 // x <- (x - sum_i V_i c_i) / norm, norm^2 = c_k - sum_i c_i^2 (V orthonormal, c_i = V_i . x, c_k = x . x); x <- 0 when
 // norm^2 <= 1e-24.  *nn = norm^2.
-__global__ void __launch_bounds__(64) k_project_normalise(const double *V, int k, const double *c, double *x, int n,
-                                                          double *nn)
+__global__ void __launch_bounds__(64) k_project_normalise(const double *V, int k, const double *c, double *x,
+                                                          unsigned n, double *nn)
 {
     grid_trigger();
     grid_wait();
@@ -148,7 +111,7 @@ __global__ void __launch_bounds__(64) k_project_normalise(const double *V, int k
             if (blockIdx.x == 0) *nn = v;
         }
     }
-    const int e = blockIdx.x * 64 + threadIdx.x;
+    const unsigned e = blockIdx.x * 64 + threadIdx.x;
     double acc = 0.0;
     if (e < n) {
 #pragma unroll 16
@@ -156,30 +119,6 @@ __global__ void __launch_bounds__(64) k_project_normalise(const double *V, int k
     }
     __syncthreads();
     if (e < n) x[e] = (x[e] - acc) * scale;
-}
-
-// out = base + alpha * V S for longer vectors (one block column of up to kMaxCols outputs)
-__global__ void __launch_bounds__(256) k_combine_base(const double *__restrict__ V, int k, const double *__restrict__ S,
-                                                      int r, double alpha, const double *base, double *out, int64_t n)
-{
-    extern __shared__ double Ss[];
-    for (int q = threadIdx.x; q < k * r; q += blockDim.x) Ss[q] = S[q];
-    __syncthreads();
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        double acc[kMaxCols];
-#pragma unroll
-        for (int j = 0; j < kMaxCols; j++) acc[j] = 0.0;
-        for (int i = 0; i < k; i++) {
-            const double v = V[(size_t)i * n + e];
-#pragma unroll
-            for (int j = 0; j < kMaxCols; j++)
-                if (j < r) acc[j] = fma(v, Ss[i * r + j], acc[j]);
-        }
-        for (int j = 0; j < r; j++) {
-            const size_t o = (size_t)j * n + e;
-            out[o] = (base ? base[o] : 0.0) + alpha * acc[j];
-        }
-    }
 }
 
 // Cholesky G = R^T R (b x b, row-major, b <= kMaxChol) to Ri = R^{-1}; columns
@@ -224,7 +163,7 @@ __global__ void __launch_bounds__(32) k_chol_inverse(const double *G, int b, dou
     if (i == 0) *rank = rk;
 }
 
-// Residuals: HX_j -= theta_j X_j, and their squared norms (partial[j][chunk], chunk = blockIdx.x)
+// Residuals: HX_j -= theta_j X_j, and their squared norms (partial[chunk][j], chunk = blockIdx.x)
 __global__ void __launch_bounds__(256) k_residual(const double *X, const double *theta, double *HX, int64_t n,
                                                   int64_t chunk, double *partial)
 {
@@ -242,15 +181,7 @@ __global__ void __launch_bounds__(256) k_residual(const double *X, const double 
         v = fma(r, r, v);
     }
     v = block_sum<256>(v);
-    if (threadIdx.x == 0) partial[j * gridDim.x + blockIdx.x] = v;
-}
-__global__ void k_sum_rows(const double *__restrict__ partial, int nchunk, int rows, double *__restrict__ out)
-{
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= rows) return;
-    double v = 0.0;
-    for (int c = 0; c < nchunk; c++) v += partial[j * nchunk + c];
-    out[j] = v;
+    if (threadIdx.x == 0) partial[blockIdx.x * gridDim.y + j] = v;
 }
 
 // Directions: T_q = R_p / (d - theta_q) (guarded), or T_q = R_p without d; sel[2q] = p, sel[2q + 1] = theta_q
@@ -296,17 +227,11 @@ __global__ void __launch_bounds__(1024) k_normalise(double *x, int64_t n, double
     for (int64_t e = threadIdx.x; e < n; e += 1024) x[e] *= f;
     if (threadIdx.x == 0) *nn = v;
 }
-// the same for longer vectors, from the squared norm (less the squares of k projections c_i already taken out)
-__global__ void k_scale_norm(double *x, int64_t n, const double *xx, const double *c, int k, double *nn)
+// the same for longer vectors, from the squared norm
+__global__ void __launch_bounds__(256) k_scale_norm(double *x, int64_t n, const double *xx, double *nn)
 {
-    __shared__ double f;
-    if (threadIdx.x == 0) {
-        double v = *xx;
-        for (int i = 0; i < k; i++) v = fma(-c[i], c[i], v);
-        f = v > 1e-24 ? 1.0 / sqrt(v) : 0.0;
-        if (blockIdx.x == 0) *nn = v;
-    }
-    __syncthreads();
+    const double v = *xx, f = v > 1e-24 ? 1.0 / sqrt(v) : 0.0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *nn = v;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) x[e] *= f;
 }
 
@@ -326,27 +251,23 @@ cudaError_t dev_gram(const double *A, int ka, const double *B, int kb, int64_t n
                      double *partial, cudaStream_t s)
 {
     if (kb > kMaxCols || kb < 1 || ka < 1) return cudaErrorInvalidValue;
-    if (n <= kSmallN) {
-        return launch_early(k_gram_small, dim3(ka, kb), kDotThreads, 0, s, A, B, (int)n, C_dev);
-    }
-    dim3 grid(kGramChunks, (ka + kGramRows - 1) / kGramRows);
-    k_gram_partial<<<grid, 256, 0, s>>>(A, ka, B, kb, n, partial);
-    k_gram_final<<<(ka * kb + 255) / 256, 256, 0, s>>>(partial, kGramChunks, ka, kb, C_dev);
-    return cudaGetLastError();
+    const int nz = chunks(n);
+    cudaError_t e = launch_early(k_gram, dim3(ka, kb, nz), kDotThreads, 0, s, A, B, (int)n, (int)((n + nz - 1) / nz),
+                                 nz == 1 ? C_dev : partial);
+    if (e == cudaSuccess && nz > 1)
+        e = launch_early(k_sum_chunks, dim3((ka * kb + 63) / 64), 64, 0, s, (const double *)partial, nz, ka * kb, C_dev);
+    return e;
 }
 
-size_t gram_partial_doubles(int64_t n, int ka) { return n <= kSmallN ? (size_t)8 * ka : (size_t)kGramChunks * ka * kMaxCols; }
+size_t gram_partial_doubles(int64_t n, int ka) { return (size_t)chunks(n) * ka * kMaxCols; }
 
 // out (r x n) = base (r x n, or nullptr: zero; may be out) + alpha * V (k x n)^T-combination with S (k x r, device)
 cudaError_t dev_combine(const double *V, int k, const double *S_dev, int r, double alpha, const double *base,
                         double *out, int64_t n, cudaStream_t s)
 {
     if (r > kMaxCols || r < 1 || k < 1) return cudaErrorInvalidValue;
-    if (n <= kSmallN)
-        return launch_early(k_combine_small, dim3((unsigned)((n + 63) / 64), r), 64, 0, s, V, k, S_dev, r, alpha, base,
-                            out, (int)n);
-    k_combine_base<<<608, 256, sizeof(double) * k * r, s>>>(V, k, S_dev, r, alpha, base, out, n);
-    return cudaGetLastError();
+    return launch_early(k_combine, dim3((unsigned)((n + 63) / 64), r), 64, 0, s, V, k, S_dev, r, alpha, base, out,
+                        (unsigned)n);
 }
 
 cudaError_t dev_chol_inverse(const double *G, int b, double *Ri, int *rank, cudaStream_t s)
@@ -355,18 +276,18 @@ cudaError_t dev_chol_inverse(const double *G, int b, double *Ri, int *rank, cuda
     return launch_early(k_chol_inverse, dim3(1), 32, 0, s, G, b, Ri, rank);
 }
 
-// HX_j -= theta_j X_j; norms2[j] = ||HX_j||^2 (device or pinned host).  partial: 304 doubles per row.
+// HX_j -= theta_j X_j; norms2[j] = ||HX_j||^2 (device or pinned host).  partial: a double per row and chunk.
 cudaError_t dev_residual(const double *X, const double *theta, double *HX, int rows, int64_t n, double *norms2,
                          double *partial, cudaStream_t s)
 {
     if (rows < 1) return cudaErrorInvalidValue;
-    const int nchunk = (int)std::max<int64_t>(1, std::min<int64_t>(kGramChunks, (n + 2047) / 2048));
-    const int64_t chunk = (n + nchunk - 1) / nchunk;
-    const cudaError_t e =
-        launch_early(k_residual, dim3(nchunk, rows), 256, 0, s, X, theta, HX, n, chunk, nchunk == 1 ? norms2 : partial);
-    if (e != cudaSuccess) return e;
-    if (nchunk > 1) k_sum_rows<<<(rows + 31) / 32, 32, 0, s>>>(partial, nchunk, rows, norms2);
-    return cudaGetLastError();
+    const int nz = chunks(n);
+    const int64_t chunk = (n + nz - 1) / nz;
+    cudaError_t e =
+        launch_early(k_residual, dim3(nz, rows), 256, 0, s, X, theta, HX, n, chunk, nz == 1 ? norms2 : partial);
+    if (e == cudaSuccess && nz > 1)
+        e = launch_early(k_sum_chunks, dim3((rows + 63) / 64), 64, 0, s, (const double *)partial, nz, rows, norms2);
+    return e;
 }
 
 cudaError_t dev_direction(const double *R, const double *d, const double *sel, int rows, int64_t n, double *T,
@@ -386,13 +307,11 @@ cudaError_t dev_unit_vectors(double *X, int64_t n, const double *at, int r, cuda
 // x <- x / ||x|| (zero when ||x||^2 <= 1e-24); nn: the squared norm (device)
 cudaError_t dev_normalise(double *x, int64_t n, double *nn, double *partial, cudaStream_t s)
 {
-    if (n <= kSmallN) {
-        return launch_early(k_normalise, dim3(1), 1024, 0, s, x, n, nn);
-    }
+    if (chunks(n) == 1) return launch_early(k_normalise, dim3(1), 1024, 0, s, x, n, nn);
     double *xx = partial + gram_partial_doubles(n, 1);
     cudaError_t e = dev_gram(x, 1, x, 1, n, xx, partial, s);
     if (e != cudaSuccess) return e;
-    k_scale_norm<<<608, 256, 0, s>>>(x, n, xx, nullptr, 0, nn);
+    k_scale_norm<<<608, 256, 0, s>>>(x, n, xx, nn);
     return cudaGetLastError();
 }
 
@@ -400,13 +319,7 @@ cudaError_t dev_normalise(double *x, int64_t n, double *nn, double *partial, cud
 cudaError_t dev_project_normalise(const double *V, int k, const double *c, double *x, int64_t n, double *nn,
                                   cudaStream_t s)
 {
-    if (n <= kSmallN) {
-        return launch_early(k_project_normalise, dim3((unsigned)((n + 63) / 64)), 64, 0, s, V, k, c, x, (int)n, nn);
-    }
-    cudaError_t e = dev_combine(V, k, c, 1, -1.0, x, x, n, s);
-    if (e != cudaSuccess) return e;
-    k_scale_norm<<<608, 256, 0, s>>>(x, n, c + k, c, k, nn);
-    return cudaGetLastError();
+    return launch_early(k_project_normalise, dim3((unsigned)((n + 63) / 64)), 64, 0, s, V, k, c, x, (unsigned)n, nn);
 }
 
 cudaError_t dev_axpby(int64_t len, double a, const double *x, double b, double *y, cudaStream_t s)

@@ -183,13 +183,13 @@ def test_constant_basis_sizes_inside_and_outside_the_row_form(D, L, prec):
         assert elem_rel(y.cpu().numpy(), r) <= (FP64_TOL if prec == "fp64" else 5e-6)
 
 
-# N_cs 8,008 and 8,568: one block per inner product, and the chunked products
-@pytest.mark.parametrize("D,L", [(6, 10), (5, 13)])
-def test_solvers_on_both_sides_of_the_short_vector_rule(D, L):
+# N_cs 8,008 and 27,132: one and two chunks per inner product
+@pytest.mark.parametrize("D,L", [(6, 10), (6, 13)])
+def test_solvers_with_products_in_one_and_in_several_chunks(D, L):
     p = synth.chained_henon_heiles(D, L, synth.draw_omega(D, 6), 0.1)
     nev, tol = 5, 1e-9
     with sg.sg_create(p, "fp64") as ctx:
-        assert (ctx.n_cs <= 8192) == (D == 6)
+        assert (ctx.n_cs <= 16384) == (L == 10)
         ev, rn, vec, _ = sg.sg_eigs(ctx, nev, "davidson", block=4, tol=tol, max_it=300, vectors=True)
         v = vec.view(nev, ctx.n_cs)
         r = apply(ctx, v) - torch.from_numpy(np.asarray(ev)).cuda()[:, None] * v
