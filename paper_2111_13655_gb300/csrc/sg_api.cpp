@@ -196,22 +196,25 @@ sg_status plan(int D, int L, const sg_basis *basis, const sg_grid *grids,
 
 namespace sg {
 
-// Input copies small enough to stay in the caches are not made: the row
-// kernel then gathers from x itself.
+// Entry-major copies of x of at most this many values are not made: the row
+// kernel gathers from x itself, which stays in the caches, and a launch is saved
+// (mixed, 24,024 values 9.1 us without the copy and 11.4 with it; 64,350 12.4
+// and 11.7; 97,240 14.3 and 11.1).
 constexpr int64_t kDirectElems = 65536;
+// The last block settles the vectors up to this many windows, a launch beyond
+// (403 windows 9.4 us by the block and 11.8 by a launch, 684 11.1 and 13.8,
+// 1,969 22.5 and 20.0, 10,104 86.3 and 81.5: the blocks meet at the counter).
 constexpr int kTicketBlocks = 1024;
 
 cudaError_t apply_rows(sg_ctx *ctx, RowIO io, cudaStream_t s)
 {
     const sg_precision prec = ctx->prob.prec;
     cudaError_t e = cudaSuccess;
-    if (prec == SG_FP64 && io.nvec == 1) io.xs = io.x;  // x is its own entry-major copy
-    else if (!io.xs || ctx->host.n_cs * (int64_t)io.nvec <= kDirectElems) io.xs = nullptr;
+    const int vt = row_vt(ctx->host, prec);
+    if (!io.xs || ctx->host.n_cs * (int64_t)io.nvec <= kDirectElems || rows_direct(prec, vt, io.nvec)) io.xs = nullptr;
     else e = launch_row_stage(ctx->rop, io, prec, s);
-    // few blocks: the last one settles the vectors; many: the counter would be
-    // a point of contention, and a launch is short beside them
     if (!io.y || ctx->rop.nwin > kTicketBlocks) io.ticket = nullptr;
-    if (e == cudaSuccess) e = launch_rows(ctx->rop, io, prec, row_vt(ctx->host, prec), s);
+    if (e == cudaSuccess) e = launch_rows(ctx->rop, io, prec, vt, s);
     if (e == cudaSuccess && io.y && !io.ticket) e = launch_row_settle(io, ctx->rop.n, s);
     return e;
 }

@@ -12,8 +12,10 @@
 // A problem with at least this many rows fills the GPU for several waves by
 // itself: it runs as its own launches (parameters in the kernel's parameter
 // bank, windows of its own plan) inside the batch's sequence, and only the
-// smaller problems share the packed launches.
-constexpr int64_t kSoloRows = 131072;
+// smaller problems share the packed launches.  Two FP32 vectors each, packed
+// and on its own: 646,646 rows 47.8 and 46.3 us; 293,930 rows with eight small
+// problems 22.9 and 26.9.
+constexpr int64_t kSoloRows = 524288;
 
 struct sg_batch {
     std::vector<sg_ctx *> ctxs;
@@ -171,7 +173,7 @@ extern "C" sg_status sg_batch_size(const sg_batch *b, int64_t *n_cs_total, int64
     if (n_cs_total) *n_cs_total = b->cs_prefix.back();
     if (n_terms_total) *n_terms_total = b->n_terms;
     if (launches_per_apply) {
-        // row form: input copies, rows, settle; term by term: max|x|, terms, finalisation
+        // at most; row form: input copies (where made), rows, settle; term by term: max|x|, terms, finalisation
         const int l = (b->packed.empty() ? 0 : 3) + 3 * (int)(b->solo.size() + b->generic.size());
         *launches_per_apply = l;
     }
@@ -271,14 +273,18 @@ sg_status enqueue_apply(sg_batch *b, const double *x, double *y, int nvec, cudaS
         o.xs = static_cast<unsigned char *>(b->xs) + c0 * io.stride * rb;
         o.flags += (size_t)j * nvec;
         const sg_ctx *c = b->ctxs[j];
-        if ((e = sg::launch_row_stage(c->rop, o, prec, s)) != cudaSuccess ||
-            (e = sg::launch_rows(c->rop, o, prec, sg::row_vt(c->host, prec), s)) != cudaSuccess ||
+        const int vt = sg::row_vt(c->host, prec);
+        if (sg::rows_direct(prec, vt, nvec)) o.xs = nullptr;
+        if ((o.xs && (e = sg::launch_row_stage(c->rop, o, prec, s)) != cudaSuccess) ||
+            (e = sg::launch_rows(c->rop, o, prec, vt, s)) != cudaSuccess ||
             (e = sg::launch_row_settle(o, c->rop.n, s)) != cudaSuccess)
             return bfail(b, SG_ECUDA, std::string("row launch: ") + cudaGetErrorString(e));
     }
     if (!b->packed.empty()) {
         const int vt = b->fp32 ? SG_F32_VT : SG_F64_VT;
-        if ((e = sg::launch_row_stage_batch(io, prec, b->d_cs_prefix, b->stage_items, b->n_stage, s)) != cudaSuccess ||
+        if (sg::rows_direct(prec, vt, nvec)) io.xs = nullptr;
+        if ((io.xs &&
+             (e = sg::launch_row_stage_batch(io, prec, b->d_cs_prefix, b->stage_items, b->n_stage, s)) != cudaSuccess) ||
             (e = sg::launch_rows_batch(b->d_ops, b->items, b->n_items, b->cap, b->wrows, io, prec, vt,
                                        b->d_cs_prefix, s)) != cudaSuccess ||
             (e = sg::launch_row_settle_batch(io, b->d_cs_prefix, (int)b->ctxs.size(), s)) != cudaSuccess)

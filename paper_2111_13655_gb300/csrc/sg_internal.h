@@ -130,6 +130,12 @@ constexpr int kRowWindowMax = 64;  // rows per window at most
 
 // Row length (elements) of the entry-major input copy for nvec vectors.
 __host__ __device__ inline int xs_stride(int nvec) { return nvec <= 2 ? nvec : (nvec + 3) & ~3; }
+// FP64 rows with one vector per lane gather from x itself at any size: the FP64
+// pipe hides the extra sectors, and the copy is saved (8 vectors: D=10 L=8 24.2 us
+// without the copy and 27.6 with it, D=12 L=8 41.0 and 42.5, D=12 L=9 87.5 and
+// 89.9, D=12 L=10 202 and 203; 5 vectors 18.6 and 21.8, 31.0 and 33.0, 61.8 and
+// 67.6, 147 and 154).  Other types convert what they gather: 2 to 3 times slower.
+inline bool rows_direct(sg_precision prec, int vt, int nvec) { return prec == SG_FP64 && (vt == 1 || nvec == 1); }
 
 // Everything the set-up kernels and the term-by-term kernel need.
 struct alignas(16) KParams {

@@ -594,7 +594,7 @@ __global__ void __launch_bounds__(kRT, row_blocks<T>()) k_rows(const RowOp R, co
 
 // Many problems: item = (problem, window); vectors of problem j from
 // nvec * cs_prefix[j], its rows of xs from cs_prefix[j], flags from j * nvec.
-template <typename T, int VT>
+template <typename T, int VT, bool ST>
 __global__ void __launch_bounds__(kRT, kBatchBlocks) k_rows_batch(const RowOp *__restrict__ ops,
                                                                 const int2 *__restrict__ items, const RowIO io,
                                                                 int lanes, const long long *__restrict__ cs_prefix,
@@ -609,9 +609,9 @@ __global__ void __launch_bounds__(kRT, kBatchBlocks) k_rows_batch(const RowOp *_
     const size_t c0 = (size_t)cs_prefix[it.x];
     o.x += c0 * io.nvec;
     o.y += c0 * io.nvec;
-    o.xs = static_cast<const T *>(io.xs) + c0 * io.stride;
+    if (ST) o.xs = static_cast<const T *>(io.xs) + c0 * io.stride;
     o.flags += (size_t)it.x * io.nvec;
-    rows_window<T, VT, true>(R, o, R.wins[it.y], lanes, cap, smem, &bar);
+    rows_window<T, VT, ST>(R, o, R.wins[it.y], lanes, cap, smem, &bar);
 }
 
 // One Chebyshev term of a window: a thread takes a row, both vectors (the real
@@ -853,9 +853,11 @@ cudaError_t smem_limits()
     if (e == cudaSuccess) e = smem_limit(k_rows<T, 1, true>);
     if (e == cudaSuccess) e = smem_limit(k_rows<T, 2, true>);
     if (e == cudaSuccess) e = smem_limit(k_rows<T, 4, true>);
-    if (e == cudaSuccess) e = smem_limit(k_rows_batch<T, 1>);
-    if (e == cudaSuccess) e = smem_limit(k_rows_batch<T, 2>);
-    if (e == cudaSuccess) e = smem_limit(k_rows_batch<T, 4>);
+    if constexpr (sizeof(T) == 8)
+        if (e == cudaSuccess) e = smem_limit(k_rows_batch<T, 1, false>);
+    if (e == cudaSuccess) e = smem_limit(k_rows_batch<T, 1, true>);
+    if (e == cudaSuccess) e = smem_limit(k_rows_batch<T, 2, true>);
+    if (e == cudaSuccess) e = smem_limit(k_rows_batch<T, 4, true>);
     if (e == cudaSuccess) e = smem_limit(k_cheb_rows<T>);
     if (e == cudaSuccess) e = smem_limit(k_cheb_rows_batch<T>);
     return e;
@@ -888,11 +890,13 @@ cudaError_t rows_batch_t(const RowOp *ops, const int2 *items, int nitems, int ca
 {
     const size_t smem = rows_smem(cap, wrows);
     const dim3 grid((unsigned)nitems);
-    vt = fit_vt(vt, io.stride);
+    vt = io.xs ? fit_vt(vt, io.stride) : 1;
     const int l = row_lanes(io.nvec, vt);
-    if (vt == 4) return launch_early(k_rows_batch<T, 4>, grid, kRT, smem, s, ops, items, io, l, cs_prefix, cap);
-    if (vt == 2) return launch_early(k_rows_batch<T, 2>, grid, kRT, smem, s, ops, items, io, l, cs_prefix, cap);
-    return launch_early(k_rows_batch<T, 1>, grid, kRT, smem, s, ops, items, io, l, cs_prefix, cap);
+    if constexpr (sizeof(T) == 8)
+        if (!io.xs) return launch_early(k_rows_batch<T, 1, false>, grid, kRT, smem, s, ops, items, io, l, cs_prefix, cap);
+    if (vt == 4) return launch_early(k_rows_batch<T, 4, true>, grid, kRT, smem, s, ops, items, io, l, cs_prefix, cap);
+    if (vt == 2) return launch_early(k_rows_batch<T, 2, true>, grid, kRT, smem, s, ops, items, io, l, cs_prefix, cap);
+    return launch_early(k_rows_batch<T, 1, true>, grid, kRT, smem, s, ops, items, io, l, cs_prefix, cap);
 }
 
 }  // namespace
