@@ -5,8 +5,8 @@ Workload: chained Henon-Heiles, D=12, L=10, nb(l)=l+1, nq(l)=l+2, omega_i ~
 U[0.8,1.2] (seeded), lambda = 0.111803; N_cs = 646,646 compact functions,
 646,646 Smolyak terms.  One step = one sg_apply_H on a block of `nvec` real
 vectors (the block of the block-Davidson solver); one application = one real
-vector.  Mixed precision (FP32 contractions, FP64 accumulation) is the headline;
-FP64 mode is measured beside it.
+vector.  Mixed precision (FP32 products, their sums carried without rounding
+in pairs) is the headline; FP64 mode is measured beside it.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
@@ -22,6 +22,7 @@ from __future__ import annotations
 
 import argparse
 import json
+import math
 import os
 import statistics
 import subprocess
@@ -37,27 +38,44 @@ sys.path.insert(0, ROOT)
 METRIC = "Smolyak H|psi> applications/s and % roofline at D=12 L=10; mixed vs FP64; p50/p99"
 UNIT = "applications/s"
 WORKLOAD = "chained Henon-Heiles D=12 L=10 nb=l+1 nq=l+2 (N_cs=646646, 646646 terms)"
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of the term kernel
-# k_apply_fast per apply (its block-form and warp-form launches) at the
-# benchmark workload with the plan sg_tune keeps, per precision, from the
-# one-pass ncu capture of the full workload summarised in profiles/; None when
-# the kernel has changed since.
-TRAFFIC_BYTES = {"mixed": 8_849_153_280, "fp64": 23_382_741_248, "df64": 23_298_306_560}
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of the row kernel
+# k_rows per apply at the benchmark workload with the default plan, per
+# precision, from the one-pass ncu capture of the full workload summarised in
+# profiles/; None when the kernel has changed since.
+TRAFFIC_BYTES = {"mixed": 181_447_168, "fp64": 223_647_744, "df64": 258_490_112}
 # FP32 instructions of one double-float multiply-add (csrc/sg_df.cuh df_fma:
 # one multiply, three FMAs, two_sum 6, two additions): the double-float arm's
 # roofline counts these against the FP32 issue rate
 DF_INSTR_PER_FMA = 12
 # FP32 lanes per SM (the unit count of the derived FP32 peak)
 FP32_LANES_PER_SM = 128
-# kernels of one sg_apply_H at this workload: k_maxabs, k_stage_x (entry-major
-# input copy), k_apply_fast (block form over the large terms), k_apply_fast
-# (warp form over the small terms), k_finalize
-LAUNCHES_PER_APPLY = 5
+# kernels of one sg_apply_H at this workload: k_row_stage (entry-major input
+# copy), k_rows (row sums), k_row_settle (vectors with non-finite input)
+LAUNCHES_PER_APPLY = 3
+
+
+def hbm_peak_gbs():
+    """Measured copy bandwidth of this GPU model (MEASURED_PEAKS.json beside this file), or None."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+            return float(json.load(f)["hbm_gbs"])
+    except (OSError, KeyError, ValueError):
+        return None
+
+
+def row_entries(D: int, L: int) -> int:
+    """Non-zero elements of the chained Henon-Heiles H_S on nb(l) = l + 1 with
+    centred modes, less its diagonal harmonic part: the cubic couplings shift
+    one index by 1 or 3, or two neighbours by 2 and 1, and a shift by d in sum
+    leaves the C(D + L - d, D) multi-indices that have room for it."""
+    c = lambda d: math.comb(D + L - d, D) if L >= d else 0
+    return (D - 1) * (2 * c(1) + 2 * c(3) + 4 * c(3))
 
 
 def algorithmic_flops_per_vector(levels: np.ndarray, nbA=1, nbB=1, nqA=2, nqB=1, rmax=None) -> int:
-    """FLOPs of one real-vector apply of the chained Henon-Heiles operator by
-    the route the fast kernel takes, 2 flops per multiply-add.  Per term:
+    """FLOPs of one real-vector apply of the chained Henon-Heiles operator term
+    by term (Alg. 1 with the inner modes of a term tabulated), 2 flops per
+    multiply-add: what the row form does not spend.  Per term:
       - a term has a grid when two neighbouring modes (a coupled pair) both
         have nb > 1; then its last `rmax` level-1 modes (mode order) are inner
         positions (rmax = 3 for nb(1) = 2, 2 for nb(1) = 3, else 0);
@@ -127,6 +145,13 @@ class ClockSampler:
     def _read(self):
         for line in self.proc.stdout:
             self.lines.append(line.strip())
+
+    def under_load(self, step, samples=5, seconds=4.0):
+        """Runs `step` (untimed) until a few samples have come in: the timed
+        steps that follow take milliseconds, less than one sampling interval."""
+        t0 = time.perf_counter()
+        while self.proc and len(self.lines) < samples and time.perf_counter() - t0 < seconds:
+            step()
 
     def __exit__(self, *exc):
         if self.proc:
@@ -575,8 +600,8 @@ def main():
         ctx = sg.sg_create(p, prec)
         tuned = args.tune and not (args.sharding == "terms" and world > 1)
         if tuned:
-            # the library's own autotuner picks the schedule for these applies
-            # (slicing target, block/warp split, shared-memory budget) by timing
+            # the library's own autotuner picks the plan for these applies
+            # (vectors per lane, rows per window, shared-memory budget) by timing
             sg.sg_tune(ctx, nvec)
         plan = dict(sg.sg_tune_plan(ctx), tuned=bool(tuned))
         n = ctx.n_cs
@@ -590,6 +615,11 @@ def main():
         barrier()
         torch.cuda.synchronize()
         with ClockSampler(torch.cuda.current_device()) as clk:
+            def load():
+                for _ in range(100):
+                    sg.sg_apply_H(ctx, xd, yd, nvec)
+                torch.cuda.synchronize()
+            clk.under_load(load)
             times = time_device(ctx, xd, yd, nvec, steps, warm, flush, torch, sg,
                                 sharded_terms=args.sharding == "terms" and world > 1)
         barrier()
@@ -599,31 +629,36 @@ def main():
         if derr:
             raise RuntimeError(f"device error code {derr} in the {prec} apply")
         lv, _ = sg.sg_term_levels(ctx)
-        f_alg = algorithmic_flops_per_vector(lv) * nvec
+        nnz = row_entries(p.D, p.L)
+        f_alg = 2 * nnz * nvec
         ms = total_ms / steps
         units = nvec * steps if args.sharding == "terms" and world > 1 else None
-        if prec == "df64":
-            # double-float: F_alg / 2 multiply-adds of DF_INSTR_PER_FMA FP32
-            # instructions each, against the FP32 issue rate (fma rate / 2)
-            instr = f_alg / 2 * DF_INSTR_PER_FMA
-            peak = peaks["fp32"] / 2 if peaks["fp32"] else None
-            achieved = instr / (statistics.mean(times) * 1e-3) / 1e12
-            roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "T FP32-instructions/s",
-                    "frac": achieved / peak if peak else None, "traffic": TRAFFIC_BYTES[prec],
-                    "flops_per_launch": f_alg, "fp32_instructions_per_launch": instr,
-                    "peak_source": "measured",
-                    "peak_note": "half the measured FP32 fma rate (one instruction per lane per cycle); "
-                                 + str(peaks["note_fp32"])}
+        sec = statistics.mean(times) * 1e-3
+        # what an apply cannot do without: x, y, the elements of H_S with their columns, the harmonic diagonal
+        nbytes = 16 * n * nvec + nnz * (4 + (4 if prec == "mixed" else 8)) + 8 * n
+        hbm = hbm_peak_gbs()
+        roof = {"traffic": TRAFFIC_BYTES[prec], "flops_per_launch": f_alg, "bytes_per_launch": nbytes,
+                "flops_term_by_term": algorithmic_flops_per_vector(lv) * nvec}
+        if prec == "fp64":
+            # the FP64 pipe: one multiply-add per element and vector
+            peak = peaks["fp64"]
+            achieved = f_alg / sec / 1e12
+            roof.update({"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+                         "frac": achieved / peak if peak else None, "peak_source": "measured",
+                         "peak_note": peaks["note_fp64"]})
         else:
-            peak = peaks["fp32"] if prec == "mixed" else peaks["fp64"]
-            achieved = f_alg / (statistics.mean(times) * 1e-3) / 1e12
-            roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                    "frac": achieved / peak if peak else None,
-                    "traffic": TRAFFIC_BYTES[prec],
-                    "flops_per_launch": f_alg,
-                    "peak_source": "measured",
-                    "peak_note": peaks["note_fp32" if prec == "mixed" else "note_fp64"],
-                    "peak_derived": peaks["derived_fp32"] if prec == "mixed" else None}
+            achieved = nbytes / sec / 1e9
+            roof.update({"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
+                         "frac": achieved / hbm if hbm else None, "peak_source": "measured",
+                         "peak_note": "copy bandwidth"})
+            if prec == "df64":
+                # beside it: FP32 instructions of the double-float multiply-adds
+                # against the FP32 issue rate (fma rate / 2)
+                instr = nnz * nvec * DF_INSTR_PER_FMA
+                rate = peaks["fp32"] / 2 if peaks["fp32"] else None
+                roof.update({"fp32_instructions_per_launch": instr,
+                             "issue_frac": instr / sec / 1e12 / rate if rate else None,
+                             "issue_note": "against half the measured FP32 fma rate; " + str(peaks["note_fp32"])})
         results[prec] = {
             "value": (units / (total_ms * 1e-3) if units else replica_throughput(world, nvec * steps, total_ms * 1e-3)),
             "ms_per_step": ms, "steps": steps,

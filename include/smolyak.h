@@ -11,6 +11,14 @@
  * Sec. 3, Table 2), and A_l the term action of Alg. 1: basis->grid (Eq. (15)),
  * the operator on the term's direct-product grid, grid->basis (Eq. (14)).
  *
+ * The library does not visit the terms one by one: over products of one-mode
+ * operators the combination telescopes, mode by mode, into a sparse matrix over
+ * the compact basis (about 15 non-zero elements per row at D=12 L=10 for
+ * Eq. (18)), whose elements are formed on the device once per context (FP64)
+ * and whose rows an apply sums (the row form).  Problems it is not built for
+ * (L > 63, more than 65,536 distinct index shifts, or more than 64 GB of
+ * elements) are applied term by term.
+ *
  * Conventions shared by every call
  *   - Indices are 0-based.  Modes are numbered 0..D-1.
  *   - Compact vectors have N_cs entries in lexicographic order of the
@@ -95,22 +103,22 @@ typedef struct {
  *   L      Smolyak level (L^B = L^G = L, Sec. 2), 0 <= L.
  *   basis  D host structs; grids: D host structs.
  *   H      Hamiltonian; all arrays are host memory, copied (caller keeps ownership).
- *   prec   SG_FP64: every step in FP64.  SG_MIXED: per-term contractions and
- *          the grid multiply in FP32, accumulation of the compact result in
- *          FP64 (exact fixed point).  SG_DF64: the contractions in double-float
- *          arithmetic (each value an unevaluated sum of two FP32 numbers,
- *          about 48 significant bits, on the FP32 pipes), accumulation as for
- *          SG_FP64; FP64-class results (relative error about 1e-14 against
- *          1e-16), for problems on the fast path only (V with monomials of one
- *          mode or of two neighbouring modes of a chain; else
- *          SG_EUNSUPPORTED); not accepted by sg_batch_create or the server.
+ *   prec   SG_FP64: every step in FP64.  SG_MIXED: elements and x in FP32,
+ *          products in FP32, four at a time, their sums carried without
+ *          rounding in a pair of FP32 numbers, the harmonic diagonal in FP64
+ *          (term by term: contractions in FP32, compact result in exact fixed
+ *          point).  SG_DF64: elements, x and sums in double-float arithmetic
+ *          (each value an unevaluated sum of two FP32 numbers, about 48
+ *          significant bits, on the FP32 pipes); FP64-class results (relative
+ *          error below 1e-13), for V with monomials of one mode or of two
+ *          neighbouring modes of a chain only (else SG_EUNSUPPORTED); not
+ *          accepted by sg_batch_create or the server.
  *   out    receives the context (owned by the caller, release with sg_destroy).
  * Setup runs on the host plus synchronous uploads on the current device.
- * The context keeps on the device M^B (4 bytes per term basis function), the
- * per-term records, images and 1D tables, and, on the fast path, the
- * inner-block tables of every term with a grid (4 bytes per value for
- * SG_MIXED, 8 for SG_FP64 and SG_DF64; 6.65 / 13.1 GB at D=12 L=10,
- * nq = l+2).  sg_size reports the total.
+ * The context keeps on the device the row operator (per element a 4-byte
+ * column and a value of 4 bytes for SG_MIXED, 8 for SG_FP64 and SG_DF64, rows
+ * filled up to multiples of four elements; 16 bytes per row beside them), the
+ * term levels and the 1D tables.  sg_size reports the total.
  * Limits of this build (SG_EUNSUPPORTED): nb(L), nq(L) <= 32, N_cs < 2^31,
  * at most 256 monomials with at most 8 factors each, powers <= 16.
  */
@@ -129,9 +137,10 @@ sg_status sg_plan(int D, int L, const sg_basis *basis, const sg_grid *grids,
 
 /* Sizes: n_cs = N_cs (compact basis), n_terms = N_st, n_s = N_s (sum of term
  * basis sizes, Sec. 2, Eq. (11)), n_grid = sum of term grid sizes, bytes_device =
- * device memory held by the context (for a context made by sg_plan: the tables
- * sg_create would allocate for the same problem, without the apply workspace,
- * which grows with the block size).  Any pointer may be NULL. */
+ * device memory held by the context (for a context made by sg_plan: an upper
+ * bound of what sg_create would hold for the same problem, without the apply
+ * workspace, which grows with the block size; it is the bound of a term-by-term
+ * schedule where that is the larger).  Any pointer may be NULL. */
 sg_status sg_size(const sg_ctx *ctx, int64_t *n_cs, int64_t *n_terms, int64_t *n_s,
                   int64_t *n_grid, int64_t *bytes_device);
 
@@ -142,12 +151,15 @@ sg_status sg_size(const sg_ctx *ctx, int64_t *n_cs, int64_t *n_terms, int64_t *n
  *   nvec   >= 1.  A complex vector is passed as two real vectors.
  * Enqueued on `stream`; the result is ready when the stream reaches it.
  * The first call with a larger nvec than before synchronises `stream` and
- * allocates the context's workspace for that many vectors: the fixed-point
- * accumulators (1 word per element for SG_MIXED, 4 otherwise) and, on the
- * fast path, an entry-major copy of x in the contraction type (rows of nvec
- * rounded up to 4 values), which every apply rewrites before its terms
- * gather from it.  Calls on one context must be ordered (one stream, or
- * synchronised streams): they share that workspace.
+ * allocates the context's workspace for that many vectors: an entry-major copy
+ * of x in the value type (rows of nvec rounded up to 4 values), which applies
+ * of more than 65,536 values rewrite before their rows gather from it (SG_FP64
+ * only when sg_tune chose more than one vector per lane)
+ * (term by term: the fixed-point accumulators, 1 word per element for
+ * SG_MIXED, 4 otherwise).  Calls on one context must be ordered (one stream,
+ * or synchronised streams): they share that workspace.
+ * A vector that holds a NaN or an infinity gives NaN in all of y's entries for
+ * that vector, and device error 201.
  */
 sg_status sg_apply_H(sg_ctx *ctx, const double *x, double *y, int nvec, void *stream);
 
@@ -161,14 +173,16 @@ sg_status sg_apply_H_host(sg_ctx *ctx, const double *x_host, double *y_host, int
                           void *stream);
 
 /*
- * Term-sharded apply: the terms of Eq. (16) are independent (the term loop of
- * Alg. 1; the paper's parallel scheme 1, Alg. 2, splits them over MPI ranks
- * and sums the partial results).  Part `part` of `nparts` takes the terms at
- * processing positions p = part (mod nparts) -- the processing order is by
- * decreasing cost, so the parts are balanced -- and adds their contributions
- * exactly into fixed-point accumulators; summing the accumulators of all parts
- * as 64-bit integers (wrapping) and finishing gives bitwise the result of
- * sg_apply_H, whatever nparts.  A multi-GPU apply runs one part per GPU (each
+ * Sharded apply (the paper's parallel scheme 1, Alg. 2, splits the terms over
+ * MPI ranks and sums the partial results).  In the row form part `part` of
+ * `nparts` takes every nparts-th window of rows and adds the bit pattern of
+ * each row's sum (an FP64 number) as an integer into the accumulator of that
+ * row, to which no other part adds; term by term it takes the terms at
+ * processing positions p = part (mod nparts) -- the order is by decreasing
+ * cost -- and adds their contributions exactly in fixed point.  Either way
+ * summing the accumulators of all parts as 64-bit integers (wrapping) and
+ * finishing gives bitwise the result of sg_apply_H, whatever nparts, provided
+ * each part is added once.  A multi-GPU apply runs one part per GPU (each
  * with its own context of the same problem and the same x), one integer
  * all-reduce (sum) of acc, and sg_apply_H_finish.
  *
@@ -180,8 +194,9 @@ sg_status sg_apply_H_host(sg_ctx *ctx, const double *x_host, double *y_host, int
  * sg_apply_H_finish -- y = H_S x from the summed accumulators of all parts
  *   (and the harmonic part applied in the compact basis); clears acc to zero.
  *   x, y as for sg_apply_H (x the same vectors the parts were given).
- * sg_part_size -- the terms of a part and their summed cost estimate (host;
- *   also on contexts made by sg_plan).  Any output may be NULL.
+ * sg_part_size -- the terms at the processing positions of a part and their
+ *   summed cost estimate (host; also on contexts made by sg_plan): the balance
+ *   of the term-by-term split.  Any output may be NULL.
  * Both device calls are enqueued on `stream`.
  */
 sg_status sg_apply_H_part(sg_ctx *ctx, const double *x, int nvec, int part, int nparts, int64_t *acc,
@@ -195,8 +210,9 @@ sg_status sg_part_size(const sg_ctx *ctx, int part, int nparts, int64_t *n_terms
  * apply H (e.g. a process whose device memory is all held by another
  * allocator, or a loop that cannot take the synchronisation a cudaMalloc may
  * bring).  It is not part of the method of the paper, which has no counterpart.
- *   The fixed-point accumulators and per-vector exponents that sg_apply_H
- *   keeps in context-owned device memory come here from one array of
+ *   The workspace that sg_apply_H keeps in context-owned device memory (the
+ *   entry-major copy of x and per-vector flags; term by term the fixed-point
+ *   accumulators and per-vector exponents) comes here from one array of
  *   SG_NOALLOC_SCRATCH_BYTES compiled into the library; every GPU that loads
  *   the library holds it until the process exits.  The call allocates nothing.
  *   Limits: nvec <= SG_NOALLOC_MAX_NVEC and nvec * N_cs <= SG_NOALLOC_MAX_ELEMS
@@ -219,12 +235,10 @@ sg_status sg_apply_H_noalloc(sg_ctx *ctx, const double *x, double *y, int nvec, 
 
 /*
  * Batches: y_j = H_S^(j) x_j for many independent problems j in one apply
- * (Eq. (16) per problem).  The terms of every problem are independent work
- * (Sec. 3: the term loop of Alg. 1 and its parallel schemes), so the terms of
- * all problems that share a kernel variant run in one launch per form (block /
- * warp), ordered by estimated cost over all problems; small problems fill the
- * gaps that large ones leave.  Problems outside the fast path (potentials with
- * monomials over three or more modes) get one launch each.
+ * (Eq. (16) per problem).  The row windows of all problems run in one launch,
+ * the largest first; small problems fill the gaps that large ones leave.
+ * Problems of at least 524,288 basis functions run as launches of their own,
+ * as do those outside the row form.
  *
  * sg_batch_create -- n (1..65535) contexts made by sg_create on the current
  *   device, all of one precision (else SG_EINVAL; SG_DF64 contexts:
@@ -232,13 +246,14 @@ sg_status sg_apply_H_noalloc(sg_ctx *ctx, const double *x, double *y, int nvec, 
  *   device tables: destroy it before any of them.  The contexts' own
  *   workspaces are not used, so sg_apply_H on a member stays valid.
  * sg_batch_size -- total N_cs and terms over the problems; kernel launches
- *   of one sg_apply_H_batch.
+ *   of one sg_apply_H_batch (at most).
  * sg_apply_H_batch -- x, y: DEVICE, problem after problem, problem j's nvec
  *   vectors (each N_cs^(j) doubles, column after column) starting at
  *   nvec * (N_cs^(0) + ... + N_cs^(j-1)).  y is overwritten; x and y must not
  *   overlap.  1 <= nvec <= 65535.  Results are bitwise those of sg_apply_H
- *   on each context.  The batch owns its workspace (fixed-point accumulators,
- *   32 bytes per vector entry), grown on the first call with a larger nvec.
+ *   on each context.  The batch owns its workspace (the entry-major copy of x,
+ *   and the fixed-point accumulators of problems outside the row form), grown
+ *   on the first call with a larger nvec.
  *   Enqueued on `stream`.
  */
 typedef struct sg_batch sg_batch;
@@ -250,30 +265,26 @@ const char *sg_batch_last_error(const sg_batch *b);
 void sg_batch_destroy(sg_batch *b);
 
 /*
- * sg_tune -- measured choice of the term schedule of a context's fast path
- * (no counterpart in the paper, whose scheme balances MPI ranks by timing).
+ * sg_tune -- measured choice of the plan of a context's row form (no
+ * counterpart in the paper, whose scheme balances MPI ranks by timing).
  * Three knobs of the plan are searched one after another, each candidate
  * timed on nvec-vector applies (median of three after one warm-up) on
  * `stream`, the fastest kept:
- *   - the slicing target (1, 2, 4): a term whose grid leaves room for fewer
- *     than that many vectors per chunk is sliced over its leading outer
- *     positions, else it runs unsliced in more, smaller chunks;
- *   - the block/warp split (1, 2, 4): terms that fit a quarter of a block's
- *     shared memory with that many vectors per chunk run one per warp;
- *   - the shared-memory budget of a block, in KB (52, 70, 104 for SG_MIXED;
- *     70, 104 for SG_FP64 and SG_DF64): more vectors per chunk, fewer
- *     resident blocks.
- * Only the term records, the split and the work-area capacities change;
- * results change by rounding only.  Synchronous; allocates and frees
- * 2 * nvec * N_cs doubles of scratch.  No other work may use the context
- * meanwhile.  A batch made from the context before sg_tune refuses to apply
- * (SG_EINVAL) until it is recreated.
- *   nvec 1..64; slice_vt (out, may be NULL): the slicing target kept (0 when
- *   the context uses the generic kernel, which has no schedule to choose);
- *   ms (out, may be NULL): its time per apply.
- * sg_tune_plan -- the plan a context uses now (tuned or default): slicing
- *   target, block/warp split, shared-memory budget in KB (zeros for the
- *   generic kernel).  Any pointer may be NULL.
+ *   - slice_vt (1, 2, 4): vectors per lane of a row sum;
+ *   - warp_vt (1, 2, 4): rows per window, in units of 16;
+ *   - smem_kb: the shared memory that four blocks may share, in KB (52, 70,
+ *     104 for SG_MIXED; 70, 104 for SG_FP64 and SG_DF64): it bounds the
+ *     entries of a window.
+ * (The names are those of an earlier schedule's knobs.)  Only the windows and
+ * the launch shape change, not the order of any sum.  Synchronous; allocates
+ * and frees 2 * nvec * N_cs doubles of scratch.  No other work may use the
+ * context meanwhile.  A batch made from the context before sg_tune refuses to
+ * apply (SG_EINVAL) until it is recreated.
+ *   nvec 1..64; slice_vt (out, may be NULL): the value kept (0 for a context
+ *   without a plan to choose: outside the row form, or with monomials other
+ *   than those SG_DF64 accepts); ms (out, may be NULL): its time per apply.
+ * sg_tune_plan -- the plan a context uses now (tuned or default; zeros for a
+ *   context without one).  Any pointer may be NULL.
  */
 sg_status sg_tune(sg_ctx *ctx, int nvec, int *slice_vt, double *ms, void *stream);
 sg_status sg_tune_plan(const sg_ctx *ctx, int *slice_vt, int *warp_vt, int *smem_kb);
@@ -295,16 +306,16 @@ sg_status sg_tune_plan(const sg_ctx *ctx, int *slice_vt, int *warp_vt, int *smem
  *
  * Each engine iteration retires finished requests, admits queued requests
  * first come first served while their planned device memory fits the budget,
- * then applies H_S to every active request's current Chebyshev vector in one
- * sg_apply_H_batch and advances every recurrence by one term in one fused
- * kernel.  Requests that arrive while others run join at the next iteration.
+ * then applies H_S to every active request's current Chebyshev vector and
+ * advances every recurrence by one term, in one launch over all requests' rows
+ * (a batched apply and an update while eigen requests are active).  Requests that arrive while others run join at the next iteration.
  * A request's results are bitwise the same alone and in any mix (its applies,
  * updates and logged sums do not depend on the other requests).
  *
  * sg_server_create -- precision of every request's contexts (SG_FP64 or
  *   SG_MIXED; else SG_EINVAL); hbm_budget_bytes:
  *   the planned device memory of the active requests never exceeds it
- *   (context tables, M^B, batch items, four state vectors, batch and context
+ *   (the bound sg_size gives for a plan, batch items, state vectors, batch and context
  *   workspaces, logs).  Transient set-up buffers of an admission (the
  *   spectral-bound Krylov run, about 80 vectors) are not counted.
  * sg_server_submit -- copies the request (the caller's arrays may be freed on
@@ -315,7 +326,7 @@ sg_status sg_tune_plan(const sg_ctx *ctx, int *slice_vt, int *warp_vt, int *smem
  *   product state of `factors` (as sg_product_state, leading dimension ld).
  *   Logs: <psi|psi> and <psi|H psi>/<psi|psi> at the start of each step.
  * sg_server_submit_eigs -- copies and plans an eigen request and queues it;
- *   SG_EBUDGET if it alone needs more than the budget (context tables, M^B,
+ *   SG_EBUDGET if it alone needs more than the budget (its plan's bound,
  *   its batch slots, the Davidson basis of max(3 nev, nev + 6 block) vectors
  *   and its images, Ritz vectors, eigenvectors).
  * sg_server_progress -- runs up to max_iters engine iterations (fewer if
@@ -436,7 +447,11 @@ sg_status sg_device_error(sg_ctx *ctx, int *code);
  *   method  SG_DAVIDSON: block Davidson, diagonal preconditioner
  *           (E_k - theta)^-1 with E_k the harmonic energies of the split modes
  *           (none when no mode is split), restart at max(3 nev, nev + 6 block)
- *           vectors.  SG_LANCZOS: block Krylov with full reorthogonalisation and
+ *           vectors.  It starts from the unit vectors of the lowest harmonic
+ *           energies and one random vector, and carries `block` Ritz pairs
+ *           beyond nev; after convergence it makes one more expansion, by the
+ *           residuals of the pairs beyond nev, so that no state is missed that
+ *           the start block does not couple to.  SG_LANCZOS: block Krylov with full reorthogonalisation and
  *           Rayleigh-Ritz, at most 320 basis vectors; a block of size >= the
  *           largest multiplicity resolves degenerate eigenvalues.
  *   block   1..8 vectors per operator application (<= 0: min(nev, 8)).
@@ -446,7 +461,8 @@ sg_status sg_device_error(sg_ctx *ctx, int *code);
  *   evecs   DEVICE, nev * N_cs (out; may be NULL).
  * Synchronous.  SG_ENOCONV when fewer than nev pairs converged (evals, resid and
  * evecs then hold the current approximations).  Allocates its workspace
- * (device memory of about 2 * max(3 nev, nev + 6 block) vectors for Davidson).
+ * (device memory of about 2 * max(3 nev, nev + 6 block) + 3 (nev + block)
+ * vectors for Davidson).
  * With a SG_MIXED context the applications are FP32-accurate; use
  * sg_eigs_refine with a SG_FP64 context of the same problem to refine.
  */
@@ -489,7 +505,7 @@ sg_status sg_product_state(const sg_ctx *ctx, const double *factors, int ld, dou
 /*
  * sg_measure_peak -- measured arithmetic throughput of the current device (no
  * counterpart in the paper; it supplies the denominators of the roofline
- * fractions of the operator action, which is bound by CUDA-core arithmetic).
+ * fractions of the operator action's FP64 form).
  * Every SM runs 32 warps of register-resident multiply-add chains for about
  * `seconds` (0 < seconds <= 60); the result counts 2 flops per multiply-add.
  *   kind        SG_PEAK_FP32: scalar FP32 fma; SG_PEAK_FP32X2: the packed

@@ -272,7 +272,7 @@ def sg_apply_H_noalloc(ctx: Ctx, x, y, nvec: int = None, stream=None) -> None:
 
 
 def acc_words(ctx: Ctx, nvec: int) -> int:
-    """int64 words of the fixed-point accumulators of nvec vectors (sg_apply_H_part)."""
+    """int64 words of the accumulators of nvec vectors (sg_apply_H_part)."""
     return ctx.n_cs * nvec * (1 if ctx.precision == SG_MIXED else 4)
 
 
@@ -413,16 +413,16 @@ def sg_propagate(ctx: Ctx, psi, dt: float, nsteps: int, order: int = 64, stream=
 
 
 def sg_tune(ctx: Ctx, nvec: int = 8, stream=None):
-    """Measured choice of the fast path's plan (slicing target, block/warp
-    split, shared-memory budget per block) for nvec-vector applies; returns
-    (slicing target kept, ms per apply).  sg_tune_plan reports the whole plan."""
+    """Measured choice of the row kernels' plan (vectors per lane, rows per
+    window, shared-memory budget) for nvec-vector applies; returns
+    (vectors per lane kept, ms per apply).  sg_tune_plan reports the whole plan."""
     vt, ms = ctypes.c_int(), ctypes.c_double()
     _check(lib().sg_tune(ctx.ptr, int(nvec), ctypes.byref(vt), ctypes.byref(ms), _stream_ptr(stream)), ctx)
     return vt.value, ms.value
 
 
 def sg_tune_plan(ctx: Ctx) -> dict:
-    """The plan the context uses now: slicing target, block/warp split, KB per block."""
+    """The plan the context uses now: vectors per lane, rows per window / 16, KB that four blocks may share."""
     a, b, c = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
     _check(lib().sg_tune_plan(ctx.ptr, ctypes.byref(a), ctypes.byref(b), ctypes.byref(c)), ctx)
     return {"slice_vt": a.value, "warp_vt": b.value, "smem_kb": c.value}

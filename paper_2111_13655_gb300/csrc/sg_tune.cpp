@@ -5,7 +5,8 @@
 // over its candidates with the others at their best so far), every candidate
 // timed on real applies of the caller's block size:
 //   1. vectors per lane (1, 2, 4): wider loads of the input copy and fewer
-//      lanes per row, against more rows in flight;
+//      lanes per row, against more rows in flight (FP64 with one vector per
+//      lane makes no copy: rows_direct);
 //   2. rows per window, in units of 16 (1, 2, 4): how many rows a block takes;
 //   3. the shared memory that SG_ROW_SHARE resident blocks may use: a window
 //      ends early where its entries would exceed its part.

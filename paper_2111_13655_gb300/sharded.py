@@ -1,8 +1,9 @@
 """Term-sharded H_S x over the ranks of a torch.distributed group (one GPU each).
 
 Every rank holds a context of the same problem and the same input vectors.
-Rank r adds the terms at processing positions p = r (mod world) into int64
-fixed-point accumulators (sg_apply_H_part); one all-reduce (sum) of the
+Rank r adds its part of the sum into int64 accumulators (sg_apply_H_part: the
+rows of every world-th window, or the terms at positions p = r (mod world) of a
+problem applied term by term); one all-reduce (sum) of the
 accumulators -- the paper's MPI sum of partial results (Alg. 2) -- and
 sg_apply_H_finish give every rank y, bitwise the single-GPU sg_apply_H
 whatever the number of ranks (integer sums are associative).  Integer sums
