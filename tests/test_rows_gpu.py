@@ -204,3 +204,30 @@ def test_solvers_with_products_in_one_and_in_several_chunks(D, L):
         c, s = np.cos(0.5 * ev[0]), np.sin(0.5 * ev[0])
         want = torch.cat([c * v[0], -s * v[0]])
         assert float((psi - want).abs().max()) <= 1e-8    # residual 1e-9 times the time, and rounding
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed", "df64"])
+@pytest.mark.parametrize("name", list(SIZES))
+def test_captured_applies_replay_bitwise(name, prec):
+    """The launches wait for one another on the device; in a caller's graph, with a kernel of the caller's before and
+    after each apply, they keep that order (x is overwritten in between)."""
+    p, nvec = SIZES[name], 5
+    with sg.sg_create(p, prec) as ctx:
+        x0 = torch.from_numpy(synth.random_vectors(ctx.n_cs, nvec, 12)).cuda()
+        want1 = apply(ctx, x0)
+        want2 = apply(ctx, want1 * 0.125)
+        x, y = torch.zeros_like(x0), torch.zeros_like(x0)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            s = torch.cuda.current_stream()
+            sg.sg_apply_H(ctx, x, y, nvec, stream=s)
+            first = y.clone()
+            x.copy_(y * 0.125)
+            sg.sg_apply_H(ctx, x, y, nvec, stream=s)
+        for _ in range(3):
+            x.copy_(x0)
+            g.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(first, want1) and torch.equal(y, want2)
+        assert sg.sg_device_error(ctx) == 0
