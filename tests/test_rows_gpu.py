@@ -183,8 +183,8 @@ def test_constant_basis_sizes_inside_and_outside_the_row_form(D, L, prec):
         assert elem_rel(y.cpu().numpy(), r) <= (FP64_TOL if prec == "fp64" else 5e-6)
 
 
-# N_cs 8,008 and 27,132: one and two chunks per inner product
-@pytest.mark.parametrize("D,L", [(6, 10), (6, 13)])
+# N_cs 8,008, 27,132 and 74,613: one, two and five chunks per inner product; grouped and plain column sums
+@pytest.mark.parametrize("D,L", [(6, 10), (6, 13), (6, 16)])
 def test_solvers_with_products_in_one_and_in_several_chunks(D, L):
     p = synth.chained_henon_heiles(D, L, synth.draw_omega(D, 6), 0.1)
     nev, tol = 5, 1e-9
