@@ -277,9 +277,13 @@ void sg_batch_destroy(sg_batch *b);
  *     entries of a window.
  * (The names are those of an earlier schedule's knobs.)  Only the windows and
  * the launch shape change, not the order of any sum.  Synchronous; allocates
- * and frees 2 * nvec * N_cs doubles of scratch.  No other work may use the
- * context meanwhile.  A batch made from the context before sg_tune refuses to
- * apply (SG_EINVAL) until it is recreated.
+ * and frees 2 * nvec * N_cs doubles of scratch, and forms each candidate's row
+ * operator beside the one in force: a candidate for which there is no memory is
+ * not taken, and SG_ENOMEM (the fastest plan no longer fits) leaves the plan
+ * that sg_tune_plan then reports.  No other work may use the context meanwhile.
+ * A batch made from the context before sg_tune refuses to apply (SG_EINVAL)
+ * until it is recreated; a caller's graph with applies captured before sg_tune
+ * names the released operator and has to be captured again.
  *   nvec 1..64; slice_vt (out, may be NULL): the value kept (0 for a context
  *   without a plan to choose: outside the row form, or with monomials other
  *   than those SG_DF64 accepts); ms (out, may be NULL): its time per apply.

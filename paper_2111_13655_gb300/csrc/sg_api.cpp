@@ -208,6 +208,7 @@ constexpr int kTicketBlocks = 1024;
 
 cudaError_t apply_rows(sg_ctx *ctx, RowIO io, cudaStream_t s)
 {
+    if (ctx->rop.nwin <= 0) return cudaErrorInvalidValue;  // nothing would write y
     const sg_precision prec = ctx->prob.prec;
     cudaError_t e = cudaSuccess;
     const int vt = row_vt(ctx->host, prec);
@@ -228,9 +229,9 @@ void free_rows(sg_ctx *ctx)
     ctx->rop = RowOp{};
 }
 
+// The earlier operator is released once the new one is complete: a failure leaves it in force.
 cudaError_t build_rows(sg_ctx *ctx)
 {
-    free_rows(ctx);
     const HostTables &T = ctx->host;
     const KParams &kp = ctx->kp;
     const sg_precision prec = ctx->prob.prec;
@@ -262,7 +263,6 @@ cudaError_t build_rows(sg_ctx *ctx)
         C.add(W.wins);
         e = B.put(&plan);
         if (e == cudaSuccess) e = C.put(&own, (size_t)W.bytes, &rec);
-        if (own) ctx->row_allocs.push_back(own);
         RowOp R{};
         if (e == cudaSuccess) {
             R.wins = reinterpret_cast<const RowWin *>(own);
@@ -278,16 +278,21 @@ cudaError_t build_rows(sg_ctx *ctx)
         R.n = (int)n;
         R.cap = W.cap;
         R.wrows = W.wrows;
-        ctx->rop = R;
-        ctx->win_entries.resize(W.wins.size());
-        for (size_t w = 0; w < W.wins.size(); w++) ctx->win_entries[w] = W.wins[w].nent;
-        ctx->row_bytes = (int64_t)(rec + W.bytes);
-        ctx->bytes_device += ctx->row_bytes;
+        if (e == cudaSuccess) {
+            ctx->plan_version++;  // before anything that a batch may still point to is released
+            free_rows(ctx);
+            ctx->row_allocs.push_back(own);
+            ctx->rop = R;
+            ctx->win_entries.resize(W.wins.size());
+            for (size_t w = 0; w < W.wins.size(); w++) ctx->win_entries[w] = W.wins[w].nent;
+            ctx->row_bytes = (int64_t)(rec + W.bytes);
+            ctx->bytes_device += ctx->row_bytes;
+        }
     }
     if (set) cudaFree(set);
     if (plan) cudaFree(plan);
     if (e != cudaSuccess) {
-        free_rows(ctx);
+        if (own) cudaFree(own);
         (void)cudaGetLastError();  // reported here; not by a later launch
     }
     return e;

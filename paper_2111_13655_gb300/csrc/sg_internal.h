@@ -373,7 +373,7 @@ struct sg_ctx {
     int acc_nvec = 0;
     double *pin = nullptr;    // pinned host memory of the solvers' small matrices
     size_t pin_doubles = 0;
-    int plan_version = 0;     // incremented whenever sg_tune installs a plan
+    int plan_version = 0;     // incremented whenever a plan or a row operator is installed
     std::string last_error;
 };
 
@@ -388,7 +388,8 @@ inline bool sg_on_ctx_device(const sg_ctx *ctx)
 namespace sg {
 
 // Row operator of a context (sg_api.cpp): forms it with the context's plan
-// (replacing an earlier one), releases it, and enqueues one apply or part.
+// (then replacing an earlier one, which a failure leaves in force), releases
+// it, and enqueues one apply or part.
 cudaError_t build_rows(sg_ctx *ctx);
 void free_rows(sg_ctx *ctx);
 cudaError_t apply_rows(sg_ctx *ctx, RowIO io, cudaStream_t s);

@@ -34,15 +34,26 @@ struct Tuner {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t err = cudaSuccess;
 
-    // Cuts the row operator into the windows of p.  False on a CUDA error.
+    // Cuts the row operator into the windows of p.  False when that fails: the
+    // operator in force, and the plan that it was cut by, stay.  The new operator
+    // is formed beside the old one; without the memory for both, p is not taken
+    // (no error of the tuner's: err stays clear).
     bool install(const Plan &p)
     {
         sg::HostTables &T = ctx->host;
+        const int vt = T.slice_vt, units = T.warp_vt, budget = T.fbudget;
+        const bool same = sg::row_window_units(T) == p.warp_vt && sg::row_budget(T, ctx->prob.prec) == p.smem_kb * 1024;
         T.slice_vt = p.slice_vt;
-        const bool same = ctx->rop.nwin > 0 && T.warp_vt == p.warp_vt && T.fbudget == p.smem_kb * 1024;
         T.warp_vt = p.warp_vt;
         T.fbudget = p.smem_kb * 1024;
-        if (!same && (err = sg::build_rows(ctx)) != cudaSuccess) return false;
+        const cudaError_t e = same ? cudaSuccess : sg::build_rows(ctx);
+        if (e != cudaSuccess) {
+            T.slice_vt = vt;
+            T.warp_vt = units;
+            T.fbudget = budget;
+            if (e != cudaErrorMemoryAllocation) err = e;
+            return false;
+        }
         ctx->plan_version++;
         return true;
     }
@@ -125,8 +136,9 @@ extern "C" sg_status sg_tune(sg_ctx *ctx, int nvec, int *slice_vt, double *ms_ou
     const cudaError_t keep_err = tu.err;
     tu.err = cudaSuccess;
     if (!tu.install(ok ? best : original) && st == SG_OK) {
-        st = tu.err != cudaSuccess ? SG_ECUDA : SG_EINVAL;
-        if (st == SG_EINVAL) ctx->last_error = "sg_tune: the kept plan could not be installed";
+        st = tu.err != cudaSuccess ? SG_ECUDA : SG_ENOMEM;
+        if (st == SG_ENOMEM)
+            ctx->last_error = "sg_tune: no memory to install the fastest plan; the plan in force (sg_tune_plan) stays";
     }
     if (tu.e0) cudaEventDestroy(tu.e0);
     if (tu.e1) cudaEventDestroy(tu.e1);
