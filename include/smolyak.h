@@ -17,7 +17,9 @@
  * Eq. (18)), whose elements are formed on the device once per context (FP64)
  * and whose rows an apply sums (the row form).  Problems it is not built for
  * (L > 63, more than 65,536 distinct index shifts, or more than 64 GB of
- * elements) are applied term by term.
+ * elements), and those whose elements the device has no memory for when the
+ * context is made (not SG_DF64: SG_ENOMEM), are applied term by term: the same
+ * sum, its rounding apart, in a small part of the memory.
  *
  * Conventions shared by every call
  *   - Indices are 0-based.  Modes are numbered 0..D-1.

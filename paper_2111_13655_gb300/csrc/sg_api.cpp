@@ -31,7 +31,10 @@ sg_status upload(sg_ctx *ctx, const std::vector<T> &v, const T **dst)
     void *p = nullptr;
     size_t bytes = std::max<size_t>(1, v.size()) * sizeof(T);
     cudaError_t e = cudaMalloc(&p, bytes);
-    if (e != cudaSuccess) return fail(ctx, SG_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();  // reported here; not by a later launch
+        return fail(ctx, SG_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    }
     ctx->allocations.push_back(p);
     ctx->bytes_device += (int64_t)bytes;
     if (!v.empty()) {
@@ -54,17 +57,80 @@ void free_workspace(sg_ctx *ctx)
     ctx->acc_nvec = 0;
 }
 
-void free_all(sg_ctx *ctx)
+void free_tables(sg_ctx *ctx)
 {
     for (void *p : ctx->allocations) cudaFree(p);
     ctx->allocations.clear();
     sg::free_rows(ctx);
+    ctx->bytes_device = 0;
+}
+
+void free_all(sg_ctx *ctx)
+{
+    free_tables(ctx);
     if (ctx->stage_x) cudaFree(ctx->stage_x);
     if (ctx->stage_y) cudaFree(ctx->stage_y);
     ctx->stage_x = ctx->stage_y = nullptr;
     if (ctx->pin) cudaFreeHost(ctx->pin);
     ctx->pin = nullptr;
     free_workspace(ctx);
+}
+
+// What the row form's set-up kernels and the index map read, and the harmonic energies.
+cudaError_t upload_row_tables(sg_ctx *ctx)
+{
+    const sg::HostTables &T = ctx->host;
+    sg::KParams &kp = ctx->kp;
+    sg::Arena A;
+    const int zero = 0;
+    const size_t rank = A.add(T.rank_tab), lmin = A.add(T.lmin_tab), lvl = A.add(T.lvl), tab = A.add(T.tabd),
+                 es = A.add(T.esplit), err = A.add(&zero, 1);
+    unsigned char *base = nullptr;
+    const cudaError_t e = A.put(&base);
+    if (base) ctx->allocations.push_back(base);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();  // reported here; not by a later launch
+        return e;
+    }
+    ctx->bytes_device += (int64_t)A.host.size();
+    kp.rank_tab = reinterpret_cast<const int *>(base + rank);
+    kp.lmin_tab = base + lmin;
+    kp.lvl = reinterpret_cast<const sg::LevelInfo *>(base + lvl);
+    kp.tabd = reinterpret_cast<const double *>(base + tab);
+    kp.esplit = reinterpret_cast<const double *>(base + es);
+    kp.err = reinterpret_cast<int *>(base + err);
+    return cudaSuccess;
+}
+
+// The tables of the term-by-term kernel.
+sg_status upload_term_tables(sg_ctx *ctx)
+{
+    const sg::HostTables &T = ctx->host;
+    const sg::Problem &p = ctx->prob;
+    sg::KParams &kp = ctx->kp;
+    const std::vector<float> tabf(T.tabd.begin(), T.tabd.end());
+    const std::vector<int> zero(1, 0);
+    const int *errp = nullptr;
+    sg_status st;
+    if ((st = upload(ctx, T.levels, &kp.levels)) != SG_OK ||
+        (st = upload(ctx, T.coefs, &kp.coefs)) != SG_OK ||
+        (st = upload(ctx, T.order, &kp.order)) != SG_OK ||
+        (st = upload(ctx, T.rank_tab, &kp.rank_tab)) != SG_OK ||
+        (st = upload(ctx, T.lmin_tab, &kp.lmin_tab)) != SG_OK ||
+        (st = upload(ctx, T.lvl, &kp.lvl)) != SG_OK ||
+        (st = upload(ctx, T.tabd, &kp.tabd)) != SG_OK ||
+        (st = upload(ctx, tabf, &kp.tabf)) != SG_OK ||
+        (st = upload(ctx, p.mcoef, &kp.mcoef)) != SG_OK ||
+        (st = upload(ctx, p.mnfac, &kp.mnfac)) != SG_OK ||
+        (st = upload(ctx, p.mfoff, &kp.mfoff)) != SG_OK ||
+        (st = upload(ctx, p.mfmode, &kp.mfmode)) != SG_OK ||
+        (st = upload(ctx, p.mfpow, &kp.mfpow)) != SG_OK ||
+        (st = upload(ctx, T.harm_mono, &kp.harm_mono)) != SG_OK ||
+        (st = upload(ctx, T.esplit, &kp.esplit)) != SG_OK ||
+        (st = upload(ctx, zero, &errp)) != SG_OK)
+        return st;
+    kp.err = const_cast<int *>(errp);
+    return SG_OK;
 }
 
 // Apply workspace for nvec vectors.  Row form: per-vector flags (zero between
@@ -334,86 +400,39 @@ sg_status sg_create(int D, int L, const sg_basis *basis, const sg_grid *grids,
     sg_status st0 = plan(D, L, basis, grids, H, prec, smem_optin, &ctx);
     if (st0 != SG_OK) return st0;
     ctx->device = device;
-    Problem &p = ctx->prob;
-    HostTables &T = ctx->host;
-    KParams &kp = ctx->kp;
-    sg_status st = SG_OK;
-    if (T.rows) {
-        // what the row form's set-up kernels and the index map read, and the harmonic energies
-        sg::Arena A;
-        const int zero = 0;
-        const size_t rank = A.add(T.rank_tab), lmin = A.add(T.lmin_tab), lvl = A.add(T.lvl), tab = A.add(T.tabd),
-                     es = A.add(T.esplit), err = A.add(&zero, 1);
-        unsigned char *base = nullptr;
-        e = A.put(&base);
-        if (base) ctx->allocations.push_back(base);
-        if (e != cudaSuccess) {
-            st = fail(nullptr, e == cudaErrorMemoryAllocation ? SG_ENOMEM : SG_ECUDA,
-                      std::string("cudaMalloc: ") + cudaGetErrorString(e));
-            free_all(ctx);
-            delete ctx;
-            return st;
-        }
-        ctx->bytes_device += (int64_t)A.host.size();
-        kp.rank_tab = reinterpret_cast<const int *>(base + rank);
-        kp.lmin_tab = base + lmin;
-        kp.lvl = reinterpret_cast<const LevelInfo *>(base + lvl);
-        kp.tabd = reinterpret_cast<const double *>(base + tab);
-        kp.esplit = reinterpret_cast<const double *>(base + es);
-        kp.err = reinterpret_cast<int *>(base + err);
-    } else {
-        const std::vector<float> tabf(T.tabd.begin(), T.tabd.end());
-        const std::vector<int> zero(1, 0);
-        const int *errp = nullptr;
-        if ((st = upload(ctx, T.levels, &kp.levels)) != SG_OK ||
-            (st = upload(ctx, T.coefs, &kp.coefs)) != SG_OK ||
-            (st = upload(ctx, T.order, &kp.order)) != SG_OK ||
-            (st = upload(ctx, T.rank_tab, &kp.rank_tab)) != SG_OK ||
-            (st = upload(ctx, T.lmin_tab, &kp.lmin_tab)) != SG_OK ||
-            (st = upload(ctx, T.lvl, &kp.lvl)) != SG_OK ||
-            (st = upload(ctx, T.tabd, &kp.tabd)) != SG_OK ||
-            (st = upload(ctx, tabf, &kp.tabf)) != SG_OK ||
-            (st = upload(ctx, p.mcoef, &kp.mcoef)) != SG_OK ||
-            (st = upload(ctx, p.mnfac, &kp.mnfac)) != SG_OK ||
-            (st = upload(ctx, p.mfoff, &kp.mfoff)) != SG_OK ||
-            (st = upload(ctx, p.mfmode, &kp.mfmode)) != SG_OK ||
-            (st = upload(ctx, p.mfpow, &kp.mfpow)) != SG_OK ||
-            (st = upload(ctx, T.harm_mono, &kp.harm_mono)) != SG_OK ||
-            (st = upload(ctx, T.esplit, &kp.esplit)) != SG_OK ||
-            (st = upload(ctx, zero, &errp)) != SG_OK) {
-            g_create_error = ctx->last_error;
-            free_all(ctx);
-            delete ctx;
-            return st;
-        }
-        kp.err = const_cast<int *>(errp);
-    }
+    auto give_up = [&](sg_status st) {
+        free_all(ctx);
+        delete ctx;
+        return st;
+    };
     ctx->has_device = true;
-    if (p.prec == SG_DF64 && (!T.rows || !term_form(p, T).fits)) {
-        st = fail(nullptr, SG_EUNSUPPORTED,
-                  "SG_DF64 needs the pair form (a potential with one- and two-mode monomials of a chain)");
-        free_all(ctx);
-        delete ctx;
-        return st;
-    }
+    HostTables &T = ctx->host;
+    if (prec == SG_DF64 && (!T.rows || !term_form(ctx->prob, T).fits))
+        return give_up(fail(nullptr, SG_EUNSUPPORTED,
+                            "SG_DF64 needs the pair form (a potential with one- and two-mode monomials of a chain)"));
     if (T.rows) {
-        e = build_rows(ctx);
-        if (e == cudaErrorMemoryAllocation) {
-            st = fail(nullptr, SG_ENOMEM, std::string("cudaMalloc (row operator): ") + cudaGetErrorString(e));
-            free_all(ctx);
-            delete ctx;
-            return st;
-        }
+        e = upload_row_tables(ctx);
+        if (e == cudaSuccess) e = build_rows(ctx);
         if (e == cudaSuccess) e = configure_rows();
-    } else {
-        ctx->smem_bytes = apply_smem_bytes(kp, ctx->fp32);
-        e = configure_kernels(ctx->smem_bytes, ctx->fp32);
+        if (e == cudaErrorMemoryAllocation && prec == SG_DF64)
+            return give_up(fail(nullptr, SG_ENOMEM, std::string("cudaMalloc (row operator): ") + cudaGetErrorString(e)));
+        if (e == cudaErrorMemoryAllocation) {
+            // no room for the rows: term by term, whose tables are a small part of them
+            T.rows = false;
+            free_tables(ctx);
+        } else if (e != cudaSuccess) {
+            return give_up(cuda_fail(nullptr, e, "context set-up"));
+        }
     }
-    if (e != cudaSuccess) {
-        st = cuda_fail(nullptr, e, "context set-up");
-        free_all(ctx);
-        delete ctx;
-        return st;
+    if (!T.rows) {
+        const sg_status st = upload_term_tables(ctx);
+        if (st != SG_OK) {
+            g_create_error = ctx->last_error;
+            return give_up(st);
+        }
+        ctx->smem_bytes = apply_smem_bytes(ctx->kp, ctx->fp32);
+        e = configure_kernels(ctx->smem_bytes, ctx->fp32);
+        if (e != cudaSuccess) return give_up(cuda_fail(nullptr, e, "context set-up"));
     }
     *out = ctx;
     return SG_OK;

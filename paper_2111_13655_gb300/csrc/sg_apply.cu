@@ -1,6 +1,6 @@
 // Term-by-term Smolyak operator action on the GPU (sm_103a), for the problems
-// whose row form (sg_rows.cu) is not built: levels above kRowMaxL, or more
-// index shifts or entries than it holds.
+// whose row form (sg_rows.cu) is not built: levels above kRowMaxL, more index
+// shifts or entries than it holds, or no device memory for its elements.
 //
 // One thread block per Smolyak term (terms ordered most-expensive first).  For
 // term l the block performs Alg. 1 of arXiv 2111.13655:
