@@ -112,9 +112,9 @@ typedef struct {
  *          point).  SG_DF64: elements, x and sums in double-float arithmetic
  *          (each value an unevaluated sum of two FP32 numbers, about 48
  *          significant bits, on the FP32 pipes); FP64-class results (relative
- *          error below 1e-13), for V with monomials of one mode or of two
- *          neighbouring modes of a chain only (else SG_EUNSUPPORTED); not
- *          accepted by sg_batch_create or the server.
+ *          error below 1e-13), for V with monomials of one or two modes, in
+ *          at most 64 pairs of modes, in the row form only (else
+ *          SG_EUNSUPPORTED); not accepted by sg_batch_create or the server.
  *   out    receives the context (owned by the caller, release with sg_destroy).
  * Setup runs on the host plus synchronous uploads on the current device.
  * The context keeps on the device the row operator (per element a 4-byte
@@ -139,10 +139,11 @@ sg_status sg_plan(int D, int L, const sg_basis *basis, const sg_grid *grids,
 
 /* Sizes: n_cs = N_cs (compact basis), n_terms = N_st, n_s = N_s (sum of term
  * basis sizes, Sec. 2, Eq. (11)), n_grid = sum of term grid sizes, bytes_device =
- * device memory held by the context (for a context made by sg_plan: an upper
- * bound of what sg_create would hold for the same problem, without the apply
- * workspace, which grows with the block size; it is the bound of a term-by-term
- * schedule where that is the larger).  Any pointer may be NULL. */
+ * device memory held by the context (for a context made by sg_plan: what
+ * sg_create would hold for the same problem, from above and within some 20%:
+ * rows are filled up to multiples of four elements, which a plan counts at its
+ * most; without the apply workspace, which grows with the block size).  Any
+ * pointer may be NULL. */
 sg_status sg_size(const sg_ctx *ctx, int64_t *n_cs, int64_t *n_terms, int64_t *n_s,
                   int64_t *n_grid, int64_t *bytes_device);
 

@@ -368,11 +368,15 @@ int64_t planned_device_bytes(const sg_ctx *ctx)
 {
     const HostTables &T = ctx->host;
     const Problem &p = ctx->prob;
-    auto b = [](const auto &v) { return (int64_t)v.size() * (int64_t)sizeof(v[0]); };
-    int64_t bytes = b(T.levels) + b(T.coefs) + b(T.order) + b(T.rank_tab) + b(T.lmin_tab) + b(T.lvl) +
-                    b(T.tabd) * 3 / 2 + b(p.mcoef) + b(p.mnfac) + b(p.mfoff) + b(p.mfmode) + b(p.mfpow) +
-                    b(T.harm_mono) + b(T.esplit);
-    return bytes + std::max(term_form(p, T).bytes, row_form_bytes(T, p.prec));
+    auto b = [](const auto &v) { return std::max<int64_t>(1, (int64_t)v.size()) * (int64_t)sizeof(v[0]); };
+    const int64_t terms = b(T.levels) + b(T.coefs) + b(T.order) + b(T.rank_tab) + b(T.lmin_tab) + b(T.lvl) +
+                          b(T.tabd) * 3 / 2 + b(p.mcoef) + b(p.mnfac) + b(p.mfoff) + b(p.mfmode) + b(p.mfpow) +
+                          b(T.harm_mono) + b(T.esplit) + (int64_t)sizeof(int);
+    if (!T.rows) return terms;
+    // every table in the arenas of upload_row_tables and build_rows starts at a multiple of 256 bytes
+    const int64_t rows = b(T.rank_tab) + b(T.lmin_tab) + b(T.lvl) + b(T.tabd) + b(T.esplit) + (int64_t)sizeof(int) +
+                         7 * 256 + row_form_bytes(T, p.prec);
+    return std::max(terms, rows);
 }
 
 }  // namespace sg
@@ -407,9 +411,9 @@ sg_status sg_create(int D, int L, const sg_basis *basis, const sg_grid *grids,
     };
     ctx->has_device = true;
     HostTables &T = ctx->host;
-    if (prec == SG_DF64 && (!T.rows || !term_form(ctx->prob, T).fits))
+    if (prec == SG_DF64 && (!T.rows || !T.pairs))
         return give_up(fail(nullptr, SG_EUNSUPPORTED,
-                            "SG_DF64 needs the pair form (a potential with one- and two-mode monomials of a chain)"));
+                            "SG_DF64 needs the row form of a potential with monomials of one and two modes (at most 64 pairs)"));
     if (T.rows) {
         e = upload_row_tables(ctx);
         if (e == cudaSuccess) e = build_rows(ctx);

@@ -40,7 +40,7 @@ constexpr int kAcc32LsbBelowMax = 40;
 // 64-bit words per accumulated entry of a context's precision
 __host__ __device__ constexpr int acc_words(bool fp32) { return fp32 ? 1 : kAccDigits; }
 
-constexpr int kMaxPairs = 64;  // coupled mode pairs of the pair form (below)
+constexpr int kMaxPairs = 64;  // coupled mode pairs of a pair potential
 
 // ---------------------------------------------------------------------------
 // The row form of H_S (sg_rows.cu, sg_rows_setup.cpp).  With U_i(l) the
@@ -206,10 +206,7 @@ struct HostTables {
     std::vector<double> tabd;
     std::vector<int> harm_mono;      // [D]
     std::vector<double> esplit;      // [n_cs]
-    // pair form: every monomial touches at most two modes, in at most kMaxPairs pairs
-    bool fast = false;
-    int nb1 = 0, nq1 = 0;            // uniform sizes of level 1 (0 if modes differ)
-    std::vector<int> pair_modes;     // [npairs][2]
+    bool pairs = false;  // every monomial touches at most two modes, in at most kMaxPairs pairs
     // row form (see RowShifts); rows = false: the term-by-term kernel applies H_S
     bool rows = false;
     int64_t row_nnz = 0;             // entries of the row operator
@@ -241,13 +238,6 @@ cudaError_t launch_apply_terms(const KParams &kp, bool fp32, const double *x, co
                                cudaStream_t stream);
 cudaError_t launch_finalize(const KParams &kp, bool fp32, const double *x, double *y, int nvec,
                             const long long *maxbits, cudaStream_t stream);
-
-// Size of the problem in its term-by-term form (sg_setup.cpp).
-struct TermForm {
-    bool fits;      // every term fits the shared memory of its form
-    int64_t bytes;  // M^B, inner-block tables, records, images
-};
-TermForm term_form(const Problem &p, const HostTables &T);
 
 // Row form, host half (sg_rows_setup.cpp).
 void build_row_shifts(const Problem &p, HostTables *T);
@@ -342,7 +332,9 @@ sg_status davidson_routed(sg_ctx *ctx, cudaStream_t stream, const ApplyFn &apply
                           int max_it, double *evals, double *resid, double *evecs, int *nconv, std::string *err);
 // J_0..J_kmax at x (Miller's backward recurrence).
 std::vector<double> bessel_j(int kmax, double x);
-// Device bytes sg_create would allocate for a planned context (tables, records, M^B).
+// Device bytes that sg_create keeps for a planned context, from above: the row
+// operator and its tables, or the term-by-term tables where these are larger
+// (a context may be made with them when the row operator does not fit).
 int64_t planned_device_bytes(const sg_ctx *ctx);
 
 }  // namespace sg

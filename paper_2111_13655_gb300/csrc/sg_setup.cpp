@@ -97,14 +97,11 @@ std::string gauss_hermite(int n, std::vector<double> *x, std::vector<double> *wf
     return "";
 }
 
-// Pair form: every monomial touches at most two modes, in at most kMaxPairs
-// mode pairs; the pairs, and the sizes of level 1 where all modes share them.
-static void find_pairs(const Problem &p, HostTables *Tp)
+// Whether every monomial touches at most two modes, in at most kMaxPairs mode
+// pairs: the potentials that SG_DF64 and sg_tune take.
+static bool pair_potential(const Problem &p)
 {
-    HostTables &T = *Tp;
-    const int D = p.D, Lp = p.L + 1;
-    T.fast = false;
-    T.pair_modes.clear();
+    std::vector<std::pair<int, int>> pairs;
     for (int m = 0; m < (int)p.mcoef.size(); m++) {
         int a = -1, b = -1;
         for (int f = p.mfoff[m]; f < p.mfoff[m + 1]; f++) {
@@ -112,23 +109,13 @@ static void find_pairs(const Problem &p, HostTables *Tp)
             if (i == a || i == b) continue;
             if (a < 0) a = i;
             else if (b < 0) b = i;
-            else return;
+            else return false;
         }
         if (b < 0) continue;
-        if (a > b) std::swap(a, b);
-        bool seen = false;
-        for (size_t q = 0; q < T.pair_modes.size(); q += 2)
-            seen |= T.pair_modes[q] == a && T.pair_modes[q + 1] == b;
-        if (!seen) { T.pair_modes.push_back(a); T.pair_modes.push_back(b); }
+        const std::pair<int, int> ab(std::min(a, b), std::max(a, b));
+        if (std::find(pairs.begin(), pairs.end(), ab) == pairs.end()) pairs.push_back(ab);
     }
-    if (T.pair_modes.size() / 2 > (size_t)kMaxPairs) return;
-    T.nb1 = T.nq1 = 0;
-    if (p.L >= 1) {
-        T.nb1 = T.lvl[1].nb; T.nq1 = T.lvl[1].nq;
-        for (int i = 1; i < D; i++)
-            if (T.lvl[(size_t)i * Lp + 1].nb != T.nb1 || T.lvl[(size_t)i * Lp + 1].nq != T.nq1) { T.nb1 = T.nq1 = 0; break; }
-    }
-    T.fast = true;
+    return pairs.size() <= (size_t)kMaxPairs;
 }
 
 std::string build_tables(const Problem &p, int smem_budget, int rb, HostTables *out)
@@ -413,117 +400,9 @@ std::string build_tables(const Problem &p, int smem_budget, int rb, HostTables *
     T.pcost.resize(T.n_terms);
     for (int64_t q = 0; q < T.n_terms; q++) T.pcost[q] = cost[T.order[q]];
 
-    find_pairs(p, &T);
+    T.pairs = pair_potential(p);
     build_row_shifts(p, &T);
     return "";
-}
-
-}  // namespace sg
-
-namespace sg {
-
-// Size of the problem term by term: per term its compact indices (M^B), its
-// record, its 1D matrices and pair tables, and the table of its inner blocks
-// (up to three level-1 modes of a term with coupled modes, one symmetric block
-// per grid point of its other modes).  It is what sg_size reports for a planned
-// context and what the request server admits by: an upper bound of the row
-// operator that sg_create allocates, and independent of its layout.
-// `fits` tells whether every term fits a block's shared memory (slicing its
-// leading outer modes, at most 64 functions per slice): pair potentials where
-// one does not are outside the double-float mode and the tuner.
-TermForm term_form(const Problem &p, const HostTables &T)
-{
-    TermForm F{T.fast, 0};
-    if (!T.fast) return F;
-    const int D = p.D, Lp = p.L + 1;
-    const int rb = p.prec == SG_MIXED ? 4 : 8, U = 16 / rb;
-    const int rmax = T.nb1 == 2 ? 3 : T.nb1 == 3 ? 2 : 0, slice_max = 64;
-    const int np = (int)T.pair_modes.size() / 2;
-    auto LI = [&](int i, int l) -> const LevelInfo & { return T.lvl[(size_t)i * Lp + l]; };
-    auto pad = [U](int64_t n) { return (n + U - 1) / U * U; };
-
-    struct Plan {
-        int na, R, mode[kMaxD], nprs, ninds;
-        int64_t NB, NBin, gsize, mat;
-    };
-    auto plan = [&](int64_t t, Plan &P) {
-        const uint8_t *lt = &T.levels[(size_t)t * T.Dpad];
-        bool inner[kMaxD] = {false};
-        P.nprs = P.ninds = 0;
-        P.gsize = 0;
-        for (int q = 0; q < np; q++) {
-            const int a = T.pair_modes[2 * q], b = T.pair_modes[2 * q + 1];
-            const bool aa = LI(a, lt[a]).nb > 1, ab = LI(b, lt[b]).nb > 1;
-            if (aa && ab) { P.nprs++; P.gsize += LI(a, lt[a]).nq * LI(b, lt[b]).nq; }
-            else if (aa || ab) P.ninds++;
-        }
-        P.R = P.na = 0;
-        for (int i = D - 1; i >= 0 && P.R < (P.nprs ? rmax : 0); i--) {
-            const LevelInfo &li = LI(i, lt[i]);
-            if (li.nb > 1 && li.nb == T.nb1 && li.nq == T.nq1) { inner[i] = true; P.R++; }
-        }
-        P.NB = P.NBin = 1;
-        P.mat = 0;
-        for (int i = 0; i < D; i++) {
-            const LevelInfo &li = LI(i, lt[i]);
-            if (li.nb <= 1) continue;
-            P.NB *= li.nb;
-            P.mat += 2 * li.nb * li.nq + li.nb * li.nb;
-            if (inner[i]) P.NBin *= li.nb;
-            else P.mode[P.na++] = i;
-        }
-        std::stable_sort(P.mode, P.mode + P.na, [&](int x, int y) {  // by 1/nb - 1/nq
-            const LevelInfo &u = LI(x, lt[x]), &w = LI(y, lt[y]);
-            return (int64_t)(u.nq - u.nb) * w.nb * w.nq < (int64_t)(w.nq - w.nb) * u.nb * u.nq;
-        });
-    };
-    auto need = [&](const Plan &P, int64_t stage, bool sliced) {
-        return pad((P.NB * U + 3) / 4) + (sliced || !P.nprs ? 2 : 1) * pad(P.NB) + (P.nprs ? 2 * pad(stage) : 0);
-    };
-    Plan P;
-    int64_t gcap = 1, mcap = 1, units = 1;
-    for (int64_t t = 0; t < T.n_terms; t++) {
-        plan(t, P);
-        const int m = P.na + P.R;
-        const int64_t u = 3 + m + P.nprs + (P.ninds + 1) / 2;
-        gcap = std::max(gcap, P.gsize);
-        mcap = std::max(mcap, P.mat);
-        units = std::max(units, u);
-        int64_t blocks = 0;
-        if (P.nprs) {
-            int64_t grid = 1;
-            for (int j = 0; j < P.na; j++) grid *= LI(P.mode[j], T.levels[(size_t)t * T.Dpad + P.mode[j]]).nq;
-            const int64_t tri = P.NBin * (P.NBin + 1) / 2;
-            blocks = pad((P.NBin == 1 ? 1 : pad(tri)) * grid);
-        }
-        F.bytes += 4 * P.NB + 16 * u + rb * (P.mat + P.gsize + blocks);
-    }
-    F.bytes += (T.n_terms + 1) * (3 * (int64_t)sizeof(long long) + sizeof(unsigned));
-    const int64_t budget = 1024 * (int64_t)(rb == 4 ? 52 : 70);
-    const int64_t head = (rb * (mcap + gcap + 2 * slice_max) + 15) & ~(int64_t)15;
-    const int64_t work = (budget - head - 1024) / rb;
-    const int64_t record = (work * rb - 16 * units) / 16 * 16;  // scratch of a record at the end of the work area
-    if (work < 2 * T.maxnb + 64 || work * rb < 16 * (3 + (int64_t)kMaxD + 2 * np)) { F.fits = false; return F; }
-    for (int64_t t = 0; t < T.n_terms && F.fits; t++) {
-        plan(t, P);
-        const uint8_t *lt = &T.levels[(size_t)t * T.Dpad];
-        bool ok = 4 * P.NB <= record;
-        if (ok && P.nprs) {
-            ok = false;
-            int64_t nbo = 1;
-            for (int s = 0; s <= P.na && !ok; s++) {
-                if (s > 0) nbo *= LI(P.mode[s - 1], lt[P.mode[s - 1]]).nb;
-                if (nbo > slice_max) break;
-                int64_t stage = P.NBin;
-                for (int j = s; j < P.na; j++) stage *= LI(P.mode[j], lt[P.mode[j]]).nq;
-                ok = need(P, stage, s > 0) <= work;
-            }
-        } else if (ok) {
-            ok = need(P, 0, false) <= work;
-        }
-        F.fits = ok;
-    }
-    return F;
 }
 
 }  // namespace sg

@@ -86,7 +86,7 @@ extern "C" sg_status sg_tune(sg_ctx *ctx, int nvec, int *slice_vt, double *ms_ou
     if (!sg_on_ctx_device(ctx)) { ctx->last_error = std::string("sg_tune: ") + "the current CUDA device is not the one the context was made on"; return SG_EINVAL; }
     if (nvec < 1 || nvec > 64) { ctx->last_error = "sg_tune: need 1 <= nvec <= 64"; return SG_EINVAL; }
     sg::HostTables &T = ctx->host;
-    if (!T.rows || !sg::term_form(ctx->prob, T).fits) {  // not a pair potential: the default plan
+    if (!T.rows || !T.pairs) {  // not a pair potential: the default plan
         if (slice_vt) *slice_vt = 0;
         if (ms_out) *ms_out = 0.0;
         return SG_OK;
@@ -159,7 +159,7 @@ extern "C" sg_status sg_tune_plan(const sg_ctx *ctx, int *slice_vt, int *warp_vt
 {
     if (!ctx) return SG_EINVAL;
     const sg::HostTables &T = ctx->host;
-    const bool plan = T.rows && sg::term_form(ctx->prob, T).fits;
+    const bool plan = T.rows && T.pairs;
     if (slice_vt) *slice_vt = plan ? sg::row_vt(T, ctx->prob.prec) : 0;
     if (warp_vt) *warp_vt = plan ? sg::row_window_units(T) : 0;
     if (smem_kb) *smem_kb = plan ? sg::row_budget(T, ctx->prob.prec) / 1024 : 0;
