@@ -322,9 +322,11 @@ sg_status sg_tune_plan(const sg_ctx *ctx, int *slice_vt, int *warp_vt, int *smem
  * sg_server_create -- precision of every request's contexts (SG_FP64 or
  *   SG_MIXED; else SG_EINVAL); hbm_budget_bytes:
  *   the planned device memory of the active requests never exceeds it
- *   (the bound sg_size gives for a plan, batch items, state vectors, batch and context
- *   workspaces, logs).  Transient set-up buffers of an admission (the
- *   spectral-bound Krylov run, about 80 vectors) are not counted.
+ *   (the bound sg_size gives for a plan, batch slots with their state vectors
+ *   and workspace, the context's workspace, logs, weights).  Transient set-up
+ *   buffers are not counted: the spectral-bound Krylov run of an admission
+ *   (about 80 vectors) and, when the set of active requests changes, the state
+ *   vectors of the set before.
  * sg_server_submit -- copies the request (the caller's arrays may be freed on
  *   return), plans it on the host, and queues it; *id identifies it.
  *   SG_EBUDGET if the request alone needs more than the budget.
@@ -334,8 +336,8 @@ sg_status sg_tune_plan(const sg_ctx *ctx, int *slice_vt, int *warp_vt, int *smem
  *   Logs: <psi|psi> and <psi|H psi>/<psi|psi> at the start of each step.
  * sg_server_submit_eigs -- copies and plans an eigen request and queues it;
  *   SG_EBUDGET if it alone needs more than the budget (its plan's bound,
- *   its batch slots, the Davidson basis of max(3 nev, nev + 6 block) vectors
- *   and its images, Ritz vectors, eigenvectors).
+ *   its batch slots, everything a Davidson run of sg_eigs allocates,
+ *   eigenvectors).
  * sg_server_progress -- runs up to max_iters engine iterations (fewer if
  *   nothing is active); returns the numbers of active and queued requests.
  *   Synchronous.

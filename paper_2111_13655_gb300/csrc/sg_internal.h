@@ -245,7 +245,8 @@ int row_vt(const HostTables &T, sg_precision prec);      // vectors per lane of 
 int row_window_units(const HostTables &T);               // rows per window / 16 of the plan
 int row_budget(const HostTables &T, sg_precision prec);  // shared memory that SG_ROW_SHARE blocks may use (bytes)
 int row_value_bytes(sg_precision prec);                  // bytes of a stored element
-// Upper bound of the device bytes of the row operator.
+// Upper bounds of the row operator's windows and of its device bytes.
+int64_t row_form_windows(const HostTables &T, sg_precision prec);
 int64_t row_form_bytes(const HostTables &T, sg_precision prec);
 struct RowWindows {
     std::vector<RowWin> wins;
@@ -330,6 +331,8 @@ sg_status chebyshev_bounds(sg_ctx *ctx, cudaStream_t stream, double *emin, doubl
 using ApplyFn = std::function<sg_status(const double *x, double *y, int r)>;
 sg_status davidson_routed(sg_ctx *ctx, cudaStream_t stream, const ApplyFn &apply, int nev, int block, double tol,
                           int max_it, double *evals, double *resid, double *evecs, int *nconv, std::string *err);
+// Device bytes that davidson_routed holds on n-entry vectors (eigenvectors and the routed apply's buffers apart).
+int64_t davidson_device_bytes(int64_t n, int nev, int block);
 // J_0..J_kmax at x (Miller's backward recurrence).
 std::vector<double> bessel_j(int kmax, double x);
 // Device bytes that sg_create keeps for a planned context, from above: the row

@@ -165,14 +165,21 @@ int row_window_rows(int64_t n, int units)
     return w;
 }
 
+// (every row filled up by up to three entries)
+static int64_t most_entries(const HostTables &T) { return T.row_nnz + 3 * T.n_cs; }
+
+int64_t row_form_windows(const HostTables &T, sg_precision prec)
+{
+    if (!T.rows) return 0;
+    // a window for every 16 rows, and one more for every 4 KB of entries that may end one early
+    return T.n_cs / 16 + 1 + most_entries(T) * (4 + row_value_bytes(prec)) / 4096;
+}
+
 int64_t row_form_bytes(const HostTables &T, sg_precision prec)
 {
     if (!T.rows) return 0;
-    // a window for every 16 rows, and one more for every 4 KB of entries that may end one early;
-    // every row filled up by up to three entries
-    const int64_t ent = T.row_nnz + 3 * T.n_cs, eb = 4 + row_value_bytes(prec);
-    const int64_t nwin = T.n_cs / 16 + 1 + ent * eb / 4096;
-    return ent * eb + 8 * T.n_cs + nwin * (8 + (int64_t)sizeof(RowWin));
+    return most_entries(T) * (4 + row_value_bytes(prec)) + 8 * T.n_cs +
+           row_form_windows(T, prec) * (8 + (int64_t)sizeof(RowWin));
 }
 
 // entries of a row with its last group of four filled

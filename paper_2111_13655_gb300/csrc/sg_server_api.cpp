@@ -182,6 +182,26 @@ sg_status make_ctx(Req *r, sg_precision prec, bool device, sg_ctx **out)
                   : sg_plan(r->D, r->L, r->basis.data(), r->grids.data(), &H, prec, out);
 }
 
+// Device bytes of one two-vector slot over a planned context's problem, from
+// above: its state (relayout), the batch's tables, and the batch's workspace, in
+// which every problem has its part of the accumulators as soon as one is applied
+// term by term.
+int64_t slot_bytes(const sg_ctx *c)
+{
+    const sg::HostTables &T = c->host;
+    const int64_t n = T.n_cs, row = sg::row_value_bytes(c->prob.prec), words = sg::acc_words(c->fp32);
+    const int64_t state = 4 * 16 * n + 2 * 2 * n * row + (int64_t)sizeof(sg::ChebState) + 8;
+    const int64_t tables = 16 * (sg::row_form_windows(T, c->prob.prec) + n / 256 + 1) + (int64_t)sizeof(sg::RowOp) + 8;
+    return state + tables + 2 * n * row + 2 * n * 8 * words + 24;
+}
+// The context's own workspace for one vector, in whichever form it is applied.
+int64_t own_workspace_bytes(const sg_ctx *c)
+{
+    return c->host.n_cs * 8 * sg::acc_words(c->fp32) + 64;
+}
+// (the tables' alignment, and small allocations' granularity)
+constexpr int64_t kRequestSlack = (int64_t)1 << 20;
+
 // Spectral interval, Chebyshev weights and per-step constants of an admitted request.
 sg_status prepare(sg_server *s, Req *r)
 {
@@ -648,17 +668,16 @@ sg_status sg_server_submit(sg_server *s, const sg_prop_request *q, int64_t *id)
         delete r;
         return sfail(s, st, std::string("sg_server_submit: ") + sg_last_error(nullptr));
     }
-    int64_t n_cs = 0, n_terms = 0;
-    sg_size(plan, &n_cs, &n_terms, nullptr, nullptr, nullptr);
+    int64_t n_cs = 0;
+    sg_size(plan, &n_cs, nullptr, nullptr, nullptr, nullptr);
     r->n_cs = n_cs;
     r->psi0.assign(2 * (size_t)n_cs, 0.0);
     if (q->psi0) std::copy(q->psi0, q->psi0 + 2 * n_cs, r->psi0.begin());
     else st = sg_product_state(plan, q->factors, q->ld, r->psi0.data());
-    // tables + M^B + batch items + 4 state vectors, the batch workspace (2
-    // vectors x 4 fixed-point words), the context's own one-vector workspace
-    // (left by the spectral-bound run) + logs
-    r->bytes = sg::planned_device_bytes(plan) + 8 * n_terms + 2 * n_cs * (4 * 8 + 32) + 32 * n_cs +
-               16 * (int64_t)r->nsteps + ((int64_t)1 << 20);
+    // the context, its batch slot, its own one-vector workspace (left by the
+    // spectral-bound run), the logs and the recurrence's weights
+    r->bytes = sg::planned_device_bytes(plan) + slot_bytes(plan) + own_workspace_bytes(plan) +
+               16 * (int64_t)r->nsteps + 8 * ((int64_t)r->order + 1) + kRequestSlack;
     sg_destroy(plan);
     if (st != SG_OK) { delete r; return sfail(s, st, "sg_server_submit: bad initial-state factors"); }
     if (r->bytes > s->budget) {
@@ -709,21 +728,18 @@ sg_status sg_server_submit_eigs(sg_server *s, const sg_eig_request *q, int64_t *
         delete r;
         return sfail(s, st, std::string("sg_server_submit_eigs: ") + sg_last_error(nullptr));
     }
-    int64_t n_cs = 0, n_terms = 0;
-    sg_size(plan, &n_cs, &n_terms, nullptr, nullptr, nullptr);
-    const int64_t pb = sg::planned_device_bytes(plan);
+    int64_t n_cs = 0;
+    sg_size(plan, &n_cs, nullptr, nullptr, nullptr, nullptr);
+    // the context, its batch slots, the Davidson run and the eigenvectors
+    r->bytes = sg::planned_device_bytes(plan) + r->nslots * slot_bytes(plan);
     sg_destroy(plan);
     r->n_cs = n_cs;
     if (r->nev > n_cs) {
         delete r;
         return sfail(s, SG_EINVAL, "sg_server_submit_eigs: nev exceeds N_cs");
     }
-    // tables + M^B + batch items per slot + 4 state vectors and the batch
-    // workspace per slot + the Davidson basis and its images (2 kmax vectors),
-    // Ritz vectors, residuals and directions, eigenvectors, Gram scratch
-    const int64_t kmax = std::max(3 * r->nev, r->nev + 6 * r->block);
-    const int64_t vecs = 2 * kmax + 2 * std::max(r->nev, r->block) + r->block + (r->want_vectors ? r->nev : 0);
-    r->bytes = pb + r->nslots * (8 * n_terms + 2 * n_cs * (4 * 8 + 32)) + 8 * vecs * n_cs + ((int64_t)4 << 20);
+    r->bytes += sg::davidson_device_bytes(n_cs, r->nev, r->block) + (r->want_vectors ? 8 * n_cs * r->nev : 0) +
+                kRequestSlack;
     if (r->bytes > s->budget) {
         const int64_t b = r->bytes;
         delete r;

@@ -271,6 +271,26 @@ struct Solver {
     }
 };
 
+// Vectors of a run of block_eigs: basis V and images W = H V (kmax each), Ritz
+// vectors X and their images and residuals HX (nx each), directions T (b),
+// scratch Q (rmax, the largest block orthonormalised at once).  nx0: vectors to
+// start from (0: none).
+struct EigVectors {
+    int kmax, guard, rmax;
+    size_t nx, total;
+    EigVectors(int64_t n, int nev, int b, bool davidson, int max_it, int nx0)
+    {
+        // basis size: Davidson restarts at max(3 nev, nev + 6 b); the Krylov (Lanczos)
+        // form keeps at most 320 vectors (its projected problem is solved densely)
+        kmax = (int)std::min<int64_t>(n, davidson ? std::max(3 * nev, nev + 6 * b)
+                                                  : std::min<int64_t>((int64_t)max_it * b + b, 320));
+        guard = davidson ? b : 0;
+        nx = (size_t)std::max(nev + guard, b);
+        rmax = std::min(kmax, std::max(nev + b, nx0) + 1);
+        total = 2 * (size_t)kmax + 2 * nx + b + rmax;
+    }
+};
+
 // Block Davidson (or, without preconditioner and without restart, a block
 // Lanczos-type Krylov method with full reorthogonalisation and Rayleigh-Ritz).
 // Returns the number of converged eigenpairs; evals/resid on the host, the
@@ -284,15 +304,10 @@ int block_eigs(Solver &S, int nev, int b, bool davidson, double tol, int max_it,
                double *evals, double *evecs, double *resid)
 {
     const int64_t n = S.n;
-    // basis size: Davidson restarts at max(3 nev, nev + 6 b); the Krylov (Lanczos)
-    // form keeps at most 320 vectors (its projected problem is solved densely)
-    const int kmax = (int)std::min<int64_t>(n, davidson ? std::max(3 * nev, nev + 6 * b)
-                                                        : std::min<int64_t>((int64_t)max_it * b + b, 320));
-    const int guard = davidson ? b : 0;
-    const size_t nx = (size_t)std::max(nev + guard, b);
-    const int rmax = std::min(kmax, std::max(nev + b, nx0) + 1);  // largest block orthonormalised at once
-    // one allocation: basis V, images W = H V, Ritz vectors X, their images and residuals HX, directions T, scratch Q
-    DBuf mem((2 * (size_t)kmax + 2 * nx + b + rmax) * n);
+    const EigVectors size(n, nev, b, davidson, max_it, nx0);
+    const int kmax = size.kmax, guard = size.guard;
+    const size_t nx = size.nx;
+    DBuf mem(size.total * n);
     double *const V = mem.p, *const W = V + (size_t)kmax * n, *const X = W + (size_t)kmax * n,
                  *const HX = X + nx * n, *const T = HX + nx * n, *const Q = T + (size_t)b * n;
     std::vector<double> Tm;  // projected matrix, k x k
@@ -687,6 +702,14 @@ sg_status davidson_routed(sg_ctx *ctx, cudaStream_t stream, const ApplyFn &apply
         return e.st;
     }
     return SG_OK;
+}
+
+int64_t davidson_device_bytes(int64_t n, int nev, int block)
+{
+    const int b = block <= 0 ? std::min(nev, kBlk) : std::min(block, kBlk);
+    const int kmax = std::max(3 * nev, nev + 6 * b), cols = nev + b + 1;
+    const size_t small = Solver::scratch(n, kmax, cols) + Solver::capacity(kmax, cols);
+    return (int64_t)sizeof(double) * (int64_t)(small + EigVectors(n, nev, b, true, 1, 0).total * n);
 }
 
 sg_status chebyshev_bounds(sg_ctx *ctx, cudaStream_t stream, double *emin, double *emax)

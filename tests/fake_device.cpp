@@ -7,6 +7,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -23,9 +24,11 @@ struct State {
     std::map<std::string, long> launches;
     int event = 0;
 } g;
+std::mutex lock;  // eigen requests of a server run on threads of their own
 
 cudaError_t allocate(void **p, size_t n)
 {
+    std::lock_guard<std::mutex> lk(lock);
     *p = nullptr;
     if (n >= g.min_bytes) {
         g.matching++;
@@ -43,6 +46,7 @@ cudaError_t allocate(void **p, size_t n)
 
 cudaError_t launched(const char *name)
 {
+    std::lock_guard<std::mutex> lk(lock);
     g.launches[name]++;
     return cudaSuccess;
 }
@@ -69,6 +73,7 @@ long fake_launches(const char *name) { return g.launches.count(name) ? g.launche
 cudaError_t cudaMalloc(void **p, size_t n) { return allocate(p, n); }
 cudaError_t cudaFree(void *p)
 {
+    std::lock_guard<std::mutex> lk(lock);
     auto f = g.live.find(p);
     if (f == g.live.end()) return p ? cudaErrorInvalidValue : cudaSuccess;
     std::memset(p, 0xFF, f->second);  // kept: see above
@@ -240,9 +245,9 @@ cudaError_t dev_combine(const double *, int, const double *, int, double, const 
     return cudaSuccess;
 }
 cudaError_t dev_chol_inverse(const double *, int, double *, int *, cudaStream_t) { return cudaSuccess; }
-cudaError_t dev_residual(const double *, const double *, double *, int, int64_t, double *, double *, cudaStream_t)
+cudaError_t dev_residual(const double *, const double *, double *, int rows, int64_t, double *, double *, cudaStream_t)
 {
-    return cudaSuccess;
+    return rows < 1 ? cudaErrorInvalidValue : cudaSuccess;
 }
 cudaError_t dev_direction(const double *, const double *, const double *, int, int64_t, double *, cudaStream_t)
 {
