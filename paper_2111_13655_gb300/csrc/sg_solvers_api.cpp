@@ -486,12 +486,13 @@ void propagate_rows(Solver &S, double *psi, double Ebar, double dE, double dt, c
     const sg_precision prec = S.ctx->prob.prec;
     const size_t rb = (size_t)row_value_bytes(prec);
     const bool logs = norm_log || energy_log;
-    // T_k and T_{k-1}, the partial sum, H psi, the two entry-major copies, inner products of every step, flags
-    DBuf mem(8 * n + 2 * (2 * n * rb + 7) / 8 + 8 * (size_t)nsteps + 4);
+    const size_t ndots = logs ? 8 * (size_t)nsteps : 0;
+    // T_k and T_{k-1}, the partial sum, H psi, the two entry-major copies, inner products of every logged step, flags
+    DBuf mem(8 * n + 2 * (2 * n * rb + 7) / 8 + ndots + 4);
     double *x = mem.p, *p = x + 2 * n, *acc = p + 2 * n, *y = acc + 2 * n, *c0 = y + 2 * n;
     unsigned char *xs = reinterpret_cast<unsigned char *>(c0), *xn = xs + 2 * n * rb;
     double *dots = c0 + 2 * (2 * n * rb + 7) / 8;
-    unsigned *flags = reinterpret_cast<unsigned *>(dots + 8 * (size_t)nsteps);
+    unsigned *flags = reinterpret_cast<unsigned *>(dots + ndots);
     ck(cudaMemsetAsync(flags, 0, 2 * sizeof(unsigned), S.s), "flags");
     ck(cudaMemcpyAsync(x, psi, sizeof(double) * 2 * n, cudaMemcpyDeviceToDevice, S.s), "psi copy");
     RowIO r{};
@@ -521,7 +522,7 @@ void propagate_rows(Solver &S, double *psi, double Ebar, double dE, double dt, c
     ck(launch_row_settle(f, (int)n, S.s), "settle");
     S.sync("propagate sync");
     if (!logs) return;
-    std::vector<double> h(8 * (size_t)nsteps);
+    std::vector<double> h(ndots);
     ck(cudaMemcpy(h.data(), dots, sizeof(double) * h.size(), cudaMemcpyDeviceToHost), "logs");
     for (int step = 0; step < nsteps; step++) {
         const double *q = &h[8 * (size_t)step];
