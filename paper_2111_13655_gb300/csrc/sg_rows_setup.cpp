@@ -2,7 +2,10 @@
 // shifts that its products of one-mode matrices couple, the size of the row
 // operator, and the windows its rows are cut into.
 #include <algorithm>
-#include <map>
+#include <array>
+#include <cstdlib>
+#include <cstring>
+#include <unordered_set>
 
 #include "sg_internal.h"
 
@@ -12,17 +15,53 @@ namespace {
 
 struct Factor { int mode, op; };  // op: power of Q, 0 = the kinetic matrix
 
-// Shifts k' - k at which the one-mode matrix of `op` can be non-zero at any
-// level: the Jacobi matrix of the grid is tridiagonal, with a zero diagonal
-// for a grid symmetric about Q = 0; the kinetic matrix couples k to k, k +- 2
-// wherever the basis is centred.
-void op_shifts(const Problem &p, const Factor &f, std::vector<int> *out)
+// Shifts k' - k at which the one-mode matrix of a factor can be non-zero at any
+// level: -reach, -reach + step, ..., reach.  The Jacobi matrix of the grid is
+// tridiagonal, with a zero diagonal for a grid symmetric about Q = 0; the
+// kinetic matrix couples k to k, k +- 2 wherever the basis is centred.
+struct Reach {
+    int mode, reach, step;
+    Reach(const Problem &p, int m, int op)
+        : mode(m), reach(op == 0 ? 2 : op), step(op == 0 || p.basis[m].q0 == 0.0 ? 2 : 1)
+    {
+    }
+    bool holds(int d) const
+    {
+        const int a = d < 0 ? -d : d;
+        return a <= reach && (step == 1 || (reach - a) % 2 == 0);
+    }
+    bool within(const Reach &o) const { return mode == o.mode && (o.step == 1 || step == 2) && o.holds(reach); }
+};
+// Whether every shift of product a is one of product b.
+bool within(const std::vector<Reach> &a, const std::vector<Reach> &b)
 {
-    out->clear();
-    const int reach = f.op == 0 ? 2 : f.op;
-    const int step = f.op == 0 || p.basis[f.mode].q0 == 0.0 ? 2 : 1;
-    for (int d = -reach; d <= reach; d += step) out->push_back(d);
+    for (const Reach &f : a)
+        if (std::none_of(b.begin(), b.end(), [&](const Reach &g) { return f.within(g); })) return false;
+    // b's other modes stay where they are
+    for (const Reach &g : b)
+        if (!g.holds(0) && std::none_of(a.begin(), a.end(), [&](const Reach &f) { return f.mode == g.mode; })) return false;
+    return true;
 }
+
+// A shift k' - k over all modes, as bytes whose order is that of the shifts.
+constexpr int kNoShift = 128;
+struct Shift {
+    std::array<unsigned char, kMaxD> d;
+    bool operator==(const Shift &o) const { return d == o.d; }
+};
+static_assert(kMaxLevelSize <= 127 && kMaxD % 8 == 0, "a shift per byte, eight to a word");
+struct ShiftHash {
+    size_t operator()(const Shift &s) const
+    {
+        uint64_t h = 0, w;
+        for (int i = 0; i < kMaxD; i += 8) {
+            std::memcpy(&w, s.d.data() + i, 8);
+            h = (h ^ w) * 0x9E3779B97F4A7C15ull;
+            h ^= h >> 29;
+        }
+        return (size_t)h;
+    }
+};
 
 }  // namespace
 
@@ -57,61 +96,77 @@ void build_row_shifts(const Problem &p, HostTables *Tp)
     for (int i = 0; i < D; i++)
         if (T.harm_mono[i] < 0) add_product(1.0, {{i, 0}});
 
-    // distinct shifts (sorted (mode, d) pairs) and the products behind each.
-    // A shift that needs more levels than L between its two ends never occurs.
-    std::map<std::vector<std::pair<int, int>>, std::vector<int>> shifts;
+    // Distinct shifts and the products behind each.  A shift that needs more
+    // levels than L between its two ends never occurs.
+    // They are collected from the products whose shifts are not all another's
+    // (a force field's products differ mostly in the powers: 64 six-mode
+    // products over 3,003 functions have one such, and collecting from each made
+    // a plan of 93 ms instead of 12).
     const int np = (int)T.pr_coef.size();
+    std::vector<std::vector<Reach>> prod(np);
+    for (int q = 0; q < np; q++)
+        for (int f = T.pr_off[q]; f < T.pr_off[q + 1]; f++) prod[q].emplace_back(p, T.pr_mode[f], T.pr_op[f]);
+    std::unordered_set<Shift, ShiftHash> found;
+    Shift cur;
+    cur.d.fill(kNoShift);
     for (int q = 0; q < np; q++) {
-        const int nf = T.pr_off[q + 1] - T.pr_off[q];
-        std::vector<std::vector<int>> sh(nf);
-        for (int a = 0; a < nf; a++) op_shifts(p, {T.pr_mode[T.pr_off[q] + a], T.pr_op[T.pr_off[q] + a]}, &sh[a]);
-        std::vector<std::pair<int, int>> cur;
+        bool inside = false;
+        for (int o = 0; o < np && !inside; o++)
+            inside = o != q && within(prod[q], prod[o]) && (o < q || !within(prod[o], prod[q]));
+        if (inside) continue;
         bool ok = true;
         // depth first over the factors, pruned by the levels the shifts need
-        auto walk = [&](auto &self, int a, int used) -> void {
+        auto walk = [&](auto &self, size_t a, int used) -> void {
             if (!ok) return;
-            if (a == nf) {
-                std::vector<std::pair<int, int>> key(cur);
-                std::sort(key.begin(), key.end());
-                shifts[key].push_back(q);
-                if ((int)shifts.size() > kRowMaxShifts) ok = false;
+            if (a == prod[q].size()) {
+                found.insert(cur);
+                if ((int)found.size() > kRowMaxShifts) ok = false;
                 return;
             }
-            const int mode = T.pr_mode[T.pr_off[q] + a];
-            for (int d : sh[a]) {
+            const Reach &f = prod[q][a];
+            for (int d = -f.reach; d <= f.reach; d += f.step) {
                 const int ad = d < 0 ? -d : d;
                 if (ad >= kw) continue;
-                const int lm = T.lmin_tab[(size_t)mode * kw + ad];
+                const int lm = T.lmin_tab[(size_t)f.mode * kw + ad];
                 if (lm > L || used + lm > L) continue;
-                if (d) cur.push_back({mode, d});
+                cur.d[f.mode] = (unsigned char)(kNoShift + d);
                 self(self, a + 1, used + lm);
-                if (d) cur.pop_back();
             }
+            cur.d[f.mode] = kNoShift;
         };
         walk(walk, 0, 0);
         if (!ok) return;
     }
-    // in the order of the column index: lexicographic in the dense shift
-    std::vector<const std::pair<const std::vector<std::pair<int, int>>, std::vector<int>> *> ord;
-    for (const auto &s : shifts) ord.push_back(&s);
-    auto dense_less = [D](const std::vector<std::pair<int, int>> &a, const std::vector<std::pair<int, int>> &b) {
-        size_t i = 0, j = 0;
-        for (int m = 0; m < D; m++) {
-            int x = 0, y = 0;
-            if (i < a.size() && a[i].first == m) x = a[i++].second;
-            if (j < b.size() && b[j].first == m) y = b[j++].second;
-            if (x != y) return x < y;
-        }
-        return false;
-    };
-    std::sort(ord.begin(), ord.end(), [&](const auto *a, const auto *b) { return dense_less(a->first, b->first); });
+    // in the order of the column index: lexicographic in the shift
+    std::vector<Shift> shifts(found.begin(), found.end());
+    std::sort(shifts.begin(), shifts.end(), [](const Shift &a, const Shift &b) { return a.d < b.d; });
+    // per mode and |d| the products that a move by d belongs to, a bit each
+    const int words = (np + 63) / 64;
+    std::vector<uint64_t> takes((size_t)D * kw * words, 0), all(words);
+    for (int q = 0; q < np; q++) {
+        const uint64_t bit = 1ull << (q % 64);
+        auto at = [&](int mode, int ad) -> uint64_t & { return takes[((size_t)mode * kw + ad) * words + q / 64]; };
+        for (int i = 0; i < D; i++) at(i, 0) |= bit;
+        for (const Reach &f : prod[q])
+            for (int ad = 0; ad < kw; ad++) at(f.mode, ad) = f.holds(ad) ? at(f.mode, ad) | bit : at(f.mode, ad) & ~bit;
+    }
     T.sh_off.assign(1, 0);
     T.sh_src_off.assign(1, 0);
     T.sh_mode.clear(); T.sh_d.clear(); T.sh_src.clear();
-    for (const auto *s : ord) {
-        for (const auto &md : s->first) { T.sh_mode.push_back(md.first); T.sh_d.push_back(md.second); }
+    for (const Shift &s : shifts) {
+        all.assign(words, ~0ull);
+        for (int i = 0; i < D; i++) {
+            const int d = (int)s.d[i] - kNoShift;
+            if (d) { T.sh_mode.push_back(i); T.sh_d.push_back(d); }
+            const uint64_t *t = &takes[((size_t)i * kw + std::abs(d)) * words];
+            for (int w = 0; w < words; w++) all[w] &= t[w];
+        }
         T.sh_off.push_back((int)T.sh_mode.size());
-        T.sh_src.insert(T.sh_src.end(), s->second.begin(), s->second.end());
+        for (int w = 0; w < words; w++)
+            for (uint64_t m = all[w]; m; m &= m - 1) {
+                const int q = 64 * w + __builtin_ctzll(m);
+                if (q < np) T.sh_src.push_back(q);
+            }
         T.sh_src_off.push_back((int)T.sh_src.size());
     }
 

@@ -19,11 +19,8 @@ ABSENT = ("sg_measure_peak", "sg_apply_H_noalloc")
 _loaded = None
 
 
-def load(tmp):
-    """The stand-in library, built once per session into `tmp`; skips without a host compiler or CUDA's headers."""
-    global _loaded
-    if _loaded is not None:
-        return _loaded
+def compiler():
+    """Host compiler command with CUDA's and the library's headers; skips without them."""
     cxx = shutil.which("g++") or shutil.which("c++")
     try:
         include = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc()))), "include")
@@ -31,18 +28,26 @@ def load(tmp):
         include = ""
     if not cxx or not os.path.exists(os.path.join(include, "cuda_runtime.h")):
         pytest.skip("needs a host C++ compiler and CUDA's headers")
-    flags = ["-std=c++17", "-O1", "-fPIC", "-isystem", include, "-I", build.CSRC, "-I", os.path.join(build.ROOT, "include")]
+    return [cxx, "-std=c++17", "-fPIC", "-isystem", include, "-I", build.CSRC, "-I", os.path.join(build.ROOT, "include")]
+
+
+def load(tmp):
+    """The stand-in library, built once per session into `tmp`."""
+    global _loaded
+    if _loaded is not None:
+        return _loaded
+    cxx = compiler()
 
     def compile_unit(path):
         obj = os.path.join(tmp, os.path.basename(path) + ".o")
-        subprocess.run([cxx, *flags, "-c", path, "-o", obj], check=True)
+        subprocess.run([*cxx, "-O1", "-c", path, "-o", obj], check=True)
         return obj
 
     with cf.ThreadPoolExecutor(max_workers=8) as ex:
         objs = list(ex.map(compile_unit, [os.path.join(build.CSRC, u) for u in UNITS] +
                            [os.path.join(HERE, "fake_device.cpp")]))
     so = os.path.join(tmp, "libfake.so")
-    subprocess.run([cxx, "-shared", "-Wl,-Bsymbolic", *objs, "-o", so, "-lpthread"], check=True)
+    subprocess.run([cxx[0], "-shared", "-Wl,-Bsymbolic", *objs, "-o", so, "-lpthread"], check=True)
     lib = ctypes.CDLL(so)
     for name, (res, args) in sg.SIGNATURES.items():
         if name not in ABSENT:
