@@ -333,7 +333,9 @@ cudaError_t build_rows(sg_ctx *ctx)
         if (e == cudaSuccess) {
             R.wins = reinterpret_cast<const RowWin *>(own);
             R.blob = own + rec;
-            e = launch_row_fill(kp, S, prec, R.wins, reinterpret_cast<const int *>(plan + win),
+            int most = 0;
+            for (const RowWin &w : W.wins) most = std::max(most, w.nent);
+            e = launch_row_fill(kp, S, prec, R.wins, (int)W.wins.size(), most, reinterpret_cast<const int *>(plan + win),
                                 reinterpret_cast<const int *>(plan + start), reinterpret_cast<const uint2 *>(plan + meta),
                                 own + rec, 0);
         }

@@ -263,8 +263,9 @@ int row_window_rows(int64_t n, int units);
 
 // Row form, device half (sg_rows.cu).  prec selects the element type.
 cudaError_t launch_row_count(const KParams &kp, const RowShifts &sh, int *cnt, cudaStream_t stream);
-cudaError_t launch_row_fill(const KParams &kp, const RowShifts &sh, sg_precision prec, const RowWin *wins,
-                            const int *win, const int *start, const uint2 *meta, unsigned char *blob,
+// The records of nwin windows of at most `most` entries each.
+cudaError_t launch_row_fill(const KParams &kp, const RowShifts &sh, sg_precision prec, const RowWin *wins, int nwin,
+                            int most, const int *win, const int *start, const uint2 *meta, unsigned char *blob,
                             cudaStream_t stream);
 cudaError_t configure_rows();
 // y = H_S x (io.y), or the sums of the windows of io.part into io.acc; vt: vectors per lane.

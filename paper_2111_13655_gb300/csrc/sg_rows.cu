@@ -92,40 +92,48 @@ __device__ double factor_elem(const KParams &P, int mode, int op, int l, int k, 
     const int off = op == 0 ? li.offK : li.offM + (op - 1) * li.nb * li.nb;
     return P.tabd[off + k * li.nb + k2];
 }
-__device__ double factor_diff(const KParams &P, int mode, int op, int l, int k, int k2)
-{
-    const double m = factor_elem(P, mode, op, l, k, k2);
-    return l > 0 ? m - factor_elem(P, mode, op, l - 1, k, k2) : m;
-}
-
 // sum over |l_S| <= T of prod Delta M_i(l_i)[k_i][k'_i] over the factors of
 // product q; the last factor's differences are summed in closed form
-// (sum_{l <= t} Delta M(l) = M(t)).
+// (sum_{l <= t} Delta M(l) = M(t)).  A factor's element is zero below the level
+// that holds both functions, so the sums run over the levels that remain above
+// these, `room` (of T).
 __device__ double product_elem(const KParams &P, const RowShifts &S, int q, const int *k, const int *k2, int sum)
 {
     const int f0 = S.prod_off[q], f1 = S.prod_off[q + 1];
-    int T = P.L - sum;
-    for (int f = f0; f < f1; f++) T += P.lmin_tab[S.fmode[f] * P.kw + k[S.fmode[f]]];
     if (f0 == f1) return 1.0;
-    const int last = f1 - 1, ml = S.fmode[last], ol = S.fop[last];
-    if (f1 - f0 == 1) return factor_elem(P, ml, ol, T, k[ml], k2[ml]);
-    double a[kRowMaxL + 1], b[kRowMaxL + 1];
-    {
-        const int m = S.fmode[f0], o = S.fop[f0];
-        for (int l = 0; l <= T; l++) a[l] = factor_diff(P, m, o, l, k[m], k2[m]);
+    auto first = [&](int f) {  // of the levels that hold both functions of factor f
+        const int m = S.fmode[f];
+        return (int)P.lmin_tab[m * P.kw + max(k[m], k2[m])];
+    };
+    int T = P.L - sum, low = 0;
+    for (int f = f0; f < f1; f++) {
+        T += P.lmin_tab[S.fmode[f] * P.kw + k[S.fmode[f]]];
+        low += first(f);
     }
-    for (int f = f0 + 1; f < last; f++) {
-        const int m = S.fmode[f], o = S.fop[f];
-        for (int t = 0; t <= T; t++) {
-            double v = 0.0;
-            for (int l = 0; l <= t; l++) v = fma(a[t - l], factor_diff(P, m, o, l, k[m], k2[m]), v);
-            b[t] = v;
+    const int last = f1 - 1, ml = S.fmode[last], ol = S.fop[last], room = T - low;
+    if (f1 - f0 == 1) return factor_elem(P, ml, ol, T, k[ml], k2[ml]);
+    double a[kRowMaxL + 1], d[kRowMaxL + 1];  // by level above the first
+    for (int f = f0; f < last; f++) {
+        const int m = S.fmode[f], o = S.fop[f], l0 = first(f);
+        double below = 0.0;
+        for (int j = 0; j <= room; j++) {
+            const double e = factor_elem(P, m, o, l0 + j, k[m], k2[m]);
+            d[j] = e - below;
+            below = e;
         }
-        for (int t = 0; t <= T; t++) a[t] = b[t];
+        for (int t = room; t >= 0; t--) {
+            if (f == f0) {
+                a[t] = d[t];
+                continue;
+            }
+            double v = 0.0;
+            for (int j = 0; j <= t; j++) v = fma(a[t - j], d[j], v);
+            a[t] = v;
+        }
     }
     double v = 0.0;
-    for (int l = 0; l <= T; l++)
-        if (a[l] != 0.0) v = fma(a[l], factor_elem(P, ml, ol, T - l, k[ml], k2[ml]), v);
+    for (int j = 0; j <= room; j++)
+        if (a[j] != 0.0) v = fma(a[j], factor_elem(P, ml, ol, first(last) + room - j, k[ml], k2[ml]), v);
     return v;
 }
 
@@ -147,48 +155,89 @@ template <> struct Elem<float> { static __device__ float of(double v) { return (
 template <> struct Elem<double> { static __device__ double of(double v) { return v; } };
 template <> struct Elem<df2> { static __device__ df2 of(double v) { return df_split(v); } };
 
-template <typename T>
-__global__ void __launch_bounds__(256) k_row_fill(const KParams P, const RowShifts S, const RowWin *__restrict__ wins,
-                                                  const int *__restrict__ win, const int *__restrict__ start,
-                                                  const uint2 *__restrict__ meta, unsigned char *__restrict__ blob)
+// The record's row list, and the shift of every entry in the place of its
+// column (~shift for the zero elements that fill a row's last group of four).
+__global__ void __launch_bounds__(256) k_row_place(const KParams P, const RowShifts S, const RowWin *__restrict__ wins,
+                                                   const int *__restrict__ win, const int *__restrict__ start,
+                                                   const uint2 *__restrict__ meta, unsigned char *__restrict__ blob)
 {
     const int r = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (r >= P.n_cs) return;
-    int k[kMaxD], k2[kMaxD];
+    int k[kMaxD];
     const int sum = unrank(P, r, k);
     const RowWin w = wins[win[r]];
     unsigned char *rec = blob + w.off;
     if (lane == 0) reinterpret_cast<uint2 *>(rec)[r - w.row0] = meta[r];
     int *cols = reinterpret_cast<int *>(rec + row_meta_bytes(w.nrows));
-    T *vals = reinterpret_cast<T *>(cols + w.nent);
     int at = start[r];
     for (int q0 = 0; q0 < S.nshift; q0 += 32) {
         const int q = q0 + lane;
         const bool in = q < S.nshift && shift_fits(P, S, q, k, sum);
         const unsigned m = __ballot_sync(0xffffffffu, in);
-        if (in) {
-            for (int i = 0; i < P.D; i++) k2[i] = k[i];
-            for (int e = S.off[q]; e < S.off[q + 1]; e++) k2[S.mode[e]] += S.d[e];
+        if (in) cols[at + __popc(m & ((1u << lane) - 1u))] = q;
+        at += __popc(m);
+    }
+    const int pad = (4 - ((at - start[r]) & 3)) & 3;
+    __syncwarp();
+    if (lane < pad) cols[at + lane] = ~cols[at - 1];
+}
+
+// Columns and elements, a thread per entry; a block takes kElemChunk entries of
+// a window and finds their rows' multi-indices once.  Bound by the FP64 pipe for
+// products of many modes (their levels' convolutions).  Set-up of 64 six-mode
+// products over 3,003 functions, and of the benchmark's operator (D=12 L=10):
+// one kernel with a warp per row, its lanes over the shifts, most of them idle
+// since few shifts fit a row, and sums over all levels 275 ms (the kernel there
+// 2.6 ms); sums over the levels that remain 64; lanes filled from a list of the
+// shifts that fit 27; a thread per entry 11 (0.5 + 0.8 ms), of which 6 are the
+// plan.  Chunks of 1,024 entries: 14 (0.5 + 0.6).
+constexpr int kElemThreads = 128, kElemChunk = 128;
+template <typename T>
+__global__ void __launch_bounds__(kElemThreads) k_row_elems(const KParams P, const RowShifts S,
+                                                            const RowWin *__restrict__ wins,
+                                                            const int *__restrict__ start,
+                                                            unsigned char *__restrict__ blob)
+{
+    __shared__ unsigned char index[kRowWindowMax][kMaxD];
+    __shared__ int level[kRowWindowMax];
+    const RowWin w = wins[blockIdx.x];
+    int *cols = reinterpret_cast<int *>(blob + w.off + row_meta_bytes(w.nrows));
+    T *vals = reinterpret_cast<T *>(cols + w.nent);
+    auto row_of = [&](int e) {  // the last row of the window that starts at or before entry e
+        int lo = 0, hi = w.nrows;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (start[w.row0 + mid] <= e) lo = mid;
+            else hi = mid;
+        }
+        return lo;
+    };
+    for (int e0 = blockIdx.y * kElemChunk; e0 < w.nent; e0 += gridDim.y * kElemChunk) {
+        const int e1 = min(w.nent, e0 + kElemChunk), r1 = row_of(e1 - 1);
+        int k[kMaxD], k2[kMaxD];
+        for (int r = row_of(e0) + threadIdx.x; r <= r1; r += kElemThreads) {
+            level[r] = unrank(P, w.row0 + r, k);
+            for (int i = 0; i < P.D; i++) index[r][i] = (unsigned char)k[i];
+        }
+        __syncthreads();
+        for (int e = e0 + threadIdx.x; e < e1; e += kElemThreads) {
+            const int r = row_of(e);
+            const bool fill = cols[e] < 0;
+            const int q = fill ? ~cols[e] : cols[e];
+            for (int i = 0; i < P.D; i++) k2[i] = k[i] = index[r][i];
+            for (int d = S.off[q]; d < S.off[q + 1]; d++) k2[S.mode[d]] += S.d[d];
             int c = 0, s = 0;
             for (int i = 0; i < P.D; i++) {
                 c += __ldg(P.rank_tab + (size_t)(i * (P.L + 1) + s) * P.kw + k2[i]);
                 s += P.lmin_tab[i * P.kw + k2[i]];
             }
             double v = 0.0;
-            for (int e = S.src_off[q]; e < S.src_off[q + 1]; e++)
-                v = fma(S.coef[S.src[e]], product_elem(P, S, S.src[e], k, k2, sum), v);
-            const int p = at + __popc(m & ((1u << lane) - 1u));
-            cols[p] = c;
-            vals[p] = Elem<T>::of(v);
+            for (int d = S.src_off[q]; d < S.src_off[q + 1] && !fill; d++)
+                v = fma(S.coef[S.src[d]], product_elem(P, S, S.src[d], k, k2, level[r]), v);
+            cols[e] = c;
+            vals[e] = Elem<T>::of(v);
         }
-        at += __popc(m);
-    }
-    // the row's last group of four is filled with zero elements (of its last column)
-    const int pad = (4 - ((at - start[r]) & 3)) & 3;
-    __syncwarp();
-    if (lane < pad) {
-        cols[at + lane] = cols[at - 1];
-        vals[at + lane] = Elem<T>::of(0.0);
+        __syncthreads();
     }
 }
 
@@ -907,14 +956,15 @@ cudaError_t launch_row_count(const KParams &kp, const RowShifts &sh, int *cnt, c
     return cudaGetLastError();
 }
 
-cudaError_t launch_row_fill(const KParams &kp, const RowShifts &sh, sg_precision prec, const RowWin *wins,
-                            const int *win, const int *start, const uint2 *meta, unsigned char *blob,
+cudaError_t launch_row_fill(const KParams &kp, const RowShifts &sh, sg_precision prec, const RowWin *wins, int nwin,
+                            int most, const int *win, const int *start, const uint2 *meta, unsigned char *blob,
                             cudaStream_t stream)
 {
-    const unsigned blocks = (unsigned)(((size_t)kp.n_cs * 32 + 255) / 256);
-    if (prec == SG_MIXED) k_row_fill<float><<<blocks, 256, 0, stream>>>(kp, sh, wins, win, start, meta, blob);
-    else if (prec == SG_DF64) k_row_fill<df2><<<blocks, 256, 0, stream>>>(kp, sh, wins, win, start, meta, blob);
-    else k_row_fill<double><<<blocks, 256, 0, stream>>>(kp, sh, wins, win, start, meta, blob);
+    k_row_place<<<(unsigned)(((size_t)kp.n_cs * 32 + 255) / 256), 256, 0, stream>>>(kp, sh, wins, win, start, meta, blob);
+    const dim3 grid((unsigned)nwin, (unsigned)std::max(1, std::min(512, (most + kElemChunk - 1) / kElemChunk)));
+    if (prec == SG_MIXED) k_row_elems<float><<<grid, kElemThreads, 0, stream>>>(kp, sh, wins, start, blob);
+    else if (prec == SG_DF64) k_row_elems<df2><<<grid, kElemThreads, 0, stream>>>(kp, sh, wins, start, blob);
+    else k_row_elems<double><<<grid, kElemThreads, 0, stream>>>(kp, sh, wins, start, blob);
     return cudaGetLastError();
 }
 

@@ -146,7 +146,7 @@ cudaError_t launch_row_count(const KParams &P, const RowShifts &S, int *cnt, cud
     }
     return launched("row_count");
 }
-cudaError_t launch_row_fill(const KParams &P, const RowShifts &, sg_precision prec, const RowWin *wins, const int *win,
+cudaError_t launch_row_fill(const KParams &P, const RowShifts &, sg_precision, const RowWin *wins, int, int, const int *win,
                             const int *start, const uint2 *meta, unsigned char *blob, cudaStream_t)
 {
     for (int r = 0; r < P.n_cs; r++) {
@@ -155,7 +155,6 @@ cudaError_t launch_row_fill(const KParams &P, const RowShifts &, sg_precision pr
         int *cols = reinterpret_cast<int *>(blob + w.off + row_meta_bytes(w.nrows));
         const int next = r + 1 < w.row0 + w.nrows ? start[r + 1] : w.nent;
         for (int e = start[r]; e < next; e++) cols[e] = r;
-        (void)prec;
     }
     return launched("row_fill");
 }
