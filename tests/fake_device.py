@@ -55,7 +55,7 @@ def load(tmp):
     lib.fake_fail_after.argtypes = [ctypes.c_long, ctypes.c_size_t]
     for name in ("fake_live", "fake_peak", "fake_largest"):
         getattr(lib, name).restype = ctypes.c_size_t
-    for name in ("fake_matching", "fake_launches"):
+    for name in ("fake_matching", "fake_launches", "fake_entries"):
         getattr(lib, name).restype = ctypes.c_long
     lib.fake_launches.argtypes = [ctypes.c_char_p]
     _loaded = lib

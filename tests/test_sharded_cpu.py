@@ -1,5 +1,6 @@
-"""Host side of the term-sharded apply, no GPU: the partition of the term
-list over parts, and the integer reduction of the parts' accumulators over two
+"""Host side of the sharded apply, no GPU: the partition of the term list over
+parts (problems applied term by term; the row form's windows: test_row_parts.py),
+and the integer reduction of the parts' accumulators over two
 gloo ranks (the collective a multi-GPU apply uses between its parts)."""
 import os
 import socket

@@ -1,8 +1,8 @@
-"""Term-sharded apply on one GPU: the parts of the term list (processing
-positions p = part mod nparts) accumulated separately and summed as 64-bit
-integers give bitwise the full sg_apply_H, for any number of parts (the
-integer sum is associative).  This is the arithmetic a multi-GPU apply runs
-with one part per GPU and one integer all-reduce (the MPI sum of Alg. 2)."""
+"""Sharded apply on one GPU: the parts (windows of rows w = part mod nparts),
+each row's sum added as a bit pattern into accumulators of its own part, summed
+as 64-bit integers give bitwise the full sg_apply_H, for any number of parts.
+This is the arithmetic a multi-GPU apply runs with one part per GPU and one
+integer all-reduce (the MPI sum of Alg. 2)."""
 import numpy as np
 import pytest
 
@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 PROBLEMS = {
     "D=6 L=8 nq=l+1": synth.workload_C2(),
     "D=12 L=6 nq=l+2": synth.workload_C3(L=6),
-    "general polynomial (generic kernel)": synth.polynomial_problem(
+    "general polynomial": synth.polynomial_problem(
         3, 5, [0.9, 1.1, 1.0],
         [(0.3, [(0, 1)]), (0.2, [(0, 2), (1, 2)]), (0.05, [(0, 1), (1, 1), (2, 1)]), (0.7, [])],
         q0=[0.3, -0.2, 0.1], scale=[1.3, 0.8, 1.0]),
