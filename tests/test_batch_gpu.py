@@ -1,10 +1,9 @@
 """Batched apply: many independent problems per sg_apply_H_batch.
 
-The batch runs the terms of all problems of one kernel variant in one launch,
-ordered by cost over all problems.  Every problem's arithmetic is the same as
-in its own sg_apply_H (same records, vector chunks and exact fixed-point
-compress-add), so results must agree bitwise; FP64 results are also checked
-against the literal CPU oracle.
+The batch sums the rows of all problems in one launch, the windows with most
+entries first.  Every row's sum is made as in the problem's own sg_apply_H, so
+results must agree bitwise; FP64 results are also checked against the literal
+CPU oracle.
 """
 import numpy as np
 import pytest
@@ -21,13 +20,13 @@ pytestmark = pytest.mark.gpu
 
 
 def mixed_bag():
-    """Problems of several kernel variants, with a generic-path one among them."""
+    """Problems of several shapes (with one applied term by term among them: test_terms_gpu.py)."""
     return [
         synth.workload_C1(),
         synth.workload_C2(),
         synth.workload_C3(L=5),                                  # nb = l+1, nq = l+2
         synth.chained_henon_heiles(4, 5, synth.draw_omega(4, 9), 0.2, nb_rule=(1, 2), nq_rule=(1, 2)),
-        synth.polynomial_problem(                                # three-mode monomial: generic kernel
+        synth.polynomial_problem(                                # three-mode monomial, shifted modes
             3, 5, [0.9, 1.1, 1.0],
             [(0.3, [(0, 1)]), (0.2, [(0, 2), (1, 2)]), (0.05, [(0, 1), (1, 1), (2, 1)]), (0.7, [])],
             q0=[0.3, -0.2, 0.1], scale=[1.3, 0.8, 1.0]),
