@@ -5,8 +5,8 @@ Workload: chained Henon-Heiles, D=12, L=10, nb(l)=l+1, nq(l)=l+2, omega_i ~
 U[0.8,1.2] (seeded), lambda = 0.111803; N_cs = 646,646 compact functions,
 646,646 Smolyak terms.  One step = one sg_apply_H on a block of `nvec` real
 vectors (the block of the block-Davidson solver); one application = one real
-vector.  Mixed precision (FP32 products, their sums carried without rounding
-in pairs) is the headline; FP64 mode is measured beside it.
+vector.  Mixed precision (FP32 products, added in FP32 by groups of four and
+these in pairs of FP32 numbers) is the headline; FP64 mode is measured beside it.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 

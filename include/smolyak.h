@@ -106,8 +106,8 @@ typedef struct {
  *   basis  D host structs; grids: D host structs.
  *   H      Hamiltonian; all arrays are host memory, copied (caller keeps ownership).
  *   prec   SG_FP64: every step in FP64.  SG_MIXED: elements and x in FP32,
- *          products in FP32, four at a time, their sums carried without
- *          rounding in a pair of FP32 numbers, the harmonic diagonal in FP64
+ *          products in FP32 and added in groups of four there, the groups'
+ *          sums in a pair of FP32 numbers, the harmonic diagonal in FP64
  *          (term by term: contractions in FP32, compact result in exact fixed
  *          point).  SG_DF64: elements, x and sums in double-float arithmetic
  *          (each value an unevaluated sum of two FP32 numbers, about 48

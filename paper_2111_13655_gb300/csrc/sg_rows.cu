@@ -13,9 +13,11 @@
 //      consecutive rows.
 // A row's entries are summed in column order by one lane whatever the plan,
 // the number of vectors or the batch, so every entry point gives the same bits.
-// Sums: FP64 by fma; mixed precision adds four products in FP32 and these to a
-// pair of FP32 numbers without error (two-sum), so nothing is lost in the
-// accumulation over a row; double-float as df_fma.
+// Sums: FP64 by fma; mixed precision adds four products in FP32 (a product and
+// three multiply-adds, each rounded) and these groups by two-sum into a pair of
+// FP32 numbers, whose low part collects the errors in FP32: a row's error is
+// that of its products and groups, 6.1 * 2^-24 of the sum of its terms' sizes
+// however long it is; double-float as df_fma.
 //
 // What bounds the row kernel (D=12 L=9, 8 vectors): FP64 its pipe, 83% busy;
 // mixed and double-float the latency of the gathers, with 34% and 45% of the

@@ -1,7 +1,7 @@
 """The double-float contraction mode (SG_DF64) through the C ABI.
 
-Parity with the oracle at the tolerances of tests/helpers.py (norm-wise as
-FP64, element-wise DF64_ELEM_TOL), on the literal oracle's cases and on the
+Parity with the oracle at the tolerances of tests/helpers.py (norm-wise
+DF64_TOL, element-wise DF64_ELEM_TOL), on the literal oracle's cases and on the
 benchmark workload at full size against the exact closed form; bitwise
 repeatability and the bitwise identity of every entry point (vectors one by
 one or together, the no-allocation apply); the contexts the mode refuses.
@@ -71,9 +71,8 @@ def test_df64_c3_full_size_matches_masked_galerkin():
 
 
 def test_df64_entry_points_bitwise():
-    """Exact fixed-point sum: repeats, vectors one at a time, and the
-    no-allocation apply (which gathers from x instead of the staged copy)
-    give the same bits."""
+    """A row is summed in one order: repeats, vectors one at a time, and the
+    no-allocation apply give the same bits."""
     p = synth.workload_C3(L=6)
     n = orc.n_compact(p)
     x = synth.random_vectors(n, 3, 99)
@@ -100,7 +99,7 @@ def test_df64_eigenvalues_match_the_oracle_spectrum():
 
 
 def test_df64_tuned_plan_keeps_parity():
-    """sg_tune re-plans a double-float context (slicing, split, budget); the
+    """sg_tune re-plans a double-float context (vectors per lane, rows per window, budget); the
     tuned applies stay within the tolerances and repeat bitwise."""
     p = synth.workload_C3(L=6)
     x = synth.random_vectors(orc.n_compact(p), 4, 31)
@@ -113,7 +112,7 @@ def test_df64_tuned_plan_keeps_parity():
 
 
 def test_df64_refusals():
-    """Problems off the fast path (a monomial of three modes) and batches are
+    """Potentials with a monomial of three modes, and batches, are
     refused with SG_EUNSUPPORTED, a double-float server with SG_EINVAL."""
     p3 = synth.polynomial_problem(3, 3, [1.0, 1.0, 1.0], [(0.1, [(0, 1), (1, 1), (2, 1)])])
     with pytest.raises(sg.SgError) as ei:

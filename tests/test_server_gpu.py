@@ -64,7 +64,7 @@ def test_server_matches_sg_propagate():
     assert np.max(np.abs(el - el_ref)) < 1e-11
 
 
-# mixed: measured 3.8e-7 on GB300 (FP32 contractions through 50 steps of
+# mixed: measured 3.8e-7 on GB300 (FP32 products through 50 steps of
 # order-64 Chebyshev); the bound keeps a margin above ten
 @pytest.mark.parametrize("prec,tol", [("fp64", 1e-10), ("mixed", 5e-6)])
 def test_request_matches_exact_propagator_of_the_oracle(prec, tol):

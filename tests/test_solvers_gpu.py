@@ -171,16 +171,12 @@ def test_chebyshev_6d_coupled_matches_exact_propagator_at_steps_1_50_200():
 
 def test_benchmark_workload_20_lowest_by_mixed_davidson_then_fp64_refinement():
     """D=12 L=10, nb=l+1, nq=l+2 (the benchmark workload): the 20 lowest
-    eigenvalues by block Davidson (block 8) with FP32 contractions, then FP64
+    eigenvalues by block Davidson (block 8) with FP32 products, then FP64
     refinement, against the masked-Galerkin spectrum stored by
     tests/golden/make_c3_eigs.py.  Per-eigenvalue errors are printed.
 
-    The FP32 residual floor here is ~1e-3: low-lying eigenvectors sit on small
-    k, and the k = 0 entry sums contributions of every term with coefficients
-    |D_l| up to 462 (Eq. (8)) whose signed sum is 1, so the terms' FP32
-    rounding (~6e-8 relative each) adds up to ~5e-4 there.  The mixed run is
-    asked for that (tol 1e-3, eigenvalues to ~1e-3); FP64 refinement then
-    brings every eigenvalue within 1e-8."""
+    The mixed run is asked for starting vectors (tol 1e-3, eigenvalues to
+    ~1e-3); FP64 refinement then brings every eigenvalue within 1e-8."""
     import os
     ref = np.loadtxt(os.path.join(os.path.dirname(__file__), "golden", "c3_eigs.txt"))
     p = synth.workload_C3()

@@ -1,8 +1,8 @@
-"""sg_tune: measured choice of the fast path's slicing target.
+"""sg_tune: measured choice of the row kernels' plan.
 
 After tuning, the context must still compute H_S within the parity
 tolerances (FP64 1e-12 norm-wise and element-wise against the oracles, mixed
-as in tests/helpers.py), repeatably to the bit, and report which target it
+as in tests/helpers.py), repeatably to the bit, and report which plan it
 kept."""
 import numpy as np
 import pytest

@@ -4,9 +4,9 @@ Such a caller (one whose device memory is all held by another allocator, or a
 loop that cannot take a cudaMalloc's synchronisation) gets the same y = H_S x
 as sg_apply_H, with the scratch taken from a fixed array in the library.  Each
 case calls the no-alloc entry point twice in a row, with different inputs.  Both
-entry points run the same kernels and the same exact fixed-point sum, so the
-results must be bitwise equal: any stale accumulator word left by an
-incomplete clear of the shared scratch would show.
+entry points run the same kernels and sum every row in the same order, so the
+results must be bitwise equal: a stale part of the input copy or of the flags in
+the shared scratch would show.
 This file is collected last so that a run stopping at its first failure has
 run every other test before it.
 """

@@ -1,8 +1,8 @@
-"""Batched apply with a large member: a problem with enough block-form terms
-to fill the GPU by itself runs as its own launches inside the batch's launch
-sequence (its parameters in the kernel's parameter bank), beside the packed
-launches of the small problems.  Results stay bitwise those of each problem's
-own context.  (A file of its own, run last: it holds the D=12 L=10 tables.)
+"""Batched apply with a large member: a problem with enough rows to fill the GPU
+by itself runs as its own launches inside the batch's launch sequence (its
+parameters in the kernel's parameter bank), beside the packed launches of the
+small problems.  Results stay bitwise those of each problem's own context.  (A
+file of its own, run last: it holds the D=12 L=10 operator.)
 """
 import pytest
 
