@@ -206,7 +206,7 @@ def bench_config(args, world: int) -> dict:
     """The `config` of the JSON line; the same for both arms."""
     par = f"terms sharded x{world}" if getattr(args, "sharding", "replicas") == "terms" and world > 1 \
         else f"replicas x{world}"
-    return {"workload": workload_name(args.L), "precision": "mixed (FP32 contractions, FP64 accumulation)",
+    return {"workload": workload_name(args.L), "precision": "mixed (FP32 products, sums in FP32 pairs, FP64 diagonal)",
             "vectors_per_step": args.nvec, "parallelism": par,
             "l2": "flushed between timed steps (256 MB write)"}
 
@@ -708,7 +708,7 @@ def main():
                           "plan": f.get("plan")}
                          if f else None),
                 "df64": ({"value": d["value"], "unit": UNIT, "ms_per_step": d["ms_per_step"], "steps": d["steps"],
-                          "precision": "double-float contractions (pairs of FP32, ~48 bits), FP64 accumulation",
+                          "precision": "double-float (pairs of FP32, ~48 bits), FP64 diagonal",
                           "latency_ms": d["latency_ms"], "roofline": d["roofline"], "clocks": d["clocks"],
                           "plan": d.get("plan")}
                          if d else None),

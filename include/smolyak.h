@@ -119,8 +119,9 @@ typedef struct {
  * Setup runs on the host plus synchronous uploads on the current device.
  * The context keeps on the device the row operator (per element a 4-byte
  * column and a value of 4 bytes for SG_MIXED, 8 for SG_FP64 and SG_DF64, rows
- * filled up to multiples of four elements; 16 bytes per row beside them), the
- * term levels and the 1D tables.  sg_size reports the total.
+ * filled up to multiples of four elements; 8 bytes per row beside them), the
+ * harmonic energies, the ranking tables and the 1D tables; term by term, these
+ * tables with the terms' levels and coefficients.  sg_size reports the total.
  * Limits of this build (SG_EUNSUPPORTED): nb(L), nq(L) <= 32, N_cs < 2^31,
  * at most 256 monomials with at most 8 factors each, powers <= 16.
  */
@@ -460,7 +461,10 @@ sg_status sg_device_error(sg_ctx *ctx, int *code);
  *           energies and one random vector, and carries `block` Ritz pairs
  *           beyond nev; after convergence it makes one more expansion, by the
  *           residuals of the pairs beyond nev, so that no state is missed that
- *           the start block does not couple to.  SG_LANCZOS: block Krylov with full reorthogonalisation and
+ *           the start block does not couple to.  Only pairs above tol are given
+ *           new directions: one that has met it is not polished further, and
+ *           its vector is off by about tol over the gap to the next state.
+ *           SG_LANCZOS: block Krylov with full reorthogonalisation and
  *           Rayleigh-Ritz, at most 320 basis vectors; a block of size >= the
  *           largest multiplicity resolves degenerate eigenvalues.
  *   block   1..8 vectors per operator application (<= 0: min(nev, 8)).
@@ -470,7 +474,7 @@ sg_status sg_device_error(sg_ctx *ctx, int *code);
  *   evecs   DEVICE, nev * N_cs (out; may be NULL).
  * Synchronous.  SG_ENOCONV when fewer than nev pairs converged (evals, resid and
  * evecs then hold the current approximations).  Allocates its workspace
- * (device memory of about 2 * max(3 nev, nev + 6 block) + 3 (nev + block)
+ * (device memory of about 2 * max(3 nev, nev + 6 block) + 3 nev + 4 block
  * vectors for Davidson).
  * With a SG_MIXED context the applications are FP32-accurate; use
  * sg_eigs_refine with a SG_FP64 context of the same problem to refine.

@@ -269,7 +269,7 @@ namespace sg {
 constexpr int64_t kDirectElems = 65536;
 // The last block settles the vectors up to this many windows, a launch beyond
 // (403 windows 9.4 us by the block and 11.8 by a launch, 684 11.1 and 13.8,
-// 1,969 22.5 and 20.0, 10,104 86.3 and 81.5: the blocks meet at the counter).
+// about 2,000 22.5 and 20.0, 10,104 86.3 and 81.5: the blocks meet at the counter).
 constexpr int kTicketBlocks = 1024;
 
 cudaError_t apply_rows(sg_ctx *ctx, RowIO io, cudaStream_t s)

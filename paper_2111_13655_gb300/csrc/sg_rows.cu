@@ -19,11 +19,11 @@
 // that of its products and groups, 6.1 * 2^-24 of the sum of its terms' sizes
 // however long it is; double-float as df_fma.
 //
-// What bounds the row kernel (D=12 L=9, 8 vectors): FP64 its pipe, 83% busy;
-// mixed and double-float the latency of the gathers, with 34% and 45% of the
+// What bounds the row kernel (D=12 L=9, 8 vectors): FP64 its pipe, 81% busy;
+// mixed and double-float the latency of the gathers, with 33% and 44% of the
 // issue slots and a quarter of the DRAM bandwidth used.  Against the kernel
 // that took every term through its grid: D=12 L=10 mixed 26.5 ms -> 80.6 us,
-// D=12 L=9 FP64 39.9 ms -> 90.4 us, D=12 L=8 double-float 4.36 ms -> 33.5 us.
+// D=12 L=9 FP64 39.9 ms -> 90.5 us, D=12 L=8 double-float 4.36 ms -> 28.8 us.
 #include <algorithm>
 #include <cstring>
 

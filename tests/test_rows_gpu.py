@@ -26,7 +26,7 @@ pytestmark = pytest.mark.gpu
 
 # N_cs 924: 17 vectors gathered directly, few windows.  12,870: 5 vectors
 # gathered directly, 7 from the copy, the last block settles.  125,970: the copy
-# and 1,969 windows, settled by a launch.
+# and about 2,000 windows, settled by a launch.
 SIZES = {"D=6 L=6": synth.workload_C3(L=6, D=6), "D=8 L=8": synth.workload_C3(L=8, D=8),
          "D=12 L=8": synth.workload_C3(L=8)}
 
