@@ -198,15 +198,16 @@ sg_status sg_apply_H_host(sg_ctx *ctx, const double *x_host, double *y_host, int
  * sg_apply_H_finish -- y = H_S x from the summed accumulators of all parts
  *   (and the harmonic part applied in the compact basis); clears acc to zero.
  *   x, y as for sg_apply_H (x the same vectors the parts were given).
- * sg_part_size -- the terms at the processing positions of a part and their
- *   summed cost estimate (host; also on contexts made by sg_plan): the balance
- *   of the term-by-term split.  Any output may be NULL.
+ * sg_part_size -- what a part takes (host; also on contexts made by sg_plan).
+ *   In the row form: its rows and the elements it reads (of a plan, whose
+ *   windows are not cut yet, whole windows and the mean length of a row); term
+ *   by term: its terms and their summed cost estimate.  Any output may be NULL.
  * Both device calls are enqueued on `stream`.
  */
 sg_status sg_apply_H_part(sg_ctx *ctx, const double *x, int nvec, int part, int nparts, int64_t *acc,
                           void *stream);
 sg_status sg_apply_H_finish(sg_ctx *ctx, const double *x, int64_t *acc, double *y, int nvec, void *stream);
-sg_status sg_part_size(const sg_ctx *ctx, int part, int nparts, int64_t *n_terms, int64_t *cost);
+sg_status sg_part_size(const sg_ctx *ctx, int part, int nparts, int64_t *n_items, int64_t *cost);
 
 /*
  * sg_apply_H_noalloc -- the operation of sg_apply_H, with the same arguments

@@ -302,7 +302,7 @@ def sg_apply_H_finish(ctx: Ctx, x, acc, y, nvec: int, stream=None) -> None:
 
 
 def sg_part_size(ctx: Ctx, part: int, nparts: int):
-    """(terms, summed cost estimate) of one part of a term-sharded apply (host)."""
+    """(rows, elements) of one part of a sharded apply; (terms, summed cost estimate) term by term (host)."""
     a, b = ctypes.c_int64(), ctypes.c_int64()
     _check(lib().sg_part_size(ctx.ptr, int(part), int(nparts), ctypes.byref(a), ctypes.byref(b)), ctx)
     return a.value, b.value

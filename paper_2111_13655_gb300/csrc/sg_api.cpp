@@ -352,7 +352,11 @@ cudaError_t build_rows(sg_ctx *ctx)
             ctx->row_allocs.push_back(own);
             ctx->rop = R;
             ctx->win_entries.resize(W.wins.size());
-            for (size_t w = 0; w < W.wins.size(); w++) ctx->win_entries[w] = W.wins[w].nent;
+            ctx->win_rows.resize(W.wins.size());
+            for (size_t w = 0; w < W.wins.size(); w++) {
+                ctx->win_entries[w] = W.wins[w].nent;
+                ctx->win_rows[w] = W.wins[w].nrows;
+            }
             ctx->row_bytes = (int64_t)(rec + W.bytes);
             ctx->bytes_device += ctx->row_bytes;
         }
@@ -530,16 +534,27 @@ sg_status sg_apply_H_finish(sg_ctx *ctx, const double *x, int64_t *acc, double *
     return SG_OK;
 }
 
-sg_status sg_part_size(const sg_ctx *ctx, int part, int nparts, int64_t *n_terms, int64_t *cost)
+sg_status sg_part_size(const sg_ctx *ctx, int part, int nparts, int64_t *n_items, int64_t *cost)
 {
     if (!ctx || nparts < 1 || part < 0 || part >= nparts) return SG_EINVAL;
     const sg::HostTables &T = ctx->host;
     int64_t c = 0, k = 0;
-    for (int64_t p = part; p < T.n_terms; p += nparts) {
-        c += T.pcost[(size_t)p];
-        k++;
+    if (T.rows && ctx->has_device) {
+        for (size_t w = part; w < ctx->win_entries.size(); w += nparts) {
+            c += ctx->win_entries[w];
+            k += ctx->win_rows[w];
+        }
+    } else if (T.rows) {  // not cut yet: whole windows, their rows of the mean length
+        const int64_t rows = sg::row_window_rows(T.n_cs, sg::row_window_units(T));
+        for (int64_t r = part * rows; r < T.n_cs; r += nparts * rows) k += std::min(rows, T.n_cs - r);
+        c = (int64_t)((double)T.row_nnz * k / T.n_cs);
+    } else {
+        for (int64_t p = part; p < T.n_terms; p += nparts) {
+            c += T.pcost[(size_t)p];
+            k++;
+        }
     }
-    if (n_terms) *n_terms = k;
+    if (n_items) *n_items = k;
     if (cost) *cost = c;
     return SG_OK;
 }

@@ -358,7 +358,7 @@ struct sg_ctx {
     // row operator: its buffers, and the plan's vectors per lane
     sg::RowOp rop{};
     std::vector<void *> row_allocs;
-    std::vector<int> win_entries;  // entries of each window
+    std::vector<int> win_entries, win_rows;  // entries and rows of each window
     int64_t row_bytes = 0;
     // apply workspace.  Row form: per-vector flags and the entry-major input
     // copy; term-by-term kernel: fixed-point accumulators and scale exponents

@@ -1,6 +1,6 @@
 """The parts of a sharded apply in the row form (host code on a stand-in device):
-every row belongs to one part, whatever the number of parts, and the parts hold
-about the same number of entries."""
+every row belongs to one part, whatever the number of parts, the parts hold
+about the same number of entries, and sg_part_size says how many."""
 import numpy as np
 import pytest
 
@@ -27,11 +27,14 @@ def test_parts_cover_every_row_once_and_balance_the_entries(fake, p, spread, pre
         x = np.ones((nvec, ctx.n_cs))
         words = sg.acc_words(ctx, nvec) // (ctx.n_cs * nvec)
         for nparts in (1, 2, 3, 8):
-            acc, entries = np.zeros((ctx.n_cs, nvec, words), np.int64), []
+            acc, entries, counted = np.zeros((ctx.n_cs, nvec, words), np.int64), [], []
             for part in range(nparts):
                 before = fake.fake_entries()
                 assert fake.sg_apply_H_part(ctx.ptr, x.ctypes.data, nvec, part, nparts, acc.ctypes.data, None) == sg.SG_OK
                 entries.append(fake.fake_entries() - before)
+                rows = int((acc[:, 0, 0] == 1).sum()) - sum(counted)
+                assert sg.sg_part_size(ctx, part, nparts) == (rows, entries[-1])
+                counted.append(rows)
             assert (acc[:, :, 0] == 1).all() and not acc[:, :, 1:].any(), nparts
             if spread:
                 assert max(entries) <= spread * np.mean(entries), (nparts, entries)

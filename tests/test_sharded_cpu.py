@@ -1,6 +1,6 @@
-"""Host side of the sharded apply, no GPU: the partition of the term list over
-parts (problems applied term by term; the row form's windows: test_row_parts.py),
-and the integer reduction of the parts' accumulators over two
+"""Host side of the sharded apply, no GPU: the partition of the rows, or of the
+terms of a problem applied term by term, over parts (of created contexts:
+test_row_parts.py), and the integer reduction of the parts' accumulators over two
 gloo ranks (the collective a multi-GPU apply uses between its parts)."""
 import os
 import socket
@@ -19,8 +19,21 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.mark.parametrize("nparts", [1, 2, 3, 8])
+def test_parts_cover_every_row_once_and_balance_the_elements(nparts):
+    from bench import row_entries
+    p = synth.workload_C3(L=16, D=6)
+    with sg.sg_plan(p, "mixed") as ctx:
+        sizes = [sg.sg_part_size(ctx, r, nparts) for r in range(nparts)]
+    assert sum(n for n, _ in sizes) == ctx.n_cs != ctx.n_terms
+    costs = np.array([c for _, c in sizes], float)
+    assert abs(costs.sum() / row_entries(6, 16) - 1.0) < 1e-3
+    assert costs.max() / costs.mean() < 1.02      # every nparts-th window of 64 rows
+
+
+@pytest.mark.parametrize("nparts", [1, 2, 3, 8])
 def test_parts_cover_every_term_once_and_balance_the_cost(nparts):
-    p = synth.workload_C3(L=8)
+    """L > 63: applied term by term."""
+    p = synth.polynomial_problem(3, 64, [1.0] * 3, [(0.2, [(0, 2), (1, 1)])], nb_rule=(3, 0), nq_rule=(4, 0))
     with sg.sg_plan(p, "mixed") as ctx:
         sizes = [sg.sg_part_size(ctx, r, nparts) for r in range(nparts)]
     assert sum(n for n, _ in sizes) == ctx.n_terms
