@@ -141,7 +141,7 @@ sg_status sg_plan(int D, int L, const sg_basis *basis, const sg_grid *grids,
 /* Sizes: n_cs = N_cs (compact basis), n_terms = N_st, n_s = N_s (sum of term
  * basis sizes, Sec. 2, Eq. (11)), n_grid = sum of term grid sizes, bytes_device =
  * device memory held by the context (for a context made by sg_plan: what
- * sg_create would hold for the same problem, from above and within some 20%:
+ * sg_create would hold for the same problem, from above and within some 25%:
  * rows are filled up to multiples of four elements, which a plan counts at its
  * most; without the apply workspace, which grows with the block size).  Any
  * pointer may be NULL. */
